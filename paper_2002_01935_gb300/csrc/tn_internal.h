@@ -29,8 +29,10 @@ struct Control {
     int64_t acc_exp[2];   // double-buffered exponent of the FP64 accumulator
     int64_t final_exp;    // exponent of the result after the last slice
     int32_t status;       // 0 ok; TN_ETIMEOUT etc. set by device code
-    int32_t pad;
+    uint32_t ticket;      // blocks of the running fold that are done
     int64_t slice_end;    // instances whose slice id reaches this are idle
+    double* out;          // direct folds: the call's output and its exponent
+    int64_t* out_exp;
 };
 
 // Instances: one launch runs n_inst copies of a node.  Instance i reads
@@ -291,9 +293,38 @@ struct AccumArgs {
     const int64_t* exp_r;
     double* acc;
     Control* ctl;
-    int32_t advance;  // one-block launches: slices to advance ctl->slice by (set by the launcher)
-    int32_t pad3;
+    int32_t advance;  // slices to advance ctl->slice by (set by the launcher)
+    int32_t direct;   // the call's last group writes ctl->out, the first does not read acc
 };
+
+// Adds an output digit (fastest first) to the fold's order, merged with the
+// previous one where the two are one digit of the root as well.
+inline void push_fold_digit(AccumArgs& a, int64_t dim, int64_t stride) {
+    if (dim == 1) return;
+    if (a.n_od > 0 && a.od_s[a.n_od - 1] * a.od_dim[a.n_od - 1] == stride &&
+        a.od_dim[a.n_od - 1] * dim < (int64_t(1) << 31)) {
+        a.od_dim[a.n_od - 1] *= (int32_t)dim;
+        return;
+    }
+    a.od_dim[a.n_od] = (int32_t)dim;
+    a.od_s[a.n_od] = stride;
+    ++a.n_od;
+}
+
+// Tile plan of a fold whose outputs are in another order than the root
+// (computed on the host): 2^t entries per tile, enumerated in root order by
+// src_add and in output order by dst_add, idx_add being the place in root
+// order; the u other bits step between tiles.
+constexpr int kFoldTile = 1024;
+struct FoldPlan {
+    int t, u;
+    int64_t src_add[10], dst_add[10];
+    int32_t idx_add[10];
+    int64_t rest_src[kMaxBits], rest_dst[kMaxBits];
+};
+
+// Floats of a leaf that one block of a leaf-maximum launch covers.
+constexpr int64_t kLeafPart = 16384;
 
 // Reverse sweep: add a leaf's adjoint (times 2^exp) into its gradient
 // accumulator at the slice offset; labels absent from the adjoint
@@ -392,18 +423,16 @@ cudaError_t launch_wave(const WaveItem* items, int n_items, const TileArgs* desc
                         const void* const* leaf_ptrs, bool is_c, cudaStream_t s,
                         const int4* deps = nullptr, unsigned* done = nullptr, unsigned* head = nullptr,
                         int G = 1, bool tiles = false);
-// Folds the slice group's roots into the FP64 accumulator, leaves the
-// result's exponent after the last group, and advances the slice counter by
-// `advance` (in the same launch when it is one block).
+// Folds the slice group's roots into the FP64 accumulator (direct: the last
+// group into the call's output), leaves the result's exponent after the last
+// group, and advances the slice counter by `advance`.
 cudaError_t launch_accumulate(const AccumArgs& a, bool is_c, cudaStream_t s, int advance);
-// Leaf maxima (as launch_leaf_max) and the call's control block and
-// accumulator (as launch_begin_call) in one launch after one memset.
+// Leaf maxima (as launch_leaf_max) and the call's control block (with the
+// output pointers that a direct fold writes), and n_acc doubles of the
+// accumulator cleared, in one launch.
 cudaError_t launch_call_begin(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
                               int64_t max_nfloat, Control* ctl, int64_t slice_begin, int64_t slice_end,
-                              double* acc, int64_t n_acc, cudaStream_t s);
-// Copies the accumulator (n doubles) and the final exponent to out / out_exp.
-cudaError_t launch_result(const double* acc, int64_t n, const Control* ctl, double* out, int64_t* out_exp,
-                          cudaStream_t s);
+                              double* acc, int64_t n_acc, double* result, int64_t* result_exp, cudaStream_t s);
 cudaError_t launch_begin_call(Control* ctl, int64_t slice_begin, int64_t slice_end, double* acc,
                               int64_t n_acc_doubles, cudaStream_t s);
 cudaError_t launch_begin_slice(unsigned* maxabs, int n_nodes, cudaStream_t s);

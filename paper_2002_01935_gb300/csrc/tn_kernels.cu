@@ -14,6 +14,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <cstring>
+#include <type_traits>
+
 #include "tn_internal.h"
 
 namespace tn {
@@ -168,94 +172,360 @@ cudaError_t launch_generic(const GenericArgs& a, bool is_c, cudaStream_t s) {
 // FP64 cross-slice accumulation (Sec. 4.7.1) with exponent alignment
 // --------------------------------------------------------------------------
 
-template <bool CPLX>
-__global__ void __launch_bounds__(256) k_accumulate(const __grid_constant__ AccumArgs a) {
-    // the n_inst roots of this launch are slices ctl->slice + i (i in order);
-    // fold them with one common exponent, skipping zero and idle slices
-    const int ni = a.n_inst > 1 ? a.n_inst : 1;
-    const int64_t step = (a.ctl->slice - a.ctl->slice_begin) / ni;
-    const int par = (int)(step & 1);
-    const int64_t accE = a.ctl->acc_exp[par];
+// Common part of the folds: the roots of one launch are slices ctl->slice + i
+// (i < n, in order; zero roots and idle slices are skipped) and are folded
+// with one common exponent.  The call's first group starts from zero instead
+// of reading the accumulator, and (direct folds) its last group writes the
+// caller's output instead of the accumulator: a call of one group, which is
+// every unsliced one, moves each output once.
+struct FoldState {
+    int64_t slice, slice_end, newE;
+    double fa;         // factor of the accumulator
+    int n;             // instances of this group
+    int par;
+    bool any, first, last;
+    const double* src;  // accumulator to read, nullptr: zero
+    double* dst;
+    bool idle;          // nothing to write: all roots zero, accumulator stays
+    bool vec;           // dst is 16-byte aligned
+};
+
+__device__ __forceinline__ FoldState fold_state(const AccumArgs& a) {
+    FoldState f;
+    const Control* ctl = a.ctl;
+    f.slice = ctl->slice;
+    f.slice_end = ctl->slice_end;
+    const int64_t begin = ctl->slice_begin;
+    f.n = a.n_inst > 1 ? a.n_inst : 1;
+    f.par = (int)(((f.slice - begin) / f.n) & 1);
+    f.first = a.direct && f.slice == begin;
+    f.last = f.slice + f.n >= f.slice_end;
+    const int64_t accE = ctl->acc_exp[f.par];
     const bool empty = accE == INT64_MIN;
-    int64_t newE = accE;
-    bool any = false;
-    for (int i = 0; i < ni; ++i) {
-        if (a.ctl->slice + i >= a.ctl->slice_end) break;
+    f.newE = accE;
+    f.any = false;
+    for (int i = 0; i < f.n; ++i) {
+        if (f.slice + i >= f.slice_end) break;
         const float rmax = __uint_as_float(a.max_r[(int64_t)i * a.s_is]);
-        if (!(rmax > 0.f)) continue;
         const int64_t S = a.exp_r[(int64_t)i * a.s_is];
-        newE = (empty && !any) ? S : (S > newE ? S : newE);
-        any = true;
+        if (!(rmax > 0.f)) continue;
+        f.newE = (empty && !f.any) ? S : (S > f.newE ? S : f.newE);
+        f.any = true;
     }
-    double fa = 1.0;
-    if (any && !empty) {
-        const int64_t da = accE - newE;
-        fa = ldexp(1.0, (int)(da < -2000 ? -2000 : da));
+    f.fa = 1.0;
+    if (f.any && !empty) {
+        const int64_t da = accE - f.newE;
+        f.fa = ldexp(1.0, (int)(da < -2000 ? -2000 : da));
     }
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < a.n_out; o += stride) {
-        if (!any) continue;
-        int64_t src = 0, rem = o;
-        for (int i = 0; i < a.n_od; ++i) {
-            const int64_t d = a.od_dim[i];
-            if ((d & (d - 1)) == 0) {  // power of two: mask and shift
-                src += (rem & (d - 1)) * a.od_s[i];
-                rem >>= __ffsll(d) - 1;
-            } else {
-                src += (rem % d) * a.od_s[i];
-                rem /= d;
-            }
-        }
-        double vr = 0.0, vi = 0.0;
-        if (CPLX) {
-            const double2 v = reinterpret_cast<double2*>(a.acc)[o];
-            vr = v.x * fa;
-            vi = v.y * fa;
-        } else {
-            vr = a.acc[o] * fa;
-        }
-        for (int i = 0; i < ni; ++i) {
-            if (a.ctl->slice + i >= a.ctl->slice_end) break;
-            const float rmax = __uint_as_float(a.max_r[(int64_t)i * a.s_is]);
-            if (!(rmax > 0.f)) continue;
-            const int64_t dr = a.exp_r[(int64_t)i * a.s_is] - newE;
-            const double fr = ldexp(1.0, (int)(dr < -2000 ? -2000 : dr));
-            const int64_t at = src + (int64_t)i * a.r_is;
-            if (CPLX) {
-                const float2 r = reinterpret_cast<const float2*>(a.R)[at];
-                vr += (double)r.x * fr;
-                vi += (double)r.y * fr;
-            } else {
-                vr += (double)reinterpret_cast<const float*>(a.R)[at] * fr;
-            }
-        }
-        if (CPLX)
-            reinterpret_cast<double2*>(a.acc)[o] = make_double2(vr, vi);
-        else
-            a.acc[o] = vr;
-    }
-    if (gridDim.x == 1 && a.advance) __syncthreads();  // every thread has read ctl->slice
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.ctl->acc_exp[par ^ 1] = newE;
-        // the last group of the call leaves the result's exponent
-        if (a.ctl->slice + ni >= a.ctl->slice_end) a.ctl->final_exp = newE == INT64_MIN ? 0 : newE;
-        if (gridDim.x == 1 && a.advance) a.ctl->slice += a.advance;
+    f.src = f.first ? nullptr : a.acc;
+    const bool out = a.direct && f.last;
+    f.dst = out ? ctl->out : a.acc;
+    f.idle = !f.any && !f.first && !out;
+    f.vec = (reinterpret_cast<uintptr_t>(f.dst) & 15) == 0;
+    return f;
+}
+
+// Root factor of instance i; 0 and false for a zero or idle one.
+__device__ __forceinline__ bool fold_factor(const AccumArgs& a, const FoldState& f, int i, double& fr) {
+    if (f.slice + i >= f.slice_end) return false;
+    const float rmax = __uint_as_float(a.max_r[(int64_t)i * a.s_is]);
+    if (!(rmax > 0.f)) return false;
+    const int64_t dr = a.exp_r[(int64_t)i * a.s_is] - f.newE;
+    fr = ldexp(1.0, (int)(dr < -2000 ? -2000 : dr));
+    return true;
+}
+
+template <bool CPLX>
+__device__ __forceinline__ double2 fold_start(const FoldState& f, int64_t o) {
+    if (!f.src) return make_double2(0.0, 0.0);
+    if constexpr (CPLX) {
+        const double2 v = reinterpret_cast<const double2*>(f.src)[o];
+        return make_double2(v.x * f.fa, v.y * f.fa);
+    } else {
+        return make_double2(f.src[o] * f.fa, 0.0);
     }
 }
 
+template <bool CPLX>
+__device__ __forceinline__ void fold_add(double2& v, const void* R, int64_t at, double fr) {
+    if constexpr (CPLX) {
+        const float2 r = __ldcs(reinterpret_cast<const float2*>(R) + at);
+        v.x += (double)r.x * fr;
+        v.y += (double)r.y * fr;
+    } else {
+        v.x += (double)__ldcs(reinterpret_cast<const float*>(R) + at) * fr;
+    }
+}
+
+template <bool CPLX>
+__device__ __forceinline__ void fold_store(const FoldState& f, int64_t o, double2 v) {
+    if constexpr (CPLX) {
+        if (f.vec) {
+            reinterpret_cast<double2*>(f.dst)[o] = v;
+        } else {  // a caller's buffer that only has the alignment of a double
+            f.dst[2 * o] = v.x;
+            f.dst[2 * o + 1] = v.y;
+        }
+    } else {
+        f.dst[o] = v.x;
+    }
+}
+
+// After the data: the accumulator's exponent, after the call's last group
+// the result's, and the slice counter.  Run by the last block to get here
+// (each block's reads of the control block come before its ticket), so that
+// no launch of its own is needed for them.
+__device__ __forceinline__ void fold_finish(const AccumArgs& a, const FoldState& f) {
+    __shared__ unsigned ticket;
+    if (gridDim.x > 1) {
+        __syncthreads();
+        if (threadIdx.x == 0) ticket = atomicInc(&a.ctl->ticket, gridDim.x - 1);  // wraps to 0 at the last block
+        __syncthreads();
+        if (ticket != gridDim.x - 1) return;
+    } else {
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        a.ctl->acc_exp[f.par ^ 1] = f.newE;
+        if (f.last) {
+            const int64_t e = f.newE == INT64_MIN ? 0 : f.newE;
+            a.ctl->final_exp = e;
+            if (a.direct) *a.ctl->out_exp = e;
+        }
+        a.ctl->slice = f.slice + a.advance;
+    }
+}
+
+// Root offset of output o: digits fastest first, shifts where a size is a
+// power of two, 32-bit division otherwise (outputs beyond 2^31 entries: 64).
+__device__ __forceinline__ int64_t fold_offset(const AccumArgs& a, int64_t o) {
+    int64_t src = 0;
+    if (a.n_out >= (int64_t(1) << 31)) {
+        for (int i = 0; i < a.n_od; ++i) {
+            const int64_t d = a.od_dim[i];
+            src += (o % d) * a.od_s[i];
+            o /= d;
+        }
+        return src;
+    }
+    unsigned rem = (unsigned)o;
+    for (int i = 0; i < a.n_od; ++i) {
+        const unsigned d = (unsigned)a.od_dim[i];
+        if ((d & (d - 1)) == 0) {
+            src += (int64_t)(rem & (d - 1)) * a.od_s[i];
+            rem >>= __ffs(d) - 1;
+        } else {
+            const unsigned q = rem / d;
+            src += (int64_t)(rem - q * d) * a.od_s[i];
+            rem = q;
+        }
+    }
+    return src;
+}
+
+// One thread per output; consecutive threads write consecutive outputs.
+// Bound by memory when the outputs follow the root's order (the digits are
+// merged on the host: one digit then), by latency for the few outputs of a
+// network with few or no open labels.
+template <bool CPLX>
+__global__ void __launch_bounds__(256) k_accumulate(const __grid_constant__ AccumArgs a) {
+    const FoldState f = fold_state(a);
+    constexpr int R = 4;  // outputs in flight per thread
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    if (!f.idle) {
+        for (int64_t o0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o0 < a.n_out; o0 += R * stride) {
+            double2 v[R];
+            int64_t src[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int64_t o = o0 + r * stride;
+                if (o >= a.n_out) break;
+                src[r] = fold_offset(a, o);
+                v[r] = fold_start<CPLX>(f, o);
+            }
+            for (int i = 0; i < f.n; ++i) {
+                double fr;
+                if (f.slice + i >= f.slice_end) break;
+                if (!fold_factor(a, f, i, fr)) continue;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (o0 + r * stride < a.n_out) fold_add<CPLX>(v[r], a.R, src[r] + (int64_t)i * a.r_is, fr);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (o0 + r * stride < a.n_out) fold_store<CPLX>(f, o0 + r * stride, v[r]);
+        }
+    }
+    fold_finish(a, f);
+}
+
+// Outputs in another order than the root's (power-of-two sizes): tiles of up
+// to 2^10 entries holding the lowest five index bits of either order, read
+// in root order and written in output order through shared memory, so that
+// both sides move whole 128-byte lines.  Bound by memory: 12 bytes read and
+// written per real output, 24 per complex one.  A call whose 2^13 x 2^12
+// complex root is transposed: 2146 us with one thread per output and a digit
+// loop, a cleared and re-read accumulator and a copy to the caller (947, 75
+// and 255 us of it), 1191 us with this fold, which writes the output itself.
+template <bool CPLX>
+__global__ void __launch_bounds__(256) k_accumulate_perm(const __grid_constant__ AccumArgs a,
+                                                         const __grid_constant__ FoldPlan p) {
+    using T = typename std::conditional<CPLX, float2, float>::type;
+    __shared__ T stage[kFoldTile + kFoldTile / 32];
+    __shared__ int64_t tsrc[kFoldTile], tdst[kFoldTile];
+    __shared__ uint16_t tidx[kFoldTile];
+    const FoldState f = fold_state(a);
+    if (!f.idle) {
+        const int tsz = 1 << p.t;
+        for (int i = threadIdx.x; i < tsz; i += blockDim.x) {
+            int64_t so = 0, dd = 0;
+            int idx = 0;
+            for (int j = 0; j < p.t; ++j)
+                if ((i >> j) & 1) {
+                    so += p.src_add[j];
+                    dd += p.dst_add[j];
+                    idx += p.idx_add[j];
+                }
+            tsrc[i] = so;                            // i counts the tile in root order
+            tdst[i] = dd;                            // ... and in output order
+            tidx[i] = (uint16_t)(idx + (idx >> 5));  // its place in the stage
+        }
+        __syncthreads();
+        constexpr int R = kFoldTile / 256;
+        const int64_t n_tiles = int64_t(1) << p.u;
+        for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            int64_t sb = 0, db = 0;
+            for (int j = 0; j < p.u; ++j)
+                if ((tile >> j) & 1) {
+                    sb += p.rest_src[j];
+                    db += p.rest_dst[j];
+                }
+            double2 v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = threadIdx.x + r * 256;
+                if (i < tsz) v[r] = fold_start<CPLX>(f, db + tdst[i]);
+            }
+            for (int q = 0; q < f.n; ++q) {
+                double fr;
+                if (f.slice + q >= f.slice_end) break;
+                if (!fold_factor(a, f, q, fr)) continue;
+                const T* root = reinterpret_cast<const T*>(a.R) + (int64_t)q * a.r_is + sb;
+                T ld[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = threadIdx.x + r * 256;
+                    if (i < tsz) ld[r] = __ldcs(root + tsrc[i]);
+                }
+                __syncthreads();  // the stage's previous entries have been read
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = threadIdx.x + r * 256;
+                    if (i < tsz) stage[i + (i >> 5)] = ld[r];
+                }
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = threadIdx.x + r * 256;
+                    if (i < tsz) {
+                        const T x = stage[tidx[i]];
+                        if constexpr (CPLX) {
+                            v[r].x += (double)x.x * fr;
+                            v[r].y += (double)x.y * fr;
+                        } else {
+                            v[r].x += (double)x * fr;
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = threadIdx.x + r * 256;
+                if (i < tsz) fold_store<CPLX>(f, db + tdst[i], v[r]);
+            }
+        }
+    }
+    fold_finish(a, f);
+}
+
+// Tile plan of the permuted fold; false where the plain fold serves as well:
+// few outputs, sizes other than powers of two, or outputs whose lowest 32
+// entries are contiguous in the root.
+static bool make_fold_plan(const AccumArgs& a, FoldPlan& p) {
+    if (a.n_out < kFoldTile) return false;
+    int64_t add[64];  // root stride of every output index bit
+    int n = 0;
+    for (int i = 0; i < a.n_od; ++i) {
+        const int64_t d = a.od_dim[i];
+        if (d & (d - 1)) return false;
+        for (int64_t b = 1; b < d; b <<= 1) {
+            if (n >= kMaxBits) return false;
+            add[n++] = a.od_s[i] * b;
+        }
+    }
+    bool contiguous = true;
+    for (int j = 0; j < 5; ++j) contiguous &= add[j] == (int64_t(1) << j);
+    if (contiguous) return false;
+    memset(&p, 0, sizeof(p));
+    bool in[64] = {};
+    for (int j = 0; j < 5; ++j) in[j] = true;
+    int cnt = 5;
+    int by_src[64];
+    for (int j = 0; j < n; ++j) by_src[j] = j;
+    std::sort(by_src, by_src + n, [&](int x, int y) { return add[x] < add[y]; });
+    for (int j = 0; j < 5; ++j)
+        if (!in[by_src[j]]) {
+            in[by_src[j]] = true;
+            ++cnt;
+        }
+    for (int j = 5; j < n && cnt < 10; ++j)
+        if (!in[j]) {
+            in[j] = true;
+            ++cnt;
+        }
+    int rank[64], r = 0;  // place of a tile bit in root order
+    for (int j = 0; j < n; ++j)
+        if (in[by_src[j]]) {
+            p.src_add[r] = add[by_src[j]];
+            rank[by_src[j]] = r++;
+        }
+    int t = 0;
+    for (int j = 0; j < n; ++j) {
+        if (in[j]) {
+            p.dst_add[t] = int64_t(1) << j;
+            p.idx_add[t] = 1 << rank[j];
+            ++t;
+        } else {
+            p.rest_src[p.u] = add[j];
+            p.rest_dst[p.u] = int64_t(1) << j;
+            ++p.u;
+        }
+    }
+    p.t = t;
+    return true;
+}
+
 cudaError_t launch_accumulate(const AccumArgs& a0, bool is_c, cudaStream_t s, int advance) {
-    int64_t blocks = (a0.n_out + 255) / 256;
+    AccumArgs a = a0;
+    a.advance = advance;
+    FoldPlan p;
+    if (make_fold_plan(a, p)) {
+        const int64_t tiles = a.n_out >> p.t;
+        const unsigned blocks = (unsigned)(tiles < sm_count() * 6 ? tiles : sm_count() * 6);
+        if (is_c)
+            k_accumulate_perm<true><<<blocks, 256, 0, s>>>(a, p);
+        else
+            k_accumulate_perm<false><<<blocks, 256, 0, s>>>(a, p);
+        return cudaGetLastError();
+    }
+    int64_t blocks = (a.n_out + 255) / 256;
     if (blocks > sm_count() * 8) blocks = sm_count() * 8;
     if (blocks < 1) blocks = 1;
-    AccumArgs a = a0;
-    a.advance = blocks == 1 ? advance : 0;  // one block advances the slice counter itself
     if (is_c)
         k_accumulate<true><<<(unsigned)blocks, 256, 0, s>>>(a);
     else
         k_accumulate<false><<<(unsigned)blocks, 256, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && blocks > 1 && advance) e = launch_advance(a.ctl, s, advance);
-    return e;
+    return cudaGetLastError();
 }
 
 __global__ void k_begin_call(Control* ctl, int64_t slice_begin, int64_t slice_end, double* acc,
@@ -268,6 +538,7 @@ __global__ void k_begin_call(Control* ctl, int64_t slice_begin, int64_t slice_en
         ctl->acc_exp[0] = INT64_MIN;
         ctl->acc_exp[1] = INT64_MIN;
         ctl->status = 0;
+        ctl->ticket = 0;
     }
     for (; i < n; i += (int64_t)gridDim.x * blockDim.x) acc[i] = 0.0;
 }
@@ -293,22 +564,35 @@ cudaError_t launch_advance(Control* ctl, cudaStream_t s, int step) {
 }
 
 // Largest |component| of every leaf, so that leaves are renormalised like
-// intermediates before their first contraction.  blockIdx.x: leaf,
-// blockIdx.y: one of gridDim.y interleaved parts of it.
+// intermediates before their first contraction.
 // Part blockIdx.y of leaf blockIdx.x: the largest |component| over its
 // entries, combined over the parts by atomicMax on the float bits
 // (non-negative floats order like unsigned), or stored directly when one
 // block covers the leaf and `direct` allows it (no zeroing needed then).
+// Large leaves are read 16 bytes a load, four loads in flight per thread
+// (bound by memory); a leaf that is not 16-byte aligned, and the ends, by
+// single floats.
 __device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const int64_t* nfloat, unsigned* out,
                                               int n, bool direct) {
     const int v = blockIdx.x;
     if (v >= n) return;
     const float* p = ptrs[v];
     const int64_t m = nfloat[v];
-    const int64_t first = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-    if ((int64_t)blockIdx.y * blockDim.x >= m && blockIdx.y > 0) return;
+    const bool vec = (reinterpret_cast<uintptr_t>(p) & 15) == 0 && m >= 4096;
+    const int64_t m4 = vec ? m / 4 : 0;
+    const int64_t step = (int64_t)gridDim.y * blockDim.x, first = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
+    if (blockIdx.y > 0 && (int64_t)blockIdx.y * blockDim.x >= (vec ? m4 : m)) return;  // nothing left for this part
     float lmax = 0.f;
-    for (int64_t i = first; i < m; i += (int64_t)gridDim.y * blockDim.x) lmax = fmaxf(lmax, fabsf(p[i]));
+    const float4* p4 = reinterpret_cast<const float4*>(p);
+    for (int64_t i = first; i < m4; i += 4 * step) {
+        float4 x[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = i + r * step < m4 ? p4[i + r * step] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            lmax = fmaxf(lmax, fmaxf(fmaxf(fabsf(x[r].x), fabsf(x[r].y)), fmaxf(fabsf(x[r].z), fabsf(x[r].w))));
+    }
+    for (int64_t i = 4 * m4 + first; i < m; i += step) lmax = fmaxf(lmax, fabsf(p[i]));
     __shared__ float red[32];
     for (int o = 16; o > 0; o >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lmax;
@@ -326,16 +610,24 @@ __device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const in
     }
 }
 
+// Blocks per leaf of a leaf-maximum launch.
+static unsigned leaf_parts(int64_t max_nfloat) {
+    int64_t parts = (max_nfloat + kLeafPart - 1) / kLeafPart;
+    return (unsigned)(parts < 1 ? 1 : (parts > 1024 ? 1024 : parts));
+}
+
 __global__ void __launch_bounds__(256) k_leaf_max(const float* const* ptrs, const int64_t* nfloat,
                                                   unsigned* out, int n) {
     leaf_max_part(ptrs, nfloat, out, n, false);
 }
 
-// The start of a call: leaf maxima as k_leaf_max, and (block 0) the control
-// block and the FP64 accumulator as k_begin_call.
+// The start of a call: leaf maxima as k_leaf_max, (block 0) the control block
+// with the call's output pointers, and the FP64 accumulator cleared where the
+// fold reads it (n_acc > 0).
 __global__ void __launch_bounds__(256) k_call_begin(const float* const* ptrs, const int64_t* nfloat,
                                                     unsigned* out, int n, Control* ctl, int64_t slice_begin,
-                                                    int64_t slice_end, double* acc, int64_t n_acc) {
+                                                    int64_t slice_end, double* acc, int64_t n_acc,
+                                                    double* result, int64_t* result_exp) {
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         ctl->slice = slice_begin;
         ctl->slice_begin = slice_begin;
@@ -343,6 +635,9 @@ __global__ void __launch_bounds__(256) k_call_begin(const float* const* ptrs, co
         ctl->acc_exp[0] = INT64_MIN;
         ctl->acc_exp[1] = INT64_MIN;
         ctl->status = 0;
+        ctl->ticket = 0;
+        ctl->out = result;
+        ctl->out_exp = result_exp;
     }
     {
         const int64_t nblk = (int64_t)gridDim.x * gridDim.y, bid = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
@@ -353,32 +648,15 @@ __global__ void __launch_bounds__(256) k_call_begin(const float* const* ptrs, co
 
 cudaError_t launch_call_begin(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
                               int64_t max_nfloat, Control* ctl, int64_t slice_begin, int64_t slice_end,
-                              double* acc, int64_t n_acc, cudaStream_t s) {
-    int64_t parts = (max_nfloat + 32767) / 32768;
-    parts = parts < 1 ? 1 : (parts > 256 ? 256 : parts);
+                              double* acc, int64_t n_acc, double* result, int64_t* result_exp, cudaStream_t s) {
+    const unsigned parts = leaf_parts(max_nfloat);
     if (n > 0 && parts > 1) {  // several blocks per leaf combine by atomicMax from zero
         const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned) * (size_t)n, s);
         if (e != cudaSuccess) return e;
     }
     const unsigned gx = (unsigned)(n > 0 ? n : 1);
-    k_call_begin<<<dim3(gx, (unsigned)parts), 256, 0, s>>>(ptrs, nfloat, out, n, ctl, slice_begin, slice_end, acc,
-                                                          n_acc);
-    return cudaGetLastError();
-}
-
-// The call's result: the FP64 accumulator and the exponent, to the caller's
-// device buffers (or a staging buffer for one host copy: exp after acc).
-__global__ void k_result(const double* acc, int64_t n, const Control* ctl, double* out, int64_t* out_exp) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = acc[i];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *out_exp = ctl->final_exp;
-}
-
-cudaError_t launch_result(const double* acc, int64_t n, const Control* ctl, double* out, int64_t* out_exp,
-                          cudaStream_t s) {
-    int64_t blocks = (n + 255) / 256;
-    blocks = blocks < 1 ? 1 : (blocks > sm_count() * 4 ? sm_count() * 4 : blocks);
-    k_result<<<(unsigned)blocks, 256, 0, s>>>(acc, n, ctl, out, out_exp);
+    k_call_begin<<<dim3(gx, parts), 256, 0, s>>>(ptrs, nfloat, out, n, ctl, slice_begin, slice_end, acc, n_acc, result,
+                                                 result_exp);
     return cudaGetLastError();
 }
 
@@ -387,9 +665,7 @@ cudaError_t launch_leaf_max(const float* const* ptrs, const int64_t* nfloat, uns
     if (n <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned) * (size_t)n, s);
     if (e != cudaSuccess) return e;
-    int64_t parts = (max_nfloat + 32767) / 32768;
-    parts = parts < 1 ? 1 : (parts > 256 ? 256 : parts);
-    k_leaf_max<<<dim3((unsigned)n, (unsigned)parts), 256, 0, s>>>(ptrs, nfloat, out, n);
+    k_leaf_max<<<dim3((unsigned)n, leaf_parts(max_nfloat)), 256, 0, s>>>(ptrs, nfloat, out, n);
     return cudaGetLastError();
 }
 

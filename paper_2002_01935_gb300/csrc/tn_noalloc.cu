@@ -211,18 +211,16 @@ tn_status run_noalloc(const NetDesc& d, const Plan& p, void* out, int out_mem, i
     memset(&a, 0, sizeof(a));
     a.R = ws + root.ws_off * eb;
     a.n_out = p.n_out;
-    a.n_od = (int)d.open.size();
-    if (a.n_od > kMaxDigits) {
+    if ((int)d.open.size() > kMaxDigits) {
         err = "too many open labels";
         return TN_EUNSUPPORTED;
     }
-    for (int i = 0; i < a.n_od; ++i) {
+    for (int i = 0; i < (int)d.open.size(); ++i) {
         int l = d.open[d.open.size() - 1 - i];
-        a.od_dim[i] = (int32_t)d.dims[l];
         int64_t s = 0;
         for (size_t j = 0; j < root.lab.size(); ++j)
             if (root.lab[j] == l) s = root.stride[j];
-        a.od_s[i] = s;
+        push_fold_digit(a, d.dims[l], s);
     }
     a.max_r = maxabs + (nn - 1);
     a.exp_r = exps + (nn - 1);
@@ -233,7 +231,8 @@ tn_status run_noalloc(const NetDesc& d, const Plan& p, void* out, int out_mem, i
     // every slice in order, then the result
     int64_t mx_leaf = 0;
     for (int v = 0; v < n; ++v) mx_leaf = std::max(mx_leaf, d.leaves[v].size * (d.is_complex() ? 2 : 1));
-    CK(launch_call_begin(lptr, lnf, leafmax, n, mx_leaf, ctl, 0, p.d_sliced, acc, (int64_t)acc_doubles, stream));
+    CK(launch_call_begin(lptr, lnf, leafmax, n, mx_leaf, ctl, 0, p.d_sliced, acc, (int64_t)acc_doubles,
+                         nullptr, nullptr, stream));
     for (int64_t s = 0; s < p.d_sliced; ++s) {
         CK(launch_begin_slice(maxabs, nn, stream));
         // the workspace offsets assume the plan's step order

@@ -707,9 +707,9 @@ tn_status alloc_plan(NetDesc& d, Plan& p, void* unit, std::string& err) {
     if (!ck(cudaMalloc(&p.inst_out_dev, sizeof(double) * 2 * G), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&p.inst_exp_dev, sizeof(int64_t) * G), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&p.ctl, sizeof(Control)), "cudaMalloc")) return TN_ENOMEM;
+    // a call of an unsliced tree folds straight into the caller's output
     size_t acc_doubles = (size_t)p.n_out * (d.is_complex() ? 2 : 1);
-    if (!ck(cudaMalloc(&p.acc, sizeof(double) * acc_doubles), "cudaMalloc")) return TN_ENOMEM;
-    if (!ck(cudaMalloc(&p.out_stage, sizeof(double) * (acc_doubles + 1)), "cudaMalloc")) return TN_ENOMEM;
+    if (p.d_sliced > 1 && !ck(cudaMalloc(&p.acc, sizeof(double) * acc_doubles), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaStreamCreateWithFlags(&p.cap_stream, cudaStreamNonBlocking), "stream")) return TN_ECUDA;
     if (!ck(cudaMalloc(&p.leafmax, sizeof(unsigned) * d.n), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc((void**)&p.leaf_ptr_dev, sizeof(void*) * d.n), "cudaMalloc")) return TN_ENOMEM;
@@ -786,16 +786,13 @@ tn_status alloc_plan(NetDesc& d, Plan& p, void* unit, std::string& err) {
     memset(&a, 0, sizeof(a));
     a.R = (char*)p.ws + root.ws_off * eb;
     a.n_out = p.n_out;
-    a.n_od = (int)d.open.size();
-    if (a.n_od > kMaxDigits) {
+    if ((int)d.open.size() > kMaxDigits) {
         err = "too many open labels";
         return TN_EUNSUPPORTED;
     }
-    for (int i = 0; i < a.n_od; ++i) {
-        int l = d.open[d.open.size() - 1 - i];
-        a.od_dim[i] = (int32_t)d.dims[l];
-        a.od_s[i] = stride_in(root.lab, root.stride, l);
-    }
+    for (int i = (int)d.open.size() - 1; i >= 0; --i)
+        push_fold_digit(a, d.dims[d.open[i]], stride_in(root.lab, root.stride, d.open[i]));
+    a.direct = 1;
     a.max_r = p.maxabs + (nn - 1);
     a.exp_r = p.exps + (nn - 1);
     a.acc = p.acc;
@@ -1170,8 +1167,17 @@ tn_status run_plan(NetDesc& d, Plan& p, void* unit, int64_t begin, int64_t count
     st = prepare_leaves(d, p, capturing, lp, stream, err);
     if (st != TN_OK) return st;
     const int64_t n_acc = p.n_out * (d.is_complex() ? 2 : 1);
+    // the last group's fold writes the result: to the caller's device buffers,
+    // or (host outputs) to a staging buffer [result | exponent] for one copy
+    double* res = static_cast<double*>(out);
+    int64_t* res_exp = out_exp2;
+    if (out_mem == TN_MEM_HOST) {
+        if (!p.out_stage) CK(cudaMalloc(&p.out_stage, sizeof(double) * (n_acc + 1)));
+        res = p.out_stage;
+        res_exp = reinterpret_cast<int64_t*>(p.out_stage + n_acc);
+    }
     CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leafmax, n, max_leaf_floats(d), p.ctl, begin,
-                         begin + count, p.acc, n_acc, stream));
+                         begin + count, nullptr, 0, res, res_exp, stream));
     const int64_t groups = (count + G - 1) / G;
     const bool use_graph = !o.no_graph && !capturing;
     if (use_graph) {
@@ -1184,17 +1190,12 @@ tn_status run_plan(NetDesc& d, Plan& p, void* unit, int64_t begin, int64_t count
     } else {
         for (int64_t s = 0; s < groups; ++s) CK(enqueue_slice(d, p, stream, uev, pf, pc));
     }
-    // the result: one launch to device outputs; to host outputs, one copy of
-    // [accumulator | exponent] staged on the device
     if (out_mem == TN_MEM_HOST) {
-        CK(launch_result(p.acc, n_acc, p.ctl, p.out_stage, reinterpret_cast<int64_t*>(p.out_stage + n_acc), stream));
         std::vector<double> host((size_t)n_acc + 1);
         CK(cudaMemcpyAsync(host.data(), p.out_stage, sizeof(double) * (n_acc + 1), cudaMemcpyDeviceToHost, stream));
         CK(cudaStreamSynchronize(stream));
         std::memcpy(out, host.data(), sizeof(double) * n_acc);
         std::memcpy(out_exp2, host.data() + n_acc, sizeof(int64_t));
-    } else {
-        CK(launch_result(p.acc, n_acc, p.ctl, static_cast<double*>(out), out_exp2, stream));
     }
     return TN_OK;
 }
@@ -1244,8 +1245,8 @@ tn_status run_instances(NetDesc& d, Plan& p, void* unit, int n_inst, const int64
     std::vector<const void*> lp;
     st = prepare_leaves(d, p, false, lp, stream, err);
     if (st != TN_OK) return st;
-    CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leafmax, n, max_leaf_floats(d), p.ctl, 0, 1, p.acc,
-                         0, stream));
+    CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leafmax, n, max_leaf_floats(d), p.ctl, 0, 1, nullptr,
+                         0, nullptr, nullptr, stream));
     st = ensure_graph(d, p, lp, 0, 0, err);
     if (st != TN_OK) return st;
     CK(cudaGraphLaunch(p.gexec, stream));
@@ -1453,7 +1454,7 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
             for (auto& c : cs) c.second.tile.P = p.split_buf;
     }
     // a valid control block (slice 0 of the range) for the single-node launches
-    CK(launch_begin_call(p.ctl, 0, p.d_sliced, p.acc, 0, s));
+    CK(launch_begin_call(p.ctl, 0, p.d_sliced, nullptr, 0, s));
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
