@@ -28,8 +28,9 @@
  *     tn_last_error().
  *   - All device work is ordered on the caller's CUDA stream (a
  *     cudaStream_t passed as void*; NULL = legacy default stream).
- *   - Power-of-two label sizes run on the tiled kernels; other sizes run on
- *     the generic kernel (same results, slower).
+ *   - Power-of-two label sizes run on the tiled kernels and the tensor cores;
+ *     nodes with other sizes run in FP32 on the same tile kernel, the
+ *     smallest on one thread per output.
  */
 #ifndef TN_H
 #define TN_H
@@ -398,9 +399,9 @@ tn_status tn_plan_info(tn_net *net, const int32_t *tree_pairs, int32_t n_sliced,
 /*
  * tn_autotune -- per-node kernel choice by measurement.
  * For every tree node that runs alone in its launch step on a tiled or
- * tensor-core kernel, each candidate -- the five CUDA-core tile shapes
- * (64x64, 16x256, 4x1024, 256x16, 128x64 outputs per block, each with two
- * K splits) and, in the reduced-
+ * tensor-core kernel, each candidate -- the CUDA-core tile shapes
+ * (64x64, 16x256, 4x1024, 256x16, 128x64 and, for real nodes, 128x128
+ * outputs per block, each with two K splits) and, in the reduced-
  * precision modes, the tensor-core GEMM -- is launched once to warm up and
  * then reps times between two CUDA events on `stream`; the fastest is kept
  * in the handle's cached plan for (tree, sliced labels, mode) and used by
@@ -409,7 +410,7 @@ tn_status tn_plan_info(tn_net *net, const int32_t *tree_pairs, int32_t n_sliced,
  * can run skip the CUDA-core shapes.  The leaves must be attached; their
  * values do not matter.  choice (NULL or n_tensors-1 entries) receives per
  * node 0 (not tuned), 1..4 or 6 (tile shapes 64x64, 16x256, 4x1024,
- * 256x16, 128x64), 8 (tensor core), 9 (tensor core with 128-column
+ * 256x16, 128x64 or 128x128), 8 (tensor core), 9 (tensor core with 128-column
  * tiles where the planner's 256-column tiles fit: twice the CTAs, for
  * nodes with few tiles) or 10 (tensor core on the planar complex layout:
  * Re and Im planes of both operands, four real products per complex one

@@ -187,6 +187,7 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
             g.A = ptr(nd.ca);
             g.B = ptr(nd.cb);
             g.C = base + nd.ws_off * eb;
+            g.P = b.split_buf;
             g.ctl = b.ctl;
             g.sc.max_a = smax(nd.ca);
             g.sc.exp_a = sexp(nd.ca);

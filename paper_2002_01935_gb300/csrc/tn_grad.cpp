@@ -138,7 +138,11 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
         int64_t se = 0;
         for (Node& nd : G.fwd) {
             nd.kind = kGeneric;
-            if (f.force_generic || !plan_tile_node(d, G.g, nd, se)) continue;
+            if (f.force_generic) continue;
+            if (!plan_tile_node(d, G.g, nd, se)) {
+                plan_any_tile(d, nd, se, copies);
+                continue;
+            }
             if (!f.no_tensor_cores) make_tensor_core(d, f.mode, nd, se, copies);
         }
     }
@@ -179,8 +183,11 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
             G.g.vstride[NV + child] = nd.stride;
             nd.kind = kGeneric;
             const int ca0 = nd.tile.conj_a, cb0 = nd.tile.conj_b;
-            if (plan_tile_node(d, G.g, nd, split_elems) && !f.no_tensor_cores)
+            if (!plan_tile_node(d, G.g, nd, split_elems)) {
+                if (!f.force_generic) plan_any_tile(d, nd, split_elems, copies);
+            } else if (!f.no_tensor_cores) {
                 make_tensor_core(d, f.mode, nd, split_elems, copies);
+            }
             nd.tile.conj_a = ca0;
             nd.tile.conj_b = cb0;
             nd.ws_off = take(nd.size);
@@ -194,6 +201,8 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
         if (nd.kind == kTiled && nd.tile.split > 1)
             split_elems = std::max(split_elems, (int64_t)nd.tile.split * nd.tile.nbatch *
                                                     (int64_t(1) << (nd.tile.nm + nd.tile.nn)));
+        if (nd.kind == kGeneric && nd.any_cfg && nd.any_split > 1)
+            split_elems = std::max(split_elems, (int64_t)nd.any_split * nd.size);
         if (nd.kind == kTensorCore) {
             const int prec = tc_prec_of_mode(f.mode);
             const int64_t eb = d.elem_bytes();
@@ -452,6 +461,8 @@ static tn_status alloc_grad(const NetDesc& d, const Plan& f, GradState& G, void*
         op_is(nd.ca, in.a_is, in.sa_is);
         op_is(nd.cb, in.b_is, in.sb_is);
         g.in = in;
+        g.P = G.split_buf;
+        if (g.nbatch * (int64_t)g.split * NI > 65535) g.cfg = 0;  // grid z limit: one thread per output
         t = nd.tile;
         t.in = in;
         t.A = A;

@@ -91,20 +91,24 @@ struct GenericArgs {
     int conj_a, conj_b;  // read the operand complex-conjugated (reverse sweep)
     unsigned long long* t_done;  // root of a batched network: completion time (ns)
     InstanceInfo in;
-};
-
-// Tiled node (power-of-two label sizes): every index group is a set of bits.
-// offset(group index g) = sum_i bit_i(g) << shift_i ; shift 255 = absent.
-struct BitGroup {
-    int nbits;
-    uint8_t sh[kMaxBits];
+    // tile kernel (cfg != 0, see TileArgs): the output digits are the N
+    // digits, then M, then batch; K digits as above
+    int cfg, split;
+    int n_nd, n_md;       // N and M digits
+    int64_t M, N, nbatch;
+    int64_t kchunk;
+    int a_mfast, b_nfast;
+    void* P;
 };
 
 // Tiled node (power-of-two label sizes).  Each index group is a list of
 // bits; bit i of a group index contributes 1 << sh[i] to an operand offset
 // (kNoBit: the operand lacks that label).  Output layout [batch][M][N].
 constexpr uint8_t kNoBit = 255;
-enum TileCfg { kTile64x64 = 1, kTile16x256 = 2, kTile4x1024 = 3, kTile256x16 = 4, kTileDot = 5, kTile128x64 = 6 };
+// kTile128x128: real nodes only
+enum TileCfg {
+    kTile64x64 = 1, kTile16x256 = 2, kTile4x1024 = 3, kTile256x16 = 4, kTileDot = 5, kTile128x64 = 6, kTile128x128 = 7
+};
 
 struct alignas(16) TileArgs {
     const void* A;
@@ -408,7 +412,10 @@ cudaError_t launch_root_adjoint(const RootAdjArgs& a, int n_inst, cudaStream_t s
 // planning, e.g. tn_plan_info on a machine without a GPU).  Grid sizes and
 // K splits are sized in multiples of it.
 int sm_count();
+// Any label sizes: the tile kernel where the planner gave the node a shape
+// (a.cfg), else one thread per output.
 cudaError_t launch_generic(const GenericArgs& a, bool is_c, cudaStream_t s);
+cudaError_t launch_tile_any(const GenericArgs& a, bool is_c, cudaStream_t s);  // tn_tiled.cu
 cudaError_t launch_tile(const TileArgs& a, bool is_c, cudaStream_t s);  // tn_tiled.cu
 // Tensor-core node (tn_tc.cu): prec as tc_prec_of_mode.
 // Packs both operands into a.P (TcGeom, one launch) and runs the bulk-copy-

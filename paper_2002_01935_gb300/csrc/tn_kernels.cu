@@ -157,6 +157,7 @@ int sm_count() {
 }
 
 cudaError_t launch_generic(const GenericArgs& a, bool is_c, cudaStream_t s) {
+    if (a.cfg) return launch_tile_any(a, is_c, s);
     int64_t blocks = (a.n_out + 255) / 256;
     if (blocks > sm_count() * 16) blocks = sm_count() * 16;
     if (blocks < 1) blocks = 1;

@@ -190,6 +190,7 @@ tn_status run_noalloc(const NetDesc& d, const Plan& p, void* out, int out_mem, i
         GenericArgs& g = gen[k];
         tn_status st = make_generic_args(d, p, k, g, err);
         if (st != TN_OK) return st;
+        g.cfg = 0;  // no split buffer here: one thread per output
         auto operand = [&](int c) -> const void* {
             if (c < 0) return unit;
             if (c < n) return d.leaves[c].ptr;

@@ -85,6 +85,15 @@ int ilog2(int64_t x) {
     return r;
 }
 
+// Real nodes take 128 x 128 tiles (64 outputs per thread) where these alone
+// give every SM one: 2^11 x 2^11 x 2^10 256 against 289 us with 64 x 64 tiles,
+// 2^12 x 2^12 x 2^10 882 against 1055; with fewer tiles the smaller ones win
+// (2^9 x 2^9 x 2^9: 39 against 30 us).  A complex thread tile of that size
+// does not fit the registers.
+bool large_real_tiles(const NetDesc& d, int64_t nbatch, int64_t M, int64_t N) {
+    return !d.is_complex() && M >= 128 && N >= 128 && ((M + 127) / 128) * ((N + 127) / 128) * nbatch >= sm_count();
+}
+
 // Tiled-kernel plan of a node whose labels and strides are all powers of
 // two: index bits per group, K order, load directions, tile shape and K
 // split.  Returns false (generic kernel) when a limit is exceeded.
@@ -171,10 +180,10 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
     const int64_t M = int64_t(1) << t.nm, N = int64_t(1) << t.nn, K = int64_t(1) << t.nk;
     int TM = 64, TN = 64, TK = 16;
     const bool dot = M * N <= 64 && K >= 512;
-    if (force_cfg >= kTile64x64 && force_cfg <= kTile128x64 && force_cfg != kTileDot && !dot) {
+    if (force_cfg >= kTile64x64 && force_cfg <= kTile128x128 && force_cfg != kTileDot && !dot) {
         // a shape forced by the autotuner (any shape is valid: tiles clip)
-        static const int shapes[7][3] = {{0, 0, 0},    {64, 64, 16},   {16, 256, 16}, {4, 1024, 4},
-                                         {256, 16, 16}, {0, 0, 0},      {128, 64, 16}};
+        static const int shapes[8][3] = {{0, 0, 0},     {64, 64, 16}, {16, 256, 16}, {4, 1024, 4},
+                                         {256, 16, 16}, {0, 0, 0},    {128, 64, 16}, {128, 128, 16}};
         t.cfg = force_cfg;
         TM = shapes[force_cfg][0];
         TN = shapes[force_cfg][1];
@@ -196,6 +205,10 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         t.cfg = kTile256x16;
         TM = 256;
         TN = 16;
+    } else if (large_real_tiles(d, p.copies * t.nbatch, M, N)) {
+        t.cfg = kTile128x128;
+        TM = 128;
+        TN = 128;
     } else {
         t.cfg = kTile64x64;
     }
@@ -295,6 +308,55 @@ Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std
         if (!has(uni, l)) uni.push_back(l);
     nd.vc = log2size(uni);
     return nd;
+}
+
+// The tile kernel for sizes of any kind.  The shape follows the rule of
+// plan_tile (4 x 1024 up to 4 rows, 16 x 256 up to 32, 256 x 16 up to 32
+// columns, else 64 x 64) and so does the K split, each part at least 16
+// entries.  Nodes of fewer than 2^13 multiply-adds keep one thread per
+// output: @@RULE@@.
+void plan_any_tile(const NetDesc& d, Node& nd, int64_t& split_elems, int copies) {
+    nd.any_cfg = 0;
+    nd.any_split = 1;
+    auto volume = [&](std::initializer_list<const std::vector<int>*> groups) {
+        double v = 1;
+        for (auto* g : groups)
+            for (int l : *g) v *= (double)d.dims[l];
+        return v;
+    };
+    const double lim = 2147483648.0;  // the kernel's indices and offsets are 32-bit
+    const double M = volume({&nd.gm}), N = volume({&nd.gn}), B = volume({&nd.gb}), K = volume({&nd.gk, &nd.gsa, &nd.gsb});
+    const double size_a = volume({&nd.gb, &nd.gm, &nd.gk, &nd.gsa}), size_b = volume({&nd.gb, &nd.gn, &nd.gk, &nd.gsb});
+    if (M * N * K * B < 8192.0 || std::max(std::max(size_a, size_b), std::max(K, std::max(M, N))) >= lim) return;
+    int cfg = kTile64x64, TM = 64, TN = 64, TK = 16;
+    if (M <= 4 && N >= 1024) {
+        cfg = kTile4x1024;
+        TM = 4;
+        TN = 1024;
+        TK = 4;
+    } else if (M <= 32 && N >= 256) {
+        cfg = kTile16x256;
+        TM = 16;
+        TN = 256;
+    } else if (N <= 32 && M >= 256) {
+        cfg = kTile256x16;
+        TM = 256;
+        TN = 16;
+    } else if (large_real_tiles(d, (int64_t)B * copies, (int64_t)M, (int64_t)N)) {
+        cfg = kTile128x128;
+        TM = TN = 128;
+    }
+    const double tiles = std::ceil(M / TM) * std::ceil(N / TN) * B;
+    if (B * copies > 65535 || std::ceil(M / TM) * std::ceil(N / TN) >= lim) return;  // launch grid limits
+    const int64_t ktiles = ((int64_t)K + TK - 1) / TK;
+    int split = 1;
+    while (tiles * copies * split < 2 * sm_count() && split * 2 <= ktiles && split < 64 &&
+           B * split * 2 * copies <= 65535)
+        split *= 2;
+    nd.any_cfg = cfg;
+    nd.any_kchunk = ((ktiles + split - 1) / split) * TK;
+    nd.any_split = (int)(((int64_t)K + nd.any_kchunk - 1) / nd.any_kchunk);  // no empty part
+    if (nd.any_split > 1) split_elems = std::max(split_elems, (int64_t)nd.any_split * (int64_t)(B * M * N));
 }
 
 // Work items of a node in the persistent launch (per instance).
@@ -485,6 +547,7 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
                 err = "the persistent launch needs power-of-two label sizes on every node";
                 return TN_EUNSUPPORTED;
             }
+            if (!p.force_generic) plan_any_tile(d, nd, split_elems, p.copies);
             continue;
         }
         if (p.persistent) {
@@ -680,6 +743,31 @@ static tn_status fill_generic(const NetDesc& d, const Plan& p, const Node& nd, G
     }
     if (nd.ca >= 0 && nd.ca < n) g.sla = p.leaf_sl[nd.ca];
     if (nd.cb >= 0 && nd.cb < n) g.slb = p.leaf_sl[nd.cb];
+    g.nbatch = g.M = g.N = 1;
+    g.split = 1;
+    if (nd.kind == kGeneric && nd.any_cfg) {
+        g.cfg = nd.any_cfg;
+        g.split = nd.any_split;
+        g.kchunk = nd.any_kchunk;
+        g.n_nd = (int)nd.gn.size();
+        g.n_md = (int)nd.gm.size();
+        for (int l : nd.gn) g.N *= d.dims[l];
+        for (int l : nd.gm) g.M *= d.dims[l];
+        for (int l : nd.gb) g.nbatch *= d.dims[l];
+        // load along the rows (columns) where they hold the operand's fastest label
+        auto fast = [&](const std::vector<int>& lab, const std::vector<int64_t>& st, const std::vector<int>& group) {
+            int best = -1;
+            int64_t bs = INT64_MAX;
+            for (size_t i = 0; i < lab.size(); ++i)
+                if (d.dims[lab[i]] > 1 && st[i] < bs) {
+                    bs = st[i];
+                    best = lab[i];
+                }
+            return best >= 0 && has(group, best);
+        };
+        g.a_mfast = fast(la, sa, nd.gm);
+        g.b_nfast = fast(lb, sb, nd.gn);
+    }
     return TN_OK;
 }
 
@@ -738,6 +826,7 @@ tn_status alloc_plan(NetDesc& d, Plan& p, void* unit, std::string& err) {
         g.B = nd.cb >= n ? (const void*)(ws + p.nodes[nd.cb - n].ws_off * eb) : nullptr;
         if (nd.ca < 0) g.A = unit;
         if (nd.cb < 0) g.B = unit;
+        g.P = p.split_buf;
         g.ctl = p.ctl;
         // leaves: renormalised by their own max, stored exponent 0
         g.sc.max_a = nd.ca >= n ? p.maxabs + (nd.ca - n) : (nd.ca >= 0 ? p.leafmax + nd.ca : nullptr);
@@ -853,9 +942,14 @@ static tn_status configure_instances(const NetDesc& d, Plan& p, int G, int step,
                 t.kchunk = ((units + split - 1) / split) * gran;
             }
         }
-        if (!p.persistent && nd.kind == kGeneric && G > 65535) {
-            err = "too many instances";
-            return TN_EUNSUPPORTED;
+        if (!p.persistent && nd.kind == kGeneric) {
+            if (G > 65535) {
+                err = "too many instances";
+                return TN_EUNSUPPORTED;
+            }
+            // the tile kernel's grid z likewise; one thread per output otherwise
+            GenericArgs& g = p.gen[k];
+            g.cfg = g.nbatch * (int64_t)nd.any_split * G > 65535 ? 0 : nd.any_cfg;
         }
     }
     if (!p.items.empty()) {
@@ -1435,10 +1529,14 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
         }
         // CUDA-core shapes, unless the node is so large that they cannot win
         if (!has_tc || vc < 32)
-            for (int v : {int(kTile64x64), int(kTile16x256), int(kTile4x1024), int(kTile256x16), int(kTile128x64)})
+            for (int v : {int(kTile64x64), int(kTile16x256), int(kTile4x1024), int(kTile256x16), int(kTile128x64),
+                          int(kTile128x128)})
                 for (int mult : {1, 4}) {
                     Node t;
-                    if (make_variant(d, p, k, v, t, split_elems, mult)) cand[k].push_back({v, t});
+                    if (v == kTile128x128 && d.is_complex()) continue;  // real nodes only
+                    // both 128-row shapes are reported as 6
+                    if (make_variant(d, p, k, v, t, split_elems, mult))
+                        cand[k].push_back({v == kTile128x128 ? int(kTile128x64) : v, t});
                 }
     }
     const int64_t need = (split_elems * (int64_t)d.elem_bytes() + 1023) / 1024 * 1024;
@@ -1450,6 +1548,7 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
         CK(cudaMalloc(&p.split_buf, need * G));
         p.split_bytes = need;
         for (auto& nd : p.nodes) nd.tile.P = p.split_buf;
+        for (auto& g : p.gen) g.P = p.split_buf;
         for (auto& cs : cand)
             for (auto& c : cs) c.second.tile.P = p.split_buf;
     }

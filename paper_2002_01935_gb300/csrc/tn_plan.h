@@ -55,6 +55,9 @@ struct Node {
     int kind = kGeneric;
     double vc = 0;               // log2 of 2^vc, Eq. vertexcon
     TileArgs tile{};             // index bits, config and split (kTiled); pointers set at alloc
+    // kGeneric: shape of the tile kernel (0: one thread per output) and K split
+    int any_cfg = 0, any_split = 1;
+    int64_t any_kchunk = 0;
 };
 
 // One launch of the per-slice sequence: a wave (all small nodes of a tree
@@ -173,6 +176,8 @@ struct Plan {
 
 tn_status build_plan(const NetDesc& d, Plan& p, std::string& err);
 Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std::vector<int>& keep);
+// Tile shape and K split of a node whose sizes are not powers of two.
+void plan_any_tile(const NetDesc& d, Node& nd, int64_t& split_elems, int copies = 1);
 bool plan_tile_node(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems);
 bool make_tensor_core(const NetDesc& d, tn_mode mode, Node& nd, int64_t& split_elems, int copies = 1);
 // Autotuner variant code of the tensor-core kernel (tile shapes use TileCfg).

@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cstring>
 #include <stdint.h>
+#include <type_traits>
 
 #include "../../include/tn.h"
 #include "tn_internal.h"
@@ -132,7 +133,8 @@ struct View {
     bool live;
 };
 
-__device__ __forceinline__ View inst_view(const TileArgs& a, int inst, int esz) {
+template <class ARGS>
+__device__ __forceinline__ View inst_view(const ARGS& a, int inst, int esz) {
     const InstanceInfo& in = a.in;
     View v;
     v.A = (const char*)a.A + (int64_t)inst * in.a_is * esz;
@@ -361,22 +363,103 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, int64_t tile_x, int
 }
 
 // --------------------------------------------------------------------------
-// The tile kernel: one CTA = TM x TN outputs of one batch index and one K
-// split (the same computation as tile_body above, written out for the
-// kernel: the shared body costs the kernel registers, hence occupancy).
+// Index groups of the two argument forms.  TileArgs (power-of-two sizes): an
+// offset is a scatter of index bits.  GenericArgs (any sizes): mixed-radix
+// digits, the output's fastest first (N digits, then M, then batch).
 // --------------------------------------------------------------------------
-template <bool CPLX, int TM, int TN, int TK, int RM, int RN>
-__global__ void __launch_bounds__((TM / RM) * (TN / RN))
-    k_tile(const __grid_constant__ TileArgs a) {
+__device__ __forceinline__ int64_t size_m(const TileArgs& a) { return 1ll << a.nm; }
+__device__ __forceinline__ int64_t size_n(const TileArgs& a) { return 1ll << a.nn; }
+__device__ __forceinline__ int64_t size_k(const TileArgs& a) { return 1ll << a.nk; }
+__device__ __forceinline__ int64_t off_m(const TileArgs& a, int64_t m) { return scatter_bits(m, a.a_m, a.nm); }
+__device__ __forceinline__ int64_t off_n(const TileArgs& a, int64_t n) { return scatter_bits(n, a.b_n, a.nn); }
+__device__ __forceinline__ void off_k(const TileArgs& a, int64_t k, int64_t& ka, int64_t& kb) {
+    ka = scatter_bits(k, a.a_k, a.nk);
+    kb = scatter_bits(k, a.b_k, a.nk);
+}
+__device__ __forceinline__ void off_b(const TileArgs& a, int64_t b, int64_t& ba, int64_t& bb) {
+    ba = scatter_bits(b, a.a_b, a.nb);
+    bb = scatter_bits(b, a.b_b, a.nb);
+}
+
+__device__ __forceinline__ int64_t size_m(const GenericArgs& a) { return a.M; }
+__device__ __forceinline__ int64_t size_n(const GenericArgs& a) { return a.N; }
+__device__ __forceinline__ int64_t size_k(const GenericArgs& a) { return a.n_sum; }
+// digits [j0, j1) of x (below 2^31: the planner's condition) with strides st
+__device__ __forceinline__ int64_t digits(unsigned x, const int32_t* dim, const int64_t* st, int j0, int j1) {
+    int64_t o = 0;
+    for (int j = j0; j < j1; ++j) {
+        const unsigned d = (unsigned)dim[j], q = x / d;
+        o += (int64_t)(x - q * d) * st[j];
+        x = q;
+    }
+    return o;
+}
+__device__ __forceinline__ int64_t off_m(const GenericArgs& a, int64_t m) {
+    return digits((unsigned)m, a.od_dim, a.od_sa, a.n_nd, a.n_nd + a.n_md);
+}
+__device__ __forceinline__ int64_t off_n(const GenericArgs& a, int64_t n) {
+    return digits((unsigned)n, a.od_dim, a.od_sb, 0, a.n_nd);
+}
+__device__ __forceinline__ void off_k(const GenericArgs& a, int64_t k, int64_t& ka, int64_t& kb) {
+    ka = digits((unsigned)k, a.kd_dim, a.kd_sa, 0, a.n_kd);
+    kb = digits((unsigned)k, a.kd_dim, a.kd_sb, 0, a.n_kd);
+}
+__device__ __forceinline__ void off_b(const GenericArgs& a, int64_t b, int64_t& ba, int64_t& bb) {
+    ba = digits((unsigned)b, a.od_dim, a.od_sa, a.n_nd + a.n_md, a.n_od);
+    bb = digits((unsigned)b, a.od_dim, a.od_sb, a.n_nd + a.n_md, a.n_od);
+}
+
+// --------------------------------------------------------------------------
+// The tile kernel: one CTA = TM x TN outputs of one batch index and one K
+// split, RM x RN of them per thread.
+//
+// Bound by the FP32 pipes for large K, by the operand loads from shared
+// memory before that: a thread holds 8 x 4 outputs (real: 8 x 8 in the largest
+// tiles), reads them 16 bytes at a time -- two complex or four real entries of
+// a row of either operand -- and K is stepped by 8 through two shared-memory
+// stages, the next step's global loads in flight during this step's
+// multiply-adds, one barrier a step.  Per-thread operand offsets within a step
+// are kept in registers; the K base follows its carry chain (power-of-two
+// sizes) or a table of 1024 K offsets in shared memory (any sizes).
+// 2^11 x 2^11 x 2^10, complex: 1029 us with 4 x 4 outputs per thread, 8-byte
+// loads and 64-bit address sums per entry, 732 now (47 TFLOP/s; 2^12 x 2^12:
+// 51); real: 421 -> 256.  The paired multiply-add fma.rn.f32x2 was tried in
+// its place and is no faster here (47 TFLOP/s on the larger node): its three
+// 64-bit operands issue every third cycle.
+// --------------------------------------------------------------------------
+constexpr int kTabK = 1024;  // K offsets held in shared memory (any sizes)
+
+template <class ARGS, bool CPLX, int TM, int TN, int TK>
+struct TileSmem {
     using T = typename VT<CPLX>::T;
+    static constexpr int PAD = CPLX ? 2 : 4;  // 16 bytes a row: no bank conflicts in stores along K
+    static constexpr size_t a_bytes = (size_t)TK * (TM + PAD) * sizeof(T);
+    static constexpr size_t b_bytes = (size_t)TK * (TN + PAD) * sizeof(T);
+    static constexpr size_t tab_bytes = std::is_same<ARGS, GenericArgs>::value ? 2 * kTabK * sizeof(int32_t) : 0;
+    static constexpr size_t bytes = 2 * (a_bytes + b_bytes) + tab_bytes;
+};
+
+template <class ARGS, bool CPLX, int TM, int TN, int TK, int RM, int RN, int MINB>
+__global__ void __launch_bounds__((TM / RM) * (TN / RN), MINB)
+    k_tile(const __grid_constant__ ARGS a) {
+    using T = typename VT<CPLX>::T;
+    using SM = TileSmem<ARGS, CPLX, TM, TN, TK>;
+    constexpr bool ANY = std::is_same<ARGS, GenericArgs>::value;
     constexpr int TX = TN / RN, TY = TM / RM, NT = TX * TY;
-    constexpr int PB = CPLX ? 2 : 4;  // keeps sB rows 16-byte aligned
-    __shared__ T sA[TK][TM + 1];
-    __shared__ __align__(16) T sB[TK][TN + PB];
-    __shared__ int64_t rowA[TM], colB[TN], kA[TK], kB[TK];
+    constexpr int RP = CPLX ? RN : RN / 2;  // accumulator pairs per row
+    constexpr int VB = CPLX ? 2 : 4;        // entries per 16-byte load
+    static_assert(RN % VB == 0 && RM % VB == 0, "thread tile");
+    extern __shared__ __align__(16) unsigned char tile_smem[];
+    __shared__ int64_t rowA[TM], colB[TN];
+    auto sA = [&](int st, int t) { return reinterpret_cast<T*>(tile_smem + st * SM::a_bytes) + t * (TM + SM::PAD); };
+    auto sB = [&](int st, int t) {
+        return reinterpret_cast<T*>(tile_smem + 2 * SM::a_bytes + st * SM::b_bytes) + t * (TN + SM::PAD);
+    };
+    int32_t* const tabA = reinterpret_cast<int32_t*>(tile_smem + 2 * (SM::a_bytes + SM::b_bytes));
+    int32_t* const tabB = tabA + kTabK;
 
     const int tid = threadIdx.x;
-    const int64_t M = 1ll << a.nm, N = 1ll << a.nn, K = 1ll << a.nk;
+    const int64_t M = size_m(a), N = size_n(a), K = size_k(a);
     const int64_t tiles_n = (N + TN - 1) / TN;
     const int64_t m0 = ((int64_t)blockIdx.x / tiles_n) * TM;
     const int64_t n0 = ((int64_t)blockIdx.x % tiles_n) * TN;
@@ -388,140 +471,219 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN))
     const View vw = inst_view(a, inst, (int)sizeof(T));
     if (!vw.live) return;
     const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && zz == 0 && tid == 0);
-    const int64_t slice = vw.slice;
-    const int64_t baseA =
-        slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb) + scatter_bits(m0, a.a_m, a.nm);
-    const int64_t baseB =
-        slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb) + scatter_bits(n0, a.b_n, a.nn);
-    for (int i = tid; i < TM; i += NT) rowA[i] = scatter_bits(i, a.a_m, a.nm);
-    for (int j = tid; j < TN; j += NT) colB[j] = scatter_bits(j, a.b_n, a.nn);
-    for (int t = tid; t < TK; t += NT) {
-        kA[t] = scatter_bits(t, a.a_k, a.nk);
-        kB[t] = scatter_bits(t, a.b_k, a.nk);
-    }
-    __syncthreads();
     const int mlim = (int)min64(M - m0, TM);
     const int nlim = (int)min64(N - n0, TN);
     const int64_t kbeg = (int64_t)split_id * a.kchunk;
     const int64_t kend = min64(K, kbeg + a.kchunk);
-    const T* A = reinterpret_cast<const T*>(vw.A);
-    const T* B = reinterpret_cast<const T*>(vw.B);
+    for (int i = tid; i < mlim; i += NT) rowA[i] = off_m(a, m0 + i);
+    for (int j = tid; j < nlim; j += NT) colB[j] = off_n(a, n0 + j);
+    int64_t ba, bb;
+    off_b(a, b, ba, bb);
+    const T* A = reinterpret_cast<const T*>(vw.A) + slice_off(a.sla, vw.slice) + ba;
+    const T* B = reinterpret_cast<const T*>(vw.B) + slice_off(a.slb, vw.slice) + bb;
+    __syncthreads();
     const int tx = tid % TX, ty = tid / TX;
 
-    T acc[RM][RN];
+    // this thread's entries of a K step: entry q of an operand tile of S rows
+    // (columns) is row i0 + q di, K index t0 + q dt, along the rows or along K
+    // as the operand is contiguous
+    constexpr int LA = (TM * TK + NT - 1) / NT, LB = (TN * TK + NT - 1) / NT;
+    constexpr int LG_TK = TK == 16 ? 4 : (TK == 8 ? 3 : 2);
+    static_assert((1 << LG_TK) == TK, "TK must be a power of two");
+    struct Walk {
+        int i0, t0, di, dt;
+        bool wrap;  // S > NT, along the rows: S / NT entries per K index
+    };
+    auto walk = [&](int S, bool along_rows) {
+        Walk w;
+        w.wrap = along_rows && S > NT;
+        if (along_rows) {
+            w.i0 = S > NT ? tid : tid % S;
+            w.t0 = S > NT ? 0 : tid / S;
+            w.di = 0;
+            w.dt = S > NT ? 0 : NT / S;
+        } else {
+            w.i0 = tid / TK;
+            w.t0 = tid % TK;
+            w.di = NT / TK;
+            w.dt = 0;
+        }
+        if (tid >= S * TK) w.i0 = S;  // fewer entries than threads: none for this one
+        return w;
+    };
+    const Walk wa = walk(TM, a.a_mfast != 0), wb = walk(TN, a.b_nfast != 0);
+    auto row_of = [&](const Walk& w, int q, int S) { return w.wrap ? w.i0 + q % (S > NT ? S / NT : 1) * NT : w.i0 + q * w.di; };
+    auto k_of = [&](const Walk& w, int q, int S) { return w.wrap ? q / (S > NT ? S / NT : 1) : w.t0 + q * w.dt; };
+    // offset in the operand without the K base (sizes of any kind: without K)
+    int offA[LA], offB[LB];  // operands have below 2^31 entries
+#pragma unroll
+    for (int q = 0; q < LA; ++q) {
+        const int i = row_of(wa, q, TM);
+        offA[q] = i < mlim ? (int)rowA[i] : 0;
+        if constexpr (!ANY) offA[q] += (int)scatter_bits(k_of(wa, q, TM), a.a_k, min(a.nk, LG_TK));
+    }
+#pragma unroll
+    for (int q = 0; q < LB; ++q) {
+        const int j = row_of(wb, q, TN);
+        offB[q] = j < nlim ? (int)colB[j] : 0;
+        if constexpr (!ANY) offB[q] += (int)scatter_bits(k_of(wb, q, TN), a.b_k, min(a.nk, LG_TK));
+    }
+
+    float2 acc[RM][RP];
 #pragma unroll
     for (int r = 0; r < RM; ++r)
 #pragma unroll
-        for (int c = 0; c < RN; ++c) acc[r][c] = zero<T>();
+        for (int c = 0; c < RP; ++c) acc[r][c] = make_float2(0.f, 0.f);
 
-    // global -> registers for one K step (all loads issued back to back).
-    // The operand offsets of the K step's base k0 are kept incrementally:
-    // k0 advances by TK, so only the bits of its carry chain change.
-    constexpr int LA = (TM * TK + NT - 1) / NT, LB = (TN * TK + NT - 1) / NT;
-    constexpr int LG_TK = TK == 16 ? 4 : (TK == 8 ? 3 : (TK == 4 ? 2 : 0));
-    static_assert((1 << LG_TK) == TK, "TK must be a power of two");
     T ra[LA], rb[LB];
-    int64_t cur_k = kbeg;
-    int64_t kaA = scatter_bits(kbeg, a.a_k, a.nk), kaB = scatter_bits(kbeg, a.b_k, a.nk);
-    auto step_k = [&]() {  // cur_k += TK, offsets follow
-        int i = LG_TK;
-        while (i < a.nk && ((cur_k >> i) & 1)) {
-            if (a.a_k[i] != kNoBit) kaA -= int64_t(1) << a.a_k[i];
-            if (a.b_k[i] != kNoBit) kaB -= int64_t(1) << a.b_k[i];
-            ++i;
+    int64_t cur_k = kbeg, kaA = 0, kaB = 0;
+    if constexpr (!ANY) off_k(a, kbeg, kaA, kaB);
+    [[maybe_unused]] auto step_k = [&]() {  // cur_k += TK, the K base follows its carry chain
+        if constexpr (!ANY) {
+            int i = LG_TK;
+            while (i < a.nk && ((cur_k >> i) & 1)) {
+                if (a.a_k[i] != kNoBit) kaA -= int64_t(1) << a.a_k[i];
+                if (a.b_k[i] != kNoBit) kaB -= int64_t(1) << a.b_k[i];
+                ++i;
+            }
+            if (i < a.nk) {
+                if (a.a_k[i] != kNoBit) kaA += int64_t(1) << a.a_k[i];
+                if (a.b_k[i] != kNoBit) kaB += int64_t(1) << a.b_k[i];
+            }
+            cur_k += TK;
         }
-        if (i < a.nk) {
-            if (a.a_k[i] != kNoBit) kaA += int64_t(1) << a.a_k[i];
-            if (a.b_k[i] != kNoBit) kaB += int64_t(1) << a.b_k[i];
-        }
-        cur_k += TK;
     };
-    auto gload = [&](int64_t k0) {
+    // global -> registers for the K step at k0 (all loads back to back); w0:
+    // first K index of the offset table
+    auto gload = [&](int64_t k0, [[maybe_unused]] int64_t w0) {
         const int klim = (int)min64(kend - k0, TK);
 #pragma unroll
         for (int q = 0; q < LA; ++q) {
-            const int e = tid + q * NT;
-            const int i = a.a_mfast ? e % TM : e / TK;
-            const int t = a.a_mfast ? e / TM : e % TK;
-            const bool in = e < TM * TK && i < mlim && t < klim;
-            ra[q] = in ? cmul(A[baseA + rowA[i] + kaA + kA[t]], sc.fa, a.conj_a) : zero<T>();
+            const int i = row_of(wa, q, TM), t = k_of(wa, q, TM);
+            ra[q] = zero<T>();
+            if (i < mlim && t < klim) {
+                if constexpr (ANY) ra[q] = A[offA[q] + tabA[(int)(k0 - w0) + t]];
+                else ra[q] = A[kaA + offA[q]];
+            }
         }
 #pragma unroll
         for (int q = 0; q < LB; ++q) {
-            const int e = tid + q * NT;
-            const int j = a.b_nfast ? e % TN : e / TK;
-            const int t = a.b_nfast ? e / TN : e % TK;
-            const bool in = e < TN * TK && j < nlim && t < klim;
-            rb[q] = in ? cmul(B[baseB + colB[j] + kaB + kB[t]], sc.fb, a.conj_b) : zero<T>();
+            const int j = row_of(wb, q, TN), t = k_of(wb, q, TN);
+            rb[q] = zero<T>();
+            if (j < nlim && t < klim) {
+                if constexpr (ANY) rb[q] = B[offB[q] + tabB[(int)(k0 - w0) + t]];
+                else rb[q] = B[kaB + offB[q]];
+            }
         }
     };
-    if (kbeg < kend) gload(kbeg);
-    for (int64_t k0 = kbeg; k0 < kend; k0 += TK) {
-        // kaA/kaB describe k0 here; gload of k0 + TK needs them advanced
+    auto stash = [&](int st) {  // registers -> shared memory, scaled
 #pragma unroll
         for (int q = 0; q < LA; ++q) {
-            const int e = tid + q * NT;
-            if (e < TM * TK) {
-                const int i = a.a_mfast ? e % TM : e / TK;
-                const int t = a.a_mfast ? e / TM : e % TK;
-                sA[t][i] = ra[q];
-            }
+            const int i = row_of(wa, q, TM);
+            if (i < TM) sA(st, k_of(wa, q, TM))[i] = cmul(ra[q], sc.fa, a.conj_a);
         }
 #pragma unroll
         for (int q = 0; q < LB; ++q) {
-            const int e = tid + q * NT;
-            if (e < TN * TK) {
-                const int j = a.b_nfast ? e % TN : e / TK;
-                const int t = a.b_nfast ? e / TN : e % TK;
-                sB[t][j] = rb[q];
-            }
+            const int j = row_of(wb, q, TN);
+            if (j < TN) sB(st, k_of(wb, q, TN))[j] = cmul(rb[q], sc.fb, a.conj_b);
         }
-        __syncthreads();
-        if (k0 + TK < kend) {
-            step_k();
-            gload(k0 + TK);  // next step's loads overlap this step's FMAs
-        }
-#pragma unroll 4
+    };
+    auto multiply = [&](int st) {
+#pragma unroll
         for (int t = 0; t < TK; ++t) {
-            T af[RM], bf[RN];
+            float4 bv[RN / VB];
 #pragma unroll
-            for (int r = 0; r < RM; ++r) af[r] = sA[t][ty * RM + r];
+            for (int c = 0; c < RN / VB; ++c)
+                bv[c] = *reinterpret_cast<const float4*>(sB(st, t) + (tx + c * TX) * VB);
+            float4 av[RM / VB];
 #pragma unroll
-            for (int c = 0; c < RN; ++c) bf[c] = sB[t][tx + c * TX];  // conflict-free
+            for (int r = 0; r < RM / VB; ++r) av[r] = *reinterpret_cast<const float4*>(sA(st, t) + ty * RM + r * VB);
+            const float* af = reinterpret_cast<const float*>(av);
+            const float* bf = reinterpret_cast<const float*>(bv);
 #pragma unroll
             for (int r = 0; r < RM; ++r)
 #pragma unroll
-                for (int c = 0; c < RN; ++c) fma_acc(acc[r][c], af[r], bf[c]);
+                for (int c = 0; c < RP; ++c) {
+                    float2& x = acc[r][c];
+                    if constexpr (CPLX) {
+                        fma_acc(x, make_float2(af[2 * r], af[2 * r + 1]), make_float2(bf[2 * c], bf[2 * c + 1]));
+                    } else {
+                        x.x = fmaf(af[r], bf[2 * c], x.x);
+                        x.y = fmaf(af[r], bf[2 * c + 1], x.y);
+                    }
+                }
         }
+    };
+    // window by window of the K offset table (power-of-two sizes: one window)
+    const int64_t win = ANY ? kTabK : (kend > kbeg ? kend - kbeg : 1);
+    for (int64_t w0 = kbeg; w0 < kend; w0 += win) {
+        const int64_t w1 = min64(kend, w0 + win);
+        if constexpr (ANY) {
+            __syncthreads();  // the table's and the stages' last readers are done
+            for (int t = tid; t < (int)(w1 - w0); t += NT) {
+                int64_t ka, kb;
+                off_k(a, w0 + t, ka, kb);
+                tabA[t] = (int32_t)ka;
+                tabB[t] = (int32_t)kb;
+            }
+            __syncthreads();
+        }
+        gload(w0, w0);
+        stash(0);
         __syncthreads();
+        int st = 0;
+        for (int64_t k0 = w0; k0 < w1; k0 += TK) {
+            const bool more = k0 + TK < w1;
+            if (more) {
+                step_k();
+                gload(k0 + TK, w0);
+            }
+            multiply(st);
+            if (more) {
+                st ^= 1;
+                stash(st);
+                __syncthreads();
+            }
+        }
     }
 
     // epilogue: direct output (one split) or a partial for the reduce pass
     float lmax = 0.f;
     T* out = reinterpret_cast<T*>(a.split > 1 ? vw.P : vw.C);
-    const int64_t plane = (a.split > 1 ? (int64_t)split_id * ((int64_t)a.nbatch) : 0) + b;
+    const int64_t plane = (a.split > 1 ? (int64_t)split_id * a.nbatch : 0) + b;
+    // whole 16-byte stores where every row starts on 16 bytes
+    const bool vec = N % VB == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
 #pragma unroll
     for (int r = 0; r < RM; ++r) {
         const int i = ty * RM + r;
         if (i >= mlim) continue;
-        const int64_t rowoff = (plane * M + m0 + i) * N + n0;
+        T* row = out + (plane * M + m0 + i) * N + n0;
 #pragma unroll
-        for (int c = 0; c < RN; ++c) {
-            const int j = tx + c * TX;
+        for (int c = 0; c < RN / VB; ++c) {
+            const int j = (tx + c * TX) * VB;
             if (j >= nlim) continue;
-            T v = acc[r][c];
+            float4 v = make_float4(acc[r][2 * c].x, acc[r][2 * c].y, acc[r][2 * c + 1].x, acc[r][2 * c + 1].y);
             if (a.split == 1) {
                 if (sc.resid) {
-                    if constexpr (CPLX) {
-                        v.x = ldexpf(v.x, -sc.resid);
-                        v.y = ldexpf(v.y, -sc.resid);
-                    } else {
-                        v = ldexpf(v, -sc.resid);
-                    }
+                    v.x = ldexpf(v.x, -sc.resid);
+                    v.y = ldexpf(v.y, -sc.resid);
+                    v.z = ldexpf(v.z, -sc.resid);
+                    v.w = ldexpf(v.w, -sc.resid);
                 }
-                lmax = fmaxf(lmax, absmax(v));
+                // columns beyond the node's hold zeros
+                lmax = fmaxf(fmaxf(lmax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
             }
-            out[rowoff + j] = v;
+            if (vec) {
+                *reinterpret_cast<float4*>(row + j) = v;
+            } else if constexpr (CPLX) {
+                row[j] = make_float2(v.x, v.y);
+                if (j + 1 < nlim) row[j + 1] = make_float2(v.z, v.w);
+            } else {
+                row[j] = v.x;
+                if (j + 1 < nlim) row[j + 1] = v.y;
+                if (j + 2 < nlim) row[j + 2] = v.z;
+                if (j + 3 < nlim) row[j + 3] = v.w;
+            }
         }
     }
     if (a.split == 1) {
@@ -534,11 +696,11 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN))
 // epilogue.  G threads share one output (G = 1 when the outputs alone fill
 // the GPU): thread g sums splits [g*split/G, (g+1)*split/G) in eight
 // independent chains, then the G sums are added in g order.
-template <bool CPLX>
-__global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ TileArgs a, int G) {
+template <class ARGS, bool CPLX>
+__global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ ARGS a, int G) {
     using T = typename VT<CPLX>::T;
     __shared__ T red[256];
-    const int64_t plane_sz = (int64_t)a.nbatch << (a.nm + a.nn);
+    const int64_t plane_sz = a.nbatch * size_m(a) * size_n(a);
     const View vw = inst_view(a, blockIdx.y, (int)sizeof(T));
     if (!vw.live) return;
     const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && threadIdx.x == 0);
@@ -968,13 +1130,58 @@ __global__ void __launch_bounds__(256)
 // launchers
 // --------------------------------------------------------------------------
 
-template <bool CPLX, int TM, int TN, int TK, int RM, int RN>
-static cudaError_t launch_cfg(const TileArgs& a, cudaStream_t s) {
-    const int64_t M = 1ll << a.nm, N = 1ll << a.nn;
+inline int64_t host_m(const TileArgs& a) { return int64_t(1) << a.nm; }
+inline int64_t host_n(const TileArgs& a) { return int64_t(1) << a.nn; }
+inline int64_t host_m(const GenericArgs& a) { return a.M; }
+inline int64_t host_n(const GenericArgs& a) { return a.N; }
+
+template <class ARGS, bool CPLX, int TM, int TN, int TK, int RM, int RN, int MINB>
+static cudaError_t launch_cfg(const ARGS& a, cudaStream_t s) {
+    const int64_t M = host_m(a), N = host_n(a);
     const int64_t tiles = ((M + TM - 1) / TM) * ((N + TN - 1) / TN);
     const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
     dim3 grid((unsigned)tiles, 1, (unsigned)(a.nbatch * a.split * ni));
-    k_tile<CPLX, TM, TN, TK, RM, RN><<<grid, (TM / RM) * (TN / RN), 0, s>>>(a);
+    constexpr size_t smem = TileSmem<ARGS, CPLX, TM, TN, TK>::bytes;
+    auto* kern = k_tile<ARGS, CPLX, TM, TN, TK, RM, RN, MINB>;
+    static bool configured = false;
+    if (!configured) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    kern<<<grid, (TM / RM) * (TN / RN), smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <class ARGS, bool CPLX>
+static cudaError_t launch_shape(const ARGS& a, cudaStream_t s) {
+    switch (a.cfg) {
+        case kTile64x64: return launch_cfg<ARGS, CPLX, 64, 64, 8, 8, 4, CPLX ? 3 : 4>(a, s);
+        case kTile16x256: return launch_cfg<ARGS, CPLX, 16, 256, 8, 4, 4, 2>(a, s);
+        case kTile4x1024: return launch_cfg<ARGS, CPLX, 4, 1024, 4, 4, 4, 2>(a, s);
+        case kTile256x16: return launch_cfg<ARGS, CPLX, 256, 16, 8, 4, 4, 2>(a, s);
+        case kTile128x64: return launch_cfg<ARGS, CPLX, 128, 64, 8, 8, CPLX ? 4 : 8, CPLX ? 2 : 3>(a, s);
+        case kTile128x128:
+            if constexpr (!CPLX) return launch_cfg<ARGS, CPLX, 128, 128, 8, 8, 8, 2>(a, s);
+            else return cudaErrorInvalidValue;
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// The K parts' partials summed in a fixed order.
+template <class ARGS, bool CPLX>
+static cudaError_t launch_reduce(const ARGS& a, cudaStream_t s) {
+    const int64_t n = a.nbatch * host_m(a) * host_n(a);
+    const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
+    // threads per output: enough that outputs x G fill the GPU's threads;
+    // chosen from one instance's outputs, so that every instance sums in the
+    // same order however many run side by side (results independent of the
+    // slice batch)
+    int G = 1;
+    while (G < 32 && G * 2 <= a.split && n * G < (int64_t)sm_count() * 256 * 4) G *= 2;
+    int64_t blocks = (n + 256 / G - 1) / (256 / G);
+    if (blocks > sm_count() * 8) blocks = sm_count() * 8;
+    k_split_reduce<ARGS, CPLX><<<dim3((unsigned)blocks, (unsigned)ni), 256, 0, s>>>(a, G);
     return cudaGetLastError();
 }
 
@@ -1040,46 +1247,34 @@ static DotPlan make_dot_plan(const TileArgs& a) {
 template <bool CPLX>
 static cudaError_t launch_tile_t(const TileArgs& a, cudaStream_t s) {
     cudaError_t e;
-    switch (a.cfg) {
-        case kTile64x64: e = launch_cfg<CPLX, 64, 64, 16, 4, 4>(a, s); break;
-        case kTile16x256: e = launch_cfg<CPLX, 16, 256, 16, 4, 4>(a, s); break;
-        case kTile4x1024: e = launch_cfg<CPLX, 4, 1024, 4, 4, 4>(a, s); break;
-        case kTile256x16: e = launch_cfg<CPLX, 256, 16, 16, 4, 4>(a, s); break;
-        case kTile128x64: e = launch_cfg<CPLX, 128, 64, 16, 8, 4>(a, s); break;
-        case kTileDot: {
-            const int64_t outs = 1ll << (a.nm + a.nn);
-            const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
-            constexpr size_t smem = dot_smem_bytes<CPLX>();
-            static bool configured = false;
-            if (!configured) {
-                e = cudaFuncSetAttribute(k_dot<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-                configured = true;
-            }
-            k_dot<CPLX><<<dim3((unsigned)outs, (unsigned)a.nbatch, (unsigned)(a.split * ni)), 256, smem, s>>>(
-                a, make_dot_plan(a));
-            e = cudaGetLastError();
-            break;
+    if (a.cfg == kTileDot) {
+        const int64_t outs = 1ll << (a.nm + a.nn);
+        const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
+        constexpr size_t smem = dot_smem_bytes<CPLX>();
+        static bool configured = false;
+        if (!configured) {
+            e = cudaFuncSetAttribute(k_dot<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            configured = true;
         }
-        default: return cudaErrorInvalidValue;
+        k_dot<CPLX><<<dim3((unsigned)outs, (unsigned)a.nbatch, (unsigned)(a.split * ni)), 256, smem, s>>>(
+            a, make_dot_plan(a));
+        e = cudaGetLastError();
+    } else {
+        e = launch_shape<TileArgs, CPLX>(a, s);
     }
     if (e != cudaSuccess || a.split == 1) return e;
-    const int64_t n = (int64_t)a.nbatch << (a.nm + a.nn);
-    const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
-    // threads per output: enough that outputs x G fill the GPU's threads;
-    // chosen from one instance's outputs, so that every instance sums in the
-    // same order however many run side by side (results independent of the
-    // slice batch)
-    int G = 1;
-    while (G < 32 && G * 2 <= a.split && n * G < (int64_t)sm_count() * 256 * 4) G *= 2;
-    int64_t blocks = (n + 256 / G - 1) / (256 / G);
-    if (blocks > sm_count() * 8) blocks = sm_count() * 8;
-    k_split_reduce<CPLX><<<dim3((unsigned)blocks, (unsigned)ni), 256, 0, s>>>(a, G);
-    return cudaGetLastError();
+    return launch_reduce<TileArgs, CPLX>(a, s);
 }
 
 cudaError_t launch_tile(const TileArgs& a, bool is_c, cudaStream_t s) {
     return is_c ? launch_tile_t<true>(a, s) : launch_tile_t<false>(a, s);
+}
+
+cudaError_t launch_tile_any(const GenericArgs& a, bool is_c, cudaStream_t s) {
+    const cudaError_t e = is_c ? launch_shape<GenericArgs, true>(a, s) : launch_shape<GenericArgs, false>(a, s);
+    if (e != cudaSuccess || a.split == 1) return e;
+    return is_c ? launch_reduce<GenericArgs, true>(a, s) : launch_reduce<GenericArgs, false>(a, s);
 }
 
 cudaError_t launch_wave(const WaveItem* items, int n_items, const TileArgs* descs,
