@@ -203,13 +203,14 @@ struct PackPlan {
 };
 
 // Tile plan of an inner-product node (k_dot), computed on the host: a tile
-// is 2^t K entries; entry e in A's order is at A offset sum of a_add and
-// K-order index sum of ca_add over its set bits (likewise for B); the u
-// remaining K bits step between tiles.
+// is 2^t K entries of every row of either operand; entry e in A's order is at
+// A offset sum of a_add over its set bits, and at K position (low 16 bits) and
+// row (from bit 16) sum of ca_add (likewise for B); the u remaining K bits step
+// between tiles.
 struct DotPlan {
     int t, u;
-    int64_t a_add[10], b_add[10];
-    int32_t ca_add[10], cb_add[10];
+    int64_t a_add[16], b_add[16];
+    int32_t ca_add[16], cb_add[16];
     int64_t rest_a[kMaxBits], rest_b[kMaxBits];
 };
 

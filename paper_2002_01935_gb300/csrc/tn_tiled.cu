@@ -747,28 +747,40 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
     if (a.t_done && threadIdx.x == 0) atomicMax(a.t_done, global_ns());
 }
 
-// Tiny output, long K: grid (outputs, batch, K splits); each CTA reduces its
-// K range in a fixed order; with several splits the partials go to P and
-// k_split_reduce sums them in split order (deterministic).
-// Inner-product node (few outputs, long K): out[b,m,n] = sum_k A[.., k] B[.., k].
-// The K range is cut into tiles of up to 2^(2 kDotLow) entries holding the
-// kDotLow lowest strides of A, the kDotLow lowest of B and the next K bits;
-// every tile is read twice in the operands' own orders (consecutive threads,
+// Inner-product node (at most 64 outputs, long K): out[b,m,n] = sum_k A[.., k] B[.., k].
+// One CTA computes all outputs of a batch entry over its part of K, so that
+// either operand is read once.  K is cut into tiles of 2^t entries that hold
+// the lowest strides of A and of B; a tile of an operand -- its rows times the
+// tile's K entries -- is read in the operand's own order (consecutive threads,
 // consecutive addresses) by asynchronous copies straight into shared memory,
-// where each entry lands at its K position, and multiplied there.  A ring of
-// kDotStages tiles keeps two tiles of copies in flight per CTA while a third
-// is multiplied; the tile base offsets follow the tile index by its carry
-// chain.  blockIdx.x: output, y: batch entry, z: K part x instance.
+// where each entry lands at its row and K position.  A ring of kDotStages
+// tiles keeps two tiles of copies in flight per CTA while a third is
+// multiplied; the tile base offsets follow the tile index by its carry chain.
+// Each thread multiplies RM x RN outputs over every LPG-th K entry (LPG threads
+// share a group of outputs).  blockIdx.x: `parts` consecutive K parts (short
+// parts share a CTA and its setup, each with its own partial, so that the sum
+// does not depend on the grid), y: batch entry, z: instance.
+// Bound by memory.  A node of 16 outputs over K = 2^18 in eight copies, 134 MB:
+// 262 us with one CTA per output and K part, which read each operand once per
+// row or column of the other, 80 now (call 3562 -> 2819 us, four of them).
+// One output over K = 2^28 (4.3 GB): 750 us as before, 85% of the HBM copy rate.
 constexpr int kDotLow = 5;
-constexpr int kDotTile = 1 << (2 * kDotLow);
-constexpr int kDotPad = kDotTile + kDotTile / 32;  // one padding entry per 32: no bank conflicts
 constexpr int kDotStages = 3;
+constexpr int kDotEntries = 4096;                            // of both operands in a stage
+// copies per thread and tile: one output needs half (its tile is 2^10 entries of each operand)
+__host__ __device__ constexpr int dot_per(int rm, int rn) { return kDotEntries / 256 / (rm * rn == 1 ? 2 : 1); }
+// one padding entry per 32 of a row and one a row: no bank conflicts along K or along the rows
+__host__ __device__ constexpr int dot_row(int t) { return (1 << t) + (1 << t) / 32 + 1; }
 
-template <bool CPLX>
-constexpr size_t dot_smem_bytes() {
-    using T = typename VT<CPLX>::T;
-    return (size_t)kDotStages * 2 * kDotPad * sizeof(T) + 2 * kDotTile * sizeof(int32_t) +
-           2 * kDotTile * sizeof(uint16_t);
+// K entries of a tile (log2) for an M x N node
+inline int dot_tile_bits(int nm, int nn, int nk) {
+    int t = 2 * kDotLow;
+    while (((int64_t(1) << nm) + (int64_t(1) << nn)) << t > kDotEntries) --t;
+    return t < nk ? t : nk;
+}
+
+inline size_t dot_smem_bytes(const DotPlan& dp, int rows, size_t esz) {
+    return (size_t)kDotStages * rows * dot_row(dp.t) * esz;
 }
 
 // asynchronous global -> shared copy of one 4- or 8-byte element
@@ -783,52 +795,83 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <bool CPLX>
-__global__ void __launch_bounds__(256) k_dot(const __grid_constant__ TileArgs a, const __grid_constant__ DotPlan dp) {
+__device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float2 shfl_xor(float2 v, int o) { return make_float2(shfl_xor(v.x, o), shfl_xor(v.y, o)); }
+
+template <bool CPLX, int RM, int RN>
+__global__ void __launch_bounds__(256, RM * RN == 1 ? 4 : 2)
+    k_dot(const __grid_constant__ TileArgs a, const __grid_constant__ DotPlan dp, int parts) {
     using T = typename VT<CPLX>::T;
+    constexpr int kDotPer = dot_per(RM, RN);
     extern __shared__ __align__(16) unsigned char dot_smem[];
-    T* const stg = reinterpret_cast<T*>(dot_smem);  // [stage][A, B][kDotPad]
-    int32_t* const offA = reinterpret_cast<int32_t*>(dot_smem + (size_t)kDotStages * 2 * kDotPad * sizeof(T));
-    int32_t* const offB = offA + kDotTile;
-    uint16_t* const canA = reinterpret_cast<uint16_t*>(offB + kDotTile);
-    uint16_t* const canB = canA + kDotTile;
-    __shared__ T red[256];
-    const int64_t N = 1ll << a.nn, M = 1ll << a.nm;
-    const int64_t m = (int64_t)blockIdx.x / N, n = (int64_t)blockIdx.x % N;
+    T* const stg = reinterpret_cast<T*>(dot_smem);  // [stage][rows of A, then of B][dot_row]
+    __shared__ T red[8][64];
+    const int tid = threadIdx.x;
+    const int N = 1 << a.nn, M = 1 << a.nm;
     const int64_t b = blockIdx.y;
-    const int sp = blockIdx.z % a.split;
-    const View vw = inst_view(a, blockIdx.z / a.split, (int)sizeof(T));
+    const View vw = inst_view(a, blockIdx.z, (int)sizeof(T));
     if (!vw.live) return;
-    const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && sp == 0 && threadIdx.x == 0);
+    const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && tid == 0);
     const int t = dp.t, u = dp.u, tsz = 1 << t;
-    for (int e = threadIdx.x; e < tsz; e += blockDim.x) {
-        int64_t xa = 0, xb = 0;
-        int ca = 0, cb = 0;
-        for (int w = 0; w < t; ++w)
-            if ((e >> w) & 1) {
-                xa += dp.a_add[w];
-                xb += dp.b_add[w];
-                ca += dp.ca_add[w];
-                cb += dp.cb_add[w];
-            }
-        offA[e] = (int32_t)xa;  // within one operand: the planner keeps tiled operands below 2^31 entries
-        offB[e] = (int32_t)xb;
-        canA[e] = (uint16_t)(ca + (ca >> 5));
-        canB[e] = (uint16_t)(cb + (cb >> 5));
+    const int row = dot_row(t), stage_sz = (M + N) * row;
+    // this thread's copies of a tile: entries of A in A's order, then of B
+    const int n_a = M << t, n_ab = (M + N) << t;
+    int off[kDotPer];
+    uint16_t pos[kDotPer];
+    // entries e = tid + 256 r of an operand (at most 12 bits; offsets within
+    // one operand: the planner keeps it below 2^31 entries).  Bits 0-7 are the
+    // thread's and are placed once per operand where B's entries start on a
+    // multiple of 256; every table index is a constant.
+    const int wa = t + a.nm, wb = t + a.nn;
+    auto place_a = [&](int e, int w, int& o, int& c) {
+        if (w < wa && ((e >> w) & 1)) {
+            o += (int)dp.a_add[w];
+            c += dp.ca_add[w];
+        }
+    };
+    auto place_b = [&](int e, int w, int& o, int& c) {
+        if (w < wb && ((e >> w) & 1)) {
+            o += (int)dp.b_add[w];
+            c += dp.cb_add[w];
+        }
+    };
+    const bool even = n_a >= 256;
+    int oa = 0, ca = 0, ob = 0, cb = M << 16;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        place_a(tid, w, oa, ca);
+        if (even) place_b(tid, w, ob, cb);
     }
-    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kDotPer; ++r) {
+        const int e0 = tid + r * 256;
+        int o = oa, c = ca;
+        if (e0 < n_a) {
+#pragma unroll
+            for (int w = 8; w < 12; ++w) place_a(e0, w, o, c);
+        } else {
+            o = ob;
+            c = cb;
+            if (!even) {
+#pragma unroll
+                for (int w = 0; w < 8; ++w) place_b(e0 - n_a, w, o, c);
+            }
+#pragma unroll
+            for (int w = 8; w < 12; ++w) place_b(e0 - n_a, w, o, c);
+        }
+        off[r] = o;
+        const int k = c & 0xffff;
+        pos[r] = (uint16_t)((c >> 16) * row + k + (k >> 5));
+    }
     const int64_t slice = vw.slice;
-    const int64_t baseA =
-        slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb) + scatter_bits(m, a.a_m, a.nm);
-    const int64_t baseB =
-        slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb) + scatter_bits(n, a.b_n, a.nn);
-    const T* A = reinterpret_cast<const T*>(vw.A);
-    const T* B = reinterpret_cast<const T*>(vw.B);
+    const T* A = reinterpret_cast<const T*>(vw.A) + slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb);
+    const T* B = reinterpret_cast<const T*>(vw.B) + slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb);
     const int64_t n_tiles = int64_t(1) << u;
     const int64_t per = (n_tiles + a.split - 1) / a.split;
-    const int64_t t0 = (int64_t)sp * per, t1 = min64(n_tiles, t0 + per);
+    int left = (int)min64(per, 1 << 30);  // tiles to the end of the current part
+    const int64_t t0 = (int64_t)blockIdx.x * parts * per, t1 = min64(n_tiles, t0 + parts * per);
     // offsets of the next tile to copy; advanced tile by tile along the carry chain
-    int64_t nt = t0, ba = baseA, bb = baseB;
+    int64_t nt = t0, ba = 0, bb = 0;
     for (int j = 0; j < u; ++j)
         if ((t0 >> j) & 1) {
             ba += dp.rest_a[j];
@@ -836,15 +879,11 @@ __global__ void __launch_bounds__(256) k_dot(const __grid_constant__ TileArgs a,
         }
     auto issue = [&](int stage) {
         if (nt < t1) {
-            T* sA = stg + (size_t)stage * 2 * kDotPad;
-            T* sB = sA + kDotPad;
+            T* st = stg + (size_t)stage * stage_sz;
 #pragma unroll
-            for (int r = 0; r < kDotTile / 256; ++r) {
-                const int e = threadIdx.x + r * 256;
-                if (e < tsz) {
-                    cp_async_elem<sizeof(T)>(sA + canA[e], A + ba + offA[e]);
-                    cp_async_elem<sizeof(T)>(sB + canB[e], B + bb + offB[e]);
-                }
+            for (int r = 0; r < kDotPer; ++r) {
+                const int e = tid + r * 256;
+                if (e < n_ab) cp_async_elem<sizeof(T)>(st + pos[r], (e < n_a ? A + ba : B + bb) + off[r]);
             }
             int j = 0;
             while (j < u && ((nt >> j) & 1)) {
@@ -862,54 +901,76 @@ __global__ void __launch_bounds__(256) k_dot(const __grid_constant__ TileArgs a,
     };
 #pragma unroll
     for (int q = 0; q < kDotStages - 1; ++q) issue(q);
-    T acc0 = zero<T>(), acc1 = zero<T>();
+    // output groups: LPG consecutive threads share one
+    const int groups = (M / RM) * (N / RN), lpg = 256 / groups;
+    const int g = tid / lpg, lane = tid % lpg;
+    const int gm = g / (N / RN) * RM, gn = g % (N / RN) * RN;
+    T acc[RM][RN];
+#pragma unroll
+    for (int r = 0; r < RM; ++r)
+#pragma unroll
+        for (int c = 0; c < RN; ++c) acc[r][c] = zero<T>();
     int stage = 0;
     for (int64_t tile = t0; tile < t1; ++tile) {
         issue((stage + kDotStages - 1) % kDotStages);
         cp_async_wait<kDotStages - 1>();  // this thread's copies of `tile` have landed
         __syncthreads();                  // ... and every other thread's
-        const T* sA = stg + (size_t)stage * 2 * kDotPad;
-        const T* sB = sA + kDotPad;
+        const T* sA = stg + (size_t)stage * stage_sz + gm * row;
+        const T* sB = stg + (size_t)stage * stage_sz + (M + gn) * row;
+#pragma unroll 4
+        for (int i = lane; i < tsz; i += lpg) {
+            const int ip = i + (i >> 5);
+            T av[RM], bv[RN];
 #pragma unroll
-        for (int r = 0; r < kDotTile / 256; ++r) {
-            const int i = threadIdx.x + r * 256;
-            if (i < tsz) {
-                const int ip = i + (i >> 5);
-                if (r & 1) fma_acc(acc1, cmul(sA[ip], sc.fa, a.conj_a), cmul(sB[ip], sc.fb, a.conj_b));
-                else fma_acc(acc0, cmul(sA[ip], sc.fa, a.conj_a), cmul(sB[ip], sc.fb, a.conj_b));
-            }
+            for (int r = 0; r < RM; ++r) av[r] = cmul(sA[r * row + ip], sc.fa, a.conj_a);
+#pragma unroll
+            for (int c = 0; c < RN; ++c) bv[c] = cmul(sB[c * row + ip], sc.fb, a.conj_b);
+#pragma unroll
+            for (int r = 0; r < RM; ++r)
+#pragma unroll
+                for (int c = 0; c < RN; ++c) fma_acc(acc[r][c], av[r], bv[c]);
         }
         __syncthreads();  // the stage is refilled by the next iteration's copies
         stage = (stage + 1) % kDotStages;
-    }
-    cp_async_wait<0>();
-    // fixed-order block reduction
-    red[threadIdx.x] = add(acc0, acc1);
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] = add(red[threadIdx.x], red[threadIdx.x + s]);
+        if (--left && tile + 1 < t1) continue;
+        left = (int)min64(per, 1 << 30);
+        // end of a K part.  Fixed-order reduction: the group's lanes of a
+        // warp, then its warps
+        const int span = lpg < 32 ? lpg : 32;
+#pragma unroll
+        for (int r = 0; r < RM; ++r)
+#pragma unroll
+            for (int c = 0; c < RN; ++c) {
+                T v = acc[r][c];
+                for (int o = span >> 1; o > 0; o >>= 1) v = add(v, shfl_xor(v, o));
+                if (lane % 32 == 0) red[lane / 32][(gm + r) * N + gn + c] = v;
+                acc[r][c] = zero<T>();
+            }
         __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        T v = red[0];
-        const int64_t o = (b * M + m) * N + n;
-        if (a.split > 1) {
-            reinterpret_cast<T*>(vw.P)[(int64_t)sp * (a.nbatch * M * N) + o] = v;
-            return;
-        }
-        if (sc.resid) {
-            if constexpr (CPLX) {
-                v.x = ldexpf(v.x, -sc.resid);
-                v.y = ldexpf(v.y, -sc.resid);
+        if (tid < M * N) {
+            T v = red[0][tid];
+            for (int w = 1; w < (lpg + 31) / 32; ++w) v = add(v, red[w][tid]);
+            const int64_t o = b * M * N + tid;
+            if (a.split > 1) {
+                reinterpret_cast<T*>(vw.P)[tile / per * (a.nbatch * M * N) + o] = v;
             } else {
-                v = ldexpf(v, -sc.resid);
+                if (sc.resid) {
+                    if constexpr (CPLX) {
+                        v.x = ldexpf(v.x, -sc.resid);
+                        v.y = ldexpf(v.y, -sc.resid);
+                    } else {
+                        v = ldexpf(v, -sc.resid);
+                    }
+                }
+                reinterpret_cast<T*>(vw.C)[o] = v;
+                const float mx = absmax(v);
+                if (mx > 0.f) atomicMax(vw.sc.max_c, __float_as_uint(mx));
+                if (a.t_done) atomicMax(a.t_done, global_ns());
             }
         }
-        reinterpret_cast<T*>(vw.C)[o] = v;
-        float mx = absmax(v);
-        if (mx > 0.f) atomicMax(vw.sc.max_c, __float_as_uint(mx));
-        if (a.t_done) atomicMax(a.t_done, global_ns());
+        // (the next part's first barrier comes before its reduction writes red)
     }
+    cp_async_wait<0>();
 }
 
 // One launch for the small nodes of one or more consecutive tree levels.
@@ -1185,29 +1246,40 @@ static cudaError_t launch_reduce(const ARGS& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Tile bits of an inner-product node: the kDotLow lowest strides of each
-// operand, then the lowest K positions, up to 2 * kDotLow bits; each
-// operand's order of them (ascending stride, absent bits last).
+// Tile plan of an inner-product node.  Tile bits of K: those among the kDotLow
+// lowest strides of either operand (its row bits, which are in every tile, take
+// part in that), the operands in turn, then the lowest K positions.  Then each
+// operand's order of its row and tile bits (ascending stride, absent bits last).
 static DotPlan make_dot_plan(const TileArgs& a) {
     DotPlan dp;
     memset(&dp, 0, sizeof(dp));
-    const int nk = a.nk;
+    const int nk = a.nk, t_max = dot_tile_bits(a.nm, a.nn, a.nk);
+    // by stride: K position, or -2 - i for row bit i; -1: none
     int by[2][64];
     for (int q = 0; q < 64; ++q) by[0][q] = by[1][q] = -1;
-    bool in[kMaxBits] = {};
     for (int p = 0; p < nk; ++p) {
         if (a.a_k[p] < 64) by[0][a.a_k[p]] = p;
         if (a.b_k[p] < 64) by[1][a.b_k[p]] = p;
     }
-    int cnt = 0;
-    for (int side = 0; side < 2; ++side)
-        for (int q = 0, r = 0; q < 64 && r < kDotLow; ++q)
-            if (by[side][q] >= 0) {
-                if (!in[by[side][q]]) ++cnt;
-                in[by[side][q]] = true;
-                ++r;
+    for (int i = 0; i < a.nm; ++i) by[0][a.a_m[i]] = -2 - i;
+    for (int i = 0; i < a.nn; ++i) by[1][a.b_n[i]] = -2 - i;
+    bool in[kMaxBits] = {};
+    int cnt = 0, q[2] = {0, 0}, low[2] = {0, 0};
+    for (bool more = true; more && cnt < t_max;) {
+        more = false;
+        for (int side = 0; side < 2; ++side) {
+            while (q[side] < 64 && by[side][q[side]] == -1) ++q[side];
+            if (q[side] >= 64 || low[side] >= kDotLow || cnt >= t_max) continue;
+            const int p = by[side][q[side]++];
+            ++low[side];
+            more = true;
+            if (p >= 0 && !in[p]) {
+                in[p] = true;
+                ++cnt;
             }
-    for (int p = 0; p < nk && cnt < 2 * kDotLow; ++p)
+        }
+    }
+    for (int p = 0; p < nk && cnt < t_max; ++p)
         if (!in[p]) {
             in[p] = true;
             ++cnt;
@@ -1225,44 +1297,67 @@ static DotPlan make_dot_plan(const TileArgs& a) {
         }
     }
     for (int side = 0; side < 2; ++side) {
-        const uint8_t* sh = side ? a.b_k : a.a_k;
-        int order[2 * kDotLow];
+        int64_t* add = side ? dp.b_add : dp.a_add;
+        int32_t* cad = side ? dp.cb_add : dp.ca_add;
         int w = 0;
-        for (int q = 0; q < 64; ++q)
-            if (by[side][q] >= 0 && in[by[side][q]]) order[w++] = pos[by[side][q]];
-        for (int j = 0; j < t; ++j)
-            if (sh[tk[j]] >= 64) order[w++] = j;
-        for (int i = 0; i < t; ++i) {
-            const int p = tk[order[i]];
-            const int64_t add = sh[p] != kNoBit ? int64_t(1) << sh[p] : 0;
-            (side ? dp.b_add : dp.a_add)[i] = add;
-            (side ? dp.cb_add : dp.ca_add)[i] = 1 << order[i];
+        for (int s = 0; s < 64; ++s) {
+            const int p = by[side][s];
+            if (p == -1 || (p >= 0 && !in[p])) continue;
+            add[w] = int64_t(1) << s;
+            cad[w++] = p >= 0 ? 1 << pos[p] : 1 << (16 - 2 - p);  // K position, or row << 16
         }
+        for (int j = 0; j < t; ++j)  // tile bits the operand lacks repeat its entries
+            if ((side ? a.b_k : a.a_k)[tk[j]] >= 64) {
+                add[w] = 0;
+                cad[w++] = 1 << j;
+            }
     }
     dp.t = t;
     dp.u = u;
     return dp;
 }
 
+template <bool CPLX, int RM, int RN>
+static cudaError_t launch_dot_rc(const TileArgs& a, cudaStream_t s) {
+    using T = typename VT<CPLX>::T;
+    const DotPlan dp = make_dot_plan(a);
+    const size_t smem = dot_smem_bytes(dp, (1 << a.nm) + (1 << a.nn), sizeof(T));
+    static bool configured = false;
+    if (!configured) {
+        const cudaError_t e = cudaFuncSetAttribute(k_dot<CPLX, RM, RN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(kDotStages * (kDotEntries + kDotEntries / 16) * sizeof(T)));
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
+    // parts of fewer than eight tiles: as many per CTA as make one round of
+    // resident CTAs (longer ones balance better over many rounds)
+    const int64_t slots = (int64_t)sm_count() * (RM * RN == 1 ? 4 : 2), total = (int64_t)a.split * a.nbatch * ni;
+    int parts = 1;
+    if (((int64_t(1) << dp.u) + a.split - 1) / a.split < 8)
+        parts = (int)std::min<int64_t>((total + slots - 1) / slots, a.split);
+    const unsigned blocks = (unsigned)((a.split + parts - 1) / parts);
+    k_dot<CPLX, RM, RN><<<dim3(blocks, (unsigned)a.nbatch, (unsigned)ni), 256, smem, s>>>(a, dp, parts);
+    return cudaGetLastError();
+}
+
+template <bool CPLX, int RM>
+static cudaError_t launch_dot_r(const TileArgs& a, cudaStream_t s) {
+    if (a.nn == 0) return launch_dot_rc<CPLX, RM, 1>(a, s);
+    if (a.nn == 1) return launch_dot_rc<CPLX, RM, 2>(a, s);
+    return launch_dot_rc<CPLX, RM, 4>(a, s);
+}
+
+template <bool CPLX>
+static cudaError_t launch_dot(const TileArgs& a, cudaStream_t s) {
+    if (a.nm == 0) return launch_dot_r<CPLX, 1>(a, s);
+    if (a.nm == 1) return launch_dot_r<CPLX, 2>(a, s);
+    return launch_dot_r<CPLX, 4>(a, s);
+}
+
 template <bool CPLX>
 static cudaError_t launch_tile_t(const TileArgs& a, cudaStream_t s) {
-    cudaError_t e;
-    if (a.cfg == kTileDot) {
-        const int64_t outs = 1ll << (a.nm + a.nn);
-        const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
-        constexpr size_t smem = dot_smem_bytes<CPLX>();
-        static bool configured = false;
-        if (!configured) {
-            e = cudaFuncSetAttribute(k_dot<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
-        k_dot<CPLX><<<dim3((unsigned)outs, (unsigned)a.nbatch, (unsigned)(a.split * ni)), 256, smem, s>>>(
-            a, make_dot_plan(a));
-        e = cudaGetLastError();
-    } else {
-        e = launch_shape<TileArgs, CPLX>(a, s);
-    }
+    const cudaError_t e = a.cfg == kTileDot ? launch_dot<CPLX>(a, s) : launch_shape<TileArgs, CPLX>(a, s);
     if (e != cudaSuccess || a.split == 1) return e;
     return launch_reduce<TileArgs, CPLX>(a, s);
 }
