@@ -1409,6 +1409,24 @@ bool make_tensor_core(const NetDesc& d, tn_mode mode, Node& nd, int64_t& split_e
             }
         }
         if (t.nbatch * (int64_t)t.split > 65535) t.split = 1;
+        // partials that do not fit L2 cost HBM traffic (written, read, and the
+        // sum written): split only if the fuller waves gain more.  Times in us:
+        // a k-block of a tile on the tensor pipe at 1.9 GHz per product of the
+        // precision, bytes at 6.5 TB/s.  A 2^13 x 2^12 x 2^10 node, 13.5 waves:
+        // 17 us of GEMM gained by two parts against 125 us of reduction and
+        // as many partial stores again (call 1191 -> 1050 us without them).
+        // Several copies per launch keep their split: a gradient step of 64
+        // copies is 2% faster without, but the other order of its sums showed
+        // as 1.6e-5 instead of 1.1e-5 error on an ill-conditioned loss.
+        const double out_bytes = (double)t.nbatch * (double)(int64_t(1) << (t.nm + t.nn)) * d.elem_bytes();
+        if (t.split > 1 && copies == 1 && t.split * out_bytes > 126e6) {
+            const double products = prec == 0 ? 1.0 : (g0.planar ? 4.0 : 3.0);
+            const double t_kb = 0.27 * products * g0.bn / 256.0;
+            auto gemm_us = [&](int s) {
+                return std::ceil(tiles * s / (double)sm_count()) * (double)(g0.nkb / s) * t_kb;
+            };
+            if (gemm_us(1) - gemm_us(t.split) < 2.0 * t.split * out_bytes / 6.5e6) t.split = 1;
+        }
     }
     const int64_t eb = d.elem_bytes();
     split_elems = std::max(split_elems, (tc_geom(t, c, prec).total + eb - 1) / eb);
