@@ -30,7 +30,7 @@ class _Contract(torch.autograd.Function):
         leaves = [t.detach().contiguous() for t in leaves]
         tnw.set_tensors(leaves)
         m, e = tnw.contract(pairs, sliced, mode)
-        value = m * torch.pow(torch.tensor(2.0, dtype=torch.float64, device=m.device), e.double())
+        value = m * torch.pow(2.0, e.double())
         ctx.tnw, ctx.pairs, ctx.sliced, ctx.mode = tnw, pairs, sliced, mode
         ctx.save_for_backward(*leaves)
         return value
@@ -71,8 +71,7 @@ class _ContractBatch(torch.autograd.Function):
         # forward in the sweep's state with the intermediates kept: the
         # backward reuses them unless another gradient call intervened
         mant, ex, token = tnw.contract_instances_keep(pairs, mode, n_batch, strides)
-        value = mant * torch.pow(torch.tensor(2.0, dtype=torch.float64, device=mant.device),
-                                 ex.double()).unsqueeze(1)
+        value = mant * torch.pow(2.0, ex.double()).unsqueeze(1)
         if tnw.dtype == binding.TN_C64:
             value = torch.complex(value[:, 0], value[:, 1])
         else:

@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import math
+import operator
 import os
 from typing import Dict, List, Optional, Sequence, Tuple
 
@@ -171,7 +172,11 @@ def _hold(t, stream) -> None:
 # times, and flattening a few hundred pairs costs more than the device work
 # of a small network.  An entry is reused only if the call's pair list
 # equals the kept tuple copy (tuples are immutable, so any change is seen).
-_tree_cache: Dict[int, Tuple[list, np.ndarray]] = {}
+# A list of tuples of integers is compared as a whole with a copy of the list
+# that holds the same tuples: a pair that was replaced is another object and
+# is compared by value, one that was not cannot have changed (2 us for 400
+# pairs, 45 entry by entry).
+_tree_cache: Dict[int, Tuple[list, np.ndarray, Optional[list]]] = {}
 
 
 # leaves per handle made here: the library reads 2 * (n_tensors - 1) tree
@@ -199,6 +204,8 @@ def _tree(pairs):
     if not isinstance(pairs, list):
         return _arr([x for p in pairs for x in p] or [0], np.int32)
     hit = _tree_cache.get(id(pairs))
+    if hit is not None and hit[2] is not None and hit[2] == pairs:
+        return hit[1]
     if hit is not None and len(hit[0]) == len(pairs):
         # element by element, so that a list of lists (e.g. pairs read from
         # JSON) or of numpy rows is reused like a list of tuples
@@ -212,7 +219,8 @@ def _tree(pairs):
     arr = _arr([x for p in pairs for x in p] or [0], np.int32)
     if len(_tree_cache) >= 64:
         _tree_cache.clear()
-    _tree_cache[id(pairs)] = ([(int(p[0]), int(p[1])) for p in pairs], arr)
+    plain = all(type(p) is tuple and len(p) == 2 and type(p[0]) is int and type(p[1]) is int for p in pairs)
+    _tree_cache[id(pairs)] = ([(int(p[0]), int(p[1])) for p in pairs], arr, list(pairs) if plain else None)
     return arr
 
 
@@ -371,6 +379,13 @@ class TensorNetwork:
         self.dims = dict(dims)
         self.open = list(open_labels)
         self.h = tn_create(self.dtype, self.labels, self.dims, self.open)
+        # entries of each leaf (structure only)
+        self._numels = []
+        for ls in self.labels:
+            n = 1
+            for l in ls:
+                n *= self.dims[l]
+            self._numels.append(int(n))
         self._keep: List = []
         if tensors is not None:
             self.set_tensors(tensors)
@@ -389,24 +404,31 @@ class TensorNetwork:
     def set_tensors(self, tensors) -> None:
         import torch
         want = torch.complex64 if self.dtype == TN_C64 else torch.float32
+        tensors = list(tensors)
         if len(tensors) > len(self.labels):
             raise TNError(TN_EINVAL, f"{len(tensors)} tensors for {len(self.labels)} leaves")
-        for v, t in enumerate(tensors):
-            # every call reads a whole leaf (stacked copies may hold more)
-            if t.numel() < self._leaf_numel(v):
-                raise TNError(TN_EINVAL, f"leaf {v}: {t.numel()} elements, the leaf has {self._leaf_numel(v)}")
+        # every call reads a whole leaf (stacked copies may hold more)
+        if not all(map(operator.ge, [t.numel() for t in tensors], self._numels)):
+            for v, t in enumerate(tensors):
+                if t.numel() < self._leaf_numel(v):
+                    raise TNError(TN_EINVAL,
+                                  f"leaf {v}: {t.numel()} elements, the leaf has {self._leaf_numel(v)}")
         self._keep = []
         attached = getattr(self, "_attached", None) or [None] * len(tensors)
+        usable = all([t.dtype == want for t in tensors]) and all([t.is_contiguous() for t in tensors])
+        keys = [(t.data_ptr(), TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST) for t in tensors] if usable else None
+        if keys is not None and keys == attached:
+            self._keep = tensors  # unchanged pointers need no call
+            return
         for v, t in enumerate(tensors):
             if t.dtype != want:
                 raise TypeError(f"leaf {v}: dtype {t.dtype}, expected {want}")
             if not t.is_contiguous():
                 raise ValueError(f"leaf {v} must be contiguous")
-            mem = TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST
+            key = keys[v] if keys is not None else (t.data_ptr(), TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST)
             self._keep.append(t)
-            key = (t.data_ptr(), mem)
-            if attached[v] != key:  # unchanged pointers need no call
-                tn_set_tensor(self.h, v, key[0], mem)
+            if attached[v] != key:
+                tn_set_tensor(self.h, v, key[0], key[1])
                 attached[v] = key
         self._attached = attached
 
@@ -419,10 +441,7 @@ class TensorNetwork:
     # instead of being accessed out of bounds.
 
     def _leaf_numel(self, v: int) -> int:
-        n = 1
-        for l in self.labels[v]:
-            n *= int(self.dims[l])
-        return n
+        return self._numels[v]
 
     def _extent(self, v: int, n_inst: int, strides) -> int:
         """Elements from leaf v's pointer that n_inst copies touch."""
@@ -432,13 +451,17 @@ class TensorNetwork:
     def _check_strides(self, n_inst: int, strides) -> None:
         if strides is not None and len(strides) != len(self.labels):
             raise TNError(TN_EINVAL, f"leaf_inst_stride needs {len(self.labels)} entries, got {len(strides)}")
-        for v, t in enumerate(self._keep):
-            if strides is not None and int(strides[v]) < 0:
+        more = max(int(n_inst) - 1, 0)
+        st = [int(x) for x in strides] if strides is not None else [0] * len(self.labels)
+        have = [t.numel() for t in self._keep]
+        if min(st) >= 0 and all(map(operator.ge, have, [more * x + k for x, k in zip(st, self._numels)])):
+            return
+        for v, n in enumerate(have):
+            if st[v] < 0:
                 raise TNError(TN_EINVAL, f"leaf {v}: negative instance stride")
             need = self._extent(v, n_inst, strides)
-            if t.numel() < need:
-                raise TNError(TN_EINVAL, f"leaf {v}: {t.numel()} elements attached, "
-                                         f"{n_inst} copies read {need}")
+            if n < need:
+                raise TNError(TN_EINVAL, f"leaf {v}: {n} elements attached, {n_inst} copies read {need}")
 
     def _check_grads(self, grads, n_inst: int = 1, strides=None) -> None:
         import torch

@@ -996,6 +996,7 @@ static tn_status configure_instances(const NetDesc& d, Plan& p, int G, int step,
         }
     }
     p.acc_args.n_inst = step == 1 ? G : 1;
+    p.graph_inst = p.graph_inst_h = -2;  // captured sequences hold the old layout
     p.cfg_inst = G;
     p.cfg_step = step;
     p.cfg_leaf_is = leaf_is;
@@ -1136,19 +1137,37 @@ static tn_status prepare_leaves(NetDesc& d, Plan& p, bool capturing, std::vector
         if (nd.cb >= 0 && nd.cb < n) p.gen[k].B = nd.tile.B = lp[nd.cb];
     }
     if (p.leaf_ptr_uploaded != lp) {
-        // the pointer table changes only when leaves are re-attached
+        // the pointer table changes only when leaves are re-attached; the
+        // pageable source is staged before the copy returns, and the stream
+        // orders it between the calls that read the table
         CK(cudaMemcpyAsync(p.leaf_ptr_dev, lp.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, stream));
-        CK(cudaStreamSynchronize(stream));
+        if (capturing) CK(cudaStreamSynchronize(stream));
         p.leaf_ptr_uploaded = lp;
     }
     return TN_OK;
 }
 
+// The pointers that a captured sequence holds: those of leaves read by nodes
+// with a launch of their own.  Waves read theirs from the device table, so
+// re-attaching the others (the output states of another bitstring, say) does
+// not recapture the graph.
+static std::vector<const void*> captured_leaves(const NetDesc& d, const Plan& p, const std::vector<const void*>& lp) {
+    std::vector<const void*> got;
+    for (const Step& st : p.steps) {
+        if (st.wave) continue;
+        const Node& nd = p.nodes[st.node];
+        for (int c : {nd.ca, nd.cb})
+            if (c >= 0 && c < d.n) got.push_back(lp[c]);
+    }
+    return got;
+}
+
 // (Re)capture the per-group graph when the leaves, the timing hooks or the
 // instance layout changed.
-static tn_status ensure_graph(const NetDesc& d, Plan& p, const std::vector<const void*>& lp, int pf,
+static tn_status ensure_graph(const NetDesc& d, Plan& p, const std::vector<const void*>& all_leaves, int pf,
                               int pc, std::string& err) {
     const bool h = pc > 0;
+    const std::vector<const void*> lp = captured_leaves(d, p, all_leaves);
     cudaGraph_t& graph = h ? p.graph_h : p.graph;
     cudaGraphExec_t& gexec = h ? p.gexec_h : p.gexec;
     std::vector<const void*>& gptrs = h ? p.graph_ptrs_h : p.graph_ptrs;
@@ -1622,8 +1641,7 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
         CK(cudaMemcpy(p.descs_dev, descs.data(), sizeof(TileArgs) * nn, cudaMemcpyHostToDevice));
     }
     p.cfg_inst = -1;
-    p.graph_ptrs.clear();
-    p.graph_ptrs_h.clear();
+    p.graph_inst = p.graph_inst_h = -2;
     p.tuned = true;
     return TN_OK;
 }

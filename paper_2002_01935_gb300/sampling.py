@@ -47,18 +47,22 @@ class OpenAmplitudes:
         self.first_out = net.n_tensors - len(self.fixed)
         self._leaves = [torch.from_numpy(np.array(t, order="C")).to(torch.complex64).cuda()
                         for t in net.tensors]
-        self._basis = torch.eye(2, dtype=torch.complex64, device="cuda")
+        self._basis = torch.eye(2, dtype=torch.complex64, device="cuda").unbind(0)
         self.tnw = binding.TensorNetwork(net.labels, net.dims, net.open, self._leaves, complex_=True)
 
     def __call__(self, x_u: Sequence[int]) -> np.ndarray:
+        import torch
         if len(x_u) != len(self.fixed):
             raise ValueError(f"x_u needs {len(self.fixed)} bits")
         leaves = list(self._leaves)
         for i, b in enumerate(x_u):
             leaves[self.first_out + i] = self._basis[int(b)]
         self.tnw.set_tensors(leaves)
-        m, e = self.tnw.contract(self.pairs, self.sliced, self.mode)
-        return m.cpu().numpy() * 2.0 ** int(e.cpu())
+        # host outputs: value and exponent come back in one copy
+        m, e = self.tnw.contract(self.pairs, self.sliced, self.mode,
+                                 out=torch.empty(self.tnw.out_shape, dtype=torch.complex128),
+                                 out_exp=torch.empty((), dtype=torch.int64))
+        return m.numpy() * 2.0 ** int(e)
 
     def close(self) -> None:
         self.tnw.close()
