@@ -3,11 +3,14 @@
 // Each network keeps its own contraction tree and host plan (Sec. 2 of arXiv
 // 2002.01935); the batch merges them into one forest: one workspace, one
 // renormalisation slot array, one leaf table and device-resident node
-// descriptors.  Execution goes by tree level across all networks: per level
-// one wave launch per storage type runs every small node of every network,
-// then the large nodes launch one by one.  A final kernel writes every
-// network's (mantissa, exponent) and the time its root completed.  The
-// whole sequence is captured once as a CUDA graph and replayed.  Sliced
+// descriptors.  The networks are dealt to up to kBatchGroups groups of about
+// equal cost, which run as parallel branches of one CUDA graph.  Within a
+// group execution goes by tree level across its networks: per level one wave
+// launch per storage type runs every small node, then the large nodes launch
+// one by one (a network's arena relies on that order; different networks share
+// nothing, and every group has its own packing and K-split buffer).  A final
+// kernel writes every network's (mantissa, exponent) and the time its root
+// completed.  The whole sequence is captured once and replayed.  Sliced
 // networks (Sec. 4.7.1: a tree sliced to a width cap) stay out of the forest:
 // after the graph, each runs its own slice loop -- its per-slice graph
 // replayed over its slices, several side by side, folded in FP64 -- on the
@@ -21,6 +24,8 @@
 #include "tn_batch.h"
 
 namespace tn {
+
+constexpr int kBatchGroups = 8;
 
 tn_status build_batch(BatchPlan& b, std::string& err) {
     const int N = (int)b.nets.size();
@@ -77,17 +82,47 @@ tn_status build_batch(BatchPlan& b, std::string& err) {
     b.split_bytes = split_bytes;
     b.descs.assign(descs, TileArgs{});
     b.gen.assign(descs, GenericArgs{});
-    // launch schedule: level by level across all networks
+    // groups: the mid-size nodes of a network (tens of microseconds on part of
+    // the GPU each) are a serial chain, so independent chains run side by side.
+    // 48 Ising networks of 40 to 100 spins: 1.88 ms as one chain, 0.76 in
+    // eight branches.  Bounded by the split buffers' memory (2 GiB in all).
+    int n_free = 0;
+    for (int i = 0; i < N; ++i) n_free += !b.is_sliced[i];
+    b.groups = std::max(1, std::min(kBatchGroups, n_free));
+    while (b.groups > 1 && b.groups * split_bytes > (int64_t(2) << 30)) --b.groups;
+    b.group_of.assign(N, 0);
+    {
+        // largest first to the cheapest group so far; a network costs its
+        // launches (about 10 us each) plus its multiply-adds at 20 TFLOP/s
+        std::vector<std::pair<double, int>> by_cost;
+        for (int i = 0; i < N; ++i) {
+            if (b.is_sliced[i]) continue;
+            double us = 0;
+            for (const Step& st : b.plans[i]->steps) us += st.wave ? 0.0 : 10.0;
+            us += b.plans[i]->C * (b.nets[i]->is_complex() ? 4e-7 : 1e-7);
+            by_cost.push_back({-us, i});
+        }
+        std::sort(by_cost.begin(), by_cost.end());
+        std::vector<double> load(b.groups, 0.0);
+        for (auto& c : by_cost) {
+            const int g = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+            b.group_of[c.second] = g;
+            load[g] -= c.first;
+        }
+    }
+    // launch schedule: per group, level by level across its networks
     b.steps.clear();
     b.items.clear();
-    for (int L = 1; L <= max_level; ++L) {
+    for (int gl = 0; gl < b.groups * max_level; ++gl) {
+        const int g = gl / max_level, L = gl % max_level + 1;
         for (int cp = 0; cp < 2; ++cp) {
             BatchStep w;
             w.wave = 1;
+            w.group = g;
             w.cplx = cp == 1;
             w.item_begin = (int)b.items.size();
             for (int i = 0; i < N; ++i) {
-                if (b.is_sliced[i] || b.nets[i]->is_complex() != w.cplx) continue;
+                if (b.is_sliced[i] || b.group_of[i] != g || b.nets[i]->is_complex() != w.cplx) continue;
                 const Plan& p = *b.plans[i];
                 for (size_t k = 0; k < p.nodes.size(); ++k) {
                     if (b.level[i][k] != L || !b.small[i][k]) continue;
@@ -107,13 +142,14 @@ tn_status build_batch(BatchPlan& b, std::string& err) {
             if (w.item_count) b.steps.push_back(w);
         }
         for (int i = 0; i < N; ++i) {
-            if (b.is_sliced[i]) continue;
+            if (b.is_sliced[i] || b.group_of[i] != g) continue;
             const Plan& p = *b.plans[i];
             for (size_t k = 0; k < p.nodes.size(); ++k) {
                 if (b.level[i][k] != L || b.small[i][k]) continue;
                 BatchStep s;
                 s.net = i;
                 s.node = (int)k;
+                s.group = g;
                 s.cplx = b.nets[i]->is_complex();
                 b.steps.push_back(s);
             }
@@ -132,7 +168,7 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
         return true;
     };
     if (!ck(cudaMalloc(&b.ws, b.ws_bytes), "batch workspace")) return TN_ENOMEM;
-    if (b.split_bytes && !ck(cudaMalloc(&b.split_buf, b.split_bytes), "cudaMalloc")) return TN_ENOMEM;
+    if (b.split_bytes && !ck(cudaMalloc(&b.split_buf, b.split_bytes * b.groups), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&b.maxabs, sizeof(unsigned) * std::max(b.n_slots, 1)), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&b.exps, sizeof(int64_t) * std::max(b.n_slots, 1)), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&b.ctl, sizeof(Control)), "cudaMalloc")) return TN_ENOMEM;
@@ -163,6 +199,7 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
         const int n = d.n;
         const size_t eb = d.elem_bytes();
         char* base = ws + b.ws_base[i];
+        void* split = static_cast<char*>(b.split_buf) + b.group_of[i] * b.split_bytes;
         for (int v = 0; v < n; ++v) nf[b.leaf_base[i] + v] = d.leaves[v].size * (d.is_complex() ? 2 : 1);
         for (size_t k = 0; k < p.nodes.size(); ++k) {
             const Node& nd = p.nodes[k];
@@ -187,7 +224,7 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
             g.A = ptr(nd.ca);
             g.B = ptr(nd.cb);
             g.C = base + nd.ws_off * eb;
-            g.P = b.split_buf;
+            g.P = split;
             g.ctl = b.ctl;
             g.sc.max_a = smax(nd.ca);
             g.sc.exp_a = sexp(nd.ca);
@@ -203,7 +240,7 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
             t.A = g.A;
             t.B = g.B;
             t.C = g.C;
-            t.P = b.split_buf;
+            t.P = split;
             t.sla = g.sla;
             t.slb = g.slb;
             t.ctl = b.ctl;
@@ -242,7 +279,11 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
     return TN_OK;
 }
 
-static cudaError_t enqueue_batch(BatchPlan& b, cudaStream_t s) {
+// The whole sequence on a capturing stream: the groups fork from it after the
+// common setup and join it before the results are gathered.  side, ev: one
+// stream and one event per group but the first, and one more event.
+static cudaError_t enqueue_batch(BatchPlan& b, cudaStream_t s, const std::vector<cudaStream_t>& side,
+                                 const std::vector<cudaEvent_t>& ev) {
     const int N = (int)b.nets.size();
     cudaError_t e = cudaMemsetAsync(b.maxabs, 0, sizeof(unsigned) * std::max(b.n_slots, 1), s);
     if (e != cudaSuccess) return e;
@@ -252,25 +293,58 @@ static cudaError_t enqueue_batch(BatchPlan& b, cudaStream_t s) {
         cudaSuccess)
         return e;
     if ((e = launch_begin_call(b.ctl, 0, 1, nullptr, 0, s)) != cudaSuccess) return e;
+    if (!side.empty()) {
+        if ((e = cudaEventRecord(ev.back(), s)) != cudaSuccess) return e;
+        for (cudaStream_t q : side)
+            if ((e = cudaStreamWaitEvent(q, ev.back(), 0)) != cudaSuccess) return e;
+    }
     for (const BatchStep& st : b.steps) {
+        const cudaStream_t q = st.group == 0 ? s : side[st.group - 1];
         if (st.wave) {
             e = launch_wave(b.items_dev + st.item_begin, st.item_count, b.descs_dev,
-                            reinterpret_cast<const void* const*>(b.leaf_ptr_dev), st.cplx, s);
+                            reinterpret_cast<const void* const*>(b.leaf_ptr_dev), st.cplx, q);
         } else {
             const Plan& p = *b.plans[st.net];
             const Node& nd = p.nodes[st.node];
             const int di = b.desc_base[st.net] + st.node;
             if (nd.kind == kTensorCore)
                 e = launch_tc(b.descs[di], tc_prec_of_mode(b.mode),
-                              st.cplx, s);
+                              st.cplx, q);
             else if (nd.kind == kTiled)
-                e = launch_tile(b.descs[di], st.cplx, s);
+                e = launch_tile(b.descs[di], st.cplx, q);
             else
-                e = launch_generic(b.gen[di], st.cplx, s);
+                e = launch_generic(b.gen[di], st.cplx, q);
         }
         if (e != cudaSuccess) return e;
     }
+    for (size_t g = 0; g < side.size(); ++g) {
+        if ((e = cudaEventRecord(ev[g], side[g])) != cudaSuccess) return e;
+        if ((e = cudaStreamWaitEvent(s, ev[g], 0)) != cudaSuccess) return e;
+    }
     return launch_batch_finish(b.roots_dev, N, b.out_dev, b.exp_dev, b.t_start, b.t_done, b.lat_dev, s);
+}
+
+// Captures the batch; the side streams and events only shape the graph and
+// are released again.
+static cudaError_t capture_batch(BatchPlan& b, cudaGraph_t* g) {
+    std::vector<cudaStream_t> side(b.groups - 1, nullptr);
+    std::vector<cudaEvent_t> ev(b.groups > 1 ? b.groups : 0, nullptr);
+    cudaError_t e = cudaSuccess;
+    for (auto& q : side)
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking);
+    for (auto& v : ev)
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(b.cap_stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        e = enqueue_batch(b, b.cap_stream, side, ev);
+        const cudaError_t e2 = cudaStreamEndCapture(b.cap_stream, g);
+        if (e == cudaSuccess) e = e2;
+    }
+    for (auto q : side)
+        if (q) cudaStreamDestroy(q);
+    for (auto v : ev)
+        if (v) cudaEventDestroy(v);
+    return e;
 }
 
 tn_status run_batch(BatchPlan& b, double* out, int64_t* out_exp2, uint64_t* latency_ns, int out_mem,
@@ -314,12 +388,8 @@ tn_status run_batch(BatchPlan& b, double* out, int64_t* out_exp2, uint64_t* late
         if (b.gexec) CK(cudaGraphExecDestroy(b.gexec));
         b.gexec = nullptr;
         cudaGraph_t g = nullptr;
-        CK(cudaStreamBeginCapture(b.cap_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = enqueue_batch(b, b.cap_stream);
-        cudaError_t e2 = cudaStreamEndCapture(b.cap_stream, &g);
-        CK(e);
-        CK(e2);
-        e = cudaGraphInstantiate(&b.gexec, g, 0);
+        CK(capture_batch(b, &g));
+        cudaError_t e = cudaGraphInstantiate(&b.gexec, g, 0);
         cudaGraphDestroy(g);
         CK(e);
         b.graph_ptrs = lp;

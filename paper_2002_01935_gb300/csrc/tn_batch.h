@@ -15,6 +15,7 @@ struct BatchStep {
     bool cplx = false;
     int item_begin = 0, item_count = 0;
     int net = -1, node = -1;  // single-node step
+    int group = 0;            // branch of the captured graph
 };
 
 // A sliced network of the batch: not part of the merged forest; its slices
@@ -42,8 +43,10 @@ struct BatchPlan {
     int64_t max_leaf_floats = 0;
     std::vector<TileArgs> descs;
     std::vector<GenericArgs> gen;
-    std::vector<BatchStep> steps;
+    std::vector<BatchStep> steps;  // group by group, level by level within one
     std::vector<WaveItem> items;
+    int groups = 1;                // branches; each has its own split buffer
+    std::vector<int> group_of;     // per network
     // device
     void* ws = nullptr;
     void* split_buf = nullptr;
