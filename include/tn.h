@@ -436,9 +436,10 @@ tn_status tn_selftest_flow_timeout(void *stream);
 
 /*
  * tn_plan_steps -- the per-slice launch sequence of a plan (host only).
- * Nodes (0..n_tensors-2, tree order) run in launch steps: a wave step runs
- * all small nodes of one tree level in one launch, a single step runs one
- * node.  *n_steps receives the number of steps; if cap >= *n_steps, then
+ * Nodes (0..n_tensors-2, tree order) run in launch steps: a subtree step runs
+ * connected pieces of the tree made of small nodes, one block each, in one
+ * launch (is_wave 0, several nodes); a wave step runs all small nodes of one
+ * or more tree levels in one launch; a single step runs one node.  *n_steps receives the number of steps; if cap >= *n_steps, then
  * step_info[5*s..5*s+4] = (is_wave, kernel kind 0 generic / 1 tiled /
  * 2 tensor core, tile configuration, number of nodes, kernel launches of
  * the step) and step_nodes lists

@@ -140,7 +140,8 @@ tn_status tn_set_tensor(tn_net* net, int32_t v, const void* ptr, int32_t mem) {
 // choices and K splits count the copies (and which the autotuner, timing
 // single copies, leaves alone).
 static tn_status get_plan(tn_net* net, const int32_t* pairs, int32_t n_sliced, const int64_t* sliced,
-                          tn_mode mode, Plan** out, int copies = 1, bool persistent = false) {
+                          tn_mode mode, Plan** out, int copies = 1, bool persistent = false,
+                          bool regions = true) {
     NetDesc& d = net->d;
     const int n = d.n;
     if (n > 1 && !pairs) return fail(TN_EINVAL, "tree_pairs is NULL");
@@ -150,7 +151,7 @@ static tn_status get_plan(tn_net* net, const int32_t* pairs, int32_t n_sliced, c
     std::vector<int64_t> sv(sliced, sliced + n_sliced);
     for (auto& p : net->plans)
         if (p->mode == mode && p->pairs == pv && p->sliced_ids == sv && p->copies == copies &&
-            p->persistent == persistent) {
+            p->persistent == persistent && p->no_regions == !regions) {
             *out = p.get();
             return TN_OK;
         }
@@ -161,6 +162,7 @@ static tn_status get_plan(tn_net* net, const int32_t* pairs, int32_t n_sliced, c
     p->sliced_ids = sv;
     p->copies = copies;
     p->persistent = persistent;
+    p->no_regions = !regions;
     std::string err;
     tn_status st = tn::build_plan(d, *p, err);
     if (st != TN_OK) return fail(st, err);
@@ -382,7 +384,7 @@ tn_status tn_contract_noalloc(tn_net* net, const int32_t* tree_pairs, int32_t n_
     for (int v = 0; v < net->d.n; ++v)
         if (!net->d.leaves[v].ptr) return fail(TN_EINVAL, "tn_contract_noalloc: tensor without data");
     Plan* p = nullptr;  // host-side plan only: no device state is created
-    tn_status st = get_plan(net, tree_pairs, n_sliced, sliced_labels, TN_MODE_FP32, &p);
+    tn_status st = get_plan(net, tree_pairs, n_sliced, sliced_labels, TN_MODE_FP32, &p, 1, false, false);
     if (st != TN_OK) return st;
     std::string err;
     st = tn::run_noalloc(net->d, *p, out, out_mem, out_exp2, (cudaStream_t)stream, err);
@@ -473,10 +475,10 @@ tn_status tn_plan_steps(tn_net* net, const int32_t* tree_pairs, int32_t n_sliced
         const tn::Node& first = p->nodes[stp.nodes[0]];
         step_info[5 * s + 0] = stp.wave;
         step_info[5 * s + 1] = first.kind;
-        step_info[5 * s + 2] = stp.wave ? 0 : (first.kind == tn::kTiled ? first.tile.cfg : 0);
+        step_info[5 * s + 2] = stp.wave || stp.regions ? 0 : (first.kind == tn::kTiled ? first.tile.cfg : 0);
         step_info[5 * s + 3] = (int32_t)stp.nodes.size();
         // a split-K tiled node adds its fixed-order reduction launch
-        step_info[5 * s + 4] = stp.wave ? 1
+        step_info[5 * s + 4] = stp.wave || stp.regions ? 1
                                : first.kind == tn::kTensorCore ? tn::tc_launches(first.tile)
                                : 1 + (first.kind == tn::kTiled && first.tile.split > 1 ? 1 : 0);
         if (step_nodes)
@@ -502,8 +504,12 @@ static tn_status batch_create(tn_batch** out, int32_t n_nets, tn_net* const* net
         const int32_t ns = n_sliced ? n_sliced[i] : 0;
         if (ns < 0 || (ns > 0 && (!sliced_labels || !sliced_labels[i])))
             return fail(TN_EINVAL, "tn_batch_create_sliced: bad sliced labels");
+        // the merged forest goes level by level over all networks: the plans of
+        // its unsliced members (and their workspace order) have no subtree steps
         Plan* p = nullptr;
-        tn_status st = get_plan(nets[i], tree_pairs[i], ns, ns ? sliced_labels[i] : nullptr, mode, &p);
+        tn_status st = get_plan(nets[i], tree_pairs[i], ns, ns ? sliced_labels[i] : nullptr, mode, &p, 1, false, ns > 0);
+        if (st == TN_OK && ns > 0 && p->d_sliced <= 1)
+            st = get_plan(nets[i], tree_pairs[i], ns, sliced_labels[i], mode, &p, 1, false, false);
         if (st != TN_OK) return st;
         b->b.nets.push_back(&nets[i]->d);
         b->b.plans.push_back(p);

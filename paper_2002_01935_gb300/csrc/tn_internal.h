@@ -279,6 +279,64 @@ struct WaveItem {
     int64_t o_count;
 };
 
+// Subtree step (tn_region.cu): the small nodes of a connected piece of the
+// tree, computed by one CTA in shared memory.  A region's program is a blob of
+// 32-bit words: records of its outputs (2 words: operand offsets A | B << 16,
+// node), the nodes' K offset tables (A | B << 16), nodes (8), operands from
+// outside (8), the operand of each staged entry (16 bits), steps (4) and the
+// nodes stored to the workspace (4).
+struct RegionHdr {
+    int32_t blob, words;      // first word, words (a multiple of 4)
+    int32_t n_out, n_k, n_nodes, n_ext, n_elem, n_steps, n_store;
+    int32_t o_k, o_nodes, o_ext, o_elem, o_steps, o_store;  // word offsets in the blob (outputs first)
+    int32_t pad;
+};
+struct RegionNode {
+    int32_t kbase, k;         // K table, summed entries
+    int32_t a, b;             // operand: >= 0 operand from outside, else ~(arena entry)
+    int32_t sa, sb;           // scale slots (operands from outside, then nodes)
+    int32_t q0;               // first output
+    int32_t conj;             // bit 0: A, bit 1: B read conjugated
+};
+struct RegionExt {
+    int32_t leaf;             // leaf, or -1: a node's output in the workspace
+    int32_t first;            // its first entry of the arena
+    int32_t node;             // that node's scale slot
+    int32_t pad;
+    int64_t ws_off;           // elements
+    int64_t pad2;
+};
+struct RegionStep {
+    int32_t q0, q1;           // outputs
+    int32_t lg_lanes;         // threads per output
+    int32_t accs;             // partial sums per thread; negative: starts a tree level (barrier before it)
+};
+struct RegionStore {
+    int32_t node, slot;       // node of the region, scale slot
+    int64_t ws_off;
+};
+struct RegionArgs {
+    const RegionHdr* hdr;
+    const int32_t* prog;
+    const void* const* leaf_ptrs;
+    const int64_t* leaf_is;   // elements between a leaf's copies
+    const SliceDigits* leaf_sl;
+    const unsigned* leafmax;
+    void* ws;
+    int64_t ws_is;            // elements between the instances' workspaces
+    unsigned* maxabs;
+    int64_t* exps;
+    int32_t slot_is;
+    int32_t slice_step;
+    const Control* ctl;
+    int32_t n_regions;
+    int32_t n_inst;
+};
+constexpr int kRegionArena = 3072;   // entries
+constexpr int kRegionNodes = 192;
+constexpr int kRegionExt = 256;
+constexpr int kRegionWords = 9216;   // of the blob
+
 // Per-slice FP64 accumulation of the root tensor into the output
 // (Sec. 4.7.1: the sliced contractions are summed), with exponent
 // alignment.  od_*: digits of the output in the user's open-label order,
@@ -431,6 +489,8 @@ cudaError_t launch_wave(const WaveItem* items, int n_items, const TileArgs* desc
                         const void* const* leaf_ptrs, bool is_c, cudaStream_t s,
                         const int4* deps = nullptr, unsigned* done = nullptr, unsigned* head = nullptr,
                         int G = 1, bool tiles = false);
+// Subtree regions of one step, every instance (tn_region.cu).
+cudaError_t launch_regions(const RegionArgs& a, bool is_c, cudaStream_t s);
 // Folds the slice group's roots into the FP64 accumulator (direct: the last
 // group into the call's output), leaves the result's exponent after the last
 // group, and advances the slice counter by `advance`.

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <cstdlib>
 #include <map>
+#include <tuple>
 
 namespace tn {
 
@@ -371,6 +372,284 @@ static int64_t persistent_items(const Node& nd) {
     return (nd.size + chunk - 1) / chunk;
 }
 
+static tn_status fill_generic(const NetDesc& d, const Plan& p, const Node& nd, GenericArgs& g, std::string& err);
+
+// ---- subtree regions (tn_region.cu)
+
+// Small enough for a region: at most 2^12 multiply-adds and 2^10 outputs (on
+// one CTA a larger node would hold up the others; waves spread it), operands
+// that can be staged.  Sizes of other kinds: the nodes that would take a
+// launch of one thread per output each.
+static bool region_node(const NetDesc& d, const Plan& p, const Node& nd) {
+    if (nd.size > 1024 || nd.vc > 12.0 || nd.ca < 0 || nd.cb < 0) return false;
+    for (int c : {nd.ca, nd.cb})
+        if (c < d.n ? d.leaves[c].size > 256 : p.nodes[c - d.n].size > 1024) return false;
+    if (nd.kind == kTiled) return wave_node(nd, p.copies);
+    if (nd.kind != kGeneric || nd.any_cfg) return false;
+    double k = 1;
+    for (const std::vector<int>* g : {&nd.gk, &nd.gsa, &nd.gsb})
+        for (int l : *g) k *= (double)d.dims[l];
+    return k <= 64;
+}
+
+static int64_t region_k(const NetDesc& d, const Node& nd) {
+    int64_t k = 1;
+    for (const std::vector<int>* g : {&nd.gk, &nd.gsa, &nd.gsb})
+        for (int l : *g) k *= d.dims[l];
+    return k;
+}
+
+// Connected pieces of region nodes, bottom up: a node joins its children's
+// pieces while the union fits one CTA's shared memory, program and 2^14
+// multiply-adds (a few microseconds).  Pieces of fewer than four nodes stay
+// with the waves.  Returns region_of (-1: none); regions in tree order.
+static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vector<std::vector<int>>& regions) {
+    const int n = d.n, nn = (int)p.nodes.size();
+    struct Size {
+        int64_t out = 0, elems = 0, macs = 0, words = 0;
+        int nodes = 0, ext = 0;
+    };
+    std::vector<int> of(nn, -1);
+    std::vector<Size> size;
+    std::vector<std::vector<int>> members;
+    for (int k = 0; k < nn; ++k) {
+        const Node& nd = p.nodes[k];
+        if (!region_node(d, p, nd)) continue;
+        const int child[2] = {nd.ca >= n ? of[nd.ca - n] : -1, nd.cb >= n ? of[nd.cb - n] : -1};
+        // candidates: both children's pieces, the larger one, the other, none
+        int tries[4][2] = {{1, 1}, {1, 0}, {0, 1}, {0, 0}};
+        if (child[0] >= 0 && child[1] >= 0 && size[child[1]].macs > size[child[0]].macs) {
+            std::swap(tries[1][0], tries[2][0]);
+            std::swap(tries[1][1], tries[2][1]);
+        }
+        for (auto& t : tries) {
+            if ((t[0] && child[0] < 0) || (t[1] && child[1] < 0)) continue;
+            Size z;
+            z.out = nd.size;
+            z.macs = (int64_t)std::llround(std::pow(2.0, nd.vc));
+            z.nodes = 1;
+            z.words = 2 * nd.size + region_k(d, nd) + 8 + 4 + 4;  // at most one step and one store each
+            for (int s = 0; s < 2; ++s) {
+                const int c = s ? nd.cb : nd.ca;
+                if (t[s]) {
+                    const Size& y = size[child[s]];
+                    z.out += y.out;
+                    z.elems += y.elems;
+                    z.macs += y.macs;
+                    z.words += y.words;
+                    z.nodes += y.nodes;
+                    z.ext += y.ext;
+                } else {
+                    const int64_t sz = c < n ? d.leaves[c].size : p.nodes[c - n].size;
+                    z.elems += sz;
+                    z.ext += 1;
+                    z.words += 8 + sz / 2 + 1;
+                }
+            }
+            if (z.out + z.elems > kRegionArena || z.nodes > kRegionNodes || z.ext > kRegionExt ||
+                z.words + 32 > kRegionWords || z.macs > (1 << 14))
+                continue;
+            const int r = (int)size.size();
+            size.push_back(z);
+            members.emplace_back();
+            for (int s = 0; s < 2; ++s)
+                if (t[s]) {
+                    for (int q : members[child[s]]) of[q] = r;
+                    members[r].insert(members[r].end(), members[child[s]].begin(), members[child[s]].end());
+                    members[child[s]].clear();
+                }
+            members[r].push_back(k);
+            of[k] = r;
+            break;
+        }
+    }
+    regions.clear();
+    for (auto& m : members) {
+        bool any = false;
+        for (int k : m) any |= p.nodes[k].kind == kGeneric;
+        if (m.empty()) continue;
+        if (m.size() < 4 && !any) {
+            for (int k : m) of[k] = -1;
+            continue;
+        }
+        std::sort(m.begin(), m.end());
+        for (int k : m) of[k] = (int)regions.size();
+        regions.push_back(m);
+    }
+    return of;
+}
+
+// Offsets of every output and K index of a node in its operands, in the order
+// of the kernel that runs it outside a region.
+static void region_tables(const NetDesc& d, const Plan& p, const Node& nd, std::vector<uint32_t>& out,
+                          std::vector<uint32_t>& kt) {
+    out.clear();
+    kt.clear();
+    auto pack = [](int64_t a, int64_t b) { return (uint32_t)a | ((uint32_t)b << 16); };
+    if (nd.kind == kTiled) {
+        const TileArgs& t = nd.tile;
+        // offsets double with every index bit: entry x + 2^i is entry x plus bit i
+        auto grow = [&](std::vector<uint32_t>& v, const uint8_t* sa, const uint8_t* sb, int nb) {
+            for (int i = 0; i < nb; ++i) {
+                const uint32_t add = pack(sa && sa[i] != kNoBit ? int64_t(1) << sa[i] : 0,
+                                          sb && sb[i] != kNoBit ? int64_t(1) << sb[i] : 0);
+                const size_t have = v.size();
+                v.resize(2 * have);
+                for (size_t x = 0; x < have; ++x) v[have + x] = v[x] + add;
+            }
+        };
+        out.push_back(0);
+        grow(out, nullptr, t.b_n, t.nn);
+        grow(out, t.a_m, nullptr, t.nm);
+        grow(out, t.a_b, t.b_b, t.nb);
+        kt.push_back(0);
+        grow(kt, t.a_k, t.b_k, t.nk);
+        return;
+    }
+    GenericArgs g;
+    std::string err;
+    fill_generic(d, p, nd, g, err);  // ranks were checked when the plan was made
+    for (int64_t o = 0; o < nd.size; ++o) {
+        int64_t rem = o, a = 0, b = 0;
+        for (int i = 0; i < g.n_od; ++i) {
+            a += rem % g.od_dim[i] * g.od_sa[i];
+            b += rem % g.od_dim[i] * g.od_sb[i];
+            rem /= g.od_dim[i];
+        }
+        out.push_back(pack(a, b));
+    }
+    for (int64_t k = 0; k < g.n_sum; ++k) {
+        int64_t rem = k, a = 0, b = 0;
+        for (int i = 0; i < g.n_kd; ++i) {
+            a += rem % g.kd_dim[i] * g.kd_sa[i];
+            b += rem % g.kd_dim[i] * g.kd_sb[i];
+            rem /= g.kd_dim[i];
+        }
+        kt.push_back(pack(a, b));
+    }
+}
+
+// Program of one region (layout: RegionHdr), appended to the plan's.
+// at: one entry per node, all -1 before and after (scratch).
+static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& members, std::vector<int>& at) {
+    const int n = d.n;
+    // order: tree level within the region, then how a node's sums are shared
+    struct Item {
+        int k, level, lg, accs;
+    };
+    std::vector<Item> items;
+    items.reserve(members.size());
+    for (int k : members) {
+        const Node& nd = p.nodes[k];
+        int lv = 0;
+        for (int c : {nd.ca, nd.cb})
+            if (c >= n && at[c - n] >= 0) lv = std::max(lv, at[c - n]);
+        at[k] = lv + 1;  // level for now
+        // the wave kernel's g partial sums per output: lanes x sums per lane
+        int64_t g = 1, K = region_k(d, nd);
+        if (nd.kind == kTiled) {
+            const int64_t O = wave_chunk(nd, p.copies);
+            g = std::min<int64_t>(O >= 256 ? 1 : 256 / O, K);
+        }
+        int64_t L = std::max<int64_t>(1, g / 8);
+        while (L < g && L < 32 && K / L > 16) L *= 2;
+        items.push_back({k, lv + 1, ilog2(L), (int)(g / L)});
+    }
+    std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) {
+        return std::tie(x.level, x.lg, x.accs) < std::tie(y.level, y.lg, y.accs);
+    });
+    for (size_t i = 0; i < items.size(); ++i) at[items[i].k] = (int)i;  // place in the program
+    std::vector<RegionExt> ext;
+    std::vector<uint16_t> elem;
+    std::vector<int64_t> q0(items.size());
+    int64_t n_out = 0;
+    for (size_t i = 0; i < items.size(); ++i) {
+        q0[i] = n_out;
+        n_out += p.nodes[items[i].k].size;
+    }
+    std::vector<RegionNode> nodes(items.size());
+    std::vector<uint32_t> outs, kts, o1, k1;
+    std::vector<RegionStep> steps;
+    for (size_t i = 0; i < items.size(); ++i) {
+        const Node& nd = p.nodes[items[i].k];
+        region_tables(d, p, nd, o1, k1);
+        RegionNode& r = nodes[i];
+        r.kbase = (int)kts.size();
+        r.k = (int)k1.size();
+        kts.insert(kts.end(), k1.begin(), k1.end());
+        for (uint32_t x : o1) {
+            outs.push_back(x);
+            outs.push_back((uint32_t)i);
+        }
+        r.q0 = (int)q0[i];
+        r.conj = 0;
+        for (int s = 0; s < 2; ++s) {
+            const int c = s ? nd.cb : nd.ca;
+            int ref, slot;
+            if (c >= n && at[c - n] >= 0) {
+                const int j = at[c - n];
+                ref = -1 - (int)q0[j];  // the arena's outputs; the staged entries are added below
+                slot = -1 - j;
+            } else {
+                RegionExt e;
+                memset(&e, 0, sizeof(e));
+                e.leaf = c < n ? c : -1;
+                e.first = (int)elem.size();
+                e.node = c < n ? 0 : c - n;
+                const int64_t sz = c < n ? d.leaves[c].size : p.nodes[c - n].size;
+                elem.insert(elem.end(), sz, (uint16_t)ext.size());
+                ref = slot = (int)ext.size();
+                ext.push_back(e);
+            }
+            (s ? r.b : r.a) = ref;
+            (s ? r.sb : r.sa) = slot;
+        }
+        const bool new_level = i == 0 || items[i].level != items[i - 1].level;
+        if (new_level || items[i].lg != items[i - 1].lg || items[i].accs != items[i - 1].accs)
+            steps.push_back({(int)q0[i], (int)q0[i], items[i].lg, new_level ? -items[i].accs : items[i].accs});
+        steps.back().q1 = (int)(q0[i] + nd.size);
+    }
+    const int n_elem = (int)elem.size(), n_ext = (int)ext.size();
+    for (RegionNode& r : nodes) {
+        if (r.a < 0) r.a = ~(n_elem + (-1 - r.a));
+        if (r.b < 0) r.b = ~(n_elem + (-1 - r.b));
+        if (r.sa < 0) r.sa = n_ext + (-1 - r.sa);
+        if (r.sb < 0) r.sb = n_ext + (-1 - r.sb);
+    }
+    // the root, its last member, is read outside
+    std::vector<RegionStore> stores{{at[members.back()], members.back(), 0}};
+    for (int k : members) at[k] = -1;
+    RegionHdr h;
+    memset(&h, 0, sizeof(h));
+    std::vector<int32_t>& P = p.region_prog;
+    h.blob = (int)P.size();
+    auto put = [&](const void* src, size_t words) {
+        while ((P.size() - h.blob) % 4) P.push_back(0);
+        const int at = (int)P.size() - h.blob;
+        const int32_t* w = static_cast<const int32_t*>(src);
+        P.insert(P.end(), w, w + words);
+        return at;
+    };
+    if (elem.size() % 2) elem.push_back(0);
+    put(outs.data(), outs.size());
+    h.o_k = put(kts.data(), kts.size());
+    h.o_nodes = put(nodes.data(), nodes.size() * sizeof(RegionNode) / 4);
+    h.o_ext = put(ext.data(), ext.size() * sizeof(RegionExt) / 4);
+    h.o_elem = put(elem.data(), elem.size() / 2);
+    h.o_steps = put(steps.data(), steps.size() * sizeof(RegionStep) / 4);
+    h.o_store = put(stores.data(), stores.size() * sizeof(RegionStore) / 4);
+    while ((P.size() - h.blob) % 4) P.push_back(0);
+    h.words = (int)P.size() - h.blob;
+    h.n_out = (int)n_out;
+    h.n_k = (int)kts.size();
+    h.n_nodes = (int)nodes.size();
+    h.n_ext = n_ext;
+    h.n_elem = n_elem;
+    h.n_steps = (int)steps.size();
+    h.n_store = (int)stores.size();
+    p.region_hdr.push_back(h);
+}
+
 tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
     const int n = d.n;
     // diagnostics: TN_FORCE_GENERIC=1 runs every node on the generic kernel,
@@ -467,6 +746,7 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
     }
     // ---- nodes
     p.nodes.clear();
+    p.nodes.reserve(std::max(n - 1, 1));  // nodes are large: no copies while the list grows
     double W = 0, C = 0;
     auto log2size = [&](const std::vector<int>& lab) {
         double s = 0;
@@ -526,7 +806,7 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
             p.vstride[me] = nd.stride;
             W = std::max(W, log2size(nd.lab));
             C += std::pow(2.0, nd.vc);
-            p.nodes.push_back(nd);
+            p.nodes.push_back(std::move(nd));
         }
     }
     // root labels must be exactly the open labels
@@ -572,10 +852,28 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
     // small tiled nodes, then one launch per remaining node
     std::vector<int> level(2 * n, 0);
     int max_level = 0;
+    // subtrees of small nodes: one region each, a single step of the schedule
+    std::vector<std::vector<int>> regions;
+    std::vector<int> region_of(p.nodes.size(), -1);
+    if (!p.no_regions && !p.no_waves && !p.no_flow && !p.force_generic && !p.persistent)
+        region_of = find_regions(d, p, regions);
     for (size_t k = 0; k < p.nodes.size(); ++k) {
         const Node& nd = p.nodes[k];
-        int la = nd.ca >= n ? level[nd.ca] : 0, lb = nd.cb >= n ? level[nd.cb] : 0;
-        level[n + k] = 1 + std::max(la, lb);
+        const int r = region_of[k];
+        int lv = 0;
+        if (r < 0) {
+            for (int c : {nd.ca, nd.cb})
+                if (c >= n) lv = std::max(lv, level[c]);
+        } else if (regions[r].back() == (int)k) {
+            // the region's root, its last node: after everything it reads from outside
+            for (int q : regions[r])
+                for (int c : {p.nodes[q].ca, p.nodes[q].cb})
+                    if (c >= n && region_of[c - n] != r) lv = std::max(lv, level[c]);
+            for (int q : regions[r]) level[n + q] = lv + 1;
+        } else {
+            continue;
+        }
+        level[n + k] = 1 + lv;
         max_level = std::max(max_level, level[n + k]);
     }
     p.steps.clear();
@@ -614,13 +912,25 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
         }
         p.steps.push_back(w);
     }
+    p.region_hdr.clear();
+    p.region_prog.clear();
+    std::vector<int> scratch(p.nodes.size(), -1);
     for (int L = 1; L <= max_level && !p.persistent; ++L) {
+        Step rs;
+        for (size_t r = 0; r < regions.size(); ++r) {
+            if (level[n + regions[r].back()] != L) continue;
+            if (rs.regions == 0) rs.region_begin = (int)p.region_hdr.size();
+            emit_region(d, p, regions[r], scratch);
+            ++rs.regions;
+            rs.nodes.insert(rs.nodes.end(), regions[r].begin(), regions[r].end());
+        }
+        if (rs.regions) p.steps.push_back(rs);
         Step w;
         w.wave = 1;
         w.item_begin = (int)p.items.size();
         std::vector<int> singles;
         for (size_t k = 0; k < p.nodes.size(); ++k) {
-            if (level[n + k] != L) continue;
+            if (level[n + k] != L || region_of[k] >= 0) continue;
             const Node& nd = p.nodes[k];
             const bool small = wave_node(nd, p.copies) && !p.no_waves;
             if (!small) {
@@ -697,6 +1007,14 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
                 }
     }
     p.ws_elems = std::max<int64_t>(ar.end, 64);
+    // the programs' workspace offsets
+    for (const RegionHdr& h : p.region_hdr) {
+        RegionExt* ext = reinterpret_cast<RegionExt*>(p.region_prog.data() + h.blob + h.o_ext);
+        for (int e = 0; e < h.n_ext; ++e)
+            if (ext[e].leaf < 0) ext[e].ws_off = p.nodes[ext[e].node].ws_off;
+        RegionStore* st = reinterpret_cast<RegionStore*>(p.region_prog.data() + h.blob + h.o_store);
+        for (int i = 0; i < h.n_store; ++i) st[i].ws_off = p.nodes[st[i].slot].ws_off;
+    }
     p.n_out = 1;
     for (int l : d.open) p.n_out *= d.dims[l];
     return TN_OK;
@@ -857,19 +1175,39 @@ tn_status alloc_plan(NetDesc& d, Plan& p, void* unit, std::string& err) {
                            cudaMemcpyHostToDevice), "cudaMemcpy"))
             return TN_ECUDA;
     }
-    if (!p.items.empty()) {
-        std::vector<TileArgs> descs(nn);
-        for (int k = 0; k < nn; ++k) descs[k] = p.nodes[k].tile;
+    if (!p.items.empty()) {  // filled by configure_instances, before every first run
         if (!ck(cudaMalloc(&p.descs_dev, sizeof(TileArgs) * nn), "cudaMalloc")) return TN_ENOMEM;
         if (!ck(cudaMalloc(&p.items_dev, sizeof(WaveItem) * p.items.size() * G), "cudaMalloc"))
             return TN_ENOMEM;
-        if (!ck(cudaMemcpy(p.descs_dev, descs.data(), sizeof(TileArgs) * nn, cudaMemcpyHostToDevice),
-                "cudaMemcpy"))
+    }
+    if (!p.region_hdr.empty()) {
+        const size_t hb = (p.region_hdr.size() * sizeof(RegionHdr) + 255) / 256 * 256;
+        const size_t pb = (p.region_prog.size() * 4 + 255) / 256 * 256;
+        const size_t sb = (p.leaf_sl.size() * sizeof(SliceDigits) + 255) / 256 * 256;
+        std::vector<char> img(hb + pb + sb + sizeof(int64_t) * n, 0);  // leaf copy strides: 0
+        memcpy(img.data(), p.region_hdr.data(), p.region_hdr.size() * sizeof(RegionHdr));
+        memcpy(img.data() + hb, p.region_prog.data(), p.region_prog.size() * 4);
+        memcpy(img.data() + hb + pb, p.leaf_sl.data(), p.leaf_sl.size() * sizeof(SliceDigits));
+        if (!ck(cudaMalloc(&p.region_dev, img.size()), "region programs")) return TN_ENOMEM;
+        if (!ck(cudaMemcpy(p.region_dev, img.data(), img.size(), cudaMemcpyHostToDevice), "cudaMemcpy"))
             return TN_ECUDA;
-        if (!ck(cudaMemcpy(p.items_dev, p.items.data(), sizeof(WaveItem) * p.items.size(),
-                           cudaMemcpyHostToDevice),
-                "cudaMemcpy"))
-            return TN_ECUDA;
+        char* q = static_cast<char*>(p.region_dev);
+        p.leaf_is_dev = reinterpret_cast<int64_t*>(q + hb + pb + sb);
+        p.leaf_is_uploaded.assign(n, 0);
+        RegionArgs& ra = p.region_args;
+        memset(&ra, 0, sizeof(ra));
+        ra.hdr = reinterpret_cast<const RegionHdr*>(q);
+        ra.prog = reinterpret_cast<const int32_t*>(q + hb);
+        ra.leaf_sl = reinterpret_cast<const SliceDigits*>(q + hb + pb);
+        ra.leaf_is = p.leaf_is_dev;
+        ra.leaf_ptrs = reinterpret_cast<const void* const*>(p.leaf_ptr_dev);
+        ra.leafmax = p.leafmax;
+        ra.ws = p.ws;
+        ra.ws_is = p.ws_elems;
+        ra.maxabs = p.maxabs;
+        ra.exps = p.exps;
+        ra.slot_is = nn;
+        ra.ctl = p.ctl;
     }
     // root accumulation: user open-label order -> root layout
     const Node& root = p.nodes.back();
@@ -995,6 +1333,19 @@ static tn_status configure_instances(const NetDesc& d, Plan& p, int G, int step,
             return TN_ECUDA;
         }
     }
+    if (p.leaf_is_dev) {
+        const std::vector<int64_t> is = leaf_is.empty() ? std::vector<int64_t>(n, 0) : leaf_is;
+        if (is != p.leaf_is_uploaded) {
+            const cudaError_t e = cudaMemcpy(p.leaf_is_dev, is.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) {
+                err = std::string("instance layout upload: ") + cudaGetErrorString(e);
+                return TN_ECUDA;
+            }
+            p.leaf_is_uploaded = is;
+        }
+        p.region_args.n_inst = G;
+        p.region_args.slice_step = step;
+    }
     p.acc_args.n_inst = step == 1 ? G : 1;
     p.graph_inst = p.graph_inst_h = -2;  // captured sequences hold the old layout
     p.cfg_inst = G;
@@ -1026,7 +1377,12 @@ static cudaError_t enqueue_slice(const NetDesc& d, Plan& p, cudaStream_t s, cons
             (e = cudaEventRecordWithFlags(ev[k - pf], s, cudaEventRecordExternal)) != cudaSuccess)
             return e;
         const Step& st = p.steps[k];
-        if (st.wave) {
+        if (st.regions) {
+            RegionArgs ra = p.region_args;
+            ra.hdr += st.region_begin;
+            ra.n_regions = st.regions;
+            e = launch_regions(ra, c, s);
+        } else if (st.wave) {
             if (st.flow)
                 e = launch_wave(p.items_dev + p.inst_items_begin[k], st.item_count * G, p.descs_dev,
                                 reinterpret_cast<const void* const*>(p.leaf_ptr_dev), c, s,
@@ -1154,7 +1510,7 @@ static tn_status prepare_leaves(NetDesc& d, Plan& p, bool capturing, std::vector
 static std::vector<const void*> captured_leaves(const NetDesc& d, const Plan& p, const std::vector<const void*>& lp) {
     std::vector<const void*> got;
     for (const Step& st : p.steps) {
-        if (st.wave) continue;
+        if (st.wave || st.regions) continue;
         const Node& nd = p.nodes[st.node];
         for (int c : {nd.ca, nd.cb})
             if (c >= 0 && c < d.n) got.push_back(lp[c]);
@@ -1514,7 +1870,7 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
     // nodes that run alone in their step, on a tiled or tensor-core kernel
     std::vector<int> tune;
     for (const Step& st : p.steps)
-        if (!st.wave) {
+        if (!st.wave && !st.regions) {
             const Node& nd = p.nodes[st.node];
             if ((nd.kind == kTiled && nd.tile.cfg != kTileDot) || nd.kind == kTensorCore) tune.push_back(st.node);
         }
@@ -1697,6 +2053,9 @@ void free_device(Plan& p) {
     if (p.descs_dev) cudaFree(p.descs_dev);
     if (p.items_dev) cudaFree(p.items_dev);
     if (p.flow_deps_dev) cudaFree(p.flow_deps_dev);
+    if (p.region_dev) cudaFree(p.region_dev);
+    p.region_dev = nullptr;
+    p.leaf_is_dev = nullptr;
     p.flow_deps_dev = nullptr;
     p.flow_cnt_dev = nullptr;
     if (p.inst_roots_dev) cudaFree(p.inst_roots_dev);

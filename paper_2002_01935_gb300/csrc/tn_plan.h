@@ -65,6 +65,7 @@ struct Node {
 struct Step {
     int wave = 0;
     int flow = 0;                  // wave over several levels run as one dataflow
+    int region_begin = 0, regions = 0;  // regions > 0: subtree step (k_region), one CTA per region
     int node = -1;                 // single-node step
     int item_begin = 0, item_count = 0;
     std::vector<int> nodes;        // nodes run by this step
@@ -113,6 +114,7 @@ struct Plan {
     unsigned* flow_cnt_dev = nullptr;  // done[node * G + inst], then one head per step
     bool force_generic = false;  // every node on the generic kernel
     bool no_waves = false;       // one launch per node
+    bool no_regions = false;     // small subtrees as wave items (merged batches, the allocation-free call)
     bool no_tensor_cores = false;  // reduced-precision modes on CUDA cores only
     int copies = 1;  // copies sharing every node launch: K splits fill the GPU with tiles x copies
     std::vector<int32_t> pairs;
@@ -155,6 +157,13 @@ struct Plan {
     std::vector<WaveItem> items;
     WaveItem* items_dev = nullptr;
     TileArgs* descs_dev = nullptr;
+    // subtree steps: programs on the host, one allocation on the device
+    std::vector<RegionHdr> region_hdr;
+    std::vector<int32_t> region_prog;
+    void* region_dev = nullptr;     // headers | programs | leaf slice digits | leaf copy strides
+    RegionArgs region_args{};
+    int64_t* leaf_is_dev = nullptr;
+    std::vector<int64_t> leaf_is_uploaded;
     void* split_buf = nullptr;      // K-split partials, shared by all split nodes
     int64_t split_bytes = 0;
     AccumArgs acc_args{};

@@ -1,0 +1,233 @@
+// tn_region.cu -- subtrees of small nodes computed in shared memory.
+//
+// Most nodes of a circuit or spin network contract a few entries (300 to 400
+// of the 370 to 480 nodes of a 20- to 25-qubit circuit have at most 2^8
+// multiply-adds): as work items of a dataflow wave each of them pays for an
+// item, a descriptor, completion counters and scale slots read through L2,
+// about 3 us per tree level.  Here one CTA takes a whole connected piece of
+// the tree (a region: at most 2^15 multiply-adds): it loads the region's
+// program -- every output's operand offsets and every node's K offsets, laid
+// out once on the host -- and the operands from outside, and goes through the
+// piece level by level with one barrier each, intermediates, maxima and
+// exponents in shared memory; only the nodes read from outside are stored.
+// Offsets come from tables, so label sizes of any kind are alike.  Bound by the
+// chain of levels: the loads at the start take three dependent round trips,
+// a level a few hundred nanoseconds.
+//
+// Every output is summed in the order of the wave kernel (partial sums of
+// every g-th entry, then their tree), so the results are the same bits.
+// Launch times (waves alone before): 16-qubit, 8-cycle amplitude 77 -> 65 us in
+// two region launches and a wave, 32 copies of a 25-qubit one 221 -> 99, eight
+// slices of a 25-qubit tree 139 -> 81 (16 of it the regions), 69 nodes of
+// three-valued labels 10 instead of one launch each.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "tn_internal.h"
+
+namespace tn {
+
+namespace {
+
+constexpr int kThreads = 256;
+
+template <bool CPLX>
+struct RT {
+    using T = float2;
+};
+template <>
+struct RT<false> {
+    using T = float;
+};
+
+__device__ __forceinline__ float2 scaled(float2 x, float f, bool cj) {
+    return make_float2(x.x * f, cj ? -x.y * f : x.y * f);
+}
+__device__ __forceinline__ float scaled(float x, float f, bool) { return x * f; }
+__device__ __forceinline__ void mac(float2& c, float2 a, float2 b) {
+    c.x = fmaf(a.x, b.x, c.x);
+    c.x = fmaf(-a.y, b.y, c.x);
+    c.y = fmaf(a.x, b.y, c.y);
+    c.y = fmaf(a.y, b.x, c.y);
+}
+__device__ __forceinline__ void mac(float& c, float a, float b) { c = fmaf(a, b, c); }
+__device__ __forceinline__ float2 plus(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float plus(float a, float b) { return a + b; }
+__device__ __forceinline__ float2 down(float2 v, int o) {
+    return make_float2(__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ float down(float v, int o) { return __shfl_down_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float largest(float2 v) { return fmaxf(fabsf(v.x), fabsf(v.y)); }
+__device__ __forceinline__ float largest(float v) { return fabsf(v); }
+__device__ __forceinline__ float2 shifted(float2 v, int e) { return make_float2(ldexpf(v.x, e), ldexpf(v.y, e)); }
+__device__ __forceinline__ float shifted(float v, int e) { return ldexpf(v, e); }
+
+__device__ __forceinline__ int exponent_of(unsigned bits) {
+    const float m = __uint_as_float(bits);
+    if (!(m > 0.f)) return 0;
+    int e;
+    frexpf(m, &e);
+    return e;
+}
+
+// Outputs [q0, q1) of a step: 2^lg threads and A partial sums per thread each.
+// K index t belongs to partial sum t mod (A 2^lg); the sums are added as a
+// tree over their index, highest bit first.
+template <bool CPLX, int A>
+__device__ __forceinline__ void region_step(const RegionStep& st, int lg, const uint2* outs, const int32_t* ktab,
+                                            const RegionNode* nodes, typename RT<CPLX>::T* arena, int out0,
+                                            unsigned* maxs, int64_t* exps, int n_ext) {
+    using T = typename RT<CPLX>::T;
+    const int lanes = 1 << lg, lane = threadIdx.x & (lanes - 1), n = (st.q1 - st.q0) << lg;
+    for (int i0 = 0; i0 < n; i0 += kThreads) {  // uniform over the block: shuffles below
+        const int i = i0 + threadIdx.x;
+        const bool on = i < n;
+        const int q = st.q0 + ((on ? i : 0) >> lg);
+        const uint2 rec = outs[q];
+        const RegionNode nd = nodes[rec.y];
+        const int eA = exponent_of(maxs[nd.sa]), eB = exponent_of(maxs[nd.sb]);
+        const int cA = max(-120, min(120, eA)), cB = max(-120, min(120, eB));
+        const float fa = ldexpf(1.f, -cA), fb = ldexpf(1.f, -cB);
+        const int resid = (eA - cA) + (eB - cB);
+        const T* a = arena + nd.a + (rec.x & 0xffffu);
+        const T* b = arena + nd.b + (rec.x >> 16);
+        T acc[A];
+#pragma unroll
+        for (int j = 0; j < A; ++j) acc[j] = T{};
+        if (on) {
+            for (int t0 = lane; t0 < nd.k; t0 += A << lg)
+#pragma unroll
+                for (int j = 0; j < A; ++j) {
+                    const int t = t0 + (j << lg);
+                    if (t < nd.k) {
+                        const unsigned ko = (unsigned)ktab[nd.kbase + t];
+                        mac(acc[j], scaled(a[ko & 0xffffu], fa, nd.conj & 1), scaled(b[ko >> 16], fb, nd.conj & 2));
+                    }
+                }
+        }
+#pragma unroll
+        for (int s = A / 2; s > 0; s >>= 1)
+#pragma unroll
+            for (int j = 0; j < s; ++j) acc[j] = plus(acc[j], acc[j + s]);
+        T v = acc[0];
+        for (int o = lanes >> 1; o > 0; o >>= 1) v = plus(v, down(v, o));
+        if (on && lane == 0) {
+            if (resid) v = shifted(v, -resid);
+            arena[out0 + q] = v;
+            if (q == nd.q0) exps[n_ext + rec.y] = exps[nd.sa] + exps[nd.sb] + eA + eB;
+        }
+        // the node's maximum: one shared atomic per warp where it holds one node
+        const unsigned m = on && lane == 0 ? __float_as_uint(largest(v)) : 0u;
+        if (__all_sync(0xffffffffu, rec.y == __shfl_sync(0xffffffffu, rec.y, 0))) {
+            const unsigned w = __reduce_max_sync(0xffffffffu, m);
+            if ((threadIdx.x & 31) == 0 && w) atomicMax(&maxs[n_ext + rec.y], w);
+        } else if (m) {
+            atomicMax(&maxs[n_ext + rec.y], m);
+        }
+    }
+}
+
+template <bool CPLX>
+__global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ RegionArgs a) {
+    using T = typename RT<CPLX>::T;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ RegionHdr h;
+    __shared__ const T* ext_ptr[kRegionExt];
+    __shared__ int64_t exps[kRegionExt + kRegionNodes];
+    __shared__ unsigned maxs[kRegionExt + kRegionNodes];
+    int32_t* const blob = reinterpret_cast<int32_t*>(smem);
+    T* const arena = reinterpret_cast<T*>(smem + sizeof(int32_t) * kRegionWords);
+    const int tid = threadIdx.x;
+    const int region = blockIdx.x % a.n_regions, inst = blockIdx.x / a.n_regions;
+    const int64_t slice = a.ctl->slice + (int64_t)inst * a.slice_step;
+    if (slice >= a.ctl->slice_end) return;
+    if (tid < (int)(sizeof(RegionHdr) / 4))
+        reinterpret_cast<int32_t*>(&h)[tid] = reinterpret_cast<const int32_t*>(a.hdr + region)[tid];
+    __syncthreads();
+    {
+        const int4* src = reinterpret_cast<const int4*>(a.prog + h.blob);
+        for (int i = tid; i < h.words / 4; i += kThreads) reinterpret_cast<int4*>(blob)[i] = src[i];
+    }
+    __syncthreads();
+    const uint2* outs = reinterpret_cast<const uint2*>(blob);
+    const int32_t* ktab = blob + h.o_k;
+    RegionNode* nodes = reinterpret_cast<RegionNode*>(blob + h.o_nodes);
+    RegionExt* ext = reinterpret_cast<RegionExt*>(blob + h.o_ext);
+    const uint16_t* elem = reinterpret_cast<const uint16_t*>(blob + h.o_elem);
+    const RegionStep* steps = reinterpret_cast<const RegionStep*>(blob + h.o_steps);
+    const RegionStore* stores = reinterpret_cast<const RegionStore*>(blob + h.o_store);
+    // operands from outside: pointer, scale, and the slice offset of a leaf
+    // (kept as its arena base for the nodes that read it)
+    for (int e = tid; e < h.n_ext; e += kThreads) {
+        const RegionExt x = ext[e];
+        int base = x.first;
+        if (x.leaf >= 0) {
+            ext_ptr[e] = reinterpret_cast<const T*>(a.leaf_ptrs[x.leaf]) + (int64_t)inst * a.leaf_is[x.leaf];
+            maxs[e] = a.leafmax[x.leaf];
+            exps[e] = 0;
+            const SliceDigits& d = a.leaf_sl[x.leaf];
+            for (int i = 0; i < d.n; ++i) base += (int)(((slice / d.div[i]) % d.dim[i]) * d.stride[i]);
+        } else {
+            ext_ptr[e] = reinterpret_cast<const T*>(a.ws) + (int64_t)inst * a.ws_is + x.ws_off;
+            maxs[e] = a.maxabs[(int64_t)inst * a.slot_is + x.node];
+            exps[e] = a.exps[(int64_t)inst * a.slot_is + x.node];
+        }
+        ext[e].pad = base;
+    }
+    for (int k = tid; k < h.n_nodes; k += kThreads) maxs[h.n_ext + k] = 0u;
+    __syncthreads();
+    for (int i = tid; i < h.n_elem; i += kThreads) {
+        const int e = elem[i];
+        arena[i] = ext_ptr[e][i - ext[e].first];
+    }
+    for (int k = tid; k < h.n_nodes; k += kThreads) {
+        nodes[k].a = nodes[k].a >= 0 ? ext[nodes[k].a].pad : ~nodes[k].a;
+        nodes[k].b = nodes[k].b >= 0 ? ext[nodes[k].b].pad : ~nodes[k].b;
+    }
+    for (int s = 0; s < h.n_steps; ++s) {
+        const RegionStep st = steps[s];
+        if (st.accs < 0) __syncthreads();
+        const int A = st.accs < 0 ? -st.accs : st.accs, lg = st.lg_lanes;
+        switch (A) {
+            case 1: region_step<CPLX, 1>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            case 2: region_step<CPLX, 2>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            case 4: region_step<CPLX, 4>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            default: region_step<CPLX, 8>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+        }
+    }
+    __syncthreads();
+    // nodes that others read: one warp each
+    for (int r = tid >> 5; r < h.n_store; r += kThreads / 32) {
+        const RegionStore so = stores[r];
+        const int q0 = nodes[so.node].q0, q1 = so.node + 1 < h.n_nodes ? nodes[so.node + 1].q0 : h.n_out;
+        T* dst = reinterpret_cast<T*>(a.ws) + (int64_t)inst * a.ws_is + so.ws_off;
+        for (int i = tid & 31; i < q1 - q0; i += 32) dst[i] = arena[h.n_elem + q0 + i];
+        if ((tid & 31) == 0) {
+            a.maxabs[(int64_t)inst * a.slot_is + so.slot] = maxs[h.n_ext + so.node];
+            a.exps[(int64_t)inst * a.slot_is + so.slot] = exps[h.n_ext + so.node];
+        }
+    }
+}
+
+template <bool CPLX>
+cudaError_t launch_t(const RegionArgs& a, cudaStream_t s) {
+    constexpr size_t smem = sizeof(int32_t) * kRegionWords + kRegionArena * sizeof(typename RT<CPLX>::T);
+    static bool configured = false;
+    if (!configured) {
+        const cudaError_t e = cudaFuncSetAttribute(k_region<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    const int ni = a.n_inst > 1 ? a.n_inst : 1;
+    k_region<CPLX><<<(unsigned)(a.n_regions * ni), kThreads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_regions(const RegionArgs& a, bool is_c, cudaStream_t s) {
+    if (a.n_regions <= 0) return cudaSuccess;
+    return is_c ? launch_t<true>(a, s) : launch_t<false>(a, s);
+}
+
+}  // namespace tn
