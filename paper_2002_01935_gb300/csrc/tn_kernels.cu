@@ -179,61 +179,96 @@ cudaError_t launch_generic(const GenericArgs& a, bool is_c, cudaStream_t s) {
 // of reading the accumulator, and (direct folds) its last group writes the
 // caller's output instead of the accumulator: a call of one group, which is
 // every unsliced one, moves each output once.
+constexpr int kFoldInst = 64;  // instances whose maxima and exponents are kept in shared memory
+
 struct FoldState {
     int64_t slice, slice_end, newE;
     double fa;         // factor of the accumulator
-    int n;             // instances of this group
+    int n;             // instances of this group that are live
     int par;
     bool any, first, last;
     const double* src;  // accumulator to read, nullptr: zero
     double* dst;
     bool idle;          // nothing to write: all roots zero, accumulator stays
     bool vec;           // dst is 16-byte aligned
+    bool plain;         // one root into zero: its values as they are
+    const double* fac;  // shared memory: factor of each instance, 0 for a zero root (n <= kFoldInst)
 };
 
+// Maximum and exponent of instance i of the group.
+__device__ __forceinline__ unsigned fold_max(const AccumArgs& a, int i) { return a.max_r[(int64_t)i * a.s_is]; }
+__device__ __forceinline__ int64_t fold_exp(const AccumArgs& a, int i) { return a.exp_r[(int64_t)i * a.s_is]; }
+__device__ __forceinline__ double fold_pow2(int64_t d) { return ldexp(1.0, (int)(d < -2000 ? -2000 : d)); }
+
 __device__ __forceinline__ FoldState fold_state(const AccumArgs& a) {
+    __shared__ unsigned smax[kFoldInst];
+    __shared__ int64_t sexp[kFoldInst];
+    __shared__ double sfac[kFoldInst];
     FoldState f;
     const Control* ctl = a.ctl;
+    const int group = a.n_inst > 1 ? a.n_inst : 1;
+    // one round trip for the control block and the instances' slots
+    if (threadIdx.x < kFoldInst && (int)threadIdx.x < group) {
+        smax[threadIdx.x] = fold_max(a, threadIdx.x);
+        sexp[threadIdx.x] = fold_exp(a, threadIdx.x);
+    }
     f.slice = ctl->slice;
     f.slice_end = ctl->slice_end;
-    const int64_t begin = ctl->slice_begin;
-    f.n = a.n_inst > 1 ? a.n_inst : 1;
-    f.par = (int)(((f.slice - begin) / f.n) & 1);
+    const int64_t begin = ctl->slice_begin, acc_exp0 = ctl->acc_exp[0], acc_exp1 = ctl->acc_exp[1];
+    double* const out_ptr = ctl->out;
+    __syncthreads();
+    f.n = (int)(f.slice_end - f.slice < group ? f.slice_end - f.slice : group);
+    f.par = group == 1 ? (int)((f.slice - begin) & 1) : (int)(((f.slice - begin) / group) & 1);
     f.first = a.direct && f.slice == begin;
-    f.last = f.slice + f.n >= f.slice_end;
-    const int64_t accE = ctl->acc_exp[f.par];
+    f.last = f.slice + group >= f.slice_end;
+    const int64_t accE = f.par ? acc_exp1 : acc_exp0;
     const bool empty = accE == INT64_MIN;
     f.newE = accE;
     f.any = false;
     for (int i = 0; i < f.n; ++i) {
-        if (f.slice + i >= f.slice_end) break;
-        const float rmax = __uint_as_float(a.max_r[(int64_t)i * a.s_is]);
-        const int64_t S = a.exp_r[(int64_t)i * a.s_is];
-        if (!(rmax > 0.f)) continue;
+        if (!(__uint_as_float(i < kFoldInst ? smax[i] : fold_max(a, i)) > 0.f)) continue;
+        const int64_t S = i < kFoldInst ? sexp[i] : fold_exp(a, i);
         f.newE = (empty && !f.any) ? S : (S > f.newE ? S : f.newE);
         f.any = true;
     }
-    f.fa = 1.0;
-    if (f.any && !empty) {
-        const int64_t da = accE - f.newE;
-        f.fa = ldexp(1.0, (int)(da < -2000 ? -2000 : da));
-    }
+    f.fa = f.any && !empty ? fold_pow2(accE - f.newE) : 1.0;
     f.src = f.first ? nullptr : a.acc;
     const bool out = a.direct && f.last;
-    f.dst = out ? ctl->out : a.acc;
+    f.dst = out ? out_ptr : a.acc;
     f.idle = !f.any && !f.first && !out;
     f.vec = (reinterpret_cast<uintptr_t>(f.dst) & 15) == 0;
+    f.plain = f.first && f.n == 1 && f.any;
+    f.fac = nullptr;
+    if (f.n > 1 && f.n <= kFoldInst) {  // the same factors for every output
+        if ((int)threadIdx.x < f.n)
+            sfac[threadIdx.x] =
+                __uint_as_float(smax[threadIdx.x]) > 0.f ? fold_pow2(sexp[threadIdx.x] - f.newE) : 0.0;
+        __syncthreads();
+        f.fac = sfac;
+    }
     return f;
 }
 
-// Root factor of instance i; 0 and false for a zero or idle one.
+// Root factor of instance i; false for a zero one.
 __device__ __forceinline__ bool fold_factor(const AccumArgs& a, const FoldState& f, int i, double& fr) {
-    if (f.slice + i >= f.slice_end) return false;
-    const float rmax = __uint_as_float(a.max_r[(int64_t)i * a.s_is]);
-    if (!(rmax > 0.f)) return false;
-    const int64_t dr = a.exp_r[(int64_t)i * a.s_is] - f.newE;
-    fr = ldexp(1.0, (int)(dr < -2000 ? -2000 : dr));
+    if (f.fac) {
+        fr = f.fac[i];
+        return fr != 0.0;
+    }
+    if (!(__uint_as_float(fold_max(a, i)) > 0.f)) return false;
+    fr = fold_pow2(fold_exp(a, i) - f.newE);
     return true;
+}
+
+// (double)x + 0.0 in integer operations: the FP64 pipe converts and adds about
+// two values per clock and SM, which bounds a fold of many outputs in the
+// root's order (67 us for 2^22 complex ones, 35 to 42 with this).  Zeros of either sign give +0; subnormal,
+// infinite and NaN values take the conversion.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+    if ((u << 1) == 0u) return 0.0;
+    if (e == 0u || e == 255u) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
 
 template <bool CPLX>
@@ -247,16 +282,13 @@ __device__ __forceinline__ double2 fold_start(const FoldState& f, int64_t o) {
     }
 }
 
-template <bool CPLX>
-__device__ __forceinline__ void fold_add(double2& v, const void* R, int64_t at, double fr) {
-    if constexpr (CPLX) {
-        const float2 r = __ldcs(reinterpret_cast<const float2*>(R) + at);
-        v.x += (double)r.x * fr;
-        v.y += (double)r.y * fr;
-    } else {
-        v.x += (double)__ldcs(reinterpret_cast<const float*>(R) + at) * fr;
-    }
+__device__ __forceinline__ void fold_add(double2& v, float2 r, double fr) {
+    v.x += (double)r.x * fr;
+    v.y += (double)r.y * fr;
 }
+__device__ __forceinline__ void fold_add(double2& v, float r, double fr) { v.x += (double)r * fr; }
+__device__ __forceinline__ double2 fold_plain(float2 r) { return make_double2(widen(r.x), widen(r.y)); }
+__device__ __forceinline__ double2 fold_plain(float r) { return make_double2(widen(r), 0.0); }
 
 template <bool CPLX>
 __device__ __forceinline__ void fold_store(const FoldState& f, int64_t o, double2 v) {
@@ -327,14 +359,28 @@ __device__ __forceinline__ int64_t fold_offset(const AccumArgs& a, int64_t o) {
 // One thread per output; consecutive threads write consecutive outputs.
 // Bound by memory when the outputs follow the root's order (the digits are
 // merged on the host: one digit then), by latency for the few outputs of a
-// network with few or no open labels.
-template <bool CPLX>
-__global__ void __launch_bounds__(256) k_accumulate(const __grid_constant__ AccumArgs a) {
+// network with few or no open labels: FEW loads the roots of the first eight
+// instances before anything else, so that they share one round trip with the
+// control block and the scale slots (16 outputs of eight slices side by side:
+// 19 us with one load after the other, 7 now; one output: 7.5 and 4).
+template <bool CPLX, bool FEW>
+__global__ void __launch_bounds__(256, 3) k_accumulate(const __grid_constant__ AccumArgs a) {
+    using T = typename std::conditional<CPLX, float2, float>::type;
+    const T* const root = reinterpret_cast<const T*>(a.R);
+    constexpr int R = FEW ? 1 : 4;  // outputs in flight per thread
+    constexpr int C = FEW ? 8 : 1;  // instances
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, o_first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int group = a.n_inst > 1 ? a.n_inst : 1;  // every instance of a group has its root, live or not
+    T head[C];
+    if (FEW && o_first < a.n_out) {
+        const int64_t at = fold_offset(a, o_first);
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            if (c < group) head[c] = __ldcs(root + at + (int64_t)c * a.r_is);
+    }
     const FoldState f = fold_state(a);
-    constexpr int R = 4;  // outputs in flight per thread
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     if (!f.idle) {
-        for (int64_t o0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o0 < a.n_out; o0 += R * stride) {
+        for (int64_t o0 = o_first; o0 < a.n_out; o0 += R * stride) {
             double2 v[R];
             int64_t src[R];
 #pragma unroll
@@ -342,15 +388,35 @@ __global__ void __launch_bounds__(256) k_accumulate(const __grid_constant__ Accu
                 const int64_t o = o0 + r * stride;
                 if (o >= a.n_out) break;
                 src[r] = fold_offset(a, o);
-                v[r] = fold_start<CPLX>(f, o);
+                if (!f.plain) v[r] = fold_start<CPLX>(f, o);
             }
-            for (int i = 0; i < f.n; ++i) {
-                double fr;
-                if (f.slice + i >= f.slice_end) break;
-                if (!fold_factor(a, f, i, fr)) continue;
+            if (f.plain) {
+                T ld[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    if (o0 + r * stride < a.n_out) fold_add<CPLX>(v[r], a.R, src[r] + (int64_t)i * a.r_is, fr);
+                    if (o0 + r * stride < a.n_out) ld[r] = FEW && o0 == o_first ? head[0] : __ldcs(root + src[r]);
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (o0 + r * stride < a.n_out) v[r] = fold_plain(ld[r]);
+            } else {
+                for (int i0 = 0; i0 < f.n; i0 += C) {
+                    T ld[R][C];
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int c = 0; c < C; ++c)
+                            if (o0 + r * stride < a.n_out && i0 + c < f.n)
+                                ld[r][c] = FEW && o0 == o_first && i0 == 0 ? head[c]
+                                                                          : __ldcs(root + src[r] + (int64_t)(i0 + c) * a.r_is);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        double fr;
+                        if (i0 + c >= f.n || !fold_factor(a, f, i0 + c, fr)) continue;
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            if (o0 + r * stride < a.n_out) fold_add(v[r], ld[r][c], fr);
+                    }
+                }
             }
 #pragma unroll
             for (int r = 0; r < R; ++r)
@@ -367,9 +433,10 @@ __global__ void __launch_bounds__(256) k_accumulate(const __grid_constant__ Accu
 // written per real output, 24 per complex one.  A call whose 2^13 x 2^12
 // complex root is transposed: 2146 us with one thread per output and a digit
 // loop, a cleared and re-read accumulator and a copy to the caller (947, 75
-// and 255 us of it), 1191 us with this fold, which writes the output itself.
+// and 255 us of it), 851 us with this fold, which writes the output itself
+// (159 us of it; 345 with one tile's loads and stores after the other).
 template <bool CPLX>
-__global__ void __launch_bounds__(256) k_accumulate_perm(const __grid_constant__ AccumArgs a,
+__global__ void __launch_bounds__(256, 5) k_accumulate_perm(const __grid_constant__ AccumArgs a,
                                                          const __grid_constant__ FoldPlan p) {
     using T = typename std::conditional<CPLX, float2, float>::type;
     __shared__ T stage[kFoldTile + kFoldTile / 32];
@@ -394,13 +461,62 @@ __global__ void __launch_bounds__(256) k_accumulate_perm(const __grid_constant__
         __syncthreads();
         constexpr int R = kFoldTile / 256;
         const int64_t n_tiles = int64_t(1) << p.u;
-        for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            int64_t sb = 0, db = 0;
-            for (int j = 0; j < p.u; ++j)
+        // tile bases, one bit per lane and a warp-wide sum
+        const int lane = threadIdx.x & 31;
+        auto bases = [&](int64_t tile, int64_t& sb, int64_t& db) {
+            sb = db = 0;
+            for (int j = lane; j < p.u; j += 32)
                 if ((tile >> j) & 1) {
                     sb += p.rest_src[j];
                     db += p.rest_dst[j];
                 }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sb += __shfl_xor_sync(0xffffffffu, sb, o);
+                db += __shfl_xor_sync(0xffffffffu, db, o);
+            }
+        };
+        if (f.plain) {
+            // one root into zero: the next tile's loads are in flight while
+            // this one is written
+            const T* root = reinterpret_cast<const T*>(a.R);
+            T ld[R];
+            int64_t sb, db = 0, nsb = 0, ndb = 0;
+            if (blockIdx.x < n_tiles) {
+                bases(blockIdx.x, sb, db);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = threadIdx.x + r * 256;
+                    if (i < tsz) ld[r] = __ldcs(root + sb + tsrc[i]);
+                }
+            }
+            for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = threadIdx.x + r * 256;
+                    if (i < tsz) stage[i + (i >> 5)] = ld[r];
+                }
+                __syncthreads();
+                if (tile + gridDim.x < n_tiles) {
+                    bases(tile + gridDim.x, nsb, ndb);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int i = threadIdx.x + r * 256;
+                        if (i < tsz) ld[r] = __ldcs(root + nsb + tsrc[i]);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = threadIdx.x + r * 256;
+                    if (i < tsz) fold_store<CPLX>(f, db + tdst[i], fold_plain(stage[tidx[i]]));
+                }
+                db = ndb;
+                __syncthreads();
+            }
+        }
+        for (int64_t tile = f.plain ? n_tiles : blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            int64_t sb, db;
+            bases(tile, sb, db);
             double2 v[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -409,7 +525,6 @@ __global__ void __launch_bounds__(256) k_accumulate_perm(const __grid_constant__
             }
             for (int q = 0; q < f.n; ++q) {
                 double fr;
-                if (f.slice + q >= f.slice_end) break;
                 if (!fold_factor(a, f, q, fr)) continue;
                 const T* root = reinterpret_cast<const T*>(a.R) + (int64_t)q * a.r_is + sb;
                 T ld[R];
@@ -429,13 +544,7 @@ __global__ void __launch_bounds__(256) k_accumulate_perm(const __grid_constant__
                 for (int r = 0; r < R; ++r) {
                     const int i = threadIdx.x + r * 256;
                     if (i < tsz) {
-                        const T x = stage[tidx[i]];
-                        if constexpr (CPLX) {
-                            v[r].x += (double)x.x * fr;
-                            v[r].y += (double)x.y * fr;
-                        } else {
-                            v[r].x += (double)x * fr;
-                        }
+                        fold_add(v[r], stage[tidx[i]], fr);
                     }
                 }
             }
@@ -512,7 +621,7 @@ cudaError_t launch_accumulate(const AccumArgs& a0, bool is_c, cudaStream_t s, in
     FoldPlan p;
     if (make_fold_plan(a, p)) {
         const int64_t tiles = a.n_out >> p.t;
-        const unsigned blocks = (unsigned)(tiles < sm_count() * 6 ? tiles : sm_count() * 6);
+        const unsigned blocks = (unsigned)(tiles < sm_count() * 5 ? tiles : sm_count() * 5);  // one round
         if (is_c)
             k_accumulate_perm<true><<<blocks, 256, 0, s>>>(a, p);
         else
@@ -522,10 +631,15 @@ cudaError_t launch_accumulate(const AccumArgs& a0, bool is_c, cudaStream_t s, in
     int64_t blocks = (a.n_out + 255) / 256;
     if (blocks > sm_count() * 8) blocks = sm_count() * 8;
     if (blocks < 1) blocks = 1;
-    if (is_c)
-        k_accumulate<true><<<(unsigned)blocks, 256, 0, s>>>(a);
+    const bool few = a.n_out <= 256 * blocks;
+    if (is_c && few)
+        k_accumulate<true, true><<<(unsigned)blocks, 256, 0, s>>>(a);
+    else if (is_c)
+        k_accumulate<true, false><<<(unsigned)blocks, 256, 0, s>>>(a);
+    else if (few)
+        k_accumulate<false, true><<<(unsigned)blocks, 256, 0, s>>>(a);
     else
-        k_accumulate<false><<<(unsigned)blocks, 256, 0, s>>>(a);
+        k_accumulate<false, false><<<(unsigned)blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
