@@ -313,8 +313,8 @@ Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std
 
 // The tile kernel for sizes of any kind.  The shape follows the rule of
 // plan_tile (4 x 1024 up to 4 rows, 16 x 256 up to 32, 256 x 16 up to 32
-// columns, else 64 x 64) and so does the K split, each part at least 16
-// entries.  Nodes of fewer than 2^13 multiply-adds keep one thread per
+// columns, else 64 x 64); the K split gives every SM a tile, each part at
+// least 16 entries.  Nodes of fewer than 2^13 multiply-adds keep one thread per
 // output, which is one launch of a few microseconds whatever the kernel:
 // 3^9 multiply-adds 9.6 us against 11-12 with the tile kernel, 3^14 26 against
 // 19, 5^12 562 against 79, 7 x 5 outputs over K = 3^8 1809 against 28.
@@ -353,7 +353,9 @@ void plan_any_tile(const NetDesc& d, Node& nd, int64_t& split_elems, int copies)
     if (B * copies > 65535 || std::ceil(M / TM) * std::ceil(N / TN) >= lim) return;  // launch grid limits
     const int64_t ktiles = ((int64_t)K + TK - 1) / TK;
     int split = 1;
-    while (tiles * copies * split < 2 * sm_count() && split * 2 <= ktiles && split < 64 &&
+    // (several CTAs share an SM: a split that only fills the second one costs
+    // more in its reduction -- 270 tiles over K = 180: 68 + 21 us in two parts)
+    while (tiles * copies * split < sm_count() && split * 2 <= ktiles && split < 64 &&
            B * split * 2 * copies <= 65535)
         split *= 2;
     nd.any_cfg = cfg;

@@ -1195,6 +1195,8 @@ inline int64_t host_m(const TileArgs& a) { return int64_t(1) << a.nm; }
 inline int64_t host_n(const TileArgs& a) { return int64_t(1) << a.nn; }
 inline int64_t host_m(const GenericArgs& a) { return a.M; }
 inline int64_t host_n(const GenericArgs& a) { return a.N; }
+inline int64_t host_k(const TileArgs& a) { return int64_t(1) << a.nk; }
+inline int64_t host_k(const GenericArgs& a) { return a.n_sum; }
 
 template <class ARGS, bool CPLX, int TM, int TN, int TK, int RM, int RN, int MINB>
 static cudaError_t launch_cfg(const ARGS& a, cudaStream_t s) {
@@ -1217,7 +1219,12 @@ static cudaError_t launch_cfg(const ARGS& a, cudaStream_t s) {
 template <class ARGS, bool CPLX>
 static cudaError_t launch_shape(const ARGS& a, cudaStream_t s) {
     switch (a.cfg) {
-        case kTile64x64: return launch_cfg<ARGS, CPLX, 64, 64, 8, 8, 4, CPLX ? 3 : 4>(a, s);
+        case kTile64x64:
+            // short sums are bound by loads and stores: twice the threads with
+            // half the outputs (complex, 2^12 x 2^12 outputs: K = 16 123 us with
+            // 8 x 4 outputs per thread, 109 with 4 x 4)
+            if (host_k(a) <= 32) return launch_cfg<ARGS, CPLX, 64, 64, 8, 4, 4, 3>(a, s);
+            return launch_cfg<ARGS, CPLX, 64, 64, 8, 8, 4, CPLX ? 3 : 4>(a, s);
         case kTile16x256: return launch_cfg<ARGS, CPLX, 16, 256, 8, 4, 4, 2>(a, s);
         case kTile4x1024: return launch_cfg<ARGS, CPLX, 4, 1024, 4, 4, 4, 2>(a, s);
         case kTile256x16: return launch_cfg<ARGS, CPLX, 256, 16, 8, 4, 4, 2>(a, s);
