@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <stdint.h>
 
 namespace tn {
@@ -201,6 +202,21 @@ struct PackPlan {
     int64_t rest_pos[kMaxBits];
     int64_t pos_row1;
 };
+
+// Lets a kernel use `bytes` of dynamic shared memory on the current device
+// (an attribute of every device's own copy of the kernel; ready: one bit per
+// device, of one kernel).
+template <class F>
+cudaError_t allow_shared(F* kern, size_t bytes, std::atomic<uint64_t>& ready) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+    if (ready.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) ready.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 // Tile plan of an inner-product node (k_dot), computed on the host: a tile
 // is 2^t K entries of every row of either operand; entry e in A's order is at

@@ -21,6 +21,7 @@
 // slices of a 25-qubit tree 139 -> 81 (16 of it the regions), 69 nodes of
 // three-valued labels 10 instead of one launch each.
 #include <cuda_runtime.h>
+#include <atomic>
 #include <stdint.h>
 
 #include "tn_internal.h"
@@ -212,12 +213,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
 template <bool CPLX>
 cudaError_t launch_t(const RegionArgs& a, cudaStream_t s) {
     constexpr size_t smem = sizeof(int32_t) * kRegionWords + kRegionArena * sizeof(typename RT<CPLX>::T);
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(k_region<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static std::atomic<uint64_t> ready{0};
+    const cudaError_t e = allow_shared(k_region<CPLX>, smem, ready);
+    if (e != cudaSuccess) return e;
     const int ni = a.n_inst > 1 ? a.n_inst : 1;
     k_region<CPLX><<<(unsigned)(a.n_regions * ni), kThreads, smem, s>>>(a);
     return cudaGetLastError();

@@ -18,6 +18,7 @@
 // max goes to the node's slot for its consumer.
 #include <cuda_runtime.h>
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <stdint.h>
 #include <type_traits>
@@ -1206,12 +1207,9 @@ static cudaError_t launch_cfg(const ARGS& a, cudaStream_t s) {
     dim3 grid((unsigned)tiles, 1, (unsigned)(a.nbatch * a.split * ni));
     constexpr size_t smem = TileSmem<ARGS, CPLX, TM, TN, TK>::bytes;
     auto* kern = k_tile<ARGS, CPLX, TM, TN, TK, RM, RN, MINB>;
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static std::atomic<uint64_t> ready{0};
+    const cudaError_t e = allow_shared(kern, smem, ready);
+    if (e != cudaSuccess) return e;
     kern<<<grid, (TM / RM) * (TN / RN), smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -1329,13 +1327,10 @@ static cudaError_t launch_dot_rc(const TileArgs& a, cudaStream_t s) {
     using T = typename VT<CPLX>::T;
     const DotPlan dp = make_dot_plan(a);
     const size_t smem = dot_smem_bytes(dp, (1 << a.nm) + (1 << a.nn), sizeof(T));
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(k_dot<CPLX, RM, RN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)(kDotStages * (kDotEntries + kDotEntries / 16) * sizeof(T)));
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static std::atomic<uint64_t> ready{0};
+    const cudaError_t e = allow_shared(k_dot<CPLX, RM, RN>,
+                                       kDotStages * (kDotEntries + kDotEntries / 16) * sizeof(T), ready);
+    if (e != cudaSuccess) return e;
     const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
     // parts of fewer than eight tiles: as many per CTA as make one round of
     // resident CTAs (longer ones balance better over many rounds)
