@@ -230,6 +230,15 @@ struct DotPlan {
     int64_t rest_a[kMaxBits], rest_b[kMaxBits];
 };
 
+constexpr int kDotLow = 5;         // lowest strides of either operand in a tile
+constexpr int kDotEntries = 2048;  // of both operands in a tile
+// K entries of a tile (log2) for a node of 2^nm x 2^nn outputs over 2^nk
+inline int dot_tile_bits(int nm, int nn, int nk) {
+    int t = 2 * kDotLow;
+    while (((int64_t(1) << nm) + (int64_t(1) << nn)) << t > kDotEntries) --t;
+    return t < nk ? t : nk;
+}
+
 // Tensor-core precision of a mode (tn_mode values): 0 TF32 single product
 // (4M), 1 TF32 hi+lo, 2 BF16 hi+lo, 3 TF32 single product (3M), 4 FP16
 // hi+lo (operands scaled by 2^kF16Shift).

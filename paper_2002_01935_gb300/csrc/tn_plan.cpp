@@ -229,10 +229,15 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         if (t.nbatch > 65535) return false;
         const int64_t outs = M * N * t.nbatch;
         int split = 1;
-        // 1024 K entries or more per part; at least eight parts per SM in all
-        // (several CTAs per SM keep enough loads in flight for HBM)
-        while (t.nbatch * p.copies * split < 8 * (int64_t)sm_count() && (K / (split * 2)) >= 1024 &&
-               split < 4096 && (int64_t)split * 2 * p.copies <= 65535)
+        // a K tile (2^11 entries of both operands) or more per part, four with
+        // several outputs, whose sums each part reduces; at least eight parts
+        // per SM in all (several CTAs per SM keep enough loads in flight for
+        // HBM).  2 x 32 outputs over K = 2^11: 34 us with parts of 1024 K
+        // entries (two CTAs), 10 with parts of a few tiles; 4 x 4 over 2^18 in
+        // eight slices: 161 us with parts of one tile, 89 with four.
+        const int64_t tiles = (K >> dot_tile_bits(t.nm, t.nn, t.nk)) / (M * N > 1 ? 4 : 1);
+        while (t.nbatch * p.copies * split < 8 * (int64_t)sm_count() && split * 2 <= tiles && split < 4096 &&
+               (int64_t)split * 2 * p.copies <= 65535)
             split *= 2;
         t.split = split;
         t.kchunk = ((K / split + 255) / 256) * 256;

@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
     if (a.t_done && threadIdx.x == 0) atomicMax(a.t_done, global_ns());
 }
 
-// Inner-product node (at most 64 outputs, long K): out[b,m,n] = sum_k A[.., k] B[.., k].
+// Inner-product node (2 to 64 outputs, long K): out[b,m,n] = sum_k A[.., k] B[.., k].
 // One CTA computes all outputs of a batch entry over its part of K, so that
 // either operand is read once.  K is cut into tiles of 2^t entries that hold
 // the lowest strides of A and of B; a tile of an operand -- its rows times the
@@ -763,25 +763,16 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
 // does not depend on the grid), y: batch entry, z: instance.
 // Bound by memory.  A node of 16 outputs over K = 2^18 in eight copies, 134 MB:
 // 262 us with one CTA per output and K part, which read each operand once per
-// row or column of the other, 80 now (call 3562 -> 2819 us, four of them).
-// One output over K = 2^28 (4.3 GB): 750 us as before, 85% of the HBM copy rate.
-constexpr int kDotLow = 5;
+// row or column of the other, 89 now (call 3562 -> 2819 us, four of them).
 constexpr int kDotStages = 3;
-constexpr int kDotEntries = 4096;                            // of both operands in a stage
-// copies per thread and tile: one output needs half (its tile is 2^10 entries of each operand)
-__host__ __device__ constexpr int dot_per(int rm, int rn) { return kDotEntries / 256 / (rm * rn == 1 ? 2 : 1); }
+constexpr int kDotPer = kDotEntries / 256;   // copies per thread and tile
+constexpr int kDotTile = 1 << (2 * kDotLow);  // K entries of a tile of one output
 // one padding entry per 32 of a row and one a row: no bank conflicts along K or along the rows
 __host__ __device__ constexpr int dot_row(int t) { return (1 << t) + (1 << t) / 32 + 1; }
 
-// K entries of a tile (log2) for an M x N node
-inline int dot_tile_bits(int nm, int nn, int nk) {
-    int t = 2 * kDotLow;
-    while (((int64_t(1) << nm) + (int64_t(1) << nn)) << t > kDotEntries) --t;
-    return t < nk ? t : nk;
-}
-
+// the stages, then offset (4 bytes) and stage position (2) of every entry of a tile
 inline size_t dot_smem_bytes(const DotPlan& dp, int rows, size_t esz) {
-    return (size_t)kDotStages * rows * dot_row(dp.t) * esz;
+    return (size_t)kDotStages * rows * dot_row(dp.t) * esz + (size_t)kDotEntries * 6;
 }
 
 // asynchronous global -> shared copy of one 4- or 8-byte element
@@ -800,10 +791,9 @@ __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sy
 __device__ __forceinline__ float2 shfl_xor(float2 v, int o) { return make_float2(shfl_xor(v.x, o), shfl_xor(v.y, o)); }
 
 template <bool CPLX, int RM, int RN>
-__global__ void __launch_bounds__(256, RM * RN == 1 ? 4 : 2)
+__global__ void __launch_bounds__(256, CPLX && RM * RN >= 8 ? 2 : 3)
     k_dot(const __grid_constant__ TileArgs a, const __grid_constant__ DotPlan dp, int parts) {
     using T = typename VT<CPLX>::T;
-    constexpr int kDotPer = dot_per(RM, RN);
     extern __shared__ __align__(16) unsigned char dot_smem[];
     T* const stg = reinterpret_cast<T*>(dot_smem);  // [stage][rows of A, then of B][dot_row]
     __shared__ T red[8][64];
@@ -815,55 +805,24 @@ __global__ void __launch_bounds__(256, RM * RN == 1 ? 4 : 2)
     const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && tid == 0);
     const int t = dp.t, u = dp.u, tsz = 1 << t;
     const int row = dot_row(t), stage_sz = (M + N) * row;
-    // this thread's copies of a tile: entries of A in A's order, then of B
+    // the copies of a tile: entries of A in A's order, then of B
     const int n_a = M << t, n_ab = (M + N) << t;
-    int off[kDotPer];
-    uint16_t pos[kDotPer];
-    // entries e = tid + 256 r of an operand (at most 12 bits; offsets within
-    // one operand: the planner keeps it below 2^31 entries).  Bits 0-7 are the
-    // thread's and are placed once per operand where B's entries start on a
-    // multiple of 256; every table index is a constant.
-    const int wa = t + a.nm, wb = t + a.nn;
-    auto place_a = [&](int e, int w, int& o, int& c) {
-        if (w < wa && ((e >> w) & 1)) {
-            o += (int)dp.a_add[w];
-            c += dp.ca_add[w];
-        }
-    };
-    auto place_b = [&](int e, int w, int& o, int& c) {
-        if (w < wb && ((e >> w) & 1)) {
-            o += (int)dp.b_add[w];
-            c += dp.cb_add[w];
-        }
-    };
-    const bool even = n_a >= 256;
-    int oa = 0, ca = 0, ob = 0, cb = M << 16;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-        place_a(tid, w, oa, ca);
-        if (even) place_b(tid, w, ob, cb);
-    }
-#pragma unroll
-    for (int r = 0; r < kDotPer; ++r) {
-        const int e0 = tid + r * 256;
-        int o = oa, c = ca;
-        if (e0 < n_a) {
-#pragma unroll
-            for (int w = 8; w < 12; ++w) place_a(e0, w, o, c);
-        } else {
-            o = ob;
-            c = cb;
-            if (!even) {
-#pragma unroll
-                for (int w = 0; w < 8; ++w) place_b(e0 - n_a, w, o, c);
+    int32_t* const off = reinterpret_cast<int32_t*>(stg + (size_t)kDotStages * stage_sz);
+    uint16_t* const pos = reinterpret_cast<uint16_t*>(off + kDotEntries);
+    for (int e0 = tid; e0 < n_ab; e0 += 256) {
+        const bool is_b = e0 >= n_a;
+        const int e = is_b ? e0 - n_a : e0, bits = t + (is_b ? a.nn : a.nm);
+        int o = 0, c = is_b ? M << 16 : 0;
+        for (int w = 0; w < bits; ++w)
+            if ((e >> w) & 1) {  // offsets within one operand: the planner keeps it below 2^31 entries
+                o += (int)(is_b ? dp.b_add : dp.a_add)[w];
+                c += (is_b ? dp.cb_add : dp.ca_add)[w];
             }
-#pragma unroll
-            for (int w = 8; w < 12; ++w) place_b(e0 - n_a, w, o, c);
-        }
-        off[r] = o;
         const int k = c & 0xffff;
-        pos[r] = (uint16_t)((c >> 16) * row + k + (k >> 5));
+        off[e0] = o;
+        pos[e0] = (uint16_t)((c >> 16) * row + k + (k >> 5));
     }
+    __syncthreads();
     const int64_t slice = vw.slice;
     const T* A = reinterpret_cast<const T*>(vw.A) + slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb);
     const T* B = reinterpret_cast<const T*>(vw.B) + slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb);
@@ -884,7 +843,7 @@ __global__ void __launch_bounds__(256, RM * RN == 1 ? 4 : 2)
 #pragma unroll
             for (int r = 0; r < kDotPer; ++r) {
                 const int e = tid + r * 256;
-                if (e < n_ab) cp_async_elem<sizeof(T)>(st + pos[r], (e < n_a ? A + ba : B + bb) + off[r]);
+                if (e < n_ab) cp_async_elem<sizeof(T)>(st + pos[e], (e < n_a ? A + ba : B + bb) + off[e]);
             }
             int j = 0;
             while (j < u && ((nt >> j) & 1)) {
@@ -972,6 +931,131 @@ __global__ void __launch_bounds__(256, RM * RN == 1 ? 4 : 2)
         // (the next part's first barrier comes before its reduction writes red)
     }
     cp_async_wait<0>();
+}
+
+// The one-output case: every thread multiplies its own four entries of a tile.
+// blockIdx.x: K part, y: batch entry, z: instance.  Bound by memory: K = 2^28
+// (4.3 GB) 726 us, 5.9 TB/s; as an instance of k_dot, whose loop over rows and
+// parts costs registers and instructions per copy, 820 to 1105.
+template <bool CPLX>
+__global__ void __launch_bounds__(256) k_dot_one(const __grid_constant__ TileArgs a, const __grid_constant__ DotPlan dp) {
+    using T = typename VT<CPLX>::T;
+    extern __shared__ __align__(16) unsigned char dot_smem[];
+    constexpr int kPad = kDotTile + kDotTile / 32;  // one padding entry per 32: no bank conflicts
+    T* const stg = reinterpret_cast<T*>(dot_smem);  // [stage][A, B][kPad]
+    int32_t* const offA = reinterpret_cast<int32_t*>(dot_smem + (size_t)kDotStages * 2 * kPad * sizeof(T));
+    int32_t* const offB = offA + kDotTile;
+    uint16_t* const posA = reinterpret_cast<uint16_t*>(offB + kDotTile);
+    uint16_t* const posB = posA + kDotTile;
+    __shared__ T red[256];
+    const int64_t b = blockIdx.y;
+    const int sp = blockIdx.x;
+    const View vw = inst_view(a, blockIdx.z, (int)sizeof(T));
+    if (!vw.live) return;
+    const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
+    const int t = dp.t, u = dp.u, tsz = 1 << t;
+    for (int e = threadIdx.x; e < tsz; e += 256) {
+        int xa = 0, xb = 0, pa = 0, pb = 0;
+        for (int w = 0; w < t; ++w)
+            if ((e >> w) & 1) {  // offsets within one operand: the planner keeps it below 2^31 entries
+                xa += (int)dp.a_add[w];
+                xb += (int)dp.b_add[w];
+                pa += dp.ca_add[w];
+                pb += dp.cb_add[w];
+            }
+        offA[e] = xa;
+        offB[e] = xb;
+        posA[e] = (uint16_t)(pa + (pa >> 5));
+        posB[e] = (uint16_t)(pb + (pb >> 5));
+    }
+    __syncthreads();
+    const int64_t slice = vw.slice;
+    const T* A = reinterpret_cast<const T*>(vw.A) + slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb);
+    const T* B = reinterpret_cast<const T*>(vw.B) + slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb);
+    const int64_t n_tiles = int64_t(1) << u;
+    const int64_t per = (n_tiles + a.split - 1) / a.split;
+    const int64_t t0 = (int64_t)sp * per, t1 = min64(n_tiles, t0 + per);
+    // offsets of the next tile to copy; advanced tile by tile along the carry chain
+    int64_t nt = t0, ba = 0, bb = 0;
+    for (int j = 0; j < u; ++j)
+        if ((t0 >> j) & 1) {
+            ba += dp.rest_a[j];
+            bb += dp.rest_b[j];
+        }
+    auto issue = [&](int stage) {
+        if (nt < t1) {
+            T* sA = stg + (size_t)stage * 2 * kPad;
+            T* sB = sA + kPad;
+#pragma unroll
+            for (int r = 0; r < kDotTile / 256; ++r) {
+                const int e = threadIdx.x + r * 256;
+                if (e < tsz) {
+                    cp_async_elem<sizeof(T)>(sA + posA[e], A + ba + offA[e]);
+                    cp_async_elem<sizeof(T)>(sB + posB[e], B + bb + offB[e]);
+                }
+            }
+            int j = 0;
+            while (j < u && ((nt >> j) & 1)) {
+                ba -= dp.rest_a[j];
+                bb -= dp.rest_b[j];
+                ++j;
+            }
+            if (j < u) {
+                ba += dp.rest_a[j];
+                bb += dp.rest_b[j];
+            }
+            ++nt;
+        }
+        cp_async_commit();  // one group per call, empty or not: the wait counts stay uniform
+    };
+#pragma unroll
+    for (int q = 0; q < kDotStages - 1; ++q) issue(q);
+    T acc0 = zero<T>(), acc1 = zero<T>();
+    int stage = 0;
+    for (int64_t tile = t0; tile < t1; ++tile) {
+        issue((stage + kDotStages - 1) % kDotStages);
+        cp_async_wait<kDotStages - 1>();  // this thread's copies of `tile` have landed
+        __syncthreads();                  // ... and every other thread's
+        const T* sA = stg + (size_t)stage * 2 * kPad;
+        const T* sB = sA + kPad;
+#pragma unroll
+        for (int r = 0; r < kDotTile / 256; ++r) {
+            const int i = threadIdx.x + r * 256;
+            if (i < tsz) {
+                const int ip = i + (i >> 5);
+                fma_acc(r & 1 ? acc1 : acc0, cmul(sA[ip], sc.fa, a.conj_a), cmul(sB[ip], sc.fb, a.conj_b));
+            }
+        }
+        __syncthreads();  // the stage is refilled by the next iteration's copies
+        stage = (stage + 1) % kDotStages;
+    }
+    cp_async_wait<0>();
+    // fixed-order block reduction
+    red[threadIdx.x] = add(acc0, acc1);
+    __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+        if (threadIdx.x < s) red[threadIdx.x] = add(red[threadIdx.x], red[threadIdx.x + s]);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        T v = red[0];
+        if (a.split > 1) {
+            reinterpret_cast<T*>(vw.P)[(int64_t)sp * a.nbatch + b] = v;
+            return;
+        }
+        if (sc.resid) {
+            if constexpr (CPLX) {
+                v.x = ldexpf(v.x, -sc.resid);
+                v.y = ldexpf(v.y, -sc.resid);
+            } else {
+                v = ldexpf(v, -sc.resid);
+            }
+        }
+        reinterpret_cast<T*>(vw.C)[b] = v;
+        const float mx = absmax(v);
+        if (mx > 0.f) atomicMax(vw.sc.max_c, __float_as_uint(mx));
+        if (a.t_done) atomicMax(a.t_done, global_ns());
+    }
 }
 
 // One launch for the small nodes of one or more consecutive tree levels.
@@ -1323,18 +1407,17 @@ static DotPlan make_dot_plan(const TileArgs& a) {
 }
 
 template <bool CPLX, int RM, int RN>
-static cudaError_t launch_dot_rc(const TileArgs& a, cudaStream_t s) {
+static cudaError_t launch_dot_rc(const TileArgs& a, const DotPlan& dp, cudaStream_t s) {
     using T = typename VT<CPLX>::T;
-    const DotPlan dp = make_dot_plan(a);
     const size_t smem = dot_smem_bytes(dp, (1 << a.nm) + (1 << a.nn), sizeof(T));
     static std::atomic<uint64_t> ready{0};
-    const cudaError_t e = allow_shared(k_dot<CPLX, RM, RN>,
-                                       kDotStages * (kDotEntries + kDotEntries / 16) * sizeof(T), ready);
+    const cudaError_t e = allow_shared(k_dot<CPLX, RM, RN>, kDotStages * (kDotEntries + kDotEntries / 16) * sizeof(T) +
+                                                                kDotEntries * 6, ready);
     if (e != cudaSuccess) return e;
     const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
     // parts of fewer than eight tiles: as many per CTA as make one round of
     // resident CTAs (longer ones balance better over many rounds)
-    const int64_t slots = (int64_t)sm_count() * (RM * RN == 1 ? 4 : 2), total = (int64_t)a.split * a.nbatch * ni;
+    const int64_t slots = (int64_t)sm_count() * 3, total = (int64_t)a.split * a.nbatch * ni;
     int parts = 1;
     if (((int64_t(1) << dp.u) + a.split - 1) / a.split < 8)
         parts = (int)std::min<int64_t>((total + slots - 1) / slots, a.split);
@@ -1343,18 +1426,34 @@ static cudaError_t launch_dot_rc(const TileArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+template <bool CPLX>
+static cudaError_t launch_dot_one(const TileArgs& a, const DotPlan& dp, cudaStream_t s) {
+    using T = typename VT<CPLX>::T;
+    constexpr size_t smem = (size_t)kDotStages * 2 * (kDotTile + kDotTile / 32) * sizeof(T) + kDotTile * 12;
+    static std::atomic<uint64_t> ready{0};
+    const cudaError_t e = allow_shared(k_dot_one<CPLX>, smem, ready);
+    if (e != cudaSuccess) return e;
+    const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
+    k_dot_one<CPLX><<<dim3((unsigned)a.split, (unsigned)a.nbatch, (unsigned)ni), 256, smem, s>>>(a, dp);
+    return cudaGetLastError();
+}
+
 template <bool CPLX, int RM>
-static cudaError_t launch_dot_r(const TileArgs& a, cudaStream_t s) {
-    if (a.nn == 0) return launch_dot_rc<CPLX, RM, 1>(a, s);
-    if (a.nn == 1) return launch_dot_rc<CPLX, RM, 2>(a, s);
-    return launch_dot_rc<CPLX, RM, 4>(a, s);
+static cudaError_t launch_dot_r(const TileArgs& a, const DotPlan& dp, cudaStream_t s) {
+    if (a.nn == 0) {
+        if constexpr (RM == 1) return launch_dot_one<CPLX>(a, dp, s);
+        else return launch_dot_rc<CPLX, RM, 1>(a, dp, s);
+    }
+    if (a.nn == 1) return launch_dot_rc<CPLX, RM, 2>(a, dp, s);
+    return launch_dot_rc<CPLX, RM, 4>(a, dp, s);
 }
 
 template <bool CPLX>
 static cudaError_t launch_dot(const TileArgs& a, cudaStream_t s) {
-    if (a.nm == 0) return launch_dot_r<CPLX, 1>(a, s);
-    if (a.nm == 1) return launch_dot_r<CPLX, 2>(a, s);
-    return launch_dot_r<CPLX, 4>(a, s);
+    const DotPlan dp = make_dot_plan(a);
+    if (a.nm == 0) return launch_dot_r<CPLX, 1>(a, dp, s);
+    if (a.nm == 1) return launch_dot_r<CPLX, 2>(a, dp, s);
+    return launch_dot_r<CPLX, 4>(a, dp, s);
 }
 
 template <bool CPLX>
