@@ -504,12 +504,8 @@ static tn_status batch_create(tn_batch** out, int32_t n_nets, tn_net* const* net
         const int32_t ns = n_sliced ? n_sliced[i] : 0;
         if (ns < 0 || (ns > 0 && (!sliced_labels || !sliced_labels[i])))
             return fail(TN_EINVAL, "tn_batch_create_sliced: bad sliced labels");
-        // the merged forest goes level by level over all networks: the plans of
-        // its unsliced members (and their workspace order) have no subtree steps
         Plan* p = nullptr;
-        tn_status st = get_plan(nets[i], tree_pairs[i], ns, ns ? sliced_labels[i] : nullptr, mode, &p, 1, false, ns > 0);
-        if (st == TN_OK && ns > 0 && p->d_sliced <= 1)
-            st = get_plan(nets[i], tree_pairs[i], ns, sliced_labels[i], mode, &p, 1, false, false);
+        tn_status st = get_plan(nets[i], tree_pairs[i], ns, ns ? sliced_labels[i] : nullptr, mode, &p);
         if (st != TN_OK) return st;
         b->b.nets.push_back(&nets[i]->d);
         b->b.plans.push_back(p);

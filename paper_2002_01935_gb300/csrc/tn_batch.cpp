@@ -27,6 +27,41 @@ namespace tn {
 
 constexpr int kBatchGroups = 8;
 
+// The programs of network i's subtree regions at level L, with leaves, scale
+// slots and workspace offsets of the batch.  Returns their number.
+static int add_regions(BatchPlan& b, int i, int L) {
+    const Plan& p = *b.plans[i];
+    const int64_t ws0 = b.ws_base[i] / (int64_t)b.nets[i]->elem_bytes();
+    int added = 0;
+    for (const Step& st : p.steps) {
+        if (!st.regions || p.node_level[st.nodes[0]] != L) continue;
+        for (int r = st.region_begin; r < st.region_begin + st.regions; ++r) {
+            RegionHdr h = p.region_hdr[r];
+            const int32_t* src = p.region_prog.data() + h.blob;
+            h.blob = (int)b.region_prog.size();
+            b.region_prog.insert(b.region_prog.end(), src, src + h.words);
+            RegionExt* ext = reinterpret_cast<RegionExt*>(b.region_prog.data() + h.blob + h.o_ext);
+            for (int e = 0; e < h.n_ext; ++e) {
+                if (ext[e].leaf >= 0) {
+                    ext[e].leaf += b.leaf_base[i];
+                } else {
+                    ext[e].node += b.slot_base[i];
+                    ext[e].ws_off += ws0;
+                }
+            }
+            RegionStore* so = reinterpret_cast<RegionStore*>(b.region_prog.data() + h.blob + h.o_store);
+            for (int j = 0; j < h.n_store; ++j) {
+                if (so[j].slot + 1 == (int)p.nodes.size()) so[j].done = i;  // the network's root
+                so[j].slot += b.slot_base[i];
+                so[j].ws_off += ws0;
+            }
+            b.region_hdr.push_back(h);
+            ++added;
+        }
+    }
+    return added;
+}
+
 tn_status build_batch(BatchPlan& b, std::string& err) {
     const int N = (int)b.nets.size();
     b.ws_base.assign(N, 0);
@@ -62,19 +97,13 @@ tn_status build_batch(BatchPlan& b, std::string& err) {
         b.desc_base[i] = descs;
         descs += (int)p.nodes.size();
         split_bytes = std::max(split_bytes, p.split_bytes);
-        const int n = d.n;
-        std::vector<int>& lv = b.level[i];
-        lv.assign(p.nodes.size(), 0);
-        for (size_t k = 0; k < p.nodes.size(); ++k) {
-            const Node& nd = p.nodes[k];
-            const int la = nd.ca >= n ? lv[nd.ca - n] : 0, lb = nd.cb >= n ? lv[nd.cb - n] : 0;
-            lv[k] = 1 + std::max(la, lb);
-            max_level = std::max(max_level, lv[k]);
-        }
+        // the levels of the network's own launch steps
+        b.level[i] = p.node_level;
+        for (int lv : p.node_level) max_level = std::max(max_level, lv);
         b.small[i].assign(p.nodes.size(), 0);
-        for (const Step& st : p.steps)
-            if (st.wave)
-                for (int k : st.nodes) b.small[i][k] = 1;
+        for (const Step& st : p.steps)  // 1: wave, 2: subtree region, 0: a launch of its own
+            if (st.wave || st.regions)
+                for (int k : st.nodes) b.small[i][k] = st.wave ? 1 : 2;
     }
     b.ws_bytes = std::max<int64_t>(ws, 256) + 256;  // + a unit scalar
     b.n_slots = slots;
@@ -98,7 +127,7 @@ tn_status build_batch(BatchPlan& b, std::string& err) {
         for (int i = 0; i < N; ++i) {
             if (b.is_sliced[i]) continue;
             double us = 0;
-            for (const Step& st : b.plans[i]->steps) us += st.wave ? 0.0 : 10.0;
+            for (const Step& st : b.plans[i]->steps) us += st.wave || st.regions ? 0.0 : 10.0;
             us += b.plans[i]->C * (b.nets[i]->is_complex() ? 4e-7 : 1e-7);
             by_cost.push_back({-us, i});
         }
@@ -116,6 +145,16 @@ tn_status build_batch(BatchPlan& b, std::string& err) {
     for (int gl = 0; gl < b.groups * max_level; ++gl) {
         const int g = gl / max_level, L = gl % max_level + 1;
         for (int cp = 0; cp < 2; ++cp) {
+            BatchStep rs;
+            rs.group = g;
+            rs.cplx = cp == 1;
+            rs.region_begin = (int)b.region_hdr.size();
+            for (int i = 0; i < N; ++i)
+                if (!b.is_sliced[i] && b.group_of[i] == g && b.nets[i]->is_complex() == rs.cplx)
+                    rs.regions += add_regions(b, i, L);
+            if (rs.regions) b.steps.push_back(rs);
+        }
+        for (int cp = 0; cp < 2; ++cp) {
             BatchStep w;
             w.wave = 1;
             w.group = g;
@@ -125,7 +164,7 @@ tn_status build_batch(BatchPlan& b, std::string& err) {
                 if (b.is_sliced[i] || b.group_of[i] != g || b.nets[i]->is_complex() != w.cplx) continue;
                 const Plan& p = *b.plans[i];
                 for (size_t k = 0; k < p.nodes.size(); ++k) {
-                    if (b.level[i][k] != L || !b.small[i][k]) continue;
+                    if (b.level[i][k] != L || b.small[i][k] != 1) continue;
                     const int64_t size = p.nodes[k].size;
                     const int64_t chunk = wave_chunk(p.nodes[k], N);  // many networks: throughput
                     for (int64_t o = 0; o < size; o += chunk) {
@@ -269,6 +308,15 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
     if (!ck(cudaMemcpy(b.descs_dev, b.descs.data(), sizeof(TileArgs) * b.descs.size(), cudaMemcpyHostToDevice),
             "cudaMemcpy"))
         return TN_ECUDA;
+    if (!b.region_hdr.empty()) {
+        const size_t hb = (b.region_hdr.size() * sizeof(RegionHdr) + 255) / 256 * 256;
+        std::vector<char> img(hb + b.region_prog.size() * 4);
+        memcpy(img.data(), b.region_hdr.data(), b.region_hdr.size() * sizeof(RegionHdr));
+        memcpy(img.data() + hb, b.region_prog.data(), b.region_prog.size() * 4);
+        if (!ck(cudaMalloc(&b.region_dev, img.size()), "region programs")) return TN_ENOMEM;
+        if (!ck(cudaMemcpy(b.region_dev, img.data(), img.size(), cudaMemcpyHostToDevice), "cudaMemcpy"))
+            return TN_ECUDA;
+    }
     if (!b.items.empty()) {
         if (!ck(cudaMalloc(&b.items_dev, sizeof(WaveItem) * b.items.size()), "cudaMalloc")) return TN_ENOMEM;
         if (!ck(cudaMemcpy(b.items_dev, b.items.data(), sizeof(WaveItem) * b.items.size(),
@@ -300,7 +348,23 @@ static cudaError_t enqueue_batch(BatchPlan& b, cudaStream_t s, const std::vector
     }
     for (const BatchStep& st : b.steps) {
         const cudaStream_t q = st.group == 0 ? s : side[st.group - 1];
-        if (st.wave) {
+        if (st.regions) {
+            RegionArgs ra;
+            memset(&ra, 0, sizeof(ra));
+            const char* base = static_cast<const char*>(b.region_dev);
+            ra.hdr = reinterpret_cast<const RegionHdr*>(base) + st.region_begin;
+            ra.prog = reinterpret_cast<const int32_t*>(base + (b.region_hdr.size() * sizeof(RegionHdr) + 255) / 256 * 256);
+            ra.leaf_ptrs = reinterpret_cast<const void* const*>(b.leaf_ptr_dev);
+            ra.leafmax = b.leafmax;
+            ra.ws = b.ws;
+            ra.maxabs = b.maxabs;
+            ra.exps = b.exps;
+            ra.ctl = b.ctl;
+            ra.t_done = b.t_done;
+            ra.n_regions = st.regions;
+            ra.n_inst = 1;
+            e = launch_regions(ra, st.cplx, q);
+        } else if (st.wave) {
             e = launch_wave(b.items_dev + st.item_begin, st.item_count, b.descs_dev,
                             reinterpret_cast<const void* const*>(b.leaf_ptr_dev), st.cplx, q);
         } else {
@@ -420,7 +484,7 @@ void free_batch(BatchPlan& b) {
     if (b.gexec) cudaGraphExecDestroy(b.gexec);
     if (b.cap_stream) cudaStreamDestroy(b.cap_stream);
     void* ptrs[] = {b.ws, b.split_buf, b.maxabs, b.exps, b.ctl, b.leafmax, (void*)b.leaf_ptr_dev,
-                    b.leaf_nfloat_dev, b.t_start, b.t_done, b.lat_dev, b.out_dev, b.exp_dev,
+                    b.region_dev, b.leaf_nfloat_dev, b.t_start, b.t_done, b.lat_dev, b.out_dev, b.exp_dev,
                     b.roots_dev, b.descs_dev, b.items_dev};
     for (void* q : ptrs)
         if (q) cudaFree(q);

@@ -16,6 +16,7 @@ struct BatchStep {
     int item_begin = 0, item_count = 0;
     int net = -1, node = -1;  // single-node step
     int group = 0;            // branch of the captured graph
+    int region_begin = 0, regions = 0;  // subtree regions of a level (all networks of one type)
 };
 
 // A sliced network of the batch: not part of the merged forest; its slices
@@ -47,6 +48,9 @@ struct BatchPlan {
     std::vector<WaveItem> items;
     int groups = 1;                // branches; each has its own split buffer
     std::vector<int> group_of;     // per network
+    std::vector<RegionHdr> region_hdr;  // the networks' programs with the batch's offsets
+    std::vector<int32_t> region_prog;
+    void* region_dev = nullptr;
     // device
     void* ws = nullptr;
     void* split_buf = nullptr;

@@ -309,7 +309,7 @@ struct WaveItem {
 // 32-bit words: records of its outputs (2 words: operand offsets A | B << 16,
 // node), the nodes' K offset tables (A | B << 16), nodes (8), operands from
 // outside (8), the operand of each staged entry (16 bits), steps (4) and the
-// nodes stored to the workspace (4).
+// nodes stored to the workspace (6).
 struct RegionHdr {
     int32_t blob, words;      // first word, words (a multiple of 4)
     int32_t n_out, n_k, n_nodes, n_ext, n_elem, n_steps, n_store;
@@ -339,13 +339,15 @@ struct RegionStep {
 struct RegionStore {
     int32_t node, slot;       // node of the region, scale slot
     int64_t ws_off;
+    int32_t done, pad;        // >= 0: completion time of this network of a batch
 };
 struct RegionArgs {
     const RegionHdr* hdr;
     const int32_t* prog;
     const void* const* leaf_ptrs;
-    const int64_t* leaf_is;   // elements between a leaf's copies
-    const SliceDigits* leaf_sl;
+    const int64_t* leaf_is;   // elements between a leaf's copies (nullptr: one copy)
+    const SliceDigits* leaf_sl;  // nullptr: unsliced
+    unsigned long long* t_done;  // RegionStore.done
     const unsigned* leafmax;
     void* ws;
     int64_t ws_is;            // elements between the instances' workspaces

@@ -383,12 +383,12 @@ static tn_status fill_generic(const NetDesc& d, const Plan& p, const Node& nd, G
 
 // ---- subtree regions (tn_region.cu)
 
-// Small enough for a region: at most 2^12 multiply-adds and 2^10 outputs (on
-// one CTA a larger node would hold up the others; waves spread it), operands
-// that can be staged.  Sizes of other kinds: the nodes that would take a
+// Small enough for a region: at most 2^14 multiply-adds (64 per thread, about a
+// microsecond; waves spread larger ones over the GPU) and 2^10 outputs,
+// operands that can be staged.  Sizes of other kinds: the nodes that would take a
 // launch of one thread per output each.
 static bool region_node(const NetDesc& d, const Plan& p, const Node& nd) {
-    if (nd.size > 1024 || nd.vc > 12.0 || nd.ca < 0 || nd.cb < 0) return false;
+    if (nd.size > 1024 || nd.vc > 14.0 || nd.ca < 0 || nd.cb < 0) return false;
     for (int c : {nd.ca, nd.cb})
         if (c < d.n ? d.leaves[c].size > 256 : p.nodes[c - d.n].size > 1024) return false;
     if (nd.kind == kTiled) return wave_node(nd, p.copies);
@@ -407,7 +407,7 @@ static int64_t region_k(const NetDesc& d, const Node& nd) {
 }
 
 // Connected pieces of region nodes, bottom up: a node joins its children's
-// pieces while the union fits one CTA's shared memory, program and 2^14
+// pieces while the union fits one CTA's shared memory, program and 2^16
 // multiply-adds (a few microseconds).  Pieces of fewer than four nodes stay
 // with the waves.  Returns region_of (-1: none); regions in tree order.
 static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vector<std::vector<int>>& regions) {
@@ -435,7 +435,7 @@ static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vecto
             z.out = nd.size;
             z.macs = (int64_t)std::llround(std::pow(2.0, nd.vc));
             z.nodes = 1;
-            z.words = 2 * nd.size + region_k(d, nd) + 8 + 4 + 4;  // at most one step and one store each
+            z.words = 2 * nd.size + region_k(d, nd) + 8 + 4 + 6;  // at most one step and one store each
             for (int s = 0; s < 2; ++s) {
                 const int c = s ? nd.cb : nd.ca;
                 if (t[s]) {
@@ -454,7 +454,7 @@ static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vecto
                 }
             }
             if (z.out + z.elems > kRegionArena || z.nodes > kRegionNodes || z.ext > kRegionExt ||
-                z.words + 32 > kRegionWords || z.macs > (1 << 14))
+                z.words + 32 > kRegionWords || z.macs > (1 << 16))
                 continue;
             const int r = (int)size.size();
             size.push_back(z);
@@ -624,7 +624,7 @@ static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& membe
         if (r.sb < 0) r.sb = n_ext + (-1 - r.sb);
     }
     // the root, its last member, is read outside
-    std::vector<RegionStore> stores{{at[members.back()], members.back(), 0}};
+    std::vector<RegionStore> stores{{at[members.back()], members.back(), 0, -1, 0}};
     for (int k : members) at[k] = -1;
     RegionHdr h;
     memset(&h, 0, sizeof(h));
@@ -883,6 +883,7 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
         level[n + k] = 1 + lv;
         max_level = std::max(max_level, level[n + k]);
     }
+    p.node_level.assign(level.begin() + n, level.begin() + n + p.nodes.size());
     p.steps.clear();
     p.items.clear();
     if (p.persistent) {

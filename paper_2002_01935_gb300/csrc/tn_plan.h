@@ -114,7 +114,8 @@ struct Plan {
     unsigned* flow_cnt_dev = nullptr;  // done[node * G + inst], then one head per step
     bool force_generic = false;  // every node on the generic kernel
     bool no_waves = false;       // one launch per node
-    bool no_regions = false;     // small subtrees as wave items (merged batches, the allocation-free call)
+    bool no_regions = false;     // small subtrees as wave items (the allocation-free call)
+    std::vector<int> node_level; // per node: level of its launch step (a region's nodes share one)
     bool no_tensor_cores = false;  // reduced-precision modes on CUDA cores only
     int copies = 1;  // copies sharing every node launch: K splits fill the GPU with tiles x copies
     std::vector<int32_t> pairs;

@@ -5,7 +5,7 @@
 // multiply-adds): as work items of a dataflow wave each of them pays for an
 // item, a descriptor, completion counters and scale slots read through L2,
 // about 3 us per tree level.  Here one CTA takes a whole connected piece of
-// the tree (a region: at most 2^15 multiply-adds): it loads the region's
+// the tree (a region: at most 2^16 multiply-adds): it loads the region's
 // program -- every output's operand offsets and every node's K offsets, laid
 // out once on the host -- and the operands from outside, and goes through the
 // piece level by level with one barrier each, intermediates, maxima and
@@ -163,11 +163,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
         const RegionExt x = ext[e];
         int base = x.first;
         if (x.leaf >= 0) {
-            ext_ptr[e] = reinterpret_cast<const T*>(a.leaf_ptrs[x.leaf]) + (int64_t)inst * a.leaf_is[x.leaf];
+            ext_ptr[e] = reinterpret_cast<const T*>(a.leaf_ptrs[x.leaf]) +
+                         (a.leaf_is ? (int64_t)inst * a.leaf_is[x.leaf] : 0);
             maxs[e] = a.leafmax[x.leaf];
             exps[e] = 0;
-            const SliceDigits& d = a.leaf_sl[x.leaf];
-            for (int i = 0; i < d.n; ++i) base += (int)(((slice / d.div[i]) % d.dim[i]) * d.stride[i]);
+            if (a.leaf_sl) {
+                const SliceDigits& d = a.leaf_sl[x.leaf];
+                for (int i = 0; i < d.n; ++i) base += (int)(((slice / d.div[i]) % d.dim[i]) * d.stride[i]);
+            }
         } else {
             ext_ptr[e] = reinterpret_cast<const T*>(a.ws) + (int64_t)inst * a.ws_is + x.ws_off;
             maxs[e] = a.maxabs[(int64_t)inst * a.slot_is + x.node];
@@ -206,6 +209,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
         if ((tid & 31) == 0) {
             a.maxabs[(int64_t)inst * a.slot_is + so.slot] = maxs[h.n_ext + so.node];
             a.exps[(int64_t)inst * a.slot_is + so.slot] = exps[h.n_ext + so.node];
+            if (so.done >= 0 && a.t_done) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                atomicMax(a.t_done + so.done, now);
+            }
         }
     }
 }
