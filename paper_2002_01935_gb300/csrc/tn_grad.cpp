@@ -54,6 +54,10 @@ struct GradState {
     std::vector<Step> steps;
     std::vector<WaveItem> items;
     std::vector<int> flow_deps;  // per combined node: child a, chunks, child b, chunks
+    std::vector<RegionHdr> region_hdr;  // subtree regions of the combined list
+    std::vector<int32_t> region_prog;
+    void* region_dev = nullptr;
+    RegionArgs region_args{};
     bool any_flow = false;
     // gradient accumulators (floats): leaf v at acc_off[v], one such block
     // of acc_floats per instance
@@ -229,30 +233,99 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
     // levels: the adjoint nodes come after every forward node (the forward
     // steps form one graph, the sweep another: a caller that just ran the
     // forward keeps its intermediates and runs the sweep alone)
-    std::vector<int> level(ncomb, 0);
+    // Small subtrees of either half run as regions, with every member stored:
+    // the sweep reads the forward values, the leaf gathers and other adjoint
+    // nodes the adjoints.
+    std::vector<int> region_of(ncomb, -1);
+    std::vector<std::vector<int>> regions;
+    RegionView view;
+    view.d = &d;
+    view.p = &G.g;
+    view.copies = copies;
+    view.node = cnode;
+    view.operand = [&](int v) -> RegionOperand {
+        if (v < n) return {-1, v, 0, d.leaves[v].size, 0};
+        const int pr = producer(v);
+        const int slot = v < NV ? v - n : nn + (v - NV);
+        if (v < NV) return {pr, -1, slot, G.fwd[v - n].size, G.fwd[v - n].ws_off};
+        const int64_t sz = pr >= 0 ? cnode(pr).size : f.nodes.back().size;  // (the root's adjoint has no producer)
+        return {pr, -1, slot, sz, G.adj_off[v - NV]};
+    };
+    if (!f.no_waves && !f.no_flow && !f.force_generic) {
+        find_regions(view, 0, nn, region_of, regions);
+        find_regions(view, nn, ncomb, region_of, regions);
+    }
+    std::vector<int> level(ncomb, 0), region_level(regions.size(), 0);
     int max_level = 0, fwd_levels = 0;
-    for (int c : order) {
-        const Node& nd = cnode(c);
+    // level of a node's step: after everything that it, or any member of its
+    // region, reads from outside (memoised; producers come earlier in the list)
+    std::function<int(int)> level_of = [&](int c) -> int {
+        const int r = region_of[c];
+        int& lv = r >= 0 ? region_level[r] : level[c];
+        if (lv > 0) return lv;
         int l = c < nn ? 0 : fwd_levels;
-        for (int v : {nd.ca, nd.cb}) {
-            const int pr = producer(v);
-            if (pr >= 0) l = std::max(l, level[pr]);
-        }
-        level[c] = l + 1;
-        max_level = std::max(max_level, level[c]);
+        auto visit = [&](int k) {
+            for (int v : {cnode(k).ca, cnode(k).cb}) {
+                const int pr = producer(v);
+                if (pr >= 0 && (r < 0 || region_of[pr] != r)) l = std::max(l, level_of(pr));
+            }
+        };
+        if (r >= 0)
+            for (int k : regions[r]) visit(k);
+        else
+            visit(c);
+        lv = l + 1;
+        return lv;
+    };
+    for (int c : order) {
+        const int l = level_of(c);
+        level[c] = l;
+        max_level = std::max(max_level, l);
         if (c < nn) fwd_levels = max_level;
+    }
+    // Adjoint regions run as late as their readers allow: one launch for many
+    // of them, and the waves between stay one launch.  (Forward ones are early
+    // by themselves: most of their operands are leaves.)
+    std::vector<int> last(regions.size(), max_level);
+    for (int c = ncomb - 1; c >= nn; --c) {
+        const int r = region_of[c];
+        for (int v : {cnode(c).ca, cnode(c).cb}) {
+            const int pr = producer(v);
+            if (pr < nn || region_of[pr] < 0 || region_of[pr] == r) continue;
+            last[region_of[pr]] = std::min(last[region_of[pr]], (r >= 0 ? last[r] : level[c]) - 1);
+        }
+    }
+    for (size_t r = 0; r < regions.size(); ++r) {
+        if (regions[r][0] < nn) continue;
+        region_level[r] = last[r];
+        for (int c : regions[r]) level[c] = last[r];
     }
     G.level = level;
     std::vector<std::vector<int>> at(max_level + 1);
     for (int c : order) at[level[c]].push_back(c);
     G.steps.clear();
     G.items.clear();
+    G.region_hdr.clear();
+    G.region_prog.clear();
+    std::vector<int> scratch(ncomb, -1);
     for (int L = 1; L <= max_level; ++L) {
+        Step rs;
+        for (size_t r = 0; r < regions.size(); ++r) {
+            if (region_level[r] != L) continue;
+            if (rs.regions == 0) rs.region_begin = (int)G.region_hdr.size();
+            std::vector<std::pair<int, int>> stored;
+            for (int c : regions[r]) stored.push_back({c, c < nn ? c : nn + G.bwd_target[c - nn]});
+            emit_region(view, regions[r], stored, scratch, G.region_hdr, G.region_prog);
+            ++rs.regions;
+            rs.nodes.insert(rs.nodes.end(), regions[r].begin(), regions[r].end());
+        }
+        if (rs.regions) G.steps.push_back(rs);
         Step w;
         w.wave = 1;
         w.item_begin = (int)G.items.size();
         std::vector<int> singles;
         for (int c : at[L]) {
+            if (region_of[c] >= 0) continue;
             const Node& nd = cnode(c);
             const bool small = wave_node(nd, G.plan_inst) && !f.no_waves;
             if (!small) {
@@ -553,6 +626,24 @@ static tn_status alloc_grad(const NetDesc& d, const Plan& f, GradState& G, void*
         UP(G.descs_dev, descs.data(), sizeof(TileArgs) * ncomb);
         UP(G.items_dev, items.data(), sizeof(WaveItem) * items.size());
     }
+    if (!G.region_hdr.empty()) {
+        RegionArgs& ra = G.region_args;
+        memset(&ra, 0, sizeof(ra));
+        std::vector<int64_t> is(n);
+        for (int v = 0; v < n; ++v) is[v] = G.img_is[v] / cf;
+        int64_t* is_dev = nullptr;
+        if (!ck(upload_regions(G.region_hdr, G.region_prog, f.leaf_sl, is, &G.region_dev, &is_dev, ra), "region programs"))
+            return TN_ENOMEM;
+        ra.leaf_ptrs = reinterpret_cast<const void* const*>(G.img_ptr_dev);
+        ra.leafmax = G.leafmax;
+        ra.ws = G.ws;
+        ra.ws_is = G.ws_elems;
+        ra.maxabs = G.maxabs;
+        ra.exps = G.exps;
+        ra.slot_is = G.n_slots;
+        ra.ctl = G.ctl;
+        ra.n_inst = n_inst;
+    }
     // leaf gathers: adjoint of leaf v -> its accumulator
     std::vector<LeafGradArgs> lg(n);
     G.max_grad_n = 0;
@@ -636,7 +727,7 @@ static void free_grad_device(GradState& G) {
                     (void*)G.leafmax, (void*)G.leaf_img, (void*)G.gacc, (void*)G.img_ptr_dev,
                     (void*)G.leaf_nfloat_dev, (void*)G.descs_dev, (void*)G.items_dev,
                     (void*)G.flow_deps_dev, (void*)G.flow_cnt_dev, (void*)G.lg_dev,
-                    (void*)G.copy_dev, (void*)G.adj_dev, (void*)G.perm_dev})
+                    (void*)G.copy_dev, (void*)G.adj_dev, (void*)G.perm_dev, G.region_dev})
         if (q) cudaFree(q);
     G.ws = G.split_buf = nullptr;
     G.maxabs = nullptr;
@@ -654,6 +745,7 @@ static void free_grad_device(GradState& G) {
     G.copy_dev = nullptr;
     G.adj_dev = nullptr;
     G.perm_dev = nullptr;
+    G.region_dev = nullptr;
     for (void* q : {(void*)G.roots_dev, (void*)G.val_dev, (void*)G.val_exp_dev})
         if (q) cudaFree(q);
     G.roots_dev = nullptr;
@@ -695,7 +787,12 @@ static cudaError_t enqueue_steps(const GradState& G, int k0, int k1, tn_mode mod
     cudaError_t e = cudaSuccess;
     for (int k = k0; k < k1 && e == cudaSuccess; ++k) {
         const Step& st = G.steps[k];
-        if (st.wave) {
+        if (st.regions) {
+            RegionArgs ra = G.region_args;
+            ra.hdr += st.region_begin;
+            ra.n_regions = st.regions;
+            e = launch_regions(ra, cplx, s);
+        } else if (st.wave) {
             const WaveItem* it = G.items_dev + G.inst_item_begin[k];
             if (st.flow)
                 e = launch_wave(it, st.item_count * NI, G.descs_dev, leaf_tab, cplx, s,

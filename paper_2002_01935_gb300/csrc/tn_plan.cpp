@@ -387,11 +387,12 @@ static tn_status fill_generic(const NetDesc& d, const Plan& p, const Node& nd, G
 // microsecond; waves spread larger ones over the GPU) and 2^10 outputs,
 // operands that can be staged.  Sizes of other kinds: the nodes that would take a
 // launch of one thread per output each.
-static bool region_node(const NetDesc& d, const Plan& p, const Node& nd) {
+static bool region_node(const RegionView& v, const Node& nd) {
+    const NetDesc& d = *v.d;
     if (nd.size > 1024 || nd.vc > 14.0 || nd.ca < 0 || nd.cb < 0) return false;
     for (int c : {nd.ca, nd.cb})
-        if (c < d.n ? d.leaves[c].size > 256 : p.nodes[c - d.n].size > 1024) return false;
-    if (nd.kind == kTiled) return wave_node(nd, p.copies);
+        if (v.operand(c).size > (c < d.n ? 256 : 1024)) return false;
+    if (nd.kind == kTiled) return wave_node(nd, v.copies);
     if (nd.kind != kGeneric || nd.any_cfg) return false;
     double k = 1;
     for (const std::vector<int>* g : {&nd.gk, &nd.gsa, &nd.gsb})
@@ -409,21 +410,25 @@ static int64_t region_k(const NetDesc& d, const Node& nd) {
 // Connected pieces of region nodes, bottom up: a node joins its children's
 // pieces while the union fits one CTA's shared memory, program and 2^16
 // multiply-adds (a few microseconds).  Pieces of fewer than four nodes stay
-// with the waves.  Returns region_of (-1: none); regions in tree order.
-static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vector<std::vector<int>>& regions) {
-    const int n = d.n, nn = (int)p.nodes.size();
+// with the waves.  (An adjoint node joins its parent adjoint's piece: that is
+// the operand of its own list.)
+void find_regions(const RegionView& v, int k0, int k1, std::vector<int>& of, std::vector<std::vector<int>>& regions) {
+    const NetDesc& d = *v.d;
     struct Size {
         int64_t out = 0, elems = 0, macs = 0, words = 0;
         int nodes = 0, ext = 0;
     };
-    std::vector<int> of(nn, -1);
     std::vector<Size> size;
     std::vector<std::vector<int>> members;
-    for (int k = 0; k < nn; ++k) {
-        const Node& nd = p.nodes[k];
-        if (!region_node(d, p, nd)) continue;
-        const int child[2] = {nd.ca >= n ? of[nd.ca - n] : -1, nd.cb >= n ? of[nd.cb - n] : -1};
-        // candidates: both children's pieces, the larger one, the other, none
+    std::vector<int> mine(k1 - k0, -1);  // piece of each node so far
+    for (int k = k0; k < k1; ++k) {
+        const Node& nd = v.node(k);
+        if (!region_node(v, nd)) continue;
+        const RegionOperand op[2] = {v.operand(nd.ca), v.operand(nd.cb)};
+        int child[2];
+        for (int s = 0; s < 2; ++s)
+            child[s] = op[s].producer >= k0 && op[s].producer < k1 ? mine[op[s].producer - k0] : -1;
+        // candidates: both operands' pieces, the larger one, the other, none
         int tries[4][2] = {{1, 1}, {1, 0}, {0, 1}, {0, 0}};
         if (child[0] >= 0 && child[1] >= 0 && size[child[1]].macs > size[child[0]].macs) {
             std::swap(tries[1][0], tries[2][0]);
@@ -431,13 +436,13 @@ static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vecto
         }
         for (auto& t : tries) {
             if ((t[0] && child[0] < 0) || (t[1] && child[1] < 0)) continue;
+            if (t[0] && t[1] && child[0] == child[1]) continue;  // (no tree has it)
             Size z;
             z.out = nd.size;
             z.macs = (int64_t)std::llround(std::pow(2.0, nd.vc));
             z.nodes = 1;
             z.words = 2 * nd.size + region_k(d, nd) + 8 + 4 + 6;  // at most one step and one store each
             for (int s = 0; s < 2; ++s) {
-                const int c = s ? nd.cb : nd.ca;
                 if (t[s]) {
                     const Size& y = size[child[s]];
                     z.out += y.out;
@@ -447,43 +452,40 @@ static std::vector<int> find_regions(const NetDesc& d, const Plan& p, std::vecto
                     z.nodes += y.nodes;
                     z.ext += y.ext;
                 } else {
-                    const int64_t sz = c < n ? d.leaves[c].size : p.nodes[c - n].size;
-                    z.elems += sz;
+                    z.elems += op[s].size;
                     z.ext += 1;
-                    z.words += 8 + sz / 2 + 1;
+                    z.words += 8 + op[s].size / 2 + 1;
                 }
             }
             if (z.out + z.elems > kRegionArena || z.nodes > kRegionNodes || z.ext > kRegionExt ||
                 z.words + 32 > kRegionWords || z.macs > (1 << 16))
                 continue;
-            const int r = (int)size.size();
-            size.push_back(z);
-            members.emplace_back();
-            for (int s = 0; s < 2; ++s)
-                if (t[s]) {
-                    for (int q : members[child[s]]) of[q] = r;
-                    members[r].insert(members[r].end(), members[child[s]].begin(), members[child[s]].end());
-                    members[child[s]].clear();
-                }
+            // the piece takes the place of the first one it joins
+            const int r = t[0] ? child[0] : (t[1] ? child[1] : (int)size.size());
+            if (r == (int)size.size()) {
+                size.emplace_back();
+                members.emplace_back();
+            }
+            if (t[0] && t[1]) {
+                for (int q : members[child[1]]) mine[q - k0] = r;
+                members[r].insert(members[r].end(), members[child[1]].begin(), members[child[1]].end());
+                members[child[1]].clear();
+            }
+            size[r] = z;
             members[r].push_back(k);
-            of[k] = r;
+            mine[k - k0] = r;
             break;
         }
     }
-    regions.clear();
     for (auto& m : members) {
-        bool any = false;
-        for (int k : m) any |= p.nodes[k].kind == kGeneric;
         if (m.empty()) continue;
-        if (m.size() < 4 && !any) {
-            for (int k : m) of[k] = -1;
-            continue;
-        }
+        bool any = false;
+        for (int k : m) any |= v.node(k).kind == kGeneric;
+        if (m.size() < 4 && !any) continue;
         std::sort(m.begin(), m.end());
         for (int k : m) of[k] = (int)regions.size();
         regions.push_back(m);
     }
-    return of;
 }
 
 // Offsets of every output and K index of a node in its operands, in the order
@@ -537,9 +539,10 @@ static void region_tables(const NetDesc& d, const Plan& p, const Node& nd, std::
 }
 
 // Program of one region (layout: RegionHdr), appended to the plan's.
-// at: one entry per node, all -1 before and after (scratch).
-static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& members, std::vector<int>& at) {
-    const int n = d.n;
+// at: one entry per node of the list, all -1 before and after (scratch).
+void emit_region(const RegionView& v, const std::vector<int>& members, const std::vector<std::pair<int, int>>& stored,
+                 std::vector<int>& at, std::vector<RegionHdr>& hdr, std::vector<int32_t>& P) {
+    const NetDesc& d = *v.d;
     // order: tree level within the region, then how a node's sums are shared
     struct Item {
         int k, level, lg, accs;
@@ -547,15 +550,17 @@ static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& membe
     std::vector<Item> items;
     items.reserve(members.size());
     for (int k : members) {
-        const Node& nd = p.nodes[k];
+        const Node& nd = v.node(k);
         int lv = 0;
-        for (int c : {nd.ca, nd.cb})
-            if (c >= n && at[c - n] >= 0) lv = std::max(lv, at[c - n]);
+        for (int c : {nd.ca, nd.cb}) {
+            const int pr = v.operand(c).producer;
+            if (pr >= 0 && at[pr] >= 0) lv = std::max(lv, at[pr]);
+        }
         at[k] = lv + 1;  // level for now
         // the wave kernel's g partial sums per output: lanes x sums per lane
         int64_t g = 1, K = region_k(d, nd);
         if (nd.kind == kTiled) {
-            const int64_t O = wave_chunk(nd, p.copies);
+            const int64_t O = wave_chunk(nd, v.copies);
             g = std::min<int64_t>(O >= 256 ? 1 : 256 / O, K);
         }
         int64_t L = std::max<int64_t>(1, g / 8);
@@ -572,14 +577,14 @@ static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& membe
     int64_t n_out = 0;
     for (size_t i = 0; i < items.size(); ++i) {
         q0[i] = n_out;
-        n_out += p.nodes[items[i].k].size;
+        n_out += v.node(items[i].k).size;
     }
     std::vector<RegionNode> nodes(items.size());
     std::vector<uint32_t> outs, kts, o1, k1;
     std::vector<RegionStep> steps;
     for (size_t i = 0; i < items.size(); ++i) {
-        const Node& nd = p.nodes[items[i].k];
-        region_tables(d, p, nd, o1, k1);
+        const Node& nd = v.node(items[i].k);
+        region_tables(d, *v.p, nd, o1, k1);
         RegionNode& r = nodes[i];
         r.kbase = (int)kts.size();
         r.k = (int)k1.size();
@@ -589,22 +594,22 @@ static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& membe
             outs.push_back((uint32_t)i);
         }
         r.q0 = (int)q0[i];
-        r.conj = 0;
+        r.conj = (nd.tile.conj_a ? 1 : 0) | (nd.tile.conj_b ? 2 : 0);
         for (int s = 0; s < 2; ++s) {
-            const int c = s ? nd.cb : nd.ca;
+            const RegionOperand op = v.operand(s ? nd.cb : nd.ca);
             int ref, slot;
-            if (c >= n && at[c - n] >= 0) {
-                const int j = at[c - n];
+            if (op.producer >= 0 && at[op.producer] >= 0) {
+                const int j = at[op.producer];
                 ref = -1 - (int)q0[j];  // the arena's outputs; the staged entries are added below
                 slot = -1 - j;
             } else {
                 RegionExt e;
                 memset(&e, 0, sizeof(e));
-                e.leaf = c < n ? c : -1;
+                e.leaf = op.leaf;
                 e.first = (int)elem.size();
-                e.node = c < n ? 0 : c - n;
-                const int64_t sz = c < n ? d.leaves[c].size : p.nodes[c - n].size;
-                elem.insert(elem.end(), sz, (uint16_t)ext.size());
+                e.node = op.leaf >= 0 ? 0 : op.slot;
+                e.ws_off = op.leaf >= 0 ? 0 : op.ws_off;
+                elem.insert(elem.end(), op.size, (uint16_t)ext.size());
                 ref = slot = (int)ext.size();
                 ext.push_back(e);
             }
@@ -623,12 +628,11 @@ static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& membe
         if (r.sa < 0) r.sa = n_ext + (-1 - r.sa);
         if (r.sb < 0) r.sb = n_ext + (-1 - r.sb);
     }
-    // the root, its last member, is read outside
-    std::vector<RegionStore> stores{{at[members.back()], members.back(), 0, -1, 0}};
+    std::vector<RegionStore> stores;
+    for (auto& st : stored) stores.push_back({at[st.first], st.second, v.node(st.first).ws_off, -1, 0});
     for (int k : members) at[k] = -1;
     RegionHdr h;
     memset(&h, 0, sizeof(h));
-    std::vector<int32_t>& P = p.region_prog;
     h.blob = (int)P.size();
     auto put = [&](const void* src, size_t words) {
         while ((P.size() - h.blob) % 4) P.push_back(0);
@@ -654,7 +658,31 @@ static void emit_region(const NetDesc& d, Plan& p, const std::vector<int>& membe
     h.n_elem = n_elem;
     h.n_steps = (int)steps.size();
     h.n_store = (int)stores.size();
-    p.region_hdr.push_back(h);
+    hdr.push_back(h);
+}
+
+cudaError_t upload_regions(const std::vector<RegionHdr>& hdr, const std::vector<int32_t>& prog,
+                           const std::vector<SliceDigits>& leaf_sl, const std::vector<int64_t>& leaf_is, void** dev,
+                           int64_t** leaf_is_dev, RegionArgs& ra) {
+    const size_t hb = (hdr.size() * sizeof(RegionHdr) + 255) / 256 * 256;
+    const size_t pb = (prog.size() * 4 + 255) / 256 * 256;
+    const size_t sb = (leaf_sl.size() * sizeof(SliceDigits) + 255) / 256 * 256;
+    std::vector<char> img(hb + pb + sb + sizeof(int64_t) * leaf_is.size());
+    memcpy(img.data(), hdr.data(), hdr.size() * sizeof(RegionHdr));
+    memcpy(img.data() + hb, prog.data(), prog.size() * 4);
+    memcpy(img.data() + hb + pb, leaf_sl.data(), leaf_sl.size() * sizeof(SliceDigits));
+    memcpy(img.data() + hb + pb + sb, leaf_is.data(), sizeof(int64_t) * leaf_is.size());
+    cudaError_t e = cudaMalloc(dev, img.size());
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpy(*dev, img.data(), img.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    char* q = static_cast<char*>(*dev);
+    *leaf_is_dev = reinterpret_cast<int64_t*>(q + hb + pb + sb);
+    ra.hdr = reinterpret_cast<const RegionHdr*>(q);
+    ra.prog = reinterpret_cast<const int32_t*>(q + hb);
+    ra.leaf_sl = reinterpret_cast<const SliceDigits*>(q + hb + pb);
+    ra.leaf_is = *leaf_is_dev;
+    return cudaSuccess;
 }
 
 tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
@@ -862,8 +890,17 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
     // subtrees of small nodes: one region each, a single step of the schedule
     std::vector<std::vector<int>> regions;
     std::vector<int> region_of(p.nodes.size(), -1);
+    RegionView view;
+    view.d = &d;
+    view.p = &p;
+    view.copies = p.copies;
+    view.node = [&p](int k) -> const Node& { return p.nodes[k]; };
+    view.operand = [&d, &p, n](int c) -> RegionOperand {
+        if (c < n) return {-1, c, 0, d.leaves[c].size, 0};
+        return {c - n, -1, c - n, p.nodes[c - n].size, 0};  // workspace offsets follow below
+    };
     if (!p.no_regions && !p.no_waves && !p.no_flow && !p.force_generic && !p.persistent)
-        region_of = find_regions(d, p, regions);
+        find_regions(view, 0, (int)p.nodes.size(), region_of, regions);
     for (size_t k = 0; k < p.nodes.size(); ++k) {
         const Node& nd = p.nodes[k];
         const int r = region_of[k];
@@ -928,7 +965,8 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
         for (size_t r = 0; r < regions.size(); ++r) {
             if (level[n + regions[r].back()] != L) continue;
             if (rs.regions == 0) rs.region_begin = (int)p.region_hdr.size();
-            emit_region(d, p, regions[r], scratch);
+            // the root, its last member, is read outside
+            emit_region(view, regions[r], {{regions[r].back(), regions[r].back()}}, scratch, p.region_hdr, p.region_prog);
             ++rs.regions;
             rs.nodes.insert(rs.nodes.end(), regions[r].begin(), regions[r].end());
         }
@@ -1189,25 +1227,12 @@ tn_status alloc_plan(NetDesc& d, Plan& p, void* unit, std::string& err) {
             return TN_ENOMEM;
     }
     if (!p.region_hdr.empty()) {
-        const size_t hb = (p.region_hdr.size() * sizeof(RegionHdr) + 255) / 256 * 256;
-        const size_t pb = (p.region_prog.size() * 4 + 255) / 256 * 256;
-        const size_t sb = (p.leaf_sl.size() * sizeof(SliceDigits) + 255) / 256 * 256;
-        std::vector<char> img(hb + pb + sb + sizeof(int64_t) * n, 0);  // leaf copy strides: 0
-        memcpy(img.data(), p.region_hdr.data(), p.region_hdr.size() * sizeof(RegionHdr));
-        memcpy(img.data() + hb, p.region_prog.data(), p.region_prog.size() * 4);
-        memcpy(img.data() + hb + pb, p.leaf_sl.data(), p.leaf_sl.size() * sizeof(SliceDigits));
-        if (!ck(cudaMalloc(&p.region_dev, img.size()), "region programs")) return TN_ENOMEM;
-        if (!ck(cudaMemcpy(p.region_dev, img.data(), img.size(), cudaMemcpyHostToDevice), "cudaMemcpy"))
-            return TN_ECUDA;
-        char* q = static_cast<char*>(p.region_dev);
-        p.leaf_is_dev = reinterpret_cast<int64_t*>(q + hb + pb + sb);
-        p.leaf_is_uploaded.assign(n, 0);
         RegionArgs& ra = p.region_args;
         memset(&ra, 0, sizeof(ra));
-        ra.hdr = reinterpret_cast<const RegionHdr*>(q);
-        ra.prog = reinterpret_cast<const int32_t*>(q + hb);
-        ra.leaf_sl = reinterpret_cast<const SliceDigits*>(q + hb + pb);
-        ra.leaf_is = p.leaf_is_dev;
+        p.leaf_is_uploaded.assign(n, 0);
+        if (!ck(upload_regions(p.region_hdr, p.region_prog, p.leaf_sl, p.leaf_is_uploaded, &p.region_dev,
+                               &p.leaf_is_dev, ra), "region programs"))
+            return TN_ENOMEM;
         ra.leaf_ptrs = reinterpret_cast<const void* const*>(p.leaf_ptr_dev);
         ra.leafmax = p.leafmax;
         ra.ws = p.ws;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <functional>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -184,6 +185,34 @@ struct Plan {
     std::vector<cudaGraphNode_t> prof_nodes;    // their record nodes, in order
 };
 
+// A list of nodes (children first) as the region builder sees it: a plan's
+// own, or the forward and adjoint nodes of a reverse sweep.
+struct RegionOperand {
+    int producer;     // node of the list that computes it, -1: none
+    int leaf;         // leaf, -1: none
+    int slot;         // scale slot (nodes)
+    int64_t size, ws_off;
+};
+struct RegionView {
+    const NetDesc* d;
+    const Plan* p;    // labels and strides of the vertices
+    int copies;       // sharing a launch
+    std::function<const Node&(int)> node;
+    std::function<RegionOperand(int)> operand;  // of a vertex id (>= 0)
+};
+// Regions among the nodes [k0, k1): region_of those nodes (-1: none), members
+// in list order.
+void find_regions(const RegionView& v, int k0, int k1, std::vector<int>& region_of,
+                  std::vector<std::vector<int>>& regions);
+// Program of one region, appended to hdr and prog; stored: the members that
+// are written to the workspace, with their scale slots.
+void emit_region(const RegionView& v, const std::vector<int>& members, const std::vector<std::pair<int, int>>& stored,
+                 std::vector<int>& scratch, std::vector<RegionHdr>& hdr, std::vector<int32_t>& prog);
+// Device image of programs, leaf slice digits and leaf copy strides; fills the
+// table pointers of ra.
+cudaError_t upload_regions(const std::vector<RegionHdr>& hdr, const std::vector<int32_t>& prog,
+                           const std::vector<SliceDigits>& leaf_sl, const std::vector<int64_t>& leaf_is, void** dev,
+                           int64_t** leaf_is_dev, RegionArgs& ra);
 tn_status build_plan(const NetDesc& d, Plan& p, std::string& err);
 Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std::vector<int>& keep);
 // Tile shape and K split of a node whose sizes are not powers of two.

@@ -1,8 +1,8 @@
 """Subtree regions (small connected pieces of the tree, one block each).
 
 Networks of two-valued labels: a region adds up every output in the order of
-the per-node launches (TN_NO_FLOW=1), so amplitudes, copies and slices
-are the same bits.  Networks of other label sizes take another
+the per-node launches (TN_NO_FLOW=1), so amplitudes, copies, slices and
+gradients are the same bits.  Networks of other label sizes take another
 kernel there: against the nested sum instead, with the bound of the other
 any-size tests (1e-5 of the sum of |products|).
 """
@@ -98,6 +98,36 @@ def test_same_bits_with_copies(torch, monkeypatch, name, n_inst):
         finally:
             h.close()
     assert res[0] == res[1]
+
+
+@pytest.mark.parametrize("name,n_inst,sliced", [("circuit_2x2", 1, 0), ("circuit_4x4", 1, 0), ("circuit_4x4", 1, 2),
+                                                ("circuit_4x4", 3, 0), ("circuit_3x3_open", 1, 1),
+                                                ("ising_20", 2, 0), ("ising_100", 1, 0)])
+def test_gradients_have_the_same_bits(torch, monkeypatch, name, n_inst, sliced):
+    """Both halves of the reverse sweep, and the sweep over kept values."""
+    net = NETS[name]()
+    pairs = planner.greedy_tree(net.labels, net.dims, net.open)
+    sl = labels_to_slice(net, sliced)
+    rng = np.random.default_rng(1)
+    adj = rng.standard_normal((n_inst,) + tuple(net.dims[l] for l in net.open))
+    adj = adj + 1j * rng.standard_normal(adj.shape) if net.is_complex else adj
+    res = []
+    for flow in ("0", "1"):
+        monkeypatch.setenv("TN_NO_FLOW", flow)
+        h, strides = handle(torch, net, n_inst)
+        try:
+            for _ in range(2):
+                g = h.grad_instances(pairs, sl, "fp32", n_inst, strides, adj)
+                torch.cuda.synchronize()
+                res.append([x.cpu().numpy().tobytes() for x in g])
+            if not sliced and not net.open:
+                m, e, token = h.contract_instances_keep(pairs, "fp32", n_inst, strides)
+                g = h.grad_instances(pairs, sl, "fp32", n_inst, strides, adj, kept_forward=token)
+                torch.cuda.synchronize()
+                res.append([x.cpu().numpy().tobytes() for x in g])
+        finally:
+            h.close()
+    assert res[1:] == res[:-1]
 
 
 @pytest.mark.parametrize("seed", range(24))
