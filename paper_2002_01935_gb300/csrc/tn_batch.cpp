@@ -352,7 +352,8 @@ static cudaError_t enqueue_batch(BatchPlan& b, cudaStream_t s, const std::vector
             RegionArgs ra;
             memset(&ra, 0, sizeof(ra));
             const char* base = static_cast<const char*>(b.region_dev);
-            ra.hdr = reinterpret_cast<const RegionHdr*>(base) + st.region_begin;
+            ra.hdr = reinterpret_cast<const RegionHdr*>(base);
+            set_regions(ra, b.region_hdr, st.region_begin, st.regions);
             ra.prog = reinterpret_cast<const int32_t*>(base + (b.region_hdr.size() * sizeof(RegionHdr) + 255) / 256 * 256);
             ra.leaf_ptrs = reinterpret_cast<const void* const*>(b.leaf_ptr_dev);
             ra.leafmax = b.leafmax;
@@ -361,7 +362,6 @@ static cudaError_t enqueue_batch(BatchPlan& b, cudaStream_t s, const std::vector
             ra.exps = b.exps;
             ra.ctl = b.ctl;
             ra.t_done = b.t_done;
-            ra.n_regions = st.regions;
             ra.n_inst = 1;
             e = launch_regions(ra, st.cplx, q);
         } else if (st.wave) {

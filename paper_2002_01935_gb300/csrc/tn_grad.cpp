@@ -789,8 +789,7 @@ static cudaError_t enqueue_steps(const GradState& G, int k0, int k1, tn_mode mod
         const Step& st = G.steps[k];
         if (st.regions) {
             RegionArgs ra = G.region_args;
-            ra.hdr += st.region_begin;
-            ra.n_regions = st.regions;
+            set_regions(ra, G.region_hdr, st.region_begin, st.regions);
             e = launch_regions(ra, cplx, s);
         } else if (st.wave) {
             const WaveItem* it = G.items_dev + G.inst_item_begin[k];

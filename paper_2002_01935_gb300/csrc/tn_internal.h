@@ -358,11 +358,15 @@ struct RegionArgs {
     const Control* ctl;
     int32_t n_regions;
     int32_t n_inst;
+    int32_t words, entries;   // largest blob and arena of the launch's regions
 };
-constexpr int kRegionArena = 3072;   // entries
+// Limits of a region; a launch takes the shared memory of its largest one.
+// With half of arena and words a 16-qubit amplitude is five regions and a wave
+// (99 us of launches; three regions 91).
+constexpr int kRegionArena = 6144;   // entries
 constexpr int kRegionNodes = 192;
 constexpr int kRegionExt = 256;
-constexpr int kRegionWords = 9216;   // of the blob
+constexpr int kRegionWords = 15360;   // of the blob
 
 // Per-slice FP64 accumulation of the root tensor into the output
 // (Sec. 4.7.1: the sliced contractions are summed), with exponent

@@ -661,6 +661,16 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
     hdr.push_back(h);
 }
 
+void set_regions(RegionArgs& ra, const std::vector<RegionHdr>& hdr, int begin, int count) {
+    ra.hdr += begin;
+    ra.n_regions = count;
+    ra.words = ra.entries = 0;
+    for (int r = begin; r < begin + count; ++r) {
+        ra.words = std::max(ra.words, hdr[r].words);
+        ra.entries = std::max(ra.entries, hdr[r].n_elem + hdr[r].n_out);
+    }
+}
+
 cudaError_t upload_regions(const std::vector<RegionHdr>& hdr, const std::vector<int32_t>& prog,
                            const std::vector<SliceDigits>& leaf_sl, const std::vector<int64_t>& leaf_is, void** dev,
                            int64_t** leaf_is_dev, RegionArgs& ra) {
@@ -1412,8 +1422,7 @@ static cudaError_t enqueue_slice(const NetDesc& d, Plan& p, cudaStream_t s, cons
         const Step& st = p.steps[k];
         if (st.regions) {
             RegionArgs ra = p.region_args;
-            ra.hdr += st.region_begin;
-            ra.n_regions = st.regions;
+            set_regions(ra, p.region_hdr, st.region_begin, st.regions);
             e = launch_regions(ra, c, s);
         } else if (st.wave) {
             if (st.flow)

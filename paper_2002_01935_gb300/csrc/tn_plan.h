@@ -208,6 +208,8 @@ void find_regions(const RegionView& v, int k0, int k1, std::vector<int>& region_
 // are written to the workspace, with their scale slots.
 void emit_region(const RegionView& v, const std::vector<int>& members, const std::vector<std::pair<int, int>>& stored,
                  std::vector<int>& scratch, std::vector<RegionHdr>& hdr, std::vector<int32_t>& prog);
+// Launch of the regions [begin, begin + count) of hdr.
+void set_regions(RegionArgs& ra, const std::vector<RegionHdr>& hdr, int begin, int count);
 // Device image of programs, leaf slice digits and leaf copy strides; fills the
 // table pointers of ra.
 cudaError_t upload_regions(const std::vector<RegionHdr>& hdr, const std::vector<int32_t>& prog,

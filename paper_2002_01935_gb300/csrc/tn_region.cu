@@ -11,15 +11,18 @@
 // piece level by level with one barrier each, intermediates, maxima and
 // exponents in shared memory; only the nodes read from outside are stored.
 // Offsets come from tables, so label sizes of any kind are alike.  Bound by the
-// chain of levels: the loads at the start take three dependent round trips,
-// a level a few hundred nanoseconds.
+// chain of levels (about a microsecond each; a multiply-add costs some twenty
+// instructions) after three dependent round trips for header, program and
+// operands, which come by asynchronous copies.  The steps of a level (outputs
+// of one shape of sum) are dealt to the block's warps, not run one after another.
 //
 // Every output is summed in the order of the wave kernel (partial sums of
 // every g-th entry, then their tree), so the results are the same bits.
-// Launch times (waves alone before): 16-qubit, 8-cycle amplitude 77 -> 65 us in
-// two region launches and a wave, 32 copies of a 25-qubit one 221 -> 99, eight
-// slices of a 25-qubit tree 139 -> 81 (16 of it the regions), 69 nodes of
-// three-valued labels 10 instead of one launch each.
+// Launch times (waves alone before): 16-qubit, 8-cycle amplitude 77 -> 54 us in
+// three region launches, 32 copies of a 25-qubit one 221 -> 84, eight
+// slices of a 25-qubit tree 139 -> 76 (20 of it the regions), 69 nodes of
+// three-valued labels 10 instead of one launch each, forward and reverse sweep
+// of a 20-qubit circuit in 64 copies 1022 -> 333 (104 the regions).
 #include <cuda_runtime.h>
 #include <atomic>
 #include <stdint.h>
@@ -30,7 +33,6 @@ namespace tn {
 
 namespace {
 
-constexpr int kThreads = 256;
 
 template <bool CPLX>
 struct RT {
@@ -63,32 +65,48 @@ __device__ __forceinline__ float largest(float v) { return fabsf(v); }
 __device__ __forceinline__ float2 shifted(float2 v, int e) { return make_float2(ldexpf(v.x, e), ldexpf(v.y, e)); }
 __device__ __forceinline__ float shifted(float v, int e) { return ldexpf(v, e); }
 
+// asynchronous global -> shared copies (all of a thread's are in flight at once)
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// frexpf's exponent of a maximum, 0 for 0 and NaN
 __device__ __forceinline__ int exponent_of(unsigned bits) {
+    const unsigned e = bits >> 23;  // (maxima have no sign)
+    if (e - 1u < 254u) return (int)e - 126;
     const float m = __uint_as_float(bits);
     if (!(m > 0.f)) return 0;
-    int e;
-    frexpf(m, &e);
-    return e;
+    int x;
+    frexpf(m, &x);
+    return x;
 }
+__device__ __forceinline__ float power_of_two(int e) { return __uint_as_float((unsigned)(127 + e) << 23); }  // |e| <= 126
 
 // Outputs [q0, q1) of a step: 2^lg threads and A partial sums per thread each.
 // K index t belongs to partial sum t mod (A 2^lg); the sums are added as a
-// tree over their index, highest bit first.
-template <bool CPLX, int A>
-__device__ __forceinline__ void region_step(const RegionStep& st, int lg, const uint2* outs, const int32_t* ktab,
+// tree over their index, highest bit first.  This warp's lanes are the step's
+// threads i0 .. i0 + 31, i0 + THREADS ...
+template <bool CPLX, int A, int THREADS>
+__device__ __forceinline__ void region_step(const RegionStep& st, int lg, int i0, const uint2* outs, const int32_t* ktab,
                                             const RegionNode* nodes, typename RT<CPLX>::T* arena, int out0,
                                             unsigned* maxs, int64_t* exps, int n_ext) {
     using T = typename RT<CPLX>::T;
     const int lanes = 1 << lg, lane = threadIdx.x & (lanes - 1), n = (st.q1 - st.q0) << lg;
-    for (int i0 = 0; i0 < n; i0 += kThreads) {  // uniform over the block: shuffles below
-        const int i = i0 + threadIdx.x;
+    for (; i0 < n; i0 += THREADS) {  // uniform over the warp: shuffles below
+        const int i = i0 + (threadIdx.x & 31);
         const bool on = i < n;
         const int q = st.q0 + ((on ? i : 0) >> lg);
         const uint2 rec = outs[q];
         const RegionNode nd = nodes[rec.y];
         const int eA = exponent_of(maxs[nd.sa]), eB = exponent_of(maxs[nd.sb]);
         const int cA = max(-120, min(120, eA)), cB = max(-120, min(120, eB));
-        const float fa = ldexpf(1.f, -cA), fb = ldexpf(1.f, -cB);
+        const float fa = power_of_two(-cA), fb = power_of_two(-cB);
         const int resid = (eA - cA) + (eB - cB);
         const T* a = arena + nd.a + (rec.x & 0xffffu);
         const T* b = arena + nd.b + (rec.x >> 16);
@@ -128,8 +146,8 @@ __device__ __forceinline__ void region_step(const RegionStep& st, int lg, const 
     }
 }
 
-template <bool CPLX>
-__global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ RegionArgs a) {
+template <bool CPLX, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : 3) k_region(const __grid_constant__ RegionArgs a) {
     using T = typename RT<CPLX>::T;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RegionHdr h;
@@ -137,18 +155,19 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
     __shared__ int64_t exps[kRegionExt + kRegionNodes];
     __shared__ unsigned maxs[kRegionExt + kRegionNodes];
     int32_t* const blob = reinterpret_cast<int32_t*>(smem);
-    T* const arena = reinterpret_cast<T*>(smem + sizeof(int32_t) * kRegionWords);
+    T* const arena = reinterpret_cast<T*>(smem + sizeof(int32_t) * a.words);
     const int tid = threadIdx.x;
     const int region = blockIdx.x % a.n_regions, inst = blockIdx.x / a.n_regions;
-    const int64_t slice = a.ctl->slice + (int64_t)inst * a.slice_step;
-    if (slice >= a.ctl->slice_end) return;
     if (tid < (int)(sizeof(RegionHdr) / 4))
         reinterpret_cast<int32_t*>(&h)[tid] = reinterpret_cast<const int32_t*>(a.hdr + region)[tid];
+    const int64_t slice = a.ctl->slice + (int64_t)inst * a.slice_step, slice_end = a.ctl->slice_end;
     __syncthreads();
+    if (slice >= slice_end) return;
     {
         const int4* src = reinterpret_cast<const int4*>(a.prog + h.blob);
-        for (int i = tid; i < h.words / 4; i += kThreads) reinterpret_cast<int4*>(blob)[i] = src[i];
+        for (int i = tid; i < h.words / 4; i += THREADS) copy_async<16>(reinterpret_cast<int4*>(blob) + i, src + i);
     }
+    copies_done();
     __syncthreads();
     const uint2* outs = reinterpret_cast<const uint2*>(blob);
     const int32_t* ktab = blob + h.o_k;
@@ -159,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
     const RegionStore* stores = reinterpret_cast<const RegionStore*>(blob + h.o_store);
     // operands from outside: pointer, scale, and the slice offset of a leaf
     // (kept as its arena base for the nodes that read it)
-    for (int e = tid; e < h.n_ext; e += kThreads) {
+    for (int e = tid; e < h.n_ext; e += THREADS) {
         const RegionExt x = ext[e];
         int base = x.first;
         if (x.leaf >= 0) {
@@ -178,30 +197,39 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
         }
         ext[e].pad = base;
     }
-    for (int k = tid; k < h.n_nodes; k += kThreads) maxs[h.n_ext + k] = 0u;
+    for (int k = tid; k < h.n_nodes; k += THREADS) maxs[h.n_ext + k] = 0u;
     __syncthreads();
-    for (int i = tid; i < h.n_elem; i += kThreads) {
+    for (int i = tid; i < h.n_elem; i += THREADS) {
         const int e = elem[i];
-        arena[i] = ext_ptr[e][i - ext[e].first];
+        copy_async<sizeof(T)>(arena + i, ext_ptr[e] + (i - ext[e].first));
     }
-    for (int k = tid; k < h.n_nodes; k += kThreads) {
+    for (int k = tid; k < h.n_nodes; k += THREADS) {
         nodes[k].a = nodes[k].a >= 0 ? ext[nodes[k].a].pad : ~nodes[k].a;
         nodes[k].b = nodes[k].b >= 0 ? ext[nodes[k].b].pad : ~nodes[k].b;
     }
+    copies_done();
+    // the steps of a level are independent: their warps' shares are dealt round
+    // robin over the block, so that a level takes as long as its longest step
+    int dealt = 0;
     for (int s = 0; s < h.n_steps; ++s) {
         const RegionStep st = steps[s];
-        if (st.accs < 0) __syncthreads();
+        if (st.accs < 0) {
+            __syncthreads();
+            dealt = 0;
+        }
         const int A = st.accs < 0 ? -st.accs : st.accs, lg = st.lg_lanes;
+        const int i0 = (((tid >> 5) - dealt) & (THREADS / 32 - 1)) * 32;
+        dealt += (((st.q1 - st.q0) << lg) + 31) / 32;
         switch (A) {
-            case 1: region_step<CPLX, 1>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
-            case 2: region_step<CPLX, 2>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
-            case 4: region_step<CPLX, 4>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
-            default: region_step<CPLX, 8>(st, lg, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            case 1: region_step<CPLX, 1, THREADS>(st, lg, i0, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            case 2: region_step<CPLX, 2, THREADS>(st, lg, i0, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            case 4: region_step<CPLX, 4, THREADS>(st, lg, i0, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
+            default: region_step<CPLX, 8, THREADS>(st, lg, i0, outs, ktab, nodes, arena, h.n_elem, maxs, exps, h.n_ext); break;
         }
     }
     __syncthreads();
     // nodes that others read: one warp each
-    for (int r = tid >> 5; r < h.n_store; r += kThreads / 32) {
+    for (int r = tid >> 5; r < h.n_store; r += THREADS / 32) {
         const RegionStore so = stores[r];
         const int q0 = nodes[so.node].q0, q1 = so.node + 1 < h.n_nodes ? nodes[so.node + 1].q0 : h.n_out;
         T* dst = reinterpret_cast<T*>(a.ws) + (int64_t)inst * a.ws_is + so.ws_off;
@@ -218,14 +246,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_region(const __grid_constant__ 
     }
 }
 
-template <bool CPLX>
-cudaError_t launch_t(const RegionArgs& a, cudaStream_t s) {
-    constexpr size_t smem = sizeof(int32_t) * kRegionWords + kRegionArena * sizeof(typename RT<CPLX>::T);
+template <bool CPLX, int THREADS>
+cudaError_t launch_t(const RegionArgs& a, unsigned blocks, cudaStream_t s) {
+    constexpr size_t esz = sizeof(typename RT<CPLX>::T);
     static std::atomic<uint64_t> ready{0};
-    const cudaError_t e = allow_shared(k_region<CPLX>, smem, ready);
+    const cudaError_t e =
+        allow_shared(k_region<CPLX, THREADS>, sizeof(int32_t) * kRegionWords + kRegionArena * esz, ready);
     if (e != cudaSuccess) return e;
-    const int ni = a.n_inst > 1 ? a.n_inst : 1;
-    k_region<CPLX><<<(unsigned)(a.n_regions * ni), kThreads, smem, s>>>(a);
+    k_region<CPLX, THREADS><<<blocks, THREADS, sizeof(int32_t) * a.words + a.entries * esz, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -233,7 +261,12 @@ cudaError_t launch_t(const RegionArgs& a, cudaStream_t s) {
 
 cudaError_t launch_regions(const RegionArgs& a, bool is_c, cudaStream_t s) {
     if (a.n_regions <= 0) return cudaSuccess;
-    return is_c ? launch_t<true>(a, s) : launch_t<false>(a, s);
+    const unsigned blocks = (unsigned)(a.n_regions * (a.n_inst > 1 ? a.n_inst : 1));
+    // one block per SM or fewer: twice the threads for its levels (a 16-qubit
+    // amplitude's three regions 60 -> 54 us); more: more blocks side by side
+    // (both halves of a 64-copy sweep 104 us, 134 with 512 threads)
+    if (blocks <= (unsigned)sm_count()) return is_c ? launch_t<true, 512>(a, blocks, s) : launch_t<false, 512>(a, blocks, s);
+    return is_c ? launch_t<true, 256>(a, blocks, s) : launch_t<false, 256>(a, blocks, s);
 }
 
 }  // namespace tn
