@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
 // does not depend on the grid), y: batch entry, z: instance.
 // Bound by memory.  A node of 16 outputs over K = 2^18 in eight copies, 134 MB:
 // 262 us with one CTA per output and K part, which read each operand once per
-// row or column of the other, 89 now (call 3562 -> 2819 us, four of them).
+// row or column of the other, 61 now (89 with more CTAs than fit at a time).
 constexpr int kDotStages = 3;
 constexpr int kDotPer = kDotEntries / 256;   // copies per thread and tile
 constexpr int kDotTile = 1 << (2 * kDotLow);  // K entries of a tile of one output
@@ -790,8 +790,11 @@ __device__ __forceinline__ void cp_async_wait() {
 __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float2 shfl_xor(float2 v, int o) { return make_float2(shfl_xor(v.x, o), shfl_xor(v.y, o)); }
 
+// CTAs per SM (registers: RM x RN sums per thread)
+constexpr int dot_resident(bool cplx, int outs) { return cplx && outs >= 8 ? 2 : 3; }
+
 template <bool CPLX, int RM, int RN>
-__global__ void __launch_bounds__(256, CPLX && RM * RN >= 8 ? 2 : 3)
+__global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
     k_dot(const __grid_constant__ TileArgs a, const __grid_constant__ DotPlan dp, int parts) {
     using T = typename VT<CPLX>::T;
     extern __shared__ __align__(16) unsigned char dot_smem[];
@@ -1417,7 +1420,7 @@ static cudaError_t launch_dot_rc(const TileArgs& a, const DotPlan& dp, cudaStrea
     const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
     // parts of fewer than eight tiles: as many per CTA as make one round of
     // resident CTAs (longer ones balance better over many rounds)
-    const int64_t slots = (int64_t)sm_count() * 3, total = (int64_t)a.split * a.nbatch * ni;
+    const int64_t slots = (int64_t)sm_count() * dot_resident(CPLX, RM * RN), total = (int64_t)a.split * a.nbatch * ni;
     int parts = 1;
     if (((int64_t(1) << dp.u) + a.split - 1) / a.split < 8)
         parts = (int)std::min<int64_t>((total + slots - 1) / slots, a.split);
