@@ -1099,6 +1099,10 @@ __global__ void __launch_bounds__(256)
     // K offsets: low 8 bits of the K index from kA / kB, the rest (at most
     // 6 more bits: wave nodes have nk <= 14) from kAh / kBh
     __shared__ int64_t kA[256], kB[256], kAh[64], kBh[64];
+    // output offsets: low 8 bits of the output index, and the rest of each of
+    // the item's rows of 256 outputs (at most 4): bit loops per output took
+    // longer than its sum (32 copies of seven nodes 60 -> 51 us)
+    __shared__ int64_t oA[256], oB[256], oAh[4], oBh[4];
     __shared__ T red[256];
     __shared__ int cur;
     __shared__ int loaded;  // node whose descriptor and K tables are in shared memory
@@ -1130,7 +1134,13 @@ __global__ void __launch_bounds__(256)
         const View vw = inst_view(d, it.pad, (int)sizeof(T));
         const int kt = d.nk < 8 ? (int)(1ll << d.nk) : 256;  // table covers k & 255
         const int kh = d.nk > 8 && d.nk <= 14 ? (int)(1ll << (d.nk - 8)) : 0;  // k >> 8
+        auto o_scatter = [&](int64_t o, int64_t& offA, int64_t& offB) {
+            const int64_t n = o & ((1ll << d.nn) - 1), m = (o >> d.nn) & ((1ll << d.nm) - 1), b = o >> (d.nn + d.nm);
+            offA = scatter_bits(b, d.a_b, d.nb) + scatter_bits(m, d.a_m, d.nm);
+            offB = scatter_bits(b, d.b_b, d.nb) + scatter_bits(n, d.b_n, d.nn);
+        };
         if (fresh) {
+            if (!TILES || it.o_count >= 0) o_scatter(tid, oA[tid], oB[tid]);
             for (int t = tid; t < kt; t += 256) {
                 kA[t] = scatter_bits(t, d.a_k, d.nk);
                 kB[t] = scatter_bits(t, d.b_k, d.nk);
@@ -1152,6 +1162,12 @@ __global__ void __launch_bounds__(256)
                 d.b_leaf >= 0 ? (const char*)leaf_ptrs[d.b_leaf] + (int64_t)it.pad * d.in.b_is * isz : vw.B);
             sA = slice_off(d.sla, vw.slice);
             sB = slice_off(d.slb, vw.slice);
+            if (tid < 4 && tid * 256 < it.o_count) {
+                int64_t hA, hB;
+                o_scatter((it.o_begin + tid * 256) & ~255ll, hA, hB);
+                oAh[tid] = sA + hA;
+                oBh[tid] = sB + hB;
+            }
         }
         // ---- then wait for children computed in this launch
         if (deps != nullptr && tid == 0) {
@@ -1185,7 +1201,6 @@ __global__ void __launch_bounds__(256)
                 tile_body<CPLX, 64, 64, 16, 4, 4, true>(d, it.o_begin % tiles, 0, it.o_begin / tiles, vw, A, B, sc);
         } else if (vw.live) {
             const int64_t K = 1ll << d.nk;
-            const int64_t nmask = (1ll << d.nn) - 1, mmask = (1ll << d.nm) - 1;
             const int O = (int)it.o_count;
             const int g = O >= 256 ? 1 : 256 / O;
             auto k_off = [&](int64_t t, int64_t& ka, int64_t& kb2) {
@@ -1201,10 +1216,10 @@ __global__ void __launch_bounds__(256)
                     kb2 = kB[t & 255] + (hi ? scatter_bits(hi, d.b_k, d.nk) : 0);
                 }
             };
-            auto o_off = [&](int64_t o, int64_t& offA, int64_t& offB) {
-                const int64_t n = o & nmask, m = (o >> d.nn) & mmask, b = o >> (d.nn + d.nm);
-                offA = sA + scatter_bits(b, d.a_b, d.nb) + scatter_bits(m, d.a_m, d.nm);
-                offB = sB + scatter_bits(b, d.b_b, d.nb) + scatter_bits(n, d.b_n, d.nn);
+            auto o_off = [&](int ol, int64_t& offA, int64_t& offB) {
+                const int lo = ((int)it.o_begin + ol) & 255;
+                offA = oA[lo] + oAh[ol >> 8];
+                offB = oB[lo] + oBh[ol >> 8];
             };
             // the children's scale slots and this thread's first operand
             // pair are read together (one L2 round trip, not two)
@@ -1216,7 +1231,7 @@ __global__ void __launch_bounds__(256)
             T a0 = zero<T>(), b0 = zero<T>();
             if (first) {
                 int64_t offA, offB, ka, kb2;
-                o_off(it.o_begin + tid / g, offA, offB);
+                o_off(tid / g, offA, offB);
                 k_off(tid % g, ka, kb2);
                 a0 = ld_cg<CPLX>(A + offA + ka);
                 b0 = ld_cg<CPLX>(B + offB + kb2);
@@ -1227,7 +1242,7 @@ __global__ void __launch_bounds__(256)
             for (int ol = tid / g; ol < O; ol += 256 / g) {
                 const int64_t o = it.o_begin + ol;
                 int64_t offA, offB;
-                o_off(o, offA, offB);
+                o_off(ol, offA, offB);
                 T acc = zero<T>();
 #pragma unroll 4
                 for (int64_t t = tid % g; t < K; t += g) {
