@@ -761,7 +761,8 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
 // share a group of outputs).  blockIdx.x: `parts` consecutive K parts (short
 // parts share a CTA and its setup, each with its own partial, so that the sum
 // does not depend on the grid), y: batch entry, z: instance.
-// Bound by memory.  A node of 16 outputs over K = 2^18 in eight copies, 134 MB:
+// Bound by memory for few outputs, for many by the instructions of its copies.
+// A node of 16 outputs over K = 2^18 in eight copies, 134 MB:
 // 262 us with one CTA per output and K part, which read each operand once per
 // row or column of the other, 61 now (89 with more CTAs than fit at a time).
 constexpr int kDotStages = 3;
