@@ -258,28 +258,30 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
     std::vector<int> level(ncomb, 0), region_level(regions.size(), 0);
     int max_level = 0, fwd_levels = 0;
     // level of a node's step: after everything that it, or any member of its
-    // region, reads from outside (memoised; producers come earlier in the list)
-    std::function<int(int)> level_of = [&](int c) -> int {
+    // region, reads from outside.  A forward region is read at its last member
+    // and takes its turn there, an adjoint one reads the sweep at its first.
+    auto level_of = [&](int c, int floor) {
         const int r = region_of[c];
-        int& lv = r >= 0 ? region_level[r] : level[c];
-        if (lv > 0) return lv;
-        int l = c < nn ? 0 : fwd_levels;
+        int l = floor;
         auto visit = [&](int k) {
             for (int v : {cnode(k).ca, cnode(k).cb}) {
                 const int pr = producer(v);
-                if (pr >= 0 && (r < 0 || region_of[pr] != r)) l = std::max(l, level_of(pr));
+                if (pr >= 0 && (r < 0 || region_of[pr] != r))
+                    l = std::max(l, region_of[pr] >= 0 ? region_level[region_of[pr]] : level[pr]);
             }
         };
         if (r >= 0)
             for (int k : regions[r]) visit(k);
         else
             visit(c);
-        lv = l + 1;
-        return lv;
+        return l + 1;
     };
-    for (int c : order) {
-        const int l = level_of(c);
-        level[c] = l;
+    for (int c = 0; c < ncomb; ++c) {
+        const int r = region_of[c];
+        if (r >= 0 && c != (c < nn ? regions[r].back() : regions[r].front())) continue;
+        const int l = level_of(c, c < nn ? 0 : fwd_levels);
+        if (r >= 0) region_level[r] = l;
+        for (int k : r >= 0 ? regions[r] : std::vector<int>{c}) level[k] = l;
         max_level = std::max(max_level, l);
         if (c < nn) fwd_levels = max_level;
     }
