@@ -135,8 +135,10 @@ __device__ __forceinline__ void region_step(const RegionStep& st, int lg, int i0
             arena[out0 + q] = v;
             if (q == nd.q0) exps[n_ext + rec.y] = exps[nd.sa] + exps[nd.sb] + eA + eB;
         }
-        // the node's maximum: one shared atomic per warp where it holds one node
-        const unsigned m = on && lane == 0 ? __float_as_uint(largest(v)) : 0u;
+        // the node's maximum: one shared atomic per warp where it holds one node.
+        // fmaxf leaves NaN out, as the other kernels' maxima do (as bits it would
+        // be above every number, and the fold take the node for a zero one).
+        const unsigned m = on && lane == 0 ? __float_as_uint(fmaxf(largest(v), 0.f)) : 0u;
         if (__all_sync(0xffffffffu, rec.y == __shfl_sync(0xffffffffu, rec.y, 0))) {
             const unsigned w = __reduce_max_sync(0xffffffffu, m);
             if ((threadIdx.x & 31) == 0 && w) atomicMax(&maxs[n_ext + rec.y], w);
