@@ -192,7 +192,7 @@ struct FoldState {
     bool idle;          // nothing to write: all roots zero, accumulator stays
     bool vec;           // dst is 16-byte aligned
     bool plain;         // one root into zero: its values as they are
-    const double* fac;  // shared memory: factor of each instance, 0 for a zero root (n <= kFoldInst)
+    const double* fac;  // shared memory: factor of each instance, negative for a zero root (n <= kFoldInst)
 };
 
 // Maximum and exponent of instance i of the group.
@@ -242,18 +242,19 @@ __device__ __forceinline__ FoldState fold_state(const AccumArgs& a) {
     if (f.n > 1 && f.n <= kFoldInst) {  // the same factors for every output
         if ((int)threadIdx.x < f.n)
             sfac[threadIdx.x] =
-                __uint_as_float(smax[threadIdx.x]) > 0.f ? fold_pow2(sexp[threadIdx.x] - f.newE) : 0.0;
+                __uint_as_float(smax[threadIdx.x]) > 0.f ? fold_pow2(sexp[threadIdx.x] - f.newE) : -1.0;
         __syncthreads();
         f.fac = sfac;
     }
     return f;
 }
 
-// Root factor of instance i; false for a zero one.
+// Root factor of instance i; false for a zero root.  A factor may be zero (a
+// root far below the others): its infinities and NaN still reach the sum.
 __device__ __forceinline__ bool fold_factor(const AccumArgs& a, const FoldState& f, int i, double& fr) {
     if (f.fac) {
         fr = f.fac[i];
-        return fr != 0.0;
+        return fr >= 0.0;
     }
     if (!(__uint_as_float(fold_max(a, i)) > 0.f)) return false;
     fr = fold_pow2(fold_exp(a, i) - f.newE);
