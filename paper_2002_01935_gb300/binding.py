@@ -204,8 +204,12 @@ def _tree(pairs):
     if not isinstance(pairs, list):
         return _arr([x for p in pairs for x in p] or [0], np.int32)
     hit = _tree_cache.get(id(pairs))
-    if hit is not None and hit[2] is not None and hit[2] == pairs:
-        return hit[1]
+    if hit is not None and hit[2] is not None:
+        try:
+            if hit[2] == pairs:
+                return hit[1]
+        except Exception:  # a row that does not compare with a tuple (numpy: no truth value)
+            pass
     if hit is not None and len(hit[0]) == len(pairs):
         # element by element, so that a list of lists (e.g. pairs read from
         # JSON) or of numpy rows is reused like a list of tuples
