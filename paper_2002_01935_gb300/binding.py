@@ -388,8 +388,8 @@ class TensorNetwork:
         for ls in self.labels:
             n = 1
             for l in ls:
-                n *= self.dims[l]
-            self._numels.append(int(n))
+                n *= int(self.dims[l])
+            self._numels.append(n)
         self._keep: List = []
         if tensors is not None:
             self.set_tensors(tensors)
