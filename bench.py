@@ -690,11 +690,10 @@ def run_network(args, torch, dist, rank, world, local):
             modes_cmp[md] = entry
 
     groups = 1 if args.persistent else sc
-    # our kernels per call: call setup (leaf maxima + control block) and the
-    # result copy; per slice group the steps' launches and the accumulation
-    # (which also advances the slice counter when it is one block)
-    n_out = math.prod(net.dims[l] for l in net.open)
-    launches_per_call = 2 + groups * (1 + (n_out > 256) + sum(s.get("launches", 1) for s in steps))
+    # our kernels per call: the call setup (leaf maxima + control block); per
+    # slice group the steps' launches and the fold, which also advances the
+    # slice counter and, for the last group, writes the result
+    launches_per_call = 1 + groups * (1 + sum(s.get("launches", 1) for s in steps))
     cfg = {"workload": WORKLOAD_NAMES[args.workload] + ("_simplified" if args.simplify else ""),
            "mode": mode, "W_s": info.W, "C": info.C,
            "d_sliced": info.d_sliced, "slices_per_step": sc,
@@ -723,7 +722,8 @@ def run_network(args, torch, dist, rank, world, local):
         "e2e": e2e,
         "gpu_launches": launches_per_call * args.steps,
         "modes": modes_cmp,
-        "step_profile": [{"step": k, "kind": ["generic", "tile", "tcgen05"][s["kind"]],
+        "step_profile": [{"step": k, "kind": "subtrees" if not s["wave"] and len(s["nodes"]) > 1
+                          else ["generic", "tile", "tcgen05"][s["kind"]],
                           "wave": s["wave"], "nodes": len(s["nodes"]), "ms": round(step_ms[k], 4)}
                          for k, s in enumerate(steps)],
         "clocks": clocks,

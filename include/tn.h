@@ -439,12 +439,14 @@ tn_status tn_selftest_flow_timeout(void *stream);
  * Nodes (0..n_tensors-2, tree order) run in launch steps: a subtree step runs
  * connected pieces of the tree made of small nodes, one block each, in one
  * launch (is_wave 0, several nodes); a wave step runs all small nodes of one
- * or more tree levels in one launch; a single step runs one node.  *n_steps receives the number of steps; if cap >= *n_steps, then
- * step_info[5*s..5*s+4] = (is_wave, kernel kind 0 generic / 1 tiled /
- * 2 tensor core, tile configuration, number of nodes, kernel launches of
- * the step) and step_nodes lists
- * the nodes of step 0, then step 1, ... (n_tensors-1 entries in all; may be
- * NULL).  Errors as tn_plan_info.
+ * or more tree levels in one launch; a single step runs one node.  *n_steps
+ * receives the number of steps; if cap >= *n_steps, then
+ * step_info[5*s..5*s+4] = (is_wave, kernel kind 0 any sizes / 1 tiled /
+ * 2 tensor core, tile configuration -- 0 for waves, subtrees, tensor-core
+ * nodes and nodes of any sizes that take one thread per output --, number of
+ * nodes, kernel launches of the step) and step_nodes lists the nodes of step
+ * 0, then step 1, ... (n_tensors-1 entries in all; may be NULL).  The kind of
+ * a wave or subtree step is its first node's.  Errors as tn_plan_info.
  */
 tn_status tn_plan_steps(tn_net *net, const int32_t *tree_pairs, int32_t n_sliced,
                         const int64_t *sliced_labels, tn_mode mode, int32_t cap, int32_t *n_steps,

@@ -475,12 +475,17 @@ tn_status tn_plan_steps(tn_net* net, const int32_t* tree_pairs, int32_t n_sliced
         const tn::Node& first = p->nodes[stp.nodes[0]];
         step_info[5 * s + 0] = stp.wave;
         step_info[5 * s + 1] = first.kind;
-        step_info[5 * s + 2] = stp.wave || stp.regions ? 0 : (first.kind == tn::kTiled ? first.tile.cfg : 0);
+        const bool one = !stp.wave && !stp.regions;  // a launch step of one node
+        step_info[5 * s + 2] = !one                       ? 0
+                               : first.kind == tn::kTiled ? first.tile.cfg
+                               : first.kind == tn::kGeneric ? first.any_cfg : 0;
         step_info[5 * s + 3] = (int32_t)stp.nodes.size();
-        // a split-K tiled node adds its fixed-order reduction launch
-        step_info[5 * s + 4] = stp.wave || stp.regions ? 1
+        // K parts add their fixed-order reduction launch
+        const int split = first.kind == tn::kTiled ? first.tile.split
+                          : first.kind == tn::kGeneric && first.any_cfg ? first.any_split : 1;
+        step_info[5 * s + 4] = !one                             ? 1
                                : first.kind == tn::kTensorCore ? tn::tc_launches(first.tile)
-                               : 1 + (first.kind == tn::kTiled && first.tile.split > 1 ? 1 : 0);
+                                                               : 1 + (split > 1 ? 1 : 0);
         if (step_nodes)
             for (int k : stp.nodes) step_nodes[pos++] = k;
     }
