@@ -443,8 +443,8 @@ tn_status tn_selftest_flow_timeout(void *stream);
  * receives the number of steps; if cap >= *n_steps, then
  * step_info[5*s..5*s+4] = (is_wave, kernel kind 0 any sizes / 1 tiled /
  * 2 tensor core, tile configuration -- 0 for waves, subtrees, tensor-core
- * nodes and nodes of any sizes that take one thread per output --, number of
- * nodes, kernel launches of the step) and step_nodes lists the nodes of step
+ * nodes and nodes of any sizes that take one thread per output; 16 more where
+ * an operand (a slice of a leaf) spreads over 2^31 entries --, number of nodes, kernel launches of the step) and step_nodes lists the nodes of step
  * 0, then step 1, ... (n_tensors-1 entries in all; may be NULL).  The kind of
  * a wave or subtree step is its first node's.  Errors as tn_plan_info.
  */

@@ -477,7 +477,7 @@ tn_status tn_plan_steps(tn_net* net, const int32_t* tree_pairs, int32_t n_sliced
         step_info[5 * s + 1] = first.kind;
         const bool one = !stp.wave && !stp.regions;  // a launch step of one node
         step_info[5 * s + 2] = !one                       ? 0
-                               : first.kind == tn::kTiled ? first.tile.cfg
+                               : first.kind == tn::kTiled ? first.tile.cfg + (first.tile.wide ? 16 : 0)
                                : first.kind == tn::kGeneric ? first.any_cfg : 0;
         step_info[5 * s + 3] = (int32_t)stp.nodes.size();
         // K parts add their fixed-order reduction launch

@@ -144,7 +144,7 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
             nd.kind = kGeneric;
             if (f.force_generic) continue;
             if (!plan_tile_node(d, G.g, nd, se)) {
-                plan_any_tile(d, nd, se, copies);
+                plan_any_tile(d, G.g, nd, se, copies);
                 continue;
             }
             if (!f.no_tensor_cores) make_tensor_core(d, f.mode, nd, se, copies);
@@ -188,7 +188,7 @@ static tn_status build_grad(const NetDesc& d, const Plan& f, GradState& G, int c
             nd.kind = kGeneric;
             const int ca0 = nd.tile.conj_a, cb0 = nd.tile.conj_b;
             if (!plan_tile_node(d, G.g, nd, split_elems)) {
-                if (!f.force_generic) plan_any_tile(d, nd, split_elems, copies);
+                if (!f.force_generic) plan_any_tile(d, G.g, nd, split_elems, copies);
             } else if (!f.no_tensor_cores) {
                 make_tensor_core(d, f.mode, nd, split_elems, copies);
             }

@@ -136,6 +136,8 @@ struct alignas(16) TileArgs {
     int tc_bn128;         // tensor-core node: 128-column GEMM tiles even where 256 fit
     int tc_planar;        // tensor-core node: planar complex layout (see TcGeom)
     int tc_nopair;        // tensor-core node: single-CTA GEMM even where CTA pairs apply
+    int wide;             // an operand's offsets reach 2^31 entries: kernels with 64-bit ones
+    int dot_each;         // inner-product node: one CTA per output and K part (k_dot_one)
     InstanceInfo in;
 };
 

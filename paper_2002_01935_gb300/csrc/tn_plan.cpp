@@ -95,6 +95,16 @@ bool large_real_tiles(const NetDesc& d, int64_t nbatch, int64_t M, int64_t N) {
     return !d.is_complex() && M >= 128 && N >= 128 && ((M + 127) / 128) * ((N + 127) / 128) * nbatch >= sm_count();
 }
 
+// An operand whose offsets reach 2^31 entries.  Labels of a sliced leaf keep
+// the strides of the whole leaf, so that its slice may be small and yet
+// spread over more than that.
+bool wide_operand(const NetDesc& d, const Plan& p, int c) {
+    if (c < 0) return false;
+    double last = 0;
+    for (size_t i = 0; i < p.vlab[c].size(); ++i) last += (double)(d.dims[p.vlab[c][i]] - 1) * (double)p.vstride[c][i];
+    return last >= 2147483648.0;
+}
+
 // Tiled-kernel plan of a node whose labels and strides are all powers of
 // two: index bits per group, K order, load directions, tile shape and K
 // split.  Returns false (generic kernel) when a limit is exceeded.
@@ -169,7 +179,7 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         if (!push(t.b_k, tmp, l, stride_in(lb, sb, l))) return false;
     }
     if (t.nb > 16 || t.nm > 31 || t.nn > 31 || t.nk > 40 || t.nm + t.nn > 40) return false;
-    // the kernels keep per-thread operand offsets in 32 bits
+    t.wide = wide_operand(d, p, nd.ca) || wide_operand(d, p, nd.cb);
     for (const std::vector<int>* lab : {&la, &lb}) {
         int64_t sz = 1;
         for (int l : *lab) sz *= d.dims[l];
@@ -191,6 +201,7 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         TK = shapes[force_cfg][2];
     } else if (dot) {
         t.cfg = kTileDot;
+        t.dot_each = M * N == 1 || t.wide;
         TM = (int)M;
         TN = (int)N;
     } else if (t.nm <= 2 && t.nn >= 10) {
@@ -235,8 +246,8 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         // HBM).  2 x 32 outputs over K = 2^11: 34 us with parts of 1024 K
         // entries (two CTAs), 10 with parts of a few tiles; 4 x 4 over 2^18 in
         // eight slices: 161 us with parts of one tile, 89 with four.
-        const int64_t tiles = (K >> dot_tile_bits(t.nm, t.nn, t.nk)) / (M * N > 1 ? 4 : 1);
-        while (t.nbatch * p.copies * split < 8 * (int64_t)sm_count() && split * 2 <= tiles && split < 4096 &&
+        const int64_t tiles = t.dot_each ? K >> dot_tile_bits(0, 0, t.nk) : (K >> dot_tile_bits(t.nm, t.nn, t.nk)) / 4;
+        while ((t.dot_each ? outs : t.nbatch) * p.copies * split < 8 * (int64_t)sm_count() && split * 2 <= tiles && split < 4096 &&
                (int64_t)split * 2 * p.copies <= 65535)
             split *= 2;
         t.split = split;
@@ -323,7 +334,7 @@ Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std
 // output, which is one launch of a few microseconds whatever the kernel:
 // 3^9 multiply-adds 9.6 us against 11-12 with the tile kernel, 3^14 26 against
 // 19, 5^12 562 against 79, 7 x 5 outputs over K = 3^8 1809 against 28.
-void plan_any_tile(const NetDesc& d, Node& nd, int64_t& split_elems, int copies) {
+void plan_any_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, int copies) {
     nd.any_cfg = 0;
     nd.any_split = 1;
     auto volume = [&](std::initializer_list<const std::vector<int>*> groups) {
@@ -333,6 +344,7 @@ void plan_any_tile(const NetDesc& d, Node& nd, int64_t& split_elems, int copies)
         return v;
     };
     const double lim = 2147483648.0;  // the kernel's indices and offsets are 32-bit
+    if (wide_operand(d, p, nd.ca) || wide_operand(d, p, nd.cb)) return;
     const double M = volume({&nd.gm}), N = volume({&nd.gn}), B = volume({&nd.gb}), K = volume({&nd.gk, &nd.gsa, &nd.gsb});
     const double size_a = volume({&nd.gb, &nd.gm, &nd.gk, &nd.gsa}), size_b = volume({&nd.gb, &nd.gn, &nd.gk, &nd.gsb});
     if (M * N * K * B < 8192.0 || std::max(std::max(size_a, size_b), std::max(K, std::max(M, N))) >= lim) return;
@@ -874,7 +886,7 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
                 err = "the persistent launch needs power-of-two label sizes on every node";
                 return TN_EUNSUPPORTED;
             }
-            if (!p.force_generic) plan_any_tile(d, nd, split_elems, p.copies);
+            if (!p.force_generic) plan_any_tile(d, p, nd, split_elems, p.copies);
             continue;
         }
         if (p.persistent) {

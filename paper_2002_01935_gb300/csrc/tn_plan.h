@@ -218,7 +218,7 @@ cudaError_t upload_regions(const std::vector<RegionHdr>& hdr, const std::vector<
 tn_status build_plan(const NetDesc& d, Plan& p, std::string& err);
 Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std::vector<int>& keep);
 // Tile shape and K split of a node whose sizes are not powers of two.
-void plan_any_tile(const NetDesc& d, Node& nd, int64_t& split_elems, int copies = 1);
+void plan_any_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, int copies = 1);
 bool plan_tile_node(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems);
 bool make_tensor_core(const NetDesc& d, tn_mode mode, Node& nd, int64_t& split_elems, int copies = 1);
 // Autotuner variant code of the tensor-core kernel (tile shapes use TileCfg).

@@ -363,6 +363,20 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, int64_t tile_x, int
     }
 }
 
+// Operands spread over 2^31 entries (a slice of a larger leaf): the body above,
+// whose operand offsets are 64-bit.
+template <bool CPLX, int TM, int TN, int TK>
+__global__ void __launch_bounds__((TM / 4) * (TN / 4)) k_tile_wide(const __grid_constant__ TileArgs a) {
+    using T = typename VT<CPLX>::T;
+    const int per_inst = (int)(a.nbatch * a.split);
+    const int zz = blockIdx.z % per_inst;
+    const View vw = inst_view(a, blockIdx.z / per_inst, (int)sizeof(T));
+    if (!vw.live) return;
+    const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && zz == 0 && threadIdx.x == 0);
+    tile_body<CPLX, TM, TN, TK, 4, 4, false>(a, blockIdx.x, zz % a.split, zz / a.split, vw,
+                                             reinterpret_cast<const T*>(vw.A), reinterpret_cast<const T*>(vw.B), sc);
+}
+
 // --------------------------------------------------------------------------
 // Index groups of the two argument forms.  TileArgs (power-of-two sizes): an
 // offset is a scatter of index bits.  GenericArgs (any sizes): mixed-radix
@@ -516,7 +530,7 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN), MINB)
     auto row_of = [&](const Walk& w, int q, int S) { return w.wrap ? w.i0 + q % (S > NT ? S / NT : 1) * NT : w.i0 + q * w.di; };
     auto k_of = [&](const Walk& w, int q, int S) { return w.wrap ? q / (S > NT ? S / NT : 1) : w.t0 + q * w.dt; };
     // offset in the operand without the K base (sizes of any kind: without K)
-    int offA[LA], offB[LB];  // operands have below 2^31 entries
+    int offA[LA], offB[LB];  // the planner sends operands that reach 2^31 entries elsewhere (TileArgs::wide)
 #pragma unroll
     for (int q = 0; q < LA; ++q) {
         const int i = row_of(wa, q, TM);
@@ -818,7 +832,7 @@ __global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
         const int e = is_b ? e0 - n_a : e0, bits = t + (is_b ? a.nn : a.nm);
         int o = 0, c = is_b ? M << 16 : 0;
         for (int w = 0; w < bits; ++w)
-            if ((e >> w) & 1) {  // offsets within one operand: the planner keeps it below 2^31 entries
+            if ((e >> w) & 1) {  // offsets within one operand, below 2^31 entries (TileArgs::wide)
                 o += (int)(is_b ? dp.b_add : dp.a_add)[w];
                 c += (is_b ? dp.cb_add : dp.ca_add)[w];
             }
@@ -937,33 +951,37 @@ __global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
     cp_async_wait<0>();
 }
 
-// The one-output case: every thread multiplies its own four entries of a tile.
-// blockIdx.x: K part, y: batch entry, z: instance.  Bound by memory: K = 2^28
+// One output per CTA: every thread multiplies its own four entries of a tile.
+// blockIdx.x: K part and output, y: batch entry, z: instance.  For one-output
+// nodes, and (WIDE: 64-bit offsets) for operands spread over 2^31 entries.
+// Bound by memory: one output over K = 2^28
 // (4.3 GB) 726 us, 5.9 TB/s; as an instance of k_dot, whose loop over rows and
 // parts costs registers and instructions per copy, 820 to 1105.
-template <bool CPLX>
+template <bool CPLX, bool WIDE>
 __global__ void __launch_bounds__(256) k_dot_one(const __grid_constant__ TileArgs a, const __grid_constant__ DotPlan dp) {
     using T = typename VT<CPLX>::T;
+    using O = typename std::conditional<WIDE, int64_t, int32_t>::type;  // offset within an operand
     extern __shared__ __align__(16) unsigned char dot_smem[];
     constexpr int kPad = kDotTile + kDotTile / 32;  // one padding entry per 32: no bank conflicts
     T* const stg = reinterpret_cast<T*>(dot_smem);  // [stage][A, B][kPad]
-    int32_t* const offA = reinterpret_cast<int32_t*>(dot_smem + (size_t)kDotStages * 2 * kPad * sizeof(T));
-    int32_t* const offB = offA + kDotTile;
+    O* const offA = reinterpret_cast<O*>(dot_smem + (size_t)kDotStages * 2 * kPad * sizeof(T));
+    O* const offB = offA + kDotTile;
     uint16_t* const posA = reinterpret_cast<uint16_t*>(offB + kDotTile);
     uint16_t* const posB = posA + kDotTile;
     __shared__ T red[256];
     const int64_t b = blockIdx.y;
-    const int sp = blockIdx.x;
+    const int lg_out = a.nm + a.nn, out = (int)blockIdx.x & ((1 << lg_out) - 1), sp = (int)blockIdx.x >> lg_out;
     const View vw = inst_view(a, blockIdx.z, (int)sizeof(T));
     if (!vw.live) return;
     const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
     const int t = dp.t, u = dp.u, tsz = 1 << t;
     for (int e = threadIdx.x; e < tsz; e += 256) {
-        int xa = 0, xb = 0, pa = 0, pb = 0;
+        O xa = 0, xb = 0;
+        int pa = 0, pb = 0;
         for (int w = 0; w < t; ++w)
-            if ((e >> w) & 1) {  // offsets within one operand: the planner keeps it below 2^31 entries
-                xa += (int)dp.a_add[w];
-                xb += (int)dp.b_add[w];
+            if ((e >> w) & 1) {
+                xa += (O)dp.a_add[w];
+                xb += (O)dp.b_add[w];
                 pa += dp.ca_add[w];
                 pb += dp.cb_add[w];
             }
@@ -974,8 +992,10 @@ __global__ void __launch_bounds__(256) k_dot_one(const __grid_constant__ TileArg
     }
     __syncthreads();
     const int64_t slice = vw.slice;
-    const T* A = reinterpret_cast<const T*>(vw.A) + slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb);
-    const T* B = reinterpret_cast<const T*>(vw.B) + slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb);
+    const T* A = reinterpret_cast<const T*>(vw.A) + slice_off(a.sla, slice) + scatter_bits(b, a.a_b, a.nb) +
+                 scatter_bits(out >> a.nn, a.a_m, a.nm);
+    const T* B = reinterpret_cast<const T*>(vw.B) + slice_off(a.slb, slice) + scatter_bits(b, a.b_b, a.nb) +
+                 scatter_bits(out & ((1 << a.nn) - 1), a.b_n, a.nn);
     const int64_t n_tiles = int64_t(1) << u;
     const int64_t per = (n_tiles + a.split - 1) / a.split;
     const int64_t t0 = (int64_t)sp * per, t1 = min64(n_tiles, t0 + per);
@@ -1043,8 +1063,9 @@ __global__ void __launch_bounds__(256) k_dot_one(const __grid_constant__ TileArg
     }
     if (threadIdx.x == 0) {
         T v = red[0];
+        const int64_t o = (b << lg_out) + out;
         if (a.split > 1) {
-            reinterpret_cast<T*>(vw.P)[(int64_t)sp * a.nbatch + b] = v;
+            reinterpret_cast<T*>(vw.P)[(int64_t)sp * (a.nbatch << lg_out) + o] = v;
             return;
         }
         if (sc.resid) {
@@ -1055,7 +1076,7 @@ __global__ void __launch_bounds__(256) k_dot_one(const __grid_constant__ TileArg
                 v = ldexpf(v, -sc.resid);
             }
         }
-        reinterpret_cast<T*>(vw.C)[b] = v;
+        reinterpret_cast<T*>(vw.C)[o] = v;
         const float mx = absmax(v);
         if (mx > 0.f) atomicMax(vw.sc.max_c, __float_as_uint(mx));
         if (a.t_done) atomicMax(a.t_done, global_ns());
@@ -1358,10 +1379,12 @@ static cudaError_t launch_reduce(const ARGS& a, cudaStream_t s) {
 // lowest strides of either operand (its row bits, which are in every tile, take
 // part in that), the operands in turn, then the lowest K positions.  Then each
 // operand's order of its row and tile bits (ascending stride, absent bits last).
+// (One output per CTA: no row bits, they are in the operand's base.)
 static DotPlan make_dot_plan(const TileArgs& a) {
     DotPlan dp;
     memset(&dp, 0, sizeof(dp));
-    const int nk = a.nk, t_max = dot_tile_bits(a.nm, a.nn, a.nk);
+    const int nm = a.dot_each ? 0 : a.nm, nn = a.dot_each ? 0 : a.nn;
+    const int nk = a.nk, t_max = dot_tile_bits(nm, nn, nk);
     // by stride: K position, or -2 - i for row bit i; -1: none
     int by[2][64];
     for (int q = 0; q < 64; ++q) by[0][q] = by[1][q] = -1;
@@ -1369,8 +1392,8 @@ static DotPlan make_dot_plan(const TileArgs& a) {
         if (a.a_k[p] < 64) by[0][a.a_k[p]] = p;
         if (a.b_k[p] < 64) by[1][a.b_k[p]] = p;
     }
-    for (int i = 0; i < a.nm; ++i) by[0][a.a_m[i]] = -2 - i;
-    for (int i = 0; i < a.nn; ++i) by[1][a.b_n[i]] = -2 - i;
+    for (int i = 0; i < nm; ++i) by[0][a.a_m[i]] = -2 - i;
+    for (int i = 0; i < nn; ++i) by[1][a.b_n[i]] = -2 - i;
     bool in[kMaxBits] = {};
     int cnt = 0, q[2] = {0, 0}, low[2] = {0, 0};
     for (bool more = true; more && cnt < t_max;) {
@@ -1445,23 +1468,24 @@ static cudaError_t launch_dot_rc(const TileArgs& a, const DotPlan& dp, cudaStrea
     return cudaGetLastError();
 }
 
-template <bool CPLX>
+template <bool CPLX, bool WIDE>
 static cudaError_t launch_dot_one(const TileArgs& a, const DotPlan& dp, cudaStream_t s) {
     using T = typename VT<CPLX>::T;
-    constexpr size_t smem = (size_t)kDotStages * 2 * (kDotTile + kDotTile / 32) * sizeof(T) + kDotTile * 12;
+    constexpr size_t smem = (size_t)kDotStages * 2 * (kDotTile + kDotTile / 32) * sizeof(T) + kDotTile * (WIDE ? 20 : 12);
     static std::atomic<uint64_t> ready{0};
-    const cudaError_t e = allow_shared(k_dot_one<CPLX>, smem, ready);
+    const cudaError_t e = allow_shared(k_dot_one<CPLX, WIDE>, smem, ready);
     if (e != cudaSuccess) return e;
     const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
-    k_dot_one<CPLX><<<dim3((unsigned)a.split, (unsigned)a.nbatch, (unsigned)ni), 256, smem, s>>>(a, dp);
+    const dim3 grid((unsigned)a.split << (a.nm + a.nn), (unsigned)a.nbatch, (unsigned)ni);
+    k_dot_one<CPLX, WIDE><<<grid, 256, smem, s>>>(a, dp);
     return cudaGetLastError();
 }
 
 template <bool CPLX, int RM>
 static cudaError_t launch_dot_r(const TileArgs& a, const DotPlan& dp, cudaStream_t s) {
     if (a.nn == 0) {
-        if constexpr (RM == 1) return launch_dot_one<CPLX>(a, dp, s);
-        else return launch_dot_rc<CPLX, RM, 1>(a, dp, s);
+        if constexpr (RM > 1) return launch_dot_rc<CPLX, RM, 1>(a, dp, s);
+        else return cudaErrorInvalidValue;  // one output: k_dot_one
     }
     if (a.nn == 1) return launch_dot_rc<CPLX, RM, 2>(a, dp, s);
     return launch_dot_rc<CPLX, RM, 4>(a, dp, s);
@@ -1470,14 +1494,37 @@ static cudaError_t launch_dot_r(const TileArgs& a, const DotPlan& dp, cudaStream
 template <bool CPLX>
 static cudaError_t launch_dot(const TileArgs& a, cudaStream_t s) {
     const DotPlan dp = make_dot_plan(a);
+    if (a.wide) return launch_dot_one<CPLX, true>(a, dp, s);
+    if (a.dot_each) return launch_dot_one<CPLX, false>(a, dp, s);
     if (a.nm == 0) return launch_dot_r<CPLX, 1>(a, dp, s);
     if (a.nm == 1) return launch_dot_r<CPLX, 2>(a, dp, s);
     return launch_dot_r<CPLX, 4>(a, dp, s);
 }
 
+template <bool CPLX, int TM, int TN, int TK>
+static cudaError_t launch_wide_cfg(const TileArgs& a, cudaStream_t s) {
+    const int64_t tiles = ((host_m(a) + TM - 1) / TM) * ((host_n(a) + TN - 1) / TN);
+    const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
+    const dim3 grid((unsigned)tiles, 1, (unsigned)(a.nbatch * a.split * ni));
+    k_tile_wide<CPLX, TM, TN, TK><<<grid, (TM / 4) * (TN / 4), 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <bool CPLX>
+static cudaError_t launch_wide(const TileArgs& a, cudaStream_t s) {
+    switch (a.cfg) {
+        case kTile16x256: return launch_wide_cfg<CPLX, 16, 256, 16>(a, s);
+        case kTile4x1024: return launch_wide_cfg<CPLX, 4, 1024, 4>(a, s);
+        case kTile256x16: return launch_wide_cfg<CPLX, 256, 16, 16>(a, s);
+        default: return launch_wide_cfg<CPLX, 64, 64, 16>(a, s);  // K parts do not depend on the tile
+    }
+}
+
 template <bool CPLX>
 static cudaError_t launch_tile_t(const TileArgs& a, cudaStream_t s) {
-    const cudaError_t e = a.cfg == kTileDot ? launch_dot<CPLX>(a, s) : launch_shape<TileArgs, CPLX>(a, s);
+    const cudaError_t e = a.cfg == kTileDot ? launch_dot<CPLX>(a, s)
+                          : a.wide          ? launch_wide<CPLX>(a, s)
+                                            : launch_shape<TileArgs, CPLX>(a, s);
     if (e != cudaSuccess || a.split == 1) return e;
     return launch_reduce<TileArgs, CPLX>(a, s);
 }
