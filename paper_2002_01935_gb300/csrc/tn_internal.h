@@ -528,6 +528,9 @@ cudaError_t launch_regions(const RegionArgs& a, bool is_c, cudaStream_t s);
 // group into the call's output), leaves the result's exponent after the last
 // group, and advances the slice counter by `advance`.
 cudaError_t launch_accumulate(const AccumArgs& a, bool is_c, cudaStream_t s, int advance);
+// Writes the leaf pointer table (n pointers) in stream order.  The pointers
+// travel as kernel parameters: no host memory is read after the call returns.
+cudaError_t launch_leaf_table(const void* const* ptrs, int n, const void** table, cudaStream_t s);
 // Leaf maxima (as launch_leaf_max) and the call's control block (with the
 // output pointers that a direct fold writes), and n_acc doubles of the
 // accumulator cleared, in one launch.

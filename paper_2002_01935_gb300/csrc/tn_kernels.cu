@@ -679,6 +679,27 @@ cudaError_t launch_advance(Control* ctl, cudaStream_t s, int step) {
     return cudaGetLastError();
 }
 
+constexpr int kTablePart = 500;  // pointers per launch: 4 KB of parameters
+struct LeafTablePart {
+    const void* ptr[kTablePart];
+};
+
+__global__ void __launch_bounds__(512) k_leaf_table(const __grid_constant__ LeafTablePart p, int n, const void** table) {
+    if ((int)threadIdx.x < n) table[threadIdx.x] = p.ptr[threadIdx.x];
+}
+
+cudaError_t launch_leaf_table(const void* const* ptrs, int n, const void** table, cudaStream_t s) {
+    for (int i = 0; i < n; i += kTablePart) {
+        LeafTablePart p;
+        const int m = std::min(kTablePart, n - i);
+        memcpy(p.ptr, ptrs + i, sizeof(void*) * m);
+        k_leaf_table<<<1, 512, 0, s>>>(p, m, table + i);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Largest |component| of every leaf, so that leaves are renormalised like
 // intermediates before their first contraction.
 // Part blockIdx.y of leaf blockIdx.x: the largest |component| over its

@@ -1548,10 +1548,12 @@ static tn_status prepare_leaves(NetDesc& d, Plan& p, bool capturing, std::vector
     }
     if (p.leaf_ptr_uploaded != lp) {
         // the pointer table changes only when leaves are re-attached; the
-        // pageable source is staged before the copy returns, and the stream
-        // orders it between the calls that read the table
-        CK(cudaMemcpyAsync(p.leaf_ptr_dev, lp.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, stream));
-        if (capturing) CK(cudaStreamSynchronize(stream));
+        // stream orders the write between the calls that read the table
+        if (capturing) {
+            err = "re-attached leaves need a first call outside stream capture";
+            return TN_EUNSUPPORTED;
+        }
+        CK(launch_leaf_table(lp.data(), n, reinterpret_cast<const void**>(p.leaf_ptr_dev), stream));
         p.leaf_ptr_uploaded = lp;
     }
     return TN_OK;
