@@ -201,7 +201,8 @@ typedef struct {
  * are complete when the call returns (the call synchronises the stream).
  * The first call with a new (tree, slicing, mode) plans the nodes and
  * allocates the workspace (cached in the handle; a call during stream
- * capture must reuse a cached plan).  Errors: TN_EINVAL (malformed tree,
+ * capture must reuse a cached plan and the leaves of the call before it, and
+ * its replays keep reading those).  Errors: TN_EINVAL (malformed tree,
  * sliced label open or unknown, a leaf without data), TN_EUNSUPPORTED (an
  * intermediate of the sliced tree with more than 2^40 entries, or a node of
  * more than 2^62 multiply-adds), TN_ENOMEM, TN_ECUDA, TN_ETIMEOUT.

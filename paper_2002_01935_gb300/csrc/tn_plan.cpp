@@ -1546,13 +1546,16 @@ static tn_status prepare_leaves(NetDesc& d, Plan& p, bool capturing, std::vector
         if (nd.ca >= 0 && nd.ca < n) p.gen[k].A = nd.tile.A = lp[nd.ca];
         if (nd.cb >= 0 && nd.cb < n) p.gen[k].B = nd.tile.B = lp[nd.cb];
     }
-    if (p.leaf_ptr_uploaded != lp) {
-        // the pointer table changes only when leaves are re-attached; the
-        // stream orders the write between the calls that read the table
-        if (capturing) {
-            err = "re-attached leaves need a first call outside stream capture";
-            return TN_EUNSUPPORTED;
-        }
+    if (capturing && p.leaf_ptr_uploaded != lp) {
+        err = "re-attached leaves need a first call outside stream capture";
+        return TN_EUNSUPPORTED;
+    }
+    // The pointer table changes only when leaves are re-attached; the stream
+    // orders the write between the calls that read the table.  A captured
+    // call writes its own pointers at every replay, so once there is one,
+    // direct calls write theirs every time.
+    p.captured |= capturing;
+    if (p.captured || p.leaf_ptr_uploaded != lp) {
         CK(launch_leaf_table(lp.data(), n, reinterpret_cast<const void**>(p.leaf_ptr_dev), stream));
         p.leaf_ptr_uploaded = lp;
     }
@@ -2133,6 +2136,7 @@ void free_device(Plan& p) {
     p.leaf_ptr_dev = nullptr;
     p.leaf_nfloat_dev = nullptr;
     p.leaf_ptr_uploaded.clear();
+    p.captured = false;
     p.gexec = nullptr;
     p.cap_stream = nullptr;
     p.ws = nullptr;

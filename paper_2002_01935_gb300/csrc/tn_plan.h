@@ -142,6 +142,7 @@ struct Plan {
     const float** leaf_ptr_dev = nullptr;  // device copy of the leaf pointers
     int64_t* leaf_nfloat_dev = nullptr;
     std::vector<const void*> leaf_ptr_uploaded;
+    bool captured = false;  // a caller's stream capture holds a call of this plan
     std::vector<GenericArgs> gen;
     GradState* grad = nullptr;
     // instances (slice-parallel or independent copies)
