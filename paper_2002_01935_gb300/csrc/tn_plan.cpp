@@ -1291,8 +1291,10 @@ tn_status alloc_plan(NetDesc& d, Plan& p, void* unit, std::string& err) {
 // Write the instance layout (G instances; step 1: instance i = slice s+i,
 // step 0: independent copies whose leaf v sits leaf_is[v] elements apart)
 // into every node's launch arguments, the wave items and the accumulator.
+// The device tables are written in the stream's order: earlier calls on it may
+// still be reading them.
 static tn_status configure_instances(const NetDesc& d, Plan& p, int G, int step,
-                                     const std::vector<int64_t>& leaf_is, std::string& err) {
+                                     const std::vector<int64_t>& leaf_is, cudaStream_t stream, std::string& err) {
     if (p.cfg_inst == G && p.cfg_step == step && p.cfg_leaf_is == leaf_is) return TN_OK;
     const int n = d.n;
     const int nn = (int)p.nodes.size();
@@ -1380,9 +1382,10 @@ static tn_status configure_instances(const NetDesc& d, Plan& p, int G, int step,
                 j0 = j1;
             }
         }
-        cudaError_t e = cudaMemcpy(p.descs_dev, descs.data(), sizeof(TileArgs) * nn, cudaMemcpyHostToDevice);
+        cudaError_t e = cudaMemcpyAsync(p.descs_dev, descs.data(), sizeof(TileArgs) * nn, cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess)
-            e = cudaMemcpy(p.items_dev, items.data(), sizeof(WaveItem) * items.size(), cudaMemcpyHostToDevice);
+            e = cudaMemcpyAsync(p.items_dev, items.data(), sizeof(WaveItem) * items.size(), cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the lists end with this block
         if (e != cudaSuccess) {
             err = std::string("instance layout upload: ") + cudaGetErrorString(e);
             return TN_ECUDA;
@@ -1391,7 +1394,8 @@ static tn_status configure_instances(const NetDesc& d, Plan& p, int G, int step,
     if (p.leaf_is_dev) {
         const std::vector<int64_t> is = leaf_is.empty() ? std::vector<int64_t>(n, 0) : leaf_is;
         if (is != p.leaf_is_uploaded) {
-            const cudaError_t e = cudaMemcpy(p.leaf_is_dev, is.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice);
+            cudaError_t e = cudaMemcpyAsync(p.leaf_is_dev, is.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
             if (e != cudaSuccess) {
                 err = std::string("instance layout upload: ") + cudaGetErrorString(e);
                 return TN_ECUDA;
@@ -1644,14 +1648,15 @@ static int64_t max_leaf_floats(const NetDesc& d) {
 }
 
 static tn_status upload_leaf_sizes(const NetDesc& d, Plan& p, int G, const std::vector<int64_t>& leaf_is,
-                                   std::string& err) {
+                                   cudaStream_t stream, std::string& err) {
     std::vector<int64_t> nf(d.n);
     for (int v = 0; v < d.n; ++v) {
         const int64_t is = leaf_is.empty() ? 0 : leaf_is[v];
         nf[v] = ((int64_t)(G - 1) * is + d.leaves[v].size) * (d.is_complex() ? 2 : 1);
     }
     if (nf == p.leaf_nfloat_uploaded) return TN_OK;
-    CK(cudaMemcpy(p.leaf_nfloat_dev, nf.data(), sizeof(int64_t) * d.n, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(p.leaf_nfloat_dev, nf.data(), sizeof(int64_t) * d.n, cudaMemcpyHostToDevice, stream));
+    CK(cudaStreamSynchronize(stream));
     p.leaf_nfloat_uploaded = nf;
     return TN_OK;
 }
@@ -1687,10 +1692,10 @@ tn_status run_plan(NetDesc& d, Plan& p, void* unit, int64_t begin, int64_t count
         err = "the first call with a new slice batch must run outside stream capture";
         return TN_EUNSUPPORTED;
     }
-    tn_status st = configure_instances(d, p, G, 1, std::vector<int64_t>(), err);
+    tn_status st = configure_instances(d, p, G, 1, std::vector<int64_t>(), stream, err);
     if (st != TN_OK) return st;
     if (!capturing) {
-        st = upload_leaf_sizes(d, p, 1, std::vector<int64_t>(), err);
+        st = upload_leaf_sizes(d, p, 1, std::vector<int64_t>(), stream, err);
         if (st != TN_OK) return st;
     }
     std::vector<const void*> lp;
@@ -1755,9 +1760,9 @@ tn_status run_instances(NetDesc& d, Plan& p, void* unit, int n_inst, const int64
     std::vector<int64_t> leaf_is(n, 0);
     if (leaf_is_arr)
         for (int v = 0; v < n; ++v) leaf_is[v] = leaf_is_arr[v];
-    tn_status st = configure_instances(d, p, G, 0, leaf_is, err);
+    tn_status st = configure_instances(d, p, G, 0, leaf_is, stream, err);
     if (st != TN_OK) return st;
-    st = upload_leaf_sizes(d, p, G, leaf_is, err);
+    st = upload_leaf_sizes(d, p, G, leaf_is, stream, err);
     if (st != TN_OK) return st;
     if (p.inst_roots_n != G) {
         const Node& root = p.nodes.back();
@@ -1769,7 +1774,8 @@ tn_status run_instances(NetDesc& d, Plan& p, void* unit, int n_inst, const int64
             roots[i].is_c = d.is_complex();
             roots[i].pad = 0;
         }
-        CK(cudaMemcpy(p.inst_roots_dev, roots.data(), sizeof(BatchRoot) * G, cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(p.inst_roots_dev, roots.data(), sizeof(BatchRoot) * G, cudaMemcpyHostToDevice, stream));
+        CK(cudaStreamSynchronize(stream));
         p.inst_roots_n = G;
     }
     std::vector<const void*> lp;
@@ -1935,9 +1941,9 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
         }
     if (tune.empty()) return TN_OK;
     // bind this call's leaves (their values do not matter for timing)
-    tn_status st = configure_instances(d, p, 1, 1, std::vector<int64_t>(), err);
+    tn_status st = configure_instances(d, p, 1, 1, std::vector<int64_t>(), s, err);
     if (st != TN_OK) return st;
-    st = upload_leaf_sizes(d, p, 1, std::vector<int64_t>(), err);
+    st = upload_leaf_sizes(d, p, 1, std::vector<int64_t>(), s, err);
     if (st != TN_OK) return st;
     std::vector<const void*> lp;
     st = prepare_leaves(d, p, false, lp, s, err);
