@@ -306,14 +306,19 @@ __device__ __forceinline__ void fold_store(const FoldState& f, int64_t o, double
 }
 
 // After the data: the accumulator's exponent, after the call's last group
-// the result's, and the slice counter.  Run by the last block to get here
-// (each block's reads of the control block come before its ticket), so that
-// no launch of its own is needed for them.
+// the result's, and the slice counter.  Run by the last block to get here, so
+// that no launch of its own is needed for them.  The fences order each block's
+// reads of the control block before its ticket, and the last ticket before the
+// writes.
 __device__ __forceinline__ void fold_finish(const AccumArgs& a, const FoldState& f) {
     __shared__ unsigned ticket;
     if (gridDim.x > 1) {
         __syncthreads();
-        if (threadIdx.x == 0) ticket = atomicInc(&a.ctl->ticket, gridDim.x - 1);  // wraps to 0 at the last block
+        if (threadIdx.x == 0) {
+            __threadfence();
+            ticket = atomicInc(&a.ctl->ticket, gridDim.x - 1);  // wraps to 0 at the last block
+            __threadfence();
+        }
         __syncthreads();
         if (ticket != gridDim.x - 1) return;
     } else {
