@@ -330,10 +330,24 @@ Node build_node(const NetDesc& d, const Plan& p, int id, int a, int b, const std
 // The tile kernel for sizes of any kind.  The shape follows the rule of
 // plan_tile (4 x 1024 up to 4 rows, 16 x 256 up to 32, 256 x 16 up to 32
 // columns, else 64 x 64); the K split gives every SM a tile, each part at
-// least 16 entries.  Nodes of fewer than 2^13 multiply-adds keep one thread per
-// output, which is one launch of a few microseconds whatever the kernel:
-// 3^9 multiply-adds 9.6 us against 11-12 with the tile kernel, 3^14 26 against
-// 19, 5^12 562 against 79, 7 x 5 outputs over K = 3^8 1809 against 28.
+// least 16 entries.  A node takes it where the estimates below say that it is
+// faster than one thread per output: 3^14 multiply-adds 26 us against 19, 5^12
+// 562 against 79, 7 x 5 outputs over K = 3^8 1809 against 28.  Tiles that
+// batch labels leave nearly empty cost about 6 us a round of resident blocks
+// all the same (3^9 entries of 3 x 3 outputs over K = 3: 275 us, 13 with one
+// thread per output; 3^10 entries of one product each: 752 and 8), as do short
+// sums of few outputs (9.6 us against 11-12 below 2^13 multiply-adds).
+//
+// Microseconds, fitted to nodes of 1 to 10^7 outputs over K = 1 to 3^10:
+// rounds of resident blocks, each with its setup and its K steps ...
+static double any_tile_us(const NetDesc& d, int cfg, double blocks, int64_t kchunk, int split) {
+    const double slots = (cfg == kTile64x64 ? 3.0 : 2.0) * sm_count();
+    const double steps = std::ceil((double)kchunk / (cfg == kTile4x1024 ? 4.0 : 8.0));
+    return 3.5 + std::ceil(blocks / slots) * (6.0 + steps * (d.is_complex() ? 1.2 : 0.6)) + (split > 1 ? 6.0 : 0.0);
+}
+// ... and one thread's serial sum, or all products at the launch's rate.
+static double any_generic_us(double outputs, double K) { return 7.0 + std::max(0.19 * K, outputs * (K + 3.0) / 220e3); }
+
 void plan_any_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, int copies) {
     nd.any_cfg = 0;
     nd.any_split = 1;
@@ -375,8 +389,12 @@ void plan_any_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_ele
     while (tiles * copies * split < sm_count() && split * 2 <= ktiles && split < 64 &&
            B * split * 2 * copies <= 65535)
         split *= 2;
+    const int64_t kchunk = ((ktiles + split - 1) / split) * TK;
+    if (any_tile_us(d, cfg, tiles * copies * split, std::min(kchunk, (int64_t)K), split) >=
+        any_generic_us(M * N * B * copies, K))
+        return;
     nd.any_cfg = cfg;
-    nd.any_kchunk = ((ktiles + split - 1) / split) * TK;
+    nd.any_kchunk = kchunk;
     nd.any_split = (int)(((int64_t)K + nd.any_kchunk - 1) / nd.any_kchunk);  // no empty part
     if (nd.any_split > 1) split_elems = std::max(split_elems, (int64_t)nd.any_split * (int64_t)(B * M * N));
 }

@@ -38,3 +38,18 @@ def test_any_sizes(cplx):
 def test_power_of_two():
     s = step([2] * 6, [2] * 6, [2] * 14)
     assert (s["kind"], s["launches"]) == (1, 2) and s["cfg"] > 0
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("m,n,k,b,tiled", [
+    (0, 0, 0, 10, False),  # products of single entries
+    (1, 1, 1, 6, False), (1, 1, 1, 9, False), (2, 1, 1, 7, False), (0, 0, 2, 8, False), (0, 3, 1, 7, False),
+    (2, 2, 2, 6, False), (0, 9, 0, 0, False),  # nearly empty tiles, few products
+    (1, 1, 8, 0, True), (0, 0, 10, 0, True), (0, 0, 8, 3, True), (0, 1, 5, 5, True),  # long sums
+    (5, 5, 5, 0, True), (3, 3, 4, 2, True),
+])
+def test_tiles_that_would_run_empty(m, n, k, b, tiled, cplx):
+    """Nodes of three-valued labels: the tile kernel where its tiles are filled
+    or the sums long, one thread per output elsewhere."""
+    s = step([3] * m, [3] * n, [3] * k, [3] * b, cplx)
+    assert s["kind"] == 0 and (s["cfg"] > 0) == tiled
