@@ -772,9 +772,12 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
 // tiles keeps two tiles of copies in flight per CTA while a third is
 // multiplied; the tile base offsets follow the tile index by its carry chain.
 // Each thread multiplies RM x RN outputs over every LPG-th K entry (LPG threads
-// share a group of outputs).  blockIdx.x: `parts` consecutive K parts (short
-// parts share a CTA and its setup, each with its own partial, so that the sum
-// does not depend on the grid), y: batch entry, z: instance.
+// share a group of outputs).  blockIdx.x: batch entry, y: `parts` consecutive K
+// parts (short parts share a CTA and its setup, each with its own partial, so
+// that the sum does not depend on the grid), z: instance.  The batch entries of
+// a K part run together: where they are an operand's fastest label they read
+// the same lines (16 entries over K = 2^20 and 4 outputs, complex: 1098 us with
+// the K parts of an entry together, 458 this way).
 // Bound by memory for few outputs, for many by the instructions of its copies.
 // A node of 16 outputs over K = 2^18 in eight copies, 134 MB:
 // 262 us with one CTA per output and K part, which read each operand once per
@@ -817,7 +820,7 @@ __global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
     __shared__ T red[8][64];
     const int tid = threadIdx.x;
     const int N = 1 << a.nn, M = 1 << a.nm;
-    const int64_t b = blockIdx.y;
+    const int64_t b = blockIdx.x;
     const View vw = inst_view(a, blockIdx.z, (int)sizeof(T));
     if (!vw.live) return;
     const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && tid == 0);
@@ -847,7 +850,7 @@ __global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
     const int64_t n_tiles = int64_t(1) << u;
     const int64_t per = (n_tiles + a.split - 1) / a.split;
     int left = (int)min64(per, 1 << 30);  // tiles to the end of the current part
-    const int64_t t0 = (int64_t)blockIdx.x * parts * per, t1 = min64(n_tiles, t0 + parts * per);
+    const int64_t t0 = (int64_t)blockIdx.y * parts * per, t1 = min64(n_tiles, t0 + parts * per);
     // offsets of the next tile to copy; advanced tile by tile along the carry chain
     int64_t nt = t0, ba = 0, bb = 0;
     for (int j = 0; j < u; ++j)
@@ -952,8 +955,9 @@ __global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
 }
 
 // One output per CTA: every thread multiplies its own four entries of a tile.
-// blockIdx.x: K part and output, y: batch entry, z: instance.  For one-output
-// nodes, and (WIDE: 64-bit offsets) for operands spread over 2^31 entries.
+// blockIdx.x: batch entry and output, y: K part, z: instance.  For one-output
+// nodes, several where the planner's rule says so, and (WIDE: 64-bit offsets)
+// operands spread over 2^31 entries.
 // Bound by memory: one output over K = 2^28
 // (4.3 GB) 726 us, 5.9 TB/s; as an instance of k_dot, whose loop over rows and
 // parts costs registers and instructions per copy, 820 to 1105.
@@ -969,8 +973,8 @@ __global__ void __launch_bounds__(256) k_dot_one(const __grid_constant__ TileArg
     uint16_t* const posA = reinterpret_cast<uint16_t*>(offB + kDotTile);
     uint16_t* const posB = posA + kDotTile;
     __shared__ T red[256];
-    const int64_t b = blockIdx.y;
-    const int lg_out = a.nm + a.nn, out = (int)blockIdx.x & ((1 << lg_out) - 1), sp = (int)blockIdx.x >> lg_out;
+    const int lg_out = a.nm + a.nn, out = (int)blockIdx.x & ((1 << lg_out) - 1), sp = (int)blockIdx.y;
+    const int64_t b = blockIdx.x >> lg_out;
     const View vw = inst_view(a, blockIdx.z, (int)sizeof(T));
     if (!vw.live) return;
     const Scales sc = node_scales(vw.sc, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
@@ -1464,7 +1468,7 @@ static cudaError_t launch_dot_rc(const TileArgs& a, const DotPlan& dp, cudaStrea
     if (((int64_t(1) << dp.u) + a.split - 1) / a.split < 8)
         parts = (int)std::min<int64_t>((total + slots - 1) / slots, a.split);
     const unsigned blocks = (unsigned)((a.split + parts - 1) / parts);
-    k_dot<CPLX, RM, RN><<<dim3(blocks, (unsigned)a.nbatch, (unsigned)ni), 256, smem, s>>>(a, dp, parts);
+    k_dot<CPLX, RM, RN><<<dim3((unsigned)a.nbatch, blocks, (unsigned)ni), 256, smem, s>>>(a, dp, parts);
     return cudaGetLastError();
 }
 
@@ -1476,7 +1480,7 @@ static cudaError_t launch_dot_one(const TileArgs& a, const DotPlan& dp, cudaStre
     const cudaError_t e = allow_shared(k_dot_one<CPLX, WIDE>, smem, ready);
     if (e != cudaSuccess) return e;
     const int ni = a.in.n_inst > 1 ? a.in.n_inst : 1;
-    const dim3 grid((unsigned)a.split << (a.nm + a.nn), (unsigned)a.nbatch, (unsigned)ni);
+    const dim3 grid((unsigned)a.nbatch << (a.nm + a.nn), (unsigned)a.split, (unsigned)ni);
     k_dot_one<CPLX, WIDE><<<grid, 256, smem, s>>>(a, dp);
     return cudaGetLastError();
 }
