@@ -105,6 +105,28 @@ bool wide_operand(const NetDesc& d, const Plan& p, int c) {
     return last >= 2147483648.0;
 }
 
+// Inner-product nodes: one CTA per output (and K part) instead of one for all
+// outputs.  tiles: 1024 products of one output.
+//  - One output: always.
+//  - Few tiles, two per SM: the outputs side by side are then faster than one
+//    after the other (8 x 8 outputs over K = 2^9: 8.8 us against 17, 2 x 2 over
+//    2^14 13 against 17; from 512 tiles on 17 to 20 either way or worse).
+//  - One row (column) whose operand does not fit L2 and is contiguous along K
+//    (at most 4 outputs or batch entries among 32 neighbours): it is read once
+//    in either form, in whole lines here (64 outputs over K = 2^18, real, 67 MB:
+//    54 us against 79; below 8192 tiles 1.2 to 3 times slower).
+bool dot_each_output(const TileArgs& t, int copies) {
+    if (t.nm + t.nn == 0) return true;
+    const int64_t tiles = (t.nbatch << (t.nm + t.nn)) * copies * std::max<int64_t>(1, (int64_t(1) << t.nk) / 1024);
+    if (tiles <= 2 * (int64_t)sm_count()) return true;
+    if (std::min(t.nm, t.nn) > 0 || tiles < 8192) return false;
+    const bool b = t.nm == 0;  // the operand that holds the outputs
+    int low = 0;
+    for (int i = 0; i < (b ? t.nn : t.nm); ++i) low += (b ? t.b_n : t.a_m)[i] < 5;
+    for (int i = 0; i < t.nb; ++i) low += (b ? t.b_b : t.a_b)[i] < 5;
+    return low <= 2;
+}
+
 // Tiled-kernel plan of a node whose labels and strides are all powers of
 // two: index bits per group, K order, load directions, tile shape and K
 // split.  Returns false (generic kernel) when a limit is exceeded.
@@ -201,7 +223,7 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         TK = shapes[force_cfg][2];
     } else if (dot) {
         t.cfg = kTileDot;
-        t.dot_each = M * N == 1 || t.wide;
+        t.dot_each = t.wide || dot_each_output(t, p.copies);
         TM = (int)M;
         TN = (int)N;
     } else if (t.nm <= 2 && t.nn >= 10) {
