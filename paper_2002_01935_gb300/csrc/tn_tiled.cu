@@ -1165,8 +1165,12 @@ __global__ void __launch_bounds__(256)
             offA = scatter_bits(b, d.a_b, d.nb) + scatter_bits(m, d.a_m, d.nm);
             offB = scatter_bits(b, d.b_b, d.nb) + scatter_bits(n, d.b_n, d.nn);
         };
+        // an item that is its CTA's only one, with one output per thread, enters
+        // just its own outputs, high bits and all (one bit loop, not one after
+        // the other: 2^14 outputs over K = 4 12.7 -> 11.3 us)
+        const bool direct = deps == nullptr && it.o_count <= 256;
         if (fresh) {
-            if (!TILES || it.o_count >= 0) o_scatter(tid, oA[tid], oB[tid]);
+            if (!direct && (!TILES || it.o_count >= 0)) o_scatter(tid, oA[tid], oB[tid]);
             for (int t = tid; t < kt; t += 256) {
                 kA[t] = scatter_bits(t, d.a_k, d.nk);
                 kB[t] = scatter_bits(t, d.b_k, d.nk);
@@ -1188,7 +1192,17 @@ __global__ void __launch_bounds__(256)
                 d.b_leaf >= 0 ? (const char*)leaf_ptrs[d.b_leaf] + (int64_t)it.pad * d.in.b_is * isz : vw.B);
             sA = slice_off(d.sla, vw.slice);
             sB = slice_off(d.slb, vw.slice);
-            if (tid < 4 && tid * 256 < it.o_count) {
+            if (direct) {
+                const int g = 256 / (int)it.o_count;
+                if (tid % g == 0 && tid / g < it.o_count) {
+                    const int64_t o = it.o_begin + tid / g;
+                    o_scatter(o, oA[o & 255], oB[o & 255]);
+                }
+                if (tid == 0) {
+                    oAh[0] = sA;
+                    oBh[0] = sB;
+                }
+            } else if (tid < 4 && tid * 256 < it.o_count) {
                 int64_t hA, hB;
                 o_scatter((it.o_begin + tid * 256) & ~255ll, hA, hB);
                 oAh[tid] = sA + hA;
