@@ -92,6 +92,7 @@ struct GradState {
     float* gacc = nullptr;
     const float** img_ptr_dev = nullptr;   // leaf image pointers (fixed)
     int64_t* leaf_nfloat_dev = nullptr;
+    std::vector<int64_t> leaf_nfloat;  // floats per leaf, all copies
     TileArgs* descs_dev = nullptr;
     WaveItem* items_dev = nullptr;
     int* flow_deps_dev = nullptr;
@@ -479,6 +480,7 @@ static tn_status alloc_grad(const NetDesc& d, const Plan& f, GradState& G, void*
         }
         UP(G.img_ptr_dev, ip.data(), sizeof(void*) * n);
         UP(G.leaf_nfloat_dev, nf.data(), sizeof(int64_t) * n);
+        G.leaf_nfloat = nf;
     }
     char* ws = (char*)G.ws;
     auto fwd_ptr = [&](int v) -> const void* {
@@ -955,14 +957,6 @@ static void gather_entries(const NetDesc& d, const GradState& G, int n_inst, con
     }
 }
 
-static int64_t image_max_floats(const NetDesc& d, const GradState& G, int n_inst) {
-    const int cf = d.is_complex() ? 2 : 1;
-    int64_t mx = 0;
-    for (int v = 0; v < d.n; ++v)
-        mx = std::max(mx, G.varying[v] ? G.img_is[v] * (n_inst - 1) + d.leaves[v].size * cf : d.leaves[v].size * cf);
-    return mx;
-}
-
 tn_status run_grad_forward(NetDesc& d, Plan& p, void* unit, int n_inst, const int64_t* leaf_inst_stride,
                            double* out, int64_t* out_exp2, int out_mem, cudaStream_t stream, std::string& err) {
     if (p.d_sliced != 1 || p.n_out != 1) {
@@ -978,7 +972,7 @@ tn_status run_grad_forward(NetDesc& d, Plan& p, void* unit, int n_inst, const in
     gather_entries(d, G, n_inst, leaf_inst_stride, tab);
     CK(cudaMemcpyAsync(G.copy_dev, tab.data(), sizeof(CopyEntry) * tab.size(), cudaMemcpyHostToDevice, stream));
     CK(launch_copy_table(G.copy_dev, (int)tab.size(), G.max_leaf_floats, stream));
-    CK(launch_leaf_max(G.img_ptr_dev, G.leaf_nfloat_dev, G.leafmax, d.n, stream, image_max_floats(d, G, n_inst)));
+    CK(launch_leaf_max(G.img_ptr_dev, G.leaf_nfloat_dev, G.leaf_nfloat.data(), G.leafmax, d.n, stream));
     CK(launch_begin_call(G.ctl, 0, 1, nullptr, 0, stream));
     CK(cudaGraphLaunch(G.gexec_f, stream));
     const bool host = out_mem == TN_MEM_HOST;
@@ -1050,7 +1044,7 @@ tn_status run_grad(NetDesc& d, Plan& p, void* unit, const double* adj, int adj_m
                            stream));
     if (!kept_forward) {
         CK(launch_copy_table(G.copy_dev, n_gather, G.max_leaf_floats, stream));
-        CK(launch_leaf_max(G.img_ptr_dev, G.leaf_nfloat_dev, G.leafmax, n, stream, image_max_floats(d, G, n_inst)));
+        CK(launch_leaf_max(G.img_ptr_dev, G.leaf_nfloat_dev, G.leaf_nfloat.data(), G.leafmax, n, stream));
     }
     // root adjoints
     const double* adj_src = adj;

@@ -534,14 +534,14 @@ cudaError_t launch_leaf_table(const void* const* ptrs, int n, const void** table
 // Leaf maxima (as launch_leaf_max) and the call's control block (with the
 // output pointers that a direct fold writes), and n_acc doubles of the
 // accumulator cleared, in one launch.
-cudaError_t launch_call_begin(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
-                              int64_t max_nfloat, Control* ctl, int64_t slice_begin, int64_t slice_end,
-                              double* acc, int64_t n_acc, double* result, int64_t* result_exp, cudaStream_t s);
+cudaError_t launch_call_begin(const float* const* ptrs, const int64_t* nfloat, const int64_t* nfloat_host, unsigned* out,
+                              int n, Control* ctl, int64_t slice_begin, int64_t slice_end, double* acc, int64_t n_acc,
+                              double* result, int64_t* result_exp, cudaStream_t s);
 cudaError_t launch_begin_call(Control* ctl, int64_t slice_begin, int64_t slice_end, double* acc,
                               int64_t n_acc_doubles, cudaStream_t s);
 cudaError_t launch_begin_slice(unsigned* maxabs, int n_nodes, cudaStream_t s);
 cudaError_t launch_advance(Control* ctl, cudaStream_t s, int step = 1);
-cudaError_t launch_leaf_max(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
-                            cudaStream_t s, int64_t max_nfloat);
+cudaError_t launch_leaf_max(const float* const* ptrs, const int64_t* nfloat, const int64_t* nfloat_host, unsigned* out,
+                            int n, cudaStream_t s);
 
 }  // namespace tn

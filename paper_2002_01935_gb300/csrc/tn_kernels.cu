@@ -706,24 +706,50 @@ cudaError_t launch_leaf_table(const void* const* ptrs, int n, const void** table
 }
 
 // Largest |component| of every leaf, so that leaves are renormalised like
-// intermediates before their first contraction.
-// Part blockIdx.y of leaf blockIdx.x: the largest |component| over its
-// entries, combined over the parts by atomicMax on the float bits
-// (non-negative floats order like unsigned), or stored directly when one
-// block covers the leaf and `direct` allows it (no zeroing needed then).
+// intermediates before their first contraction.  A leaf is cut into parts of
+// kLeafPart floats (at most 1024), one block each, combined by atomicMax on the
+// float bits (non-negative floats order like unsigned), or stored directly when
+// one block covers the leaf and `direct` allows it (no zeroing needed then).
+// Blocks [0, n0) are part 0 of every leaf, the others the further parts of the
+// large leaves listed in `big`, so that many small leaves beside a large one
+// add no empty blocks (300 leaves and one of 2^26 floats: 228 us with as many
+// blocks for every leaf, 51 now; 2000 and one of 2^20: 91 and 7).
 // Large leaves are read 16 bytes a load, four loads in flight per thread
 // (bound by memory); a leaf that is not 16-byte aligned, and the ends, by
 // single floats.
-__device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const int64_t* nfloat, unsigned* out,
-                                              int n, bool direct) {
-    const int v = blockIdx.x;
-    if (v >= n) return;
+constexpr int kBigLeaves = 128;
+struct BigLeaves {
+    int32_t n;
+    int32_t leaf[kBigLeaves];
+    int32_t first[kBigLeaves + 1];  // first of the leaf's further blocks
+};
+
+__host__ __device__ inline int leaf_parts(int64_t nfloat) {
+    const int64_t parts = (nfloat + kLeafPart - 1) / kLeafPart;
+    return (int)(parts < 1 ? 1 : (parts > 1024 ? 1024 : parts));
+}
+
+__device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n0,
+                                              const BigLeaves& big, bool direct) {
+    int v = blockIdx.x, part = 0;
+    if (v >= n0) {
+        const int b = v - n0;
+        if (b >= big.first[big.n]) return;
+        int lo = 0, hi = big.n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (big.first[mid] <= b) lo = mid;
+            else hi = mid - 1;
+        }
+        v = big.leaf[lo];
+        part = 1 + b - big.first[lo];
+    }
     const float* p = ptrs[v];
     const int64_t m = nfloat[v];
+    const int parts = leaf_parts(m);
     const bool vec = (reinterpret_cast<uintptr_t>(p) & 15) == 0 && m >= 4096;
     const int64_t m4 = vec ? m / 4 : 0;
-    const int64_t step = (int64_t)gridDim.y * blockDim.x, first = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-    if (blockIdx.y > 0 && (int64_t)blockIdx.y * blockDim.x >= (vec ? m4 : m)) return;  // nothing left for this part
+    const int64_t step = (int64_t)parts * blockDim.x, first = (int64_t)part * blockDim.x + threadIdx.x;
     float lmax = 0.f;
     const float4* p4 = reinterpret_cast<const float4*>(p);
     for (int64_t i = first; i < m4; i += 4 * step) {
@@ -744,7 +770,7 @@ __device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const in
         lmax = threadIdx.x < nw ? red[threadIdx.x] : 0.f;
         for (int o = 16; o > 0; o >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
         if (threadIdx.x == 0) {
-            if (direct && gridDim.y == 1)
+            if (direct && parts == 1)
                 out[v] = __float_as_uint(lmax);
             else
                 atomicMax(&out[v], __float_as_uint(lmax));
@@ -752,25 +778,34 @@ __device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const in
     }
 }
 
-// Blocks per leaf of a leaf-maximum launch.
-static unsigned leaf_parts(int64_t max_nfloat) {
-    int64_t parts = (max_nfloat + kLeafPart - 1) / kLeafPart;
-    return (unsigned)(parts < 1 ? 1 : (parts > 1024 ? 1024 : parts));
+// The next large leaves from v on; returns the number of their further blocks.
+static int next_big(const int64_t* nfloat, int n, int& v, BigLeaves& big) {
+    big.n = 0;
+    int blocks = 0;
+    for (; v < n && big.n < kBigLeaves; ++v) {
+        const int parts = leaf_parts(nfloat[v]);
+        if (parts == 1) continue;
+        big.leaf[big.n] = v;
+        big.first[big.n++] = blocks;
+        blocks += parts - 1;
+    }
+    big.first[big.n] = blocks;
+    return blocks;
 }
 
-__global__ void __launch_bounds__(256) k_leaf_max(const float* const* ptrs, const int64_t* nfloat,
-                                                  unsigned* out, int n) {
-    leaf_max_part(ptrs, nfloat, out, n, false);
+__global__ void __launch_bounds__(256) k_leaf_max(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n0,
+                                                  const __grid_constant__ BigLeaves big) {
+    leaf_max_part(ptrs, nfloat, out, n0, big, false);
 }
 
 // The start of a call: leaf maxima as k_leaf_max, (block 0) the control block
 // with the call's output pointers, and the FP64 accumulator cleared where the
 // fold reads it (n_acc > 0).
-__global__ void __launch_bounds__(256) k_call_begin(const float* const* ptrs, const int64_t* nfloat,
-                                                    unsigned* out, int n, Control* ctl, int64_t slice_begin,
-                                                    int64_t slice_end, double* acc, int64_t n_acc,
+__global__ void __launch_bounds__(256) k_call_begin(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
+                                                    const __grid_constant__ BigLeaves big, Control* ctl,
+                                                    int64_t slice_begin, int64_t slice_end, double* acc, int64_t n_acc,
                                                     double* result, int64_t* result_exp) {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->slice = slice_begin;
         ctl->slice_begin = slice_begin;
         ctl->slice_end = slice_end;
@@ -781,34 +816,50 @@ __global__ void __launch_bounds__(256) k_call_begin(const float* const* ptrs, co
         ctl->out = result;
         ctl->out_exp = result_exp;
     }
-    {
-        const int64_t nblk = (int64_t)gridDim.x * gridDim.y, bid = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-        for (int64_t i = bid * blockDim.x + threadIdx.x; i < n_acc; i += nblk * blockDim.x) acc[i] = 0.0;
-    }
-    leaf_max_part(ptrs, nfloat, out, n, true);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_acc; i += (int64_t)gridDim.x * blockDim.x)
+        acc[i] = 0.0;
+    leaf_max_part(ptrs, nfloat, out, n, big, true);
 }
 
-cudaError_t launch_call_begin(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
-                              int64_t max_nfloat, Control* ctl, int64_t slice_begin, int64_t slice_end,
-                              double* acc, int64_t n_acc, double* result, int64_t* result_exp, cudaStream_t s) {
-    const unsigned parts = leaf_parts(max_nfloat);
-    if (n > 0 && parts > 1) {  // several blocks per leaf combine by atomicMax from zero
+// The further parts of large leaves that one list does not hold.
+static cudaError_t launch_more_big(const float* const* ptrs, const int64_t* nfloat, unsigned* out,
+                                   const int64_t* nfloat_host, int n, int v, cudaStream_t s) {
+    BigLeaves big;
+    while (const int blocks = next_big(nfloat_host, n, v, big)) {
+        k_leaf_max<<<(unsigned)blocks, 256, 0, s>>>(ptrs, nfloat, out, 0, big);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_call_begin(const float* const* ptrs, const int64_t* nfloat, const int64_t* nfloat_host, unsigned* out,
+                              int n, Control* ctl, int64_t slice_begin, int64_t slice_end, double* acc, int64_t n_acc,
+                              double* result, int64_t* result_exp, cudaStream_t s) {
+    BigLeaves big;
+    int v = 0;
+    const int more = next_big(nfloat_host, n, v, big);
+    if (more) {  // several blocks per leaf combine by atomicMax from zero
         const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned) * (size_t)n, s);
         if (e != cudaSuccess) return e;
     }
-    const unsigned gx = (unsigned)(n > 0 ? n : 1);
-    k_call_begin<<<dim3(gx, parts), 256, 0, s>>>(ptrs, nfloat, out, n, ctl, slice_begin, slice_end, acc, n_acc, result,
-                                                 result_exp);
-    return cudaGetLastError();
+    k_call_begin<<<(unsigned)std::max(n + more, 1), 256, 0, s>>>(ptrs, nfloat, out, n, big, ctl, slice_begin, slice_end, acc, n_acc,
+                                                      result, result_exp);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? launch_more_big(ptrs, nfloat, out, nfloat_host, n, v, s) : e;
 }
 
-cudaError_t launch_leaf_max(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n,
-                            cudaStream_t s, int64_t max_nfloat) {
+cudaError_t launch_leaf_max(const float* const* ptrs, const int64_t* nfloat, const int64_t* nfloat_host, unsigned* out,
+                            int n, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned) * (size_t)n, s);
     if (e != cudaSuccess) return e;
-    k_leaf_max<<<dim3((unsigned)n, leaf_parts(max_nfloat)), 256, 0, s>>>(ptrs, nfloat, out, n);
-    return cudaGetLastError();
+    BigLeaves big;
+    int v = 0;
+    const int more = next_big(nfloat_host, n, v, big);
+    k_leaf_max<<<(unsigned)(n + more), 256, 0, s>>>(ptrs, nfloat, out, n, big);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? launch_more_big(ptrs, nfloat, out, nfloat_host, n, v, s) : e;
 }
 
 // Leaf adjoints of one slice, all leaves in one launch: blockIdx.y picks

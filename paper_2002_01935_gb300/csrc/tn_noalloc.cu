@@ -230,9 +230,9 @@ tn_status run_noalloc(const NetDesc& d, const Plan& p, void* out, int out_mem, i
 
     // the call: leaf maxima, control block and accumulator cleared, then
     // every slice in order, then the result
-    int64_t mx_leaf = 0;
-    for (int v = 0; v < n; ++v) mx_leaf = std::max(mx_leaf, d.leaves[v].size * (d.is_complex() ? 2 : 1));
-    CK(launch_call_begin(lptr, lnf, leafmax, n, mx_leaf, ctl, 0, p.d_sliced, acc, (int64_t)acc_doubles,
+    std::vector<int64_t> nf(n);
+    for (int v = 0; v < n; ++v) nf[v] = d.leaves[v].size * (d.is_complex() ? 2 : 1);
+    CK(launch_call_begin(lptr, lnf, nf.data(), leafmax, n, ctl, 0, p.d_sliced, acc, (int64_t)acc_doubles,
                          nullptr, nullptr, stream));
     for (int64_t s = 0; s < p.d_sliced; ++s) {
         CK(launch_begin_slice(maxabs, nn, stream));

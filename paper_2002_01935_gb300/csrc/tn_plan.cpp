@@ -1681,12 +1681,6 @@ static tn_status ensure_graph(const NetDesc& d, Plan& p, const std::vector<const
     return TN_OK;
 }
 
-static int64_t max_leaf_floats(const NetDesc& d) {
-    int64_t m = 0;
-    for (int v = 0; v < d.n; ++v) m = std::max(m, d.leaves[v].size * (d.is_complex() ? 2 : 1));
-    return m;
-}
-
 static tn_status upload_leaf_sizes(const NetDesc& d, Plan& p, int G, const std::vector<int64_t>& leaf_is,
                                    cudaStream_t stream, std::string& err) {
     std::vector<int64_t> nf(d.n);
@@ -1753,7 +1747,7 @@ tn_status run_plan(NetDesc& d, Plan& p, void* unit, int64_t begin, int64_t count
         res = p.out_stage;
         res_exp = reinterpret_cast<int64_t*>(p.out_stage + n_acc);
     }
-    CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leafmax, n, max_leaf_floats(d), p.ctl, begin,
+    CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leaf_nfloat_uploaded.data(), p.leafmax, n, p.ctl, begin,
                          begin + count, nullptr, 0, res, res_exp, stream));
     const int64_t groups = (count + G - 1) / G;
     const bool use_graph = !o.no_graph && !capturing;
@@ -1830,8 +1824,8 @@ tn_status run_instances(NetDesc& d, Plan& p, void* unit, int n_inst, const int64
     std::vector<const void*> lp;
     st = prepare_leaves(d, p, false, lp, stream, err);
     if (st != TN_OK) return st;
-    CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leafmax, n, max_leaf_floats(d), p.ctl, 0, 1, nullptr,
-                         0, nullptr, nullptr, stream));
+    CK(launch_call_begin(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leaf_nfloat_uploaded.data(), p.leafmax, n, p.ctl, 0, 1,
+                         nullptr, 0, nullptr, nullptr, stream));
     st = ensure_graph(d, p, lp, 0, 0, err);
     if (st != TN_OK) return st;
     CK(cudaGraphLaunch(p.gexec, stream));
@@ -1997,7 +1991,7 @@ tn_status autotune_plan(NetDesc& d, Plan& p, int reps, int32_t* choice, cudaStre
     std::vector<const void*> lp;
     st = prepare_leaves(d, p, false, lp, s, err);
     if (st != TN_OK) return st;
-    CK(launch_leaf_max(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leafmax, d.n, s, max_leaf_floats(d)));
+    CK(launch_leaf_max(p.leaf_ptr_dev, p.leaf_nfloat_dev, p.leaf_nfloat_uploaded.data(), p.leafmax, d.n, s));
     // candidates and the shared P buffer they need
     std::vector<std::vector<std::pair<int, Node>>> cand(nn);
     int64_t split_elems = 0;
