@@ -207,7 +207,28 @@ tn_status alloc_batch(BatchPlan& b, std::string& err) {
         return true;
     };
     if (!ck(cudaMalloc(&b.ws, b.ws_bytes), "batch workspace")) return TN_ENOMEM;
-    if (b.split_bytes && !ck(cudaMalloc(&b.split_buf, b.split_bytes * b.groups), "cudaMalloc")) return TN_ENOMEM;
+    // one packing and K-split buffer per group; fewer groups (several in one
+    // branch, one after another) where the buffers would take more than three
+    // quarters of the device's free memory
+    size_t room = 0, all = 0;
+    if (!ck(cudaMemGetInfo(&room, &all), "cudaMemGetInfo")) return TN_ECUDA;
+    int groups = b.groups;
+    while (groups > 1 && groups * b.split_bytes > (int64_t)(room / 4 * 3)) --groups;
+    while (b.split_bytes) {
+        const cudaError_t e = cudaMalloc(&b.split_buf, b.split_bytes * groups);
+        if (e == cudaSuccess) break;
+        if (groups == 1 || e != cudaErrorMemoryAllocation) {
+            ck(e, "cudaMalloc");
+            return TN_ENOMEM;
+        }
+        cudaGetLastError();  // the failure is dealt with here
+        --groups;
+    }
+    if (groups < b.groups) {  // the steps of a branch stay in their networks' order
+        b.groups = groups;
+        for (int& g : b.group_of) g %= groups;
+        for (BatchStep& st : b.steps) st.group %= groups;
+    }
     if (!ck(cudaMalloc(&b.maxabs, sizeof(unsigned) * std::max(b.n_slots, 1)), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&b.exps, sizeof(int64_t) * std::max(b.n_slots, 1)), "cudaMalloc")) return TN_ENOMEM;
     if (!ck(cudaMalloc(&b.ctl, sizeof(Control)), "cudaMalloc")) return TN_ENOMEM;
