@@ -390,7 +390,8 @@ tn_status tn_contract_instances(tn_net *net, const int32_t *tree_pairs, tn_mode 
  * Eqs. edgecon and vertexcon: out[0] = W_s (sliced width, log2 of the
  * largest tensor), out[1] = C (contraction cost of one slice), out[2] =
  * d_sliced, out[3] = FLOPs of all slices (8 C d_sliced complex, 2 C
- * d_sliced real), out[4] = workspace bytes per slice, out[5] = number of
+ * d_sliced real), out[4] = workspace bytes per slice (of tn_contract or of
+ * tn_contract_noalloc, whose launch sequences differ: the larger), out[5] = number of
  * nodes run by the tiled kernels, out[6] = by the tensor-core kernel,
  * out[7] = by the generic kernel.  Host only; no device work.
  */

@@ -398,7 +398,12 @@ tn_status tn_plan_info(tn_net* net, const int32_t* tree_pairs, int32_t n_sliced,
     Plan* p = nullptr;
     tn_status st = get_plan(net, tree_pairs, n_sliced, sliced_labels, mode, &p);
     if (st != TN_OK) return st;
-    tn::plan_info(net->d, *p, out);
+    Plan* q = p;  // the allocation-free call's plan, where it differs
+    if (!p->region_hdr.empty()) {
+        st = get_plan(net, tree_pairs, n_sliced, sliced_labels, mode, &q, 1, false, false);
+        if (st != TN_OK) return st;
+    }
+    tn::plan_info(net->d, *p, q->ws_elems, out);
     return TN_OK;
 }
 

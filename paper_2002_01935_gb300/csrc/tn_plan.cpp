@@ -1103,13 +1103,16 @@ tn_status build_plan(const NetDesc& d, Plan& p, std::string& err) {
         }
     }
     // ---- workspace liveness in execution order: a step's outputs are all
-    // allocated before any of its operands is released (they run at once)
+    // allocated before any of its operands is released (they run at once).  Of a
+    // region only the root is stored.
     Arena ar;
     for (const Step& st : p.steps) {
-        for (int k : st.nodes) p.nodes[k].ws_off = ar.alloc(p.nodes[k].size);
+        auto inside = [&](int k) { return region_of[k] >= 0 && regions[region_of[k]].back() != k; };
+        for (int k : st.nodes)
+            if (!inside(k)) p.nodes[k].ws_off = ar.alloc(p.nodes[k].size);
         for (int k : st.nodes)
             for (int c : {p.nodes[k].ca, p.nodes[k].cb})
-                if (c >= n) {
+                if (c >= n && !inside(c - n)) {
                     const Node& ch = p.nodes[c - n];
                     ar.release(ch.ws_off, ch.size);
                 }
@@ -2120,12 +2123,12 @@ tn_status make_generic_args(const NetDesc& d, const Plan& p, int k, GenericArgs&
     return fill_generic(d, p, p.nodes[k], g, err);
 }
 
-void plan_info(const NetDesc& d, const Plan& p, double out[8]) {
+void plan_info(const NetDesc& d, const Plan& p, int64_t ws_elems, double out[8]) {
     out[0] = p.W;
     out[1] = p.C;
     out[2] = (double)p.d_sliced;
     out[3] = (d.is_complex() ? 8.0 : 2.0) * p.C * (double)p.d_sliced;
-    out[4] = (double)p.ws_elems * (double)d.elem_bytes();
+    out[4] = (double)std::max(p.ws_elems, ws_elems) * (double)d.elem_bytes();
     int cnt[3] = {0, 0, 0};
     for (auto& nd : p.nodes) cnt[nd.kind]++;
     out[5] = cnt[kTiled];

@@ -258,7 +258,8 @@ tn_status run_grad(NetDesc& d, Plan& p, void* unit, const double* adj, int adj_m
 // every intermediate kept; values as tn_contract_instances.
 tn_status run_grad_forward(NetDesc& d, Plan& p, void* unit, int n_inst, const int64_t* leaf_inst_stride,
                            double* out, int64_t* out_exp2, int out_mem, cudaStream_t stream, std::string& err);
-void plan_info(const NetDesc& d, const Plan& p, double out[8]);
+// ws_elems: workspace of the same tree without subtree regions.
+void plan_info(const NetDesc& d, const Plan& p, int64_t ws_elems, double out[8]);
 void free_device(Plan& p);  // releases device state; the host plan stays valid
 void free_grad(Plan& p);
 // Generic-kernel arguments of node k (index digits, slice digits); pointers
