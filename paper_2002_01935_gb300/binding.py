@@ -383,13 +383,9 @@ class TensorNetwork:
         self.dims = dict(dims)
         self.open = list(open_labels)
         self.h = tn_create(self.dtype, self.labels, self.dims, self.open)
-        # entries of each leaf (structure only)
-        self._numels = []
-        for ls in self.labels:
-            n = 1
-            for l in ls:
-                n *= int(self.dims[l])
-            self._numels.append(n)
+        # entries of each leaf (structure only; sizes as Python integers)
+        size = {l: int(d) for l, d in self.dims.items()}
+        self._numels = [math.prod([size[l] for l in ls]) for ls in self.labels]
         self._keep: List = []
         if tensors is not None:
             self.set_tensors(tensors)
@@ -420,20 +416,26 @@ class TensorNetwork:
         self._keep = []
         attached = getattr(self, "_attached", None) or [None] * len(tensors)
         usable = all([t.dtype == want for t in tensors]) and all([t.is_contiguous() for t in tensors])
-        keys = [(t.data_ptr(), TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST) for t in tensors] if usable else None
-        if keys is not None and keys == attached:
-            self._keep = tensors  # unchanged pointers need no call
-            return
-        for v, t in enumerate(tensors):
-            if t.dtype != want:
-                raise TypeError(f"leaf {v}: dtype {t.dtype}, expected {want}")
-            if not t.is_contiguous():
-                raise ValueError(f"leaf {v} must be contiguous")
-            key = keys[v] if keys is not None else (t.data_ptr(), TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST)
-            self._keep.append(t)
-            if attached[v] != key:
-                tn_set_tensor(self.h, v, key[0], key[1])
-                attached[v] = key
+        if usable:
+            keys = [(t.data_ptr(), TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST) for t in tensors]
+            self._keep = tensors
+            if keys == attached:  # unchanged pointers need no call
+                return
+            for v, key in enumerate(keys):
+                if attached[v] != key:
+                    tn_set_tensor(self.h, v, key[0], key[1])
+                    attached[v] = key
+        else:  # up to the first leaf that cannot be attached
+            for v, t in enumerate(tensors):
+                if t.dtype != want:
+                    raise TypeError(f"leaf {v}: dtype {t.dtype}, expected {want}")
+                if not t.is_contiguous():
+                    raise ValueError(f"leaf {v} must be contiguous")
+                key = (t.data_ptr(), TN_MEM_DEVICE if t.is_cuda else TN_MEM_HOST)
+                self._keep.append(t)
+                if attached[v] != key:
+                    tn_set_tensor(self.h, v, key[0], key[1])
+                    attached[v] = key
         self._attached = attached
 
     @property

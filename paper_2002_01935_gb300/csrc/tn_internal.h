@@ -314,9 +314,9 @@ struct WaveItem {
 // nodes stored to the workspace (6).
 struct RegionHdr {
     int32_t blob, words;      // first word, words (a multiple of 4)
-    int32_t n_out, n_k, n_nodes, n_ext, n_elem, n_steps, n_store;
+    int32_t n_out, n_nodes, n_ext, n_elem, n_steps, n_store;
     int32_t o_k, o_nodes, o_ext, o_elem, o_steps, o_store;  // word offsets in the blob (outputs first)
-    int32_t pad;
+    int32_t pad[2];
 };
 struct RegionNode {
     int32_t kbase, k;         // K table, summed entries

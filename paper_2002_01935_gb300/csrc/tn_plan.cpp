@@ -476,6 +476,7 @@ void find_regions(const RegionView& v, int k0, int k1, std::vector<int>& of, std
     for (int k = k0; k < k1; ++k) {
         const Node& nd = v.node(k);
         if (!region_node(v, nd)) continue;
+        const int64_t K = region_k(d, nd);
         const RegionOperand op[2] = {v.operand(nd.ca), v.operand(nd.cb)};
         int child[2];
         for (int s = 0; s < 2; ++s)
@@ -491,9 +492,9 @@ void find_regions(const RegionView& v, int k0, int k1, std::vector<int>& of, std
             if (t[0] && t[1] && child[0] == child[1]) continue;  // (no tree has it)
             Size z;
             z.out = nd.size;
-            z.macs = (int64_t)std::llround(std::pow(2.0, nd.vc));
+            z.macs = nd.size * K;
             z.nodes = 1;
-            z.words = 2 * nd.size + region_k(d, nd) + 8 + 4 + 6;  // at most one step and one store each
+            z.words = 2 * nd.size + K + 8 + 4 + 6;  // at most one step and one store each
             for (int s = 0; s < 2; ++s) {
                 if (t[s]) {
                     const Size& y = size[child[s]];
@@ -541,30 +542,28 @@ void find_regions(const RegionView& v, int k0, int k1, std::vector<int>& of, std
 }
 
 // Offsets of every output and K index of a node in its operands, in the order
-// of the kernel that runs it outside a region.
-static void region_tables(const NetDesc& d, const Plan& p, const Node& nd, std::vector<uint32_t>& out,
-                          std::vector<uint32_t>& kt) {
-    out.clear();
-    kt.clear();
-    auto pack = [](int64_t a, int64_t b) { return (uint32_t)a | ((uint32_t)b << 16); };
+// of the kernel that runs it outside a region: written to every second word of
+// out, and to kt.
+static void region_tables(const NetDesc& d, const Plan& p, const Node& nd, int64_t K, int32_t* out, int32_t* kt) {
+    auto pack = [](int64_t a, int64_t b) { return (int32_t)((uint32_t)a | ((uint32_t)b << 16)); };
     if (nd.kind == kTiled) {
         const TileArgs& t = nd.tile;
         // offsets double with every index bit: entry x + 2^i is entry x plus bit i
-        auto grow = [&](std::vector<uint32_t>& v, const uint8_t* sa, const uint8_t* sb, int nb) {
-            for (int i = 0; i < nb; ++i) {
-                const uint32_t add = pack(sa && sa[i] != kNoBit ? int64_t(1) << sa[i] : 0,
-                                          sb && sb[i] != kNoBit ? int64_t(1) << sb[i] : 0);
-                const size_t have = v.size();
-                v.resize(2 * have);
-                for (size_t x = 0; x < have; ++x) v[have + x] = v[x] + add;
+        auto grow = [&](int32_t* v, int step, int64_t& have, const uint8_t* sa, const uint8_t* sb, int nb) {
+            for (int i = 0; i < nb; ++i, have *= 2) {
+                const int32_t add = pack(sa && sa[i] != kNoBit ? int64_t(1) << sa[i] : 0,
+                                         sb && sb[i] != kNoBit ? int64_t(1) << sb[i] : 0);
+                for (int64_t x = 0; x < have; ++x) v[(have + x) * step] = (int32_t)((uint32_t)v[x * step] + (uint32_t)add);
             }
         };
-        out.push_back(0);
-        grow(out, nullptr, t.b_n, t.nn);
-        grow(out, t.a_m, nullptr, t.nm);
-        grow(out, t.a_b, t.b_b, t.nb);
-        kt.push_back(0);
-        grow(kt, t.a_k, t.b_k, t.nk);
+        int64_t have = 1;
+        out[0] = 0;
+        grow(out, 2, have, nullptr, t.b_n, t.nn);
+        grow(out, 2, have, t.a_m, nullptr, t.nm);
+        grow(out, 2, have, t.a_b, t.b_b, t.nb);
+        have = 1;
+        kt[0] = 0;
+        grow(kt, 1, have, t.a_k, t.b_k, t.nk);
         return;
     }
     GenericArgs g;
@@ -577,16 +576,16 @@ static void region_tables(const NetDesc& d, const Plan& p, const Node& nd, std::
             b += rem % g.od_dim[i] * g.od_sb[i];
             rem /= g.od_dim[i];
         }
-        out.push_back(pack(a, b));
+        out[2 * o] = pack(a, b);
     }
-    for (int64_t k = 0; k < g.n_sum; ++k) {
+    for (int64_t k = 0; k < K; ++k) {
         int64_t rem = k, a = 0, b = 0;
         for (int i = 0; i < g.n_kd; ++i) {
             a += rem % g.kd_dim[i] * g.kd_sa[i];
             b += rem % g.kd_dim[i] * g.kd_sb[i];
             rem /= g.kd_dim[i];
         }
-        kt.push_back(pack(a, b));
+        kt[k] = pack(a, b);
     }
 }
 
@@ -598,6 +597,7 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
     // order: tree level within the region, then how a node's sums are shared
     struct Item {
         int k, level, lg, accs;
+        int64_t K;
     };
     std::vector<Item> items;
     items.reserve(members.size());
@@ -617,7 +617,7 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
         }
         int64_t L = std::max<int64_t>(1, g / 8);
         while (L < g && L < 32 && K / L > 16) L *= 2;
-        items.push_back({k, lv + 1, ilog2(L), (int)(g / L)});
+        items.push_back({k, lv + 1, ilog2(L), (int)(g / L), K});
     }
     std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) {
         return std::tie(x.level, x.lg, x.accs) < std::tie(y.level, y.lg, y.accs);
@@ -626,25 +626,31 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
     std::vector<RegionExt> ext;
     std::vector<uint16_t> elem;
     std::vector<int64_t> q0(items.size());
-    int64_t n_out = 0;
+    int64_t n_out = 0, n_k = 0;
     for (size_t i = 0; i < items.size(); ++i) {
         q0[i] = n_out;
         n_out += v.node(items[i].k).size;
+        n_k += items[i].K;
     }
+    // the blob starts with the outputs and the K tables
+    RegionHdr h;
+    memset(&h, 0, sizeof(h));
+    h.blob = (int)P.size();
+    h.o_k = (int)((2 * n_out + 3) / 4 * 4);
+    P.resize(P.size() + h.o_k + n_k);
+    int32_t* const outs = P.data() + h.blob;
+    int32_t* const kts = outs + h.o_k;
+    n_k = 0;
     std::vector<RegionNode> nodes(items.size());
-    std::vector<uint32_t> outs, kts, o1, k1;
     std::vector<RegionStep> steps;
     for (size_t i = 0; i < items.size(); ++i) {
         const Node& nd = v.node(items[i].k);
-        region_tables(d, *v.p, nd, o1, k1);
         RegionNode& r = nodes[i];
-        r.kbase = (int)kts.size();
-        r.k = (int)k1.size();
-        kts.insert(kts.end(), k1.begin(), k1.end());
-        for (uint32_t x : o1) {
-            outs.push_back(x);
-            outs.push_back((uint32_t)i);
-        }
+        r.kbase = (int)n_k;
+        r.k = (int)items[i].K;
+        region_tables(d, *v.p, nd, r.k, outs + 2 * q0[i], kts + n_k);
+        for (int64_t q = q0[i]; q < q0[i] + nd.size; ++q) outs[2 * q + 1] = (int32_t)i;
+        n_k += r.k;
         r.q0 = (int)q0[i];
         r.conj = (nd.tile.conj_a ? 1 : 0) | (nd.tile.conj_b ? 2 : 0);
         for (int s = 0; s < 2; ++s) {
@@ -683,9 +689,6 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
     std::vector<RegionStore> stores;
     for (auto& st : stored) stores.push_back({at[st.first], st.second, v.node(st.first).ws_off, -1, 0});
     for (int k : members) at[k] = -1;
-    RegionHdr h;
-    memset(&h, 0, sizeof(h));
-    h.blob = (int)P.size();
     auto put = [&](const void* src, size_t words) {
         while ((P.size() - h.blob) % 4) P.push_back(0);
         const int at = (int)P.size() - h.blob;
@@ -694,8 +697,6 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
         return at;
     };
     if (elem.size() % 2) elem.push_back(0);
-    put(outs.data(), outs.size());
-    h.o_k = put(kts.data(), kts.size());
     h.o_nodes = put(nodes.data(), nodes.size() * sizeof(RegionNode) / 4);
     h.o_ext = put(ext.data(), ext.size() * sizeof(RegionExt) / 4);
     h.o_elem = put(elem.data(), elem.size() / 2);
@@ -704,7 +705,6 @@ void emit_region(const RegionView& v, const std::vector<int>& members, const std
     while ((P.size() - h.blob) % 4) P.push_back(0);
     h.words = (int)P.size() - h.blob;
     h.n_out = (int)n_out;
-    h.n_k = (int)kts.size();
     h.n_nodes = (int)nodes.size();
     h.n_ext = n_ext;
     h.n_elem = n_elem;
