@@ -200,6 +200,28 @@ __device__ __forceinline__ unsigned fold_max(const AccumArgs& a, int i) { return
 __device__ __forceinline__ int64_t fold_exp(const AccumArgs& a, int i) { return a.exp_r[(int64_t)i * a.s_is]; }
 __device__ __forceinline__ double fold_pow2(int64_t d) { return ldexp(1.0, (int)(d < -2000 ? -2000 : d)); }
 
+// The accumulator's exponent, after the call's last group the result's, and the
+// slice counter: written by the last block to have read the control block, so
+// that no launch of its own is needed for them.  The fences order each block's
+// reads before its ticket, and the last ticket before the writes; they come
+// before the block's own stores, which they would otherwise wait for (2.2 us at
+// the end of a fold of 2^20 to 2^22 outputs).
+__device__ __forceinline__ void fold_control(const AccumArgs& a, const FoldState& f) {
+    if (gridDim.x > 1) {
+        __threadfence();
+        const unsigned ticket = atomicInc(&a.ctl->ticket, gridDim.x - 1);  // wraps to 0 at the last block
+        __threadfence();
+        if (ticket != gridDim.x - 1) return;
+    }
+    a.ctl->acc_exp[f.par ^ 1] = f.newE;
+    if (f.last) {
+        const int64_t e = f.newE == INT64_MIN ? 0 : f.newE;
+        a.ctl->final_exp = e;
+        if (a.direct) *a.ctl->out_exp = e;
+    }
+    a.ctl->slice = f.slice + a.advance;
+}
+
 __device__ __forceinline__ FoldState fold_state(const AccumArgs& a) {
     __shared__ unsigned smax[kFoldInst];
     __shared__ int64_t sexp[kFoldInst];
@@ -239,6 +261,7 @@ __device__ __forceinline__ FoldState fold_state(const AccumArgs& a) {
     f.vec = (reinterpret_cast<uintptr_t>(f.dst) & 15) == 0;
     f.plain = f.first && f.n == 1 && f.any;
     f.fac = nullptr;
+    if (threadIdx.x == 0) fold_control(a, f);  // (every thread's reads came before the barrier above)
     if (f.n > 1 && f.n <= kFoldInst) {  // the same factors for every output
         if ((int)threadIdx.x < f.n)
             sfac[threadIdx.x] =
@@ -302,36 +325,6 @@ __device__ __forceinline__ void fold_store(const FoldState& f, int64_t o, double
         }
     } else {
         f.dst[o] = v.x;
-    }
-}
-
-// After the data: the accumulator's exponent, after the call's last group
-// the result's, and the slice counter.  Run by the last block to get here, so
-// that no launch of its own is needed for them.  The fences order each block's
-// reads of the control block before its ticket, and the last ticket before the
-// writes.
-__device__ __forceinline__ void fold_finish(const AccumArgs& a, const FoldState& f) {
-    __shared__ unsigned ticket;
-    if (gridDim.x > 1) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            ticket = atomicInc(&a.ctl->ticket, gridDim.x - 1);  // wraps to 0 at the last block
-            __threadfence();
-        }
-        __syncthreads();
-        if (ticket != gridDim.x - 1) return;
-    } else {
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        a.ctl->acc_exp[f.par ^ 1] = f.newE;
-        if (f.last) {
-            const int64_t e = f.newE == INT64_MIN ? 0 : f.newE;
-            a.ctl->final_exp = e;
-            if (a.direct) *a.ctl->out_exp = e;
-        }
-        a.ctl->slice = f.slice + a.advance;
     }
 }
 
@@ -429,7 +422,6 @@ __global__ void __launch_bounds__(256, 3) k_accumulate(const __grid_constant__ A
                 if (o0 + r * stride < a.n_out) fold_store<CPLX>(f, o0 + r * stride, v[r]);
         }
     }
-    fold_finish(a, f);
 }
 
 // Outputs in another order than the root's (power-of-two sizes): tiles of up
@@ -561,7 +553,6 @@ __global__ void __launch_bounds__(256, 5) k_accumulate_perm(const __grid_constan
             }
         }
     }
-    fold_finish(a, f);
 }
 
 // Tile plan of the permuted fold; false where the plain fold serves as well:
