@@ -419,8 +419,8 @@ struct FoldPlan {
     int64_t rest_src[kMaxBits], rest_dst[kMaxBits];
 };
 
-// Floats of a leaf that one block of a leaf-maximum launch covers.
-constexpr int64_t kLeafPart = 16384;
+// Floats of a large leaf that one block of a leaf-maximum launch covers.
+constexpr int64_t kLeafPart = 8192;
 
 // Reverse sweep: add a leaf's adjoint (times 2^exp) into its gradient
 // accumulator at the slice offset; labels absent from the adjoint

@@ -697,14 +697,16 @@ cudaError_t launch_leaf_table(const void* const* ptrs, int n, const void** table
 }
 
 // Largest |component| of every leaf, so that leaves are renormalised like
-// intermediates before their first contraction.  A leaf is cut into parts of
-// kLeafPart floats (at most 1024), one block each, combined by atomicMax on the
-// float bits (non-negative floats order like unsigned), or stored directly when
-// one block covers the leaf and `direct` allows it (no zeroing needed then).
+// intermediates before their first contraction.  A leaf of more than two parts'
+// floats is cut into parts of kLeafPart (at most 1024), one block each (2^23 and
+// 2^22 complex entries: 29 us with parts of 2^14 floats, 22 with 2^13), combined
+// by atomicMax on the float bits (non-negative floats order like unsigned), or
+// stored directly when one block covers the leaf and `direct` allows it (no
+// zeroing needed then).
 // Blocks [0, n0) are part 0 of every leaf, the others the further parts of the
 // large leaves listed in `big`, so that many small leaves beside a large one
 // add no empty blocks (300 leaves and one of 2^26 floats: 228 us with as many
-// blocks for every leaf, 51 now; 2000 and one of 2^20: 91 and 7).
+// blocks for every leaf, 40 now; 2000 and one of 2^20: 91 and 5).
 // Large leaves are read 16 bytes a load, four loads in flight per thread
 // (bound by memory); a leaf that is not 16-byte aligned, and the ends, by
 // single floats.
@@ -716,8 +718,9 @@ struct BigLeaves {
 };
 
 __host__ __device__ inline int leaf_parts(int64_t nfloat) {
+    if (nfloat <= 2 * kLeafPart) return 1;  // (several would need their slot cleared by a launch of its own)
     const int64_t parts = (nfloat + kLeafPart - 1) / kLeafPart;
-    return (int)(parts < 1 ? 1 : (parts > 1024 ? 1024 : parts));
+    return (int)(parts > 1024 ? 1024 : parts);
 }
 
 __device__ __forceinline__ void leaf_max_part(const float* const* ptrs, const int64_t* nfloat, unsigned* out, int n0,
