@@ -262,12 +262,11 @@ bool plan_tile(const NetDesc& d, const Plan& p, Node& nd, int64_t& split_elems, 
         if (t.nbatch > 65535) return false;
         const int64_t outs = M * N * t.nbatch;
         int split = 1;
-        // a K tile (2^11 entries of both operands) or more per part, four with
-        // several outputs, whose sums each part reduces; at least eight parts
-        // per SM in all (several CTAs per SM keep enough loads in flight for
-        // HBM).  2 x 32 outputs over K = 2^11: 34 us with parts of 1024 K
-        // entries (two CTAs), 10 with parts of a few tiles; 4 x 4 over 2^18 in
-        // eight slices: 161 us with parts of one tile, 89 with four.
+        // a K tile (2^11 entries of both operands) or more per part, four where a
+        // part reduces several outputs; at least eight parts (times outputs, with
+        // a CTA each) per SM in all: several CTAs per SM keep enough loads in
+        // flight for HBM.  4 x 4 outputs over 2^18 in eight slices: 161 us with
+        // parts of one tile, 89 with four.
         const int64_t tiles = t.dot_each ? K >> dot_tile_bits(0, 0, t.nk) : (K >> dot_tile_bits(t.nm, t.nn, t.nk)) / 4;
         while ((t.dot_each ? outs : t.nbatch) * p.copies * split < 8 * (int64_t)sm_count() && split * 2 <= tiles && split < 4096 &&
                (int64_t)split * 2 * p.copies <= 65535)
@@ -435,9 +434,9 @@ static tn_status fill_generic(const NetDesc& d, const Plan& p, const Node& nd, G
 
 // ---- subtree regions (tn_region.cu)
 
-// Small enough for a region: at most 2^14 multiply-adds (64 per thread, about a
-// microsecond; waves spread larger ones over the GPU) and 2^10 outputs,
-// operands that can be staged.  Sizes of other kinds: the nodes that would take a
+// Small enough for a region: at most 2^14 multiply-adds (64 per thread of a
+// 256-thread block, 32 of a 512-thread one: about a microsecond; waves spread
+// larger ones over the GPU) and 2^10 outputs, operands that can be staged.  Sizes of other kinds: the nodes that would take a
 // launch of one thread per output each.
 static bool region_node(const RegionView& v, const Node& nd) {
     const NetDesc& d = *v.d;

@@ -1,10 +1,11 @@
-// tn_tiled.cu -- tiled node kernels for power-of-two label sizes (FP32 on
-// CUDA cores).
+// tn_tiled.cu -- tiled node kernels (FP32 on CUDA cores): the tile kernel for
+// label sizes of any kind, the inner-product and wave kernels for powers of two.
 //
 // A tree node contracts A and B over the shared labels (Sec. 2 of arXiv
 // 2002.01935).  With every label size a power of two, each group of labels
 // (batch, M, N, K) is a set of index bits and an operand offset is a
-// scatter of those bits to the operand's strides.  The node output is laid
+// scatter of those bits to the operand's strides (other sizes: of mixed-radix
+// digits).  The node output is laid
 // out [batch][M][N], i.e. a row-major M x N matrix per batch index, so a
 // node is a batched GEMM whose operands are read through bit scatters:
 //   C[b, m, n] = sum_k A[sA(b) + sA(m) + sA(k)] * B[sB(b) + sB(k) + sB(n)].
@@ -197,11 +198,13 @@ __device__ __forceinline__ typename VT<CPLX>::T ld_cg(const typename VT<CPLX>::T
 
 // --------------------------------------------------------------------------
 // Register-blocked tile: TM x TN outputs of one batch index and one K split;
-// TK-deep steps through shared memory.  This body serves the tile items of
-// the persistent dataflow launch (CG: operands read through L2 only -- they
-// may have been written earlier in the same launch by other CTAs); the tile
-// kernel below is the same computation.  A and B are the instance's operand
-// bases; the epilogue writes C (or the K part's partial) and the maximum.
+// TK-deep steps through one shared-memory stage, 64-bit operand offsets.  This
+// body serves the tile items of the persistent dataflow launch (CG: operands
+// read through L2 only -- they may have been written earlier in the same launch
+// by other CTAs) and k_tile_wide; the tile kernel below computes the same with
+// two stages, more outputs per thread and 32-bit offsets.  A and B are the
+// instance's operand bases; the epilogue writes C (or the K part's partial) and
+// the maximum.
 // --------------------------------------------------------------------------
 template <bool CPLX, int TM, int TN, int TK, int RM, int RN, bool CG>
 __device__ __forceinline__ void tile_body(const TileArgs& a, int64_t tile_x, int split_id, int64_t b,
@@ -363,8 +366,10 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, int64_t tile_x, int
     }
 }
 
-// Operands spread over 2^31 entries (a slice of a larger leaf): the body above,
-// whose operand offsets are 64-bit.
+// Operands spread over 2^31 entries (a slice of a larger leaf, so at least 8 GB
+// of it): the body above, whose operand offsets are 64-bit.  Bound like k_tile by
+// the FP32 pipes and shared-memory loads, at about half its rate (2^11 x 2^11 x
+// 2^10, real: 523 us, 294 in k_tile): one stage and 4 x 4 outputs per thread.
 template <bool CPLX, int TM, int TN, int TK>
 __global__ void __launch_bounds__((TM / 4) * (TN / 4)) k_tile_wide(const __grid_constant__ TileArgs a) {
     using T = typename VT<CPLX>::T;
@@ -762,7 +767,8 @@ __global__ void __launch_bounds__(256) k_split_reduce(const __grid_constant__ AR
     if (a.t_done && threadIdx.x == 0) atomicMax(a.t_done, global_ns());
 }
 
-// Inner-product node (2 to 64 outputs, long K): out[b,m,n] = sum_k A[.., k] B[.., k].
+// Inner-product node (2 to 64 outputs, long K, more than two tiles of 1024
+// products per SM: dot_each_output in tn_plan.cpp): out[b,m,n] = sum_k A[.., k] B[.., k].
 // One CTA computes all outputs of a batch entry over its part of K, so that
 // either operand is read once.  K is cut into tiles of 2^t entries that hold
 // the lowest strides of A and of B; a tile of an operand -- its rows times the
@@ -957,8 +963,8 @@ __global__ void __launch_bounds__(256, dot_resident(CPLX, RM * RN))
 // One output per CTA: every thread multiplies its own four entries of a tile.
 // blockIdx.x: batch entry and output, y: K part, z: instance.  For one-output
 // nodes, several where the planner's rule says so, and (WIDE: 64-bit offsets)
-// operands spread over 2^31 entries.
-// Bound by memory: one output over K = 2^28
+// operands spread over 2^31 entries (8 x 4 outputs over K = 2^18, real: 52 us, 30
+// in k_dot).  Bound by memory: one output over K = 2^28
 // (4.3 GB) 726 us, 5.9 TB/s; as an instance of k_dot, whose loop over rows and
 // parts costs registers and instructions per copy, 820 to 1105.
 template <bool CPLX, bool WIDE>

@@ -53,3 +53,19 @@ def test_tiles_that_would_run_empty(m, n, k, b, tiled, cplx):
     or the sums long, one thread per output elsewhere."""
     s = step([3] * m, [3] * n, [3] * k, [3] * b, cplx)
     assert s["kind"] == 0 and (s["cfg"] > 0) == tiled
+
+
+@pytest.mark.parametrize("seed", range(24))
+def test_small_networks_are_subtrees(seed):
+    """The networks of any label sizes that the GPU tests contract in regions
+    do have one: a step of several nodes that is no wave."""
+    from paper_2002_01935_gb300 import inputs, planner
+    net = inputs.random_network(5 + seed % 8, 7 + seed % 7, 400 + seed, n_open=seed % 3, max_dim=2 + seed % 4,
+                                complex_=seed % 2 == 0)
+    pairs = planner.greedy_tree(net.labels, net.dims, net.open)
+    h = binding.TensorNetwork(net.labels, net.dims, net.open, None, complex_=net.is_complex)
+    try:
+        steps = h.plan_steps(pairs, [], "fp32")
+    finally:
+        h.close()
+    assert any(not s["wave"] and len(s["nodes"]) > 1 and s["cfg"] == 0 and s["launches"] == 1 for s in steps)
